@@ -284,29 +284,47 @@ lbmk::StepParams<R> make_params(const lbm_handle* h, int from) {
         const double kappa = d.c_mref / (1.0 - om * d.c_mref);
         P.kappa_m = (R)kappa;
         for (int k = 0; k < 9; ++k) P.wk_move[k] = (R)((Q == 9 ? w9[k] : 0.25 * p.varpi) * kappa);
-        for (int k = 0; k < 9; ++k) {
-            P.wmv[k] = {P.w_move[k], P.wk_move[k]};
-            P.nwmv[k] = {-P.w_move[k], -P.wk_move[k]};
-        }
         P.om_cf = (R)(om * d.c_fref);
         P.rest_m = (R)(1.0 - om * d.c_mref);
     }
     const double phi = p.porosity;
-    P.phi = (R)phi;
     P.inv_phi = (R)(1.0 / phi);
     if (p.flow) {
-        P.drag_lin = (R)(phi * d.nu_f / d.K);
-        P.drag_forch = (R)(phi * d.F_phi / std::sqrt(d.K));
-        P.gbeta = (R)d.gbeta;
+        P.nlin = (R)(-phi * d.nu_f / d.K);
+        P.nforch = (R)(-phi * d.F_phi / std::sqrt(d.K));
+        P.fgb = (R)(phi * d.gbeta);
         P.T0 = (R)p.T_ref0;
         P.l0 = (R)d.l0;
         P.l0sq = (R)(d.l0 * d.l0);
         P.l1 = (R)d.l1;
+        P.nl1 = (R)-d.l1;
+        P.n2l0 = (R)(1.0 - 2.0 * d.l0);
+        // 1 - s from the rounded rate, so that m = m^eq is kept exactly by (1 - s) m + s m^eq
+        const R sv = (R)d.s[7];
+        P.c_v = (R)1 - sv;
+        P.k_v = (R)((double)sv / phi);
+        P.k_h = (R)((1.0 - 0.5 * (double)sv) / phi);
+        P.k_2h = (R)2 * P.k_h;
+        P.k_uu = (R)(3.0 * (double)(R)d.s[1] / phi);
+        P.k_uf = (R)(6.0 * (1.0 - 0.5 * d.s[1]) / phi);
     }
     for (int k = 0; k < 9; ++k) {
-        P.s[k] = (R)d.s[k];
-        P.eta[k] = (R)d.eta[k];
-        P.nrate[k] = {-(R)d.zeta[k], -(R)d.eta[k]};
+        P.nz[k] = -(R)d.zeta[k];
+        P.ne[k] = -(R)d.eta[k];
+    }
+    if (p.thermal_q == 5) {
+        const R za = (R)d.zeta[1], ze = (R)d.zeta[3], zp = (R)d.zeta[4];
+        const R ea = (R)d.eta[1], ee = (R)d.eta[3], ep = (R)d.eta[4];
+        P.z_j = (R)0.5 * ((R)1 - za);
+        P.z_ju = (R)(0.5 * (double)za / phi);
+        P.z_3 = (R)0.25 * ((R)1 - ze);
+        P.z_3T = (R)(0.25 * (double)ze * p.varpi * d.c_fref);
+        P.z_4 = (R)0.25 * ((R)1 - zp);
+        P.e_j = (R)0.5 * ((R)1 - ea);
+        P.e_3 = (R)0.25 * ((R)1 - ee);
+        P.e_3T = (R)(0.25 * (double)ee * p.varpi * d.c_mref);
+        P.e_4 = (R)0.25 * ((R)1 - ep);
+        P.quart_varpi = (R)(0.25 * p.varpi);
     }
     P.H_fs = (R)d.H_fs;
     P.H_fl = (R)d.H_fl;
@@ -323,8 +341,8 @@ lbmk::StepParams<R> make_params(const lbm_handle* h, int from) {
     // Eq. 9 variant: per-node zeta_alpha = 1/(1/2 + k_f(f_l)/(rho_l c_fref c_sT^2)) (Eq. A19);
     // rate k of the PCM lattice is zr_a[k] + zr_b[k] zeta_alpha (fixed, zeta_alpha, or 2 - zeta_alpha)
     P.phase_k = phase_k_of(h);
-    P.kl_c = (R)(p.k_f / (d.c_fref * d.csT2));
     P.ks_c = (R)(d.k_s / (d.c_fref * d.csT2));
+    P.kd_c = (R)((p.k_f - d.k_s) / (d.c_fref * d.csT2));
     {
         const int Q = p.thermal_q, e_role = p.zeta_e > 0.0 ? 0 : 2;
         int role[9] = {0, 1, 1, e_role, 0, 0, 0, 0, 0};
@@ -339,8 +357,10 @@ lbmk::StepParams<R> make_params(const lbm_handle* h, int from) {
             P.zr_b[k] = role[k] == 0 ? (R)0.0 : (role[k] == 1 ? (R)1.0 : (R)-1.0);
         }
     }
-    P.a_m = (R)(d.h_v / ((1.0 - phi) * d.rho_m));
-    P.x_pm = (R)(-(1.0 - phi) * d.rho_m / (phi * 1.0));
+    const double a_m = d.h_v / ((1.0 - phi) * d.rho_m);
+    P.x_now = (R)(-1.5 * a_m);
+    P.x_prev = (R)(0.5 * a_m);
+    P.x_pm = d.h_v == 0.0 ? (R)0 : (R)(-(1.0 - phi) * d.rho_m / (phi * 1.0));   // no exchange: the PCM takes nothing
     return P;
 }
 

@@ -30,15 +30,20 @@
 //     streaming and collision conserve the enthalpy to ~2^-46 instead of
 //     accumulating FP32 rounding in the isothermal mushy zone, where nothing
 //     damps it;
-//   * every other rest population is a remainder as well, and the PCM's
-//     exchange source is the opposite of the change the metal's n_0 actually
-//     took (scaled by the heat capacities), so the exchange moves no energy
-//     that the metal's rounding dropped;
+//   * every other rest population is a remainder as well (the FP32 metal's
+//     takes what its movers give up, without passing through their sum), and the
+//     PCM's exchange source is the opposite of the change the metal's n_0
+//     actually took (scaled by the heat capacities), so the exchange moves no
+//     energy that the metal's rounding dropped;
 //   * the state is chunked: [chunk][plane][kChunk] with chunks of kChunk nodes
 //     along x, so one pointer per pulled neighbour reaches all its planes;
-//   * FP32 arithmetic goes through the packed two-lane instructions of sm_100
-//     and later wherever two values take the same operations (the PCM and
-//     metal lattices, pairs of flow moments, or the two nodes of a pair).
+//   * the arithmetic is written once over a lane type (one node, or a pair of
+//     nodes in the packed two-lane FP32 instructions of sm_100 and later), with
+//     every rounding named, so that all kernels give a node the same bits;
+//   * what is conserved or nearly so is never passed through a constant or a
+//     quotient whose rounding would be the same at every node and step: FP32
+//     velocities after 200 steps of the 256^2 cavity are within 7e-7 of exact
+//     arithmetic (up to 1.8e-5 when they were).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -120,51 +125,101 @@ struct Chunk {
     static constexpr int bytes = wide_off + PL::wide * kChunk * (int)sizeof(float);
 };
 
-// A pair of values that go through the same arithmetic: the PCM and metal
-// lattices' populations and moments (x: PCM, y: metal).  With FP32 arithmetic
-// a pair operation is one packed instruction (the .f32x2 add, multiply and
-// fused multiply-add of sm_100 and later), which halves the issue slots of
-// that arithmetic; FP64 keeps two scalar operations.  Each lane is rounded as
-// the scalar operation would be.
+// ---------------------------------------------------------------------------
+// Lanes
+// ---------------------------------------------------------------------------
+// The node update is written once, over a lane type T: float or double (one
+// node per thread), or W, two neighbouring nodes of a row per thread.  A W
+// operation is one packed instruction for both nodes (the .f32x2 add, multiply
+// and fused multiply-add of sm_100 and later), which halves the issue slots of
+// the arithmetic; scalar constants broadcast, negations and lane swaps cost
+// nothing in packed operands.  Every operation names its rounding, so no
+// multiply and add are contracted by the compiler, and a node's result is the
+// same bit for bit in every kernel and lane type.
 template <typename R>
 struct alignas(2 * sizeof(R)) V2 {
     R x, y;
 };
+using W = V2<float>;
 
-template <typename R>
-__device__ __forceinline__ V2<R> add2(V2<R> a, V2<R> b) {
-    if constexpr (sizeof(R) == 4) {
-        const float2 r = __fadd2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y));
-        return {r.x, r.y};
-    } else {
-        return {a.x + b.x, a.y + b.y};
-    }
+struct Mask2 {
+    bool x, y;
+};
+
+template <typename T> struct Lane { using R = T; using Mask = bool; static constexpr int n = 1; };
+template <> struct Lane<W> { using R = float; using Mask = Mask2; static constexpr int n = 2; };
+
+template <typename T> __device__ __forceinline__ T bc(typename Lane<T>::R v) {   // broadcast
+    if constexpr (Lane<T>::n == 2) return {v, v};
+    else return v;
 }
 
-template <typename R>
-__device__ __forceinline__ V2<R> mul2(V2<R> a, V2<R> b) {
-    if constexpr (sizeof(R) == 4) {
-        const float2 r = __fmul2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y));
-        return {r.x, r.y};
-    } else {
-        return {a.x * b.x, a.y * b.y};
-    }
+__device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float vsub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double vadd(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double vsub(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ double vmul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double vfma(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float2 f2(W a) { return make_float2(a.x, a.y); }
+__device__ __forceinline__ W vadd(W a, W b) {
+    const float2 r = __fadd2_rn(f2(a), f2(b));
+    return {r.x, r.y};
 }
+__device__ __forceinline__ W vsub(W a, W b) { return vadd(a, W{-b.x, -b.y}); }
+__device__ __forceinline__ W vfma(W a, W b, W c) {
+    const float2 r = __ffma2_rn(f2(a), f2(b), f2(c));
+    return {r.x, r.y};
+}
+__device__ __forceinline__ W vmul(W a, W b) {
+    const float2 r = __fmul2_rn(f2(a), f2(b));
+    return {r.x, r.y};
+}
+// A product that goes into an error-free sum: ptxas 13.0 fuses a packed
+// multiply with the addition of its product although both name their rounding
+// (-fmad=false does not stop it), and the error taken would be another
+// number's.  One scalar multiply per lane is left alone.
+__device__ __forceinline__ float vmul_alone(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ W vmul_alone(W a, W b) { return {__fmul_rn(a.x, b.x), __fmul_rn(a.y, b.y)}; }
+__device__ __forceinline__ float vneg(float a) { return -a; }
+__device__ __forceinline__ double vneg(double a) { return -a; }
+__device__ __forceinline__ W vneg(W a) { return {-a.x, -a.y}; }
 
-template <typename R>
-__device__ __forceinline__ V2<R> fma2(V2<R> a, V2<R> b, V2<R> c) {   // a b + c, one rounding per lane
-    if constexpr (sizeof(R) == 4) {
-        const float2 r = __ffma2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y), make_float2(c.x, c.y));
-        return {r.x, r.y};
-    } else {
-        return {fma(a.x, b.x, c.x), fma(a.y, b.y, c.y)};
-    }
-}
+// with a constant factor or term
+template <typename T> __device__ __forceinline__ T vmulc(typename Lane<T>::R c, T a) { return vmul(bc<T>(c), a); }
+template <typename T> __device__ __forceinline__ T vfmac(typename Lane<T>::R c, T a, T b) { return vfma(bc<T>(c), a, b); }
+template <typename T> __device__ __forceinline__ T vaddc(T a, typename Lane<T>::R c) { return vadd(a, bc<T>(c)); }
 
-template <typename R>
-__device__ __forceinline__ V2<R> sub2(V2<R> a, V2<R> b) {   // a - b, one rounding per lane
-    return fma2(b, V2<R>{R(-1), R(-1)}, a);
+template <typename R> __device__ __forceinline__ R vsel(bool m, R a, R b) { return m ? a : b; }
+__device__ __forceinline__ W vsel(Mask2 m, W a, W b) { return {m.x ? a.x : b.x, m.y ? a.y : b.y}; }
+
+// sat(a c), min(a, c), max(a, 0)
+__device__ __forceinline__ float vsatmul(float a, float c) { return __saturatef(__fmul_rn(a, c)); }
+__device__ __forceinline__ W vsatmul(W a, float c) { return {vsatmul(a.x, c), vsatmul(a.y, c)}; }
+__device__ __forceinline__ float vminc(float a, float c) { return fminf(a, c); }
+__device__ __forceinline__ W vminc(W a, float c) { return {fminf(a.x, c), fminf(a.y, c)}; }
+__device__ __forceinline__ float vmax0(float a) { return fmaxf(a, 0.0f); }
+__device__ __forceinline__ W vmax0(W a) { return {fmaxf(a.x, 0.0f), fmaxf(a.y, 0.0f)}; }
+
+// 1/a and sqrt(a), a >= 0, in FP32: one instruction each, relative error at
+// most 1 ulp and 2^-23 (the division and the rsqrtf product they replace took
+// 5 and 8 instructions, with 2 ulp and 2^-22.4; subnormal speeds, below
+// 1e-19 lattice units, flush to zero)
+__device__ __forceinline__ float vrcp(float a) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+    return r;
 }
+__device__ __forceinline__ float vsqrt(float a) {
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+    return r;
+}
+__device__ __forceinline__ W vrcp(W a) { return {vrcp(a.x), vrcp(a.y)}; }
+__device__ __forceinline__ W vsqrt(W a) { return {vsqrt(a.x), vsqrt(a.y)}; }
+__device__ __forceinline__ double vrcp(double a) { return 1.0 / a; }
+__device__ __forceinline__ double vsqrt(double a) { return sqrt(a); }
 
 // Per-run constants, passed by value (__grid_constant__).
 template <typename R>
@@ -184,299 +239,197 @@ struct StepParams {
     R fscale, finv;      // flow deviations are stored times fscale (a power of two)
     // 16-bit modes: references of the moving thermal populations
     R w_move[9];         // w'_i: the equilibrium weight of mover i (D2Q9 w_i, D2Q5 varpi/4)
+    R wk_move[9];        // w'_i kappa_m: metal mover reference per unit of h_0
     R g0_fs, g0_fl;      // PCM rest population at solidus / liquidus equilibrium
     R cr_solid, cr_liquid;   // c_f,ref dT/dg_0 on the solid and liquid branches
     R cr_fs, cr_dsl;     // c_f,ref T_fs, c_f,ref (T_fl - T_fs)
     R inv_dg0;           // 1 / (g0_fl - g0_fs)
-    R wk_move[9];        // w'_i kappa_m: metal mover reference per unit of h_0
     R kappa_m;           // c_m,ref / (c_pm - omega c_m,ref): mover reference per unit of h_0 / w'_i
     R om_cf;             // omega c_f,ref (omega = sum of the w'_i): g_0 = H - om_cf T(H) at equilibrium
     R rest_m;            // 1 - omega c_m,ref / c_pm: h_0 = rest_m c_pm T_m at equilibrium
     // flow (Eqs. 3, 7, 16, 25)
-    R phi, inv_phi, drag_lin, drag_forch, gbeta, T0, l0, l0sq, l1;
-    R s[9];
+    R inv_phi, fgb, T0, l0, l0sq, l1;   // fgb = phi gbeta
+    R nl1, n2l0;         // -l_1, 1 - 2 l_0
+    R nlin, nforch;      // -phi nu_f / K and -phi F_phi / sqrt(K): the negated drag is nlin + nforch |u|
+    R k_uu, k_uf;        // 3 s_e / phi and 6 (1 - s_e / 2) / phi
+    R c_v, k_v, k_h, k_2h;   // 1 - s_v, s_v / phi, (1 - s_v / 2) / phi and twice that
     // thermal (Eqs. 38-39, 34, 45, App. B)
     // (c_pl = c_pm = 1 in the lattice units of Eq. 54, so they appear nowhere below)
     R H_fs, H_fl, inv_dH, T_fs, T_fl, dT_sl, inv_c_ps;   // dT_sl = T_fl - T_fs
     R c_fref, c_mref, varpi;
     R vcf, vcm;          // varpi c_f,ref and varpi c_m,ref (D2Q5 equilibria, Eqs. B2, B4)
-    R eta[9];            // metal rates (eta[0] for the FP32 rest population's relaxation)
-    V2<R> nrate[9];      // (-zeta_k, -eta_k): PCM and metal relaxation rates, negated
-    V2<R> nwmv[9];       // (-w'_k, -w'_k kappa_m): 16-bit mover references per unit of (ref, h_0)
-    V2<R> wmv[9];        // (w'_k, w'_k kappa_m)
-    R a_m;               // h_v/((1 - phi) rho_m), Eq. 47
+    R nz[9], ne[9];      // -zeta_k, -eta_k (D2Q9)
+    // D2Q5 relaxation, with the factors 1/2 (j) and 1/4 (n_3, n_4) of M^-1 folded in
+    R z_j, z_ju, z_3, z_3T, z_4;   // (1 - z_a)/2, z_a/(2 phi), (1 - z_e)/4, z_e varpi c_f,ref / 4, (1 - z_eps)/4
+    R e_j, e_3, e_3T, e_4;         // the metal's
+    R quart_varpi;       // varpi / 4
+    R x_now, x_prev;     // -1.5 a_m, 0.5 a_m with a_m = h_v/((1 - phi) rho_m): Eq. 47 and Remark III
     R x_pm;              // -a_f/a_m = -(1 - phi) rho_m/(phi rho_l): PCM source per unit of metal source
     // Eq. 9 variant: PCM rates from the node's liquid fraction
     int phase_k;         // 1: k_s != k_l, rates per node
-    R kl_c, ks_c;        // k_l, k_s over (rho_l c_fref c_sT^2)
+    R ks_c, kd_c;        // k_s and k_l - k_s over (rho_l c_fref c_sT^2)
     R zr_a[9], zr_b[9];  // PCM rate k = zr_a[k] + zr_b[k] zeta_alpha
 };
 
 enum : unsigned int { STATUS_UNSTABLE = 1u };
 
-// Error-free transformations (IEEE round-to-nearest, no contraction).
+// ---------------------------------------------------------------------------
+// Error-free sums
+// ---------------------------------------------------------------------------
+// The rounding error of s = fl(a + b) (Knuth's TwoSum, the sum already taken).
+template <typename T>
+__device__ __forceinline__ T sum_err(T a, T b, T s) {
+    const T bb = vsub(s, a);
+    return vadd(vsub(a, vsub(s, bb)), vsub(b, bb));
+}
+
+template <typename T>
 struct FF {
-    float hi, lo;
+    T hi, lo;
 };
 
-__device__ __forceinline__ FF two_sum(float a, float b) {        // Knuth
-    const float s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-    return {s, e};
+template <typename T>
+__device__ __forceinline__ FF<T> fast_two_sum(T a, T b) {   // Dekker, |a| >= |b|
+    const T s = vadd(a, b);
+    return {s, vsub(b, vsub(s, a))};
 }
 
-__device__ __forceinline__ FF fast_two_sum(float a, float b) {   // Dekker, |a| >= |b|
-    const float s = __fadd_rn(a, b);
-    return {s, __fsub_rn(b, __fsub_rn(s, a))};
+// v[1] + ... + v[Q-1] by pairs, opposite directions first (the sums that the
+// moments need too).
+template <int Q, typename T>
+__device__ __forceinline__ T mover_sum(const T* v) {
+    const T s = vadd(vadd(v[1], v[3]), vadd(v[2], v[4]));
+    if constexpr (Q == 5) return s;
+    else return vadd(s, vadd(vadd(v[5], v[7]), vadd(v[6], v[8])));
 }
 
-__device__ __forceinline__ FF ff_add(FF a, float b) {
-    const FF s = two_sum(a.hi, b);
-    return fast_two_sum(s.hi, __fadd_rn(s.lo, a.lo));
-}
-
-
-// a.hi + a.lo + sign * (v[1] + ... + v[Q-1]) as a float-float pair: each term
-// enters through TwoSum, the rounding errors gather in one float, and the pair
-// is normalised once at the end (a compensated sum; its error is of the order
-// of (Q - 1) u^2 |sum|, u = 2^-24).
-template <int Q>
-__device__ __forceinline__ FF ff_accumulate(FF a, const float* v, float sign) {
-    float s = a.hi, c = a.lo;
-#pragma unroll
-    for (int i = 1; i < Q; ++i) {
-        const FF t = two_sum(s, sign * v[i]);
-        s = t.hi;
-        c = __fadd_rn(c, t.lo);
+// The same, and the sum of the rounding errors made on the way.
+template <int Q, typename T>
+__device__ __forceinline__ FF<T> mover_sum_ff(const T* v) {
+    const T a = vadd(v[1], v[3]), b = vadd(v[2], v[4]), s = vadd(a, b);
+    T e = vadd(vadd(sum_err(v[1], v[3], a), sum_err(v[2], v[4], b)), sum_err(a, b, s));
+    if constexpr (Q == 5) {
+        return {s, e};
+    } else {
+        const T c = vadd(v[5], v[7]), d = vadd(v[6], v[8]), r = vadd(c, d), t = vadd(s, r);
+        e = vadd(e, vadd(vadd(sum_err(v[5], v[7], c), sum_err(v[6], v[8], d)), sum_err(c, d, r)));
+        return {t, vadd(e, sum_err(s, r, t))};
     }
-    return fast_two_sum(s, c);
 }
 
 // ---------------------------------------------------------------------------
 // Transforms
 // ---------------------------------------------------------------------------
 
-template <typename R>
-__device__ __forceinline__ void m_from_f9(const R* f, R* m) {
-    const R s14 = f[1] + f[2] + f[3] + f[4];
-    const R s58 = f[5] + f[6] + f[7] + f[8];
-    const R dx = f[1] - f[3], dy = f[2] - f[4];
-    const R ax = f[5] - f[6] - f[7] + f[8];
-    const R ay = f[5] + f[6] - f[7] - f[8];
-    m[0] = f[0] + s14 + s58;
-    m[1] = R(-4) * f[0] - s14 + R(2) * s58;
-    m[2] = R(4) * f[0] - R(2) * s14 + s58;
-    m[3] = dx + ax;
-    m[4] = R(-2) * dx + ax;
-    m[5] = dy + ay;
-    m[6] = R(-2) * dy + ay;
-    m[7] = f[1] - f[2] + f[3] - f[4];
-    m[8] = f[5] - f[6] + f[7] - f[8];
+// Eq. 13: m = M f (rho, e, eps, j_x, q_x, j_y, q_y, p_xx, p_xy).
+template <typename T>
+__device__ __forceinline__ void m_from_f9(const T* f, T* m) {
+    const T a = vadd(f[1], f[3]), b = vadd(f[2], f[4]), c = vadd(f[5], f[7]), d = vadd(f[6], f[8]);
+    const T dx = vsub(f[1], f[3]), dy = vsub(f[2], f[4]), ec = vsub(f[5], f[7]), ed = vsub(f[6], f[8]);
+    const T s14 = vadd(a, b), s58 = vadd(c, d);
+    const T ax = vsub(ec, ed), ay = vadd(ec, ed);
+    m[0] = vadd(f[0], vadd(s14, s58));
+    m[1] = vfmac<T>(-4, f[0], vfmac<T>(2, s58, vneg(s14)));
+    m[2] = vfmac<T>(-2, s14, vfmac<T>(4, f[0], s58));
+    m[3] = vadd(dx, ax);
+    m[4] = vfmac<T>(-2, dx, ax);
+    m[5] = vadd(dy, ay);
+    m[6] = vfmac<T>(-2, dy, ay);
+    m[7] = vsub(a, b);
+    m[8] = vsub(c, d);
 }
 
 // f = M^-1 m, every f scaled by SC (a power of two: the 16-bit flow storage
-// scale, folded into the row norms).
-template <typename R, int SC = 1>
-__device__ __forceinline__ void f_from_m9(const R* m, R* f) {
+// scale, folded into the row norms).  The conserved moments come back without
+// the rounding of 1/9 and 1/6 (which would grow the momentum by 3e-8 a step in
+// FP32): f_0 and the axis populations' odd part are the remainders to m_0 and
+// to m_3 / 2, m_5 / 2.
+template <typename T, int SC = 1>
+__device__ __forceinline__ void f_from_m9(const T* m, T* f) {
+    using R = typename Lane<T>::R;
     constexpr double s = SC;
-    const R A = m[0] * R(s / 9.0), B = m[1] * R(s / 36.0), C = m[2] * R(s / 36.0);
-    const R DX = m[3] * R(s / 6.0), QX = m[4] * R(s / 12.0);
-    const R DY = m[5] * R(s / 6.0), QY = m[6] * R(s / 12.0);
-    const R P = m[7] * R(s * 0.25), S = m[8] * R(s * 0.25);
-    f[0] = A - R(4) * B + R(4) * C;
-    const R b1 = A - B - R(2) * C;
-    f[1] = b1 + DX - R(2) * QX + P;
-    f[3] = b1 - DX + R(2) * QX + P;
-    f[2] = b1 + DY - R(2) * QY - P;
-    f[4] = b1 - DY + R(2) * QY - P;
-    const R b5 = A + R(2) * B + C;
-    const R X = DX + QX, Y = DY + QY;
-    f[5] = b5 + X + Y + S;
-    f[6] = b5 - X + Y - S;
-    f[7] = b5 - X - Y + S;
-    f[8] = b5 + X - Y - S;
+    const T A = vmulc<T>(R(s / 9.0), m[0]);
+    const T b1 = vfmac<T>(R(-s / 18.0), m[2], vfmac<T>(R(-s / 36.0), m[1], A));
+    const T b5 = vfmac<T>(R(s / 36.0), m[2], vfmac<T>(R(s / 18.0), m[1], A));
+    const T b15 = vadd(b1, b5);
+    f[0] = SC == 1 ? vfmac<T>(R(-4), b15, m[0]) : vfmac<T>(R(s), m[0], vmulc<T>(R(-4), b15));
+    const T X = vfmac<T>(R(s / 12.0), m[4], vmulc<T>(R(s / 6.0), m[3]));
+    const T Y = vfmac<T>(R(s / 12.0), m[6], vmulc<T>(R(s / 6.0), m[5]));
+    const T tx = vfmac<T>(R(-2), X, vmulc<T>(R(s * 0.5), m[3]));
+    const T ty = vfmac<T>(R(-2), Y, vmulc<T>(R(s * 0.5), m[5]));
+    const T bp = vfmac<T>(R(s * 0.25), m[7], b1), bm = vfmac<T>(R(-s * 0.25), m[7], b1);
+    f[1] = vadd(bp, tx);
+    f[3] = vsub(bp, tx);
+    f[2] = vadd(bm, ty);
+    f[4] = vsub(bm, ty);
+    const T gp = vfmac<T>(R(s * 0.25), m[8], b5), gm = vfmac<T>(R(-s * 0.25), m[8], b5);
+    const T hp = vadd(X, Y), hm = vsub(Y, X);
+    f[5] = vadd(gp, hp);
+    f[7] = vsub(gp, hp);
+    f[6] = vadd(gm, hm);
+    f[8] = vsub(gm, hm);
 }
 
-// Eq. 13 on the population pairs (f1, f2), (f3, f4), (f5, f6), (f7, f8) (the
-// D2Q9 order of Eq. 11): m_0 and the moment pairs (e, eps), (j_x, j_y),
-// (q_x, q_y), (p_xx, p_xy).
-template <typename R>
-__device__ __forceinline__ void m_from_f9p(R f0, const V2<R>* F, R& m0, V2<R>* m) {
-    const V2<R> A = add2(F[0], F[1]);   // (f1 + f3, f2 + f4)
-    const V2<R> D = sub2(F[0], F[1]);   // (f1 - f3, f2 - f4)
-    const V2<R> B = add2(F[2], F[3]);   // (f5 + f7, f6 + f8)
-    const V2<R> E = sub2(F[2], F[3]);   // (f5 - f7, f6 - f8)
-    const R s14 = A.x + A.y, s58 = B.x + B.y;
-    const V2<R> a = {E.x - E.y, E.x + E.y};   // (f5 - f6 - f7 + f8, f5 + f6 - f7 - f8)
-    m0 = f0 + s14 + s58;
-    m[0] = {R(-4) * f0 - s14 + R(2) * s58, R(4) * f0 - R(2) * s14 + s58};
-    m[1] = add2(D, a);
-    m[2] = fma2(V2<R>{R(-2), R(-2)}, D, a);
-    m[3] = {A.x - A.y, B.x - B.y};
-}
-
-// f = M^-1 m on the same pairs, every f scaled by SC (as f_from_m9).
-template <typename R, int SC = 1>
-__device__ __forceinline__ void f_from_m9p(R m0, const V2<R>* m, R& f0, V2<R>* F) {
-    constexpr double s = SC;
-    const R A = m0 * R(s / 9.0);
-    const V2<R> BC = mul2(m[0], V2<R>{R(s / 36.0), R(s / 36.0)});   // (B, C)
-    const V2<R> D = mul2(m[1], V2<R>{R(s / 6.0), R(s / 6.0)});      // (DX, DY)
-    const V2<R> Q = mul2(m[2], V2<R>{R(s / 12.0), R(s / 12.0)});    // (QX, QY)
-    const V2<R> PS = mul2(m[3], V2<R>{R(s * 0.25), R(s * 0.25)});   // (P, S)
-    f0 = A - R(4) * BC.x + R(4) * BC.y;
-    const R b1 = A - BC.x - R(2) * BC.y;
-    const R b5 = A + R(2) * BC.x + BC.y;
-    const V2<R> T = fma2(V2<R>{R(-2), R(-2)}, Q, D);   // (DX - 2 QX, DY - 2 QY)
-    const V2<R> X = add2(D, Q);                         // (DX + QX, DY + QY)
-    const V2<R> bp = {b1 + PS.x, b1 - PS.x};
-    F[0] = add2(bp, T);                                 // (f1, f2)
-    F[1] = sub2(bp, T);                                 // (f3, f4)
-    const V2<R> G = {b5 + PS.y, b5 - PS.y}, H = {X.x + X.y, X.y - X.x};
-    F[2] = add2(G, H);                                  // (f5, f6)
-    F[3] = sub2(G, H);                                  // (f7, f8)
-}
-
-// Eq. B1 and its inverse on (PCM, metal) pairs: n = M g for D2Q5 with
-// n_0 = g_0 + ((g_1 + g_3) + (g_2 + g_4)), n_1 = g_1 - g_3, n_2 = g_2 - g_4,
+// Eq. B1: n_0 = sum g, n_1 = g_1 - g_3, n_2 = g_2 - g_4,
 // n_3 = g_1 + g_2 + g_3 + g_4, n_4 = g_1 - g_2 + g_3 - g_4.
-template <typename R>
-__device__ __forceinline__ void m_from_f5(const V2<R>* g, V2<R>* n) {
-    const V2<R> a = add2(g[1], g[3]), b = add2(g[2], g[4]);
-    n[1] = sub2(g[1], g[3]);
-    n[2] = sub2(g[2], g[4]);
-    n[3] = add2(a, b);
-    n[4] = sub2(a, b);
-    n[0] = add2(g[0], n[3]);
-}
-
-template <typename R>
-__device__ __forceinline__ void f_from_m5(const V2<R>* n, V2<R>* g) {
-    const V2<R> qu = {R(0.25), R(0.25)}, h = {R(0.5), R(0.5)}, mh = {R(-0.5), R(-0.5)};
-    const V2<R> p = mul2(add2(n[3], n[4]), qu), q = mul2(sub2(n[3], n[4]), qu);
-    g[0] = sub2(n[0], n[3]);
-    g[1] = fma2(h, n[1], p);
-    g[3] = fma2(mh, n[1], p);
-    g[2] = fma2(h, n[2], q);
-    g[4] = fma2(mh, n[2], q);
-}
-
-template <typename R, int Q>
-__device__ __forceinline__ void fwd2(const V2<R>* v, V2<R>* m) {
+template <typename T, int Q>
+__device__ __forceinline__ void thermal_moments(const T* g, T* n) {
     if constexpr (Q == 5) {
-        m_from_f5(v, m);
+        const T a = vadd(g[1], g[3]), b = vadd(g[2], g[4]);
+        n[1] = vsub(g[1], g[3]);
+        n[2] = vsub(g[2], g[4]);
+        n[3] = vadd(a, b);
+        n[4] = vsub(a, b);
+        n[0] = vadd(g[0], n[3]);
     } else {
-        R a[9], b[9], ma[9], mb[9];
-#pragma unroll
-        for (int k = 0; k < 9; ++k) { a[k] = v[k].x; b[k] = v[k].y; }
-        m_from_f9(a, ma);
-        m_from_f9(b, mb);
-#pragma unroll
-        for (int k = 0; k < 9; ++k) m[k] = {ma[k], mb[k]};
-    }
-}
-
-template <typename R, int Q>
-__device__ __forceinline__ void inv2(const V2<R>* m, V2<R>* v) {
-    if constexpr (Q == 5) {
-        f_from_m5(m, v);
-    } else {
-        R a[9], b[9], va[9], vb[9];
-#pragma unroll
-        for (int k = 0; k < 9; ++k) { a[k] = m[k].x; b[k] = m[k].y; }
-        f_from_m9(a, va);
-        f_from_m9(b, vb);
-#pragma unroll
-        for (int k = 0; k < 9; ++k) v[k] = {va[k], vb[k]};
+        m_from_f9(g, n);
     }
 }
 
 // ---------------------------------------------------------------------------
-// Equilibrium moments
+// Equations of state
 // ---------------------------------------------------------------------------
-
-// Eq. 34 (D2Q9) / Eq. B2 (D2Q5)
-template <typename R, int Q>
-__device__ __forceinline__ void neq_pcm(const StepParams<R>& P, R H, R T, R ux, R uy, R* ne) {
-    const R t = T * P.inv_phi;   // c_pl T / phi
-    const R jx = t * ux, jy = t * uy;
-    if constexpr (Q == 9) {
-        ne[0] = H;
-        ne[1] = R(-4) * H + R(2) * P.c_fref * T;
-        ne[2] = R(4) * H - R(3) * P.c_fref * T;
-        ne[3] = jx; ne[4] = -jx; ne[5] = jy; ne[6] = -jy;
-        ne[7] = R(0); ne[8] = R(0);
-    } else {
-        ne[0] = H; ne[1] = jx; ne[2] = jy; ne[3] = P.vcf * T; ne[4] = R(0);
-    }
-}
-
-// Eq. 45 (D2Q9) / Eq. B4 (D2Q5)
-template <typename R, int Q>
-__device__ __forceinline__ void neq_metal(const StepParams<R>& P, R Tm, R* ne) {
-    if constexpr (Q == 9) {
-        const R e = Tm;   // c_pm T_m
-        ne[0] = e;
-        ne[1] = R(-4) * e + R(2) * P.c_mref * Tm;
-        ne[2] = R(4) * e - R(3) * P.c_mref * Tm;
-#pragma unroll
-        for (int k = 3; k < 9; ++k) ne[k] = R(0);
-    } else {
-        ne[0] = Tm; ne[1] = R(0); ne[2] = R(0); ne[3] = P.vcm * Tm; ne[4] = R(0);   // ne[0] = c_pm T_m
-    }
-}
-
-template <typename R>
-__device__ __forceinline__ R sat01(R x) {
-    if constexpr (sizeof(R) == 4) return __saturatef(x);
-    else return fmin(fmax(x, R(0)), R(1));
-}
 
 // Eqs. 38-39 without branches: f_l = clamp((H - H_s)/(H_l - H_s), 0, 1) and
 // T = min(H/c_ps, T_s) + f_l (T_l - T_s) + max(H - H_l, 0)/c_pl, which is
 // H/c_ps below the solidus, T_s + f_l (T_l - T_s) in the mushy zone and
 // T_l + (H - H_l)/c_pl above the liquidus (c_pl = 1).
-template <typename R>
-__device__ __forceinline__ void enthalpy_state(const StepParams<R>& P, R H, R& T, R& fl) {
-    fl = sat01((H - P.H_fs) * P.inv_dH);
-    T = fmin(H * P.inv_c_ps, P.T_fs) + fl * P.dT_sl + fmax(H - P.H_fl, R(0));
+template <typename T>
+__device__ __forceinline__ void enthalpy_state(const StepParams<float>& P, T H, T& Tf, T& fl) {
+    fl = vsatmul(vaddc(H, -P.H_fs), P.inv_dH);
+    Tf = vadd(vfmac<T>(P.dT_sl, fl, vminc(vmulc<T>(P.inv_c_ps, H), P.T_fs)), vmax0(vaddc(H, -P.H_fl)));
+}
+
+__device__ __forceinline__ void enthalpy_state(const StepParams<double>& P, double H, double& Tf, double& fl) {
+    fl = fmin(fmax((H - P.H_fs) * P.inv_dH, 0.0), 1.0);
+    Tf = fmin(H * P.inv_c_ps, P.T_fs) + fl * P.dT_sl + fmax(H - P.H_fl, 0.0);
 }
 
 // c_f,ref T at equilibrium as a function of the PCM rest population g_0: the
 // inverse of g_0 = H - omega c_f,ref T(H) with T(H) from Eq. 38 (16-bit modes).
-template <typename R>
-__device__ __forceinline__ R pcm_ref(const StepParams<R>& P, R g0) {
-    // the three branches as in enthalpy_state: solid slope up to g0_fs, a linear
-    // rise of c_f,ref (T_fl - T_fs) across the mushy zone, liquid slope above g0_fl
-    return fmin(g0 * P.cr_solid, P.cr_fs) + sat01((g0 - P.g0_fs) * P.inv_dg0) * P.cr_dsl +
-           fmax(g0 - P.g0_fl, R(0)) * P.cr_liquid;
-}
-
-template <typename R>
-__device__ __forceinline__ R fast_rcp(R x) {
-    if constexpr (sizeof(R) == 4) return __fdividef(1.0f, x);
-    else return R(1) / x;
-}
-
-template <typename R>
-__device__ __forceinline__ R fast_sqrt(R x) {   // x >= 0
-    if constexpr (sizeof(R) == 4) return x > 0.0f ? x * rsqrtf(x) : 0.0f;
-    else return sqrt(x);
+// The three branches as in enthalpy_state: solid slope up to g0_fs, a linear
+// rise of c_f,ref (T_fl - T_fs) across the mushy zone, liquid slope above g0_fl.
+template <typename T>
+__device__ __forceinline__ T pcm_ref(const StepParams<float>& P, T g0) {
+    const T a = vfmac<T>(P.cr_dsl, vsatmul(vaddc(g0, -P.g0_fs), P.inv_dg0), vminc(vmulc<T>(P.cr_solid, g0), P.cr_fs));
+    return vfmac<T>(P.cr_liquid, vmax0(vaddc(g0, -P.g0_fl)), a);
 }
 
 // ---------------------------------------------------------------------------
 // Node state
 // ---------------------------------------------------------------------------
 
-template <int M, int QT, bool FLOW>
+template <int M, int QT, bool FLOW, typename T>
 struct NodeState {
-    using R = typename ModeTraits<M>::R;
-    R mp[FLOW ? 9 : 1];  // moments of f+ minus r (after the wall rule)
-    V2<R> th[QT];        // moments of (g, h) (after the wall rule); th[0] = (H, c_pm T_m) (high parts)
-    R Hlo, Elo;          // low parts of H and c_pm T_m (error-free bookkeeping; 0 where unused)
-    R H, Tf, fl, Tm, rho, drho, ux, uy, um, Gy;   // um = |u|
+    T mp[FLOW ? 9 : 1];  // moments of f+ minus r, times kFlowScale<M> (after the wall rule)
+    T n[QT], k[QT];      // PCM and metal moments (after the wall rule); n[0] = H (high part), k[0] = c_pm T_m = T_m
+    T Hlo, Elo;          // low parts of H and c_pm T_m (error-free bookkeeping; 0 where unused)
+    T h0, hs;            // metal rest population and the sum of its movers: k[0] = h0 + hs before rounding (FP32)
+    T Tf, fl, rho, drho, ux, uy, um, G;   // um = |u|, G = phi G_y (Eq. 7)
 };
+
+// the lane's type in a mode's one-node kernels
+template <int M> using Node1 = typename ModeTraits<M>::R;
 
 template <int M>
 __device__ __forceinline__ typename ModeTraits<M>::R ldb(const typename ModeTraits<M>::B* p) {
@@ -489,18 +442,46 @@ __device__ __forceinline__ void stb(typename ModeTraits<M>::B* p, R v) {
     *p = from_f<B>(v);
 }
 
-// The nine flow populations of one node (f_0 and the pairs of f_from_m9p);
-// PS: elements from one plane to the next (kChunk in a state copy, where the
-// inlined constant folds into the addresses).
-template <int M>
-__device__ __forceinline__ void store_flow(typename ModeTraits<M>::B* db, typename ModeTraits<M>::R f0,
-                                           const V2<typename ModeTraits<M>::R>* F, int PS = kChunk) {
-    stb<M>(db, f0);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        stb<M>(db + (2 * j + 1) * PS, F[j].x);
-        stb<M>(db + (2 * j + 2) * PS, F[j].y);
+// Two adjacent elements of a plane, as stored (16-bit: one 32-bit access; FP32: 64-bit).
+__device__ __forceinline__ W unpack2(__half2 v) {
+    const float2 f = __half22float2(v);
+    return {f.x, f.y};
+}
+__device__ __forceinline__ W unpack2(__nv_bfloat162 v) {
+    const float2 f = __bfloat1622float2(v);
+    return {f.x, f.y};
+}
+__device__ __forceinline__ W unpack2(float2 v) { return {v.x, v.y}; }
+template <typename B> struct Two;
+template <> struct Two<__half> { using type = __half2; };
+template <> struct Two<__nv_bfloat16> { using type = __nv_bfloat162; };
+template <> struct Two<float> { using type = float2; };
+
+// Stores v at p (the lanes adjacent); returns the values as a reader decodes them.
+template <int M, typename T>
+__device__ __forceinline__ T put(typename ModeTraits<M>::B* p, T v) {
+    if constexpr (Lane<T>::n == 1) {
+        const typename ModeTraits<M>::B b = from_f<typename ModeTraits<M>::B>(v);
+        *p = b;
+        return to_f(b);
+    } else if constexpr (M == MODE_F16) {
+        const __half2 h = __floats2half2_rn(v.x, v.y);
+        *reinterpret_cast<__half2*>(p) = h;
+        return unpack2(h);
+    } else if constexpr (M == MODE_BF16) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(v.x, v.y);
+        *reinterpret_cast<__nv_bfloat162*>(p) = h;
+        return unpack2(h);
+    } else {
+        *reinterpret_cast<float2*>(p) = f2(v);
+        return v;
     }
+}
+template <typename R> __device__ __forceinline__ void put_real(R* p, R v) { *p = v; }
+__device__ __forceinline__ void put_real(float* p, W v) { *reinterpret_cast<float2*>(p) = f2(v); }
+template <typename T, typename R> __device__ __forceinline__ T get_real(const R* p) {
+    if constexpr (Lane<T>::n == 2) return unpack2(*reinterpret_cast<const float2*>(p));
+    else return *p;
 }
 
 // Byte offset, within a state copy, of the chunk holding node (x, y).
@@ -586,254 +567,449 @@ struct PullAt {
     }
 };
 
-// Flow moments of the pulled populations (Eqs. 13, 15), deviation form.  A
-// is the accessor of the pulled neighbourhood: PullAt (the state copy in
-// global memory) or a staged copy in shared memory.
-template <int M, int QT, bool FLOW, typename A>
-__device__ __forceinline__ void pull_flow(const StepParams<typename ModeTraits<M>::R>& P, const A& a,
-                                          NodeState<M, QT, FLOW>& n) {
-    using R = typename ModeTraits<M>::R;
-    if constexpr (FLOW) {
-        R f0 = a.bulk(0, 0);
-        V2<R> F[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) F[j] = {a.bulk(2 * j + 1, 2 * j + 1), a.bulk(2 * j + 2, 2 * j + 2)};
-        if constexpr (M == MODE_F16) {
-            constexpr R is = R(1.0 / 1024.0);
-            f0 *= is;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) F[j] = mul2(F[j], V2<R>{is, is});
+// The same around the node pair (x0, x0 + 1), x0 even (both nodes in one
+// chunk): own reads the pair's two adjacent elements, west the elements of
+// x0 - 1 and x0, east those of x0 + 1 and x0 + 2.
+template <int M, int QT>
+struct PairAt {
+    using B = typename ModeTraits<M>::B;
+    using CH = Chunk<M, QT, true>;
+    static constexpr int es = (int)sizeof(B);
+    const char* row[3];
+    int cm, cp, w0, wm, wp;   // west, east and wide elements, from the pair's bulk plane 0
+    __device__ __forceinline__ PairAt(const StepParams<float>& P, int x0, int ys) {
+        const int xm = x0 == 0 ? P.nx - 1 : x0 - 1;       // west of x0
+        const int xp = x0 + 2 >= P.nx ? 0 : x0 + 2;       // east of x0 + 1
+        const int ym = ys == 0 ? P.ny - 1 : ys - 1;
+        const int yp = ys == P.ny - 1 ? 0 : ys + 1;
+        const int rb = P.cpr * CH::bytes;
+        const int c0 = col_off<M, QT, true>(x0);
+        const char* own = P.src + ((long long)ys * rb + c0);
+        row[0] = own + (long long)(ym - ys) * rb;
+        row[1] = own;
+        row[2] = own + (long long)(yp - ys) * rb;
+        cm = col_off<M, QT, true>(xm) - c0;
+        cp = col_off<M, QT, true>(xp) - c0;
+        if constexpr (kSplit<M>) {
+            w0 = col_off<M, QT, true, true>(x0) - c0;
+            wm = col_off<M, QT, true, true>(xm) - c0;
+            wp = col_off<M, QT, true, true>(xp) - c0;
         }
-        V2<R> m[4];
-        m_from_f9p(f0, F, n.mp[0], m);
-        n.mp[1] = m[0].x; n.mp[2] = m[0].y;
-        n.mp[3] = m[1].x; n.mp[5] = m[1].y;
-        n.mp[4] = m[2].x; n.mp[6] = m[2].y;
-        n.mp[7] = m[3].x; n.mp[8] = m[3].y;
+    }
+    __device__ __forceinline__ static float one(const char* p) { return ldb<M>(reinterpret_cast<const B*>(p)); }
+    __device__ __forceinline__ static float onew(const char* p) { return __ldg(reinterpret_cast<const float*>(p)); }
+    __device__ __forceinline__ W bulk(int q, int plane) const {
+        const char* r = row[src_row(q)] + plane * kChunk * es;
+        if (src_col(q) == 0) return {one(r + cm), one(r)};
+        if (src_col(q) == 2) return {one(r + es), one(r + cp)};
+        return unpack2(__ldg(reinterpret_cast<const typename Two<B>::type*>(r)));
+    }
+    __device__ __forceinline__ W wide(int q, int w) const {
+        const char* r = row[src_row(q)] + w * kChunk * 4;
+        if (src_col(q) == 0) return {onew(r + wm), onew(r + w0)};
+        if (src_col(q) == 2) return {onew(r + w0 + 4), onew(r + wp)};
+        return unpack2(__ldg(reinterpret_cast<const float2*>(r + w0)));
+    }
+};
+
+// Flow moments of the pulled populations (Eqs. 13, 15), deviation form, as
+// stored (times kFlowScale<M>).  A is the accessor of the pulled
+// neighbourhood: PullAt or PairAt (the state copy in global memory) or
+// PullTile (a staged copy in shared memory).
+template <int M, int QT, bool FLOW, typename T, typename A>
+__device__ __forceinline__ void pull_flow(const A& a, NodeState<M, QT, FLOW, T>& n) {
+    if constexpr (FLOW) {
+        T f[9];
+#pragma unroll
+        for (int q = 0; q < 9; ++q) f[q] = a.bulk(q, q);
+        m_from_f9(f, n.mp);
     }
 }
 
 // PCM and metal moments of the pulled populations (Eqs. 33, 44, B1).
-template <int M, int QT, bool FLOW, typename A>
+template <int M, int QT, bool FLOW, typename T, typename A>
 __device__ __forceinline__ void pull_thermal(const StepParams<typename ModeTraits<M>::R>& P, const A& a,
-                                             NodeState<M, QT, FLOW>& n) {
-    using R = typename ModeTraits<M>::R;
+                                             NodeState<M, QT, FLOW, T>& n) {
     using PL = Planes<M, QT, FLOW>;
-    V2<R> t[QT];   // (g_q, h_q)
+    T g[QT], h[QT];
     if constexpr (kSplit<M>) {
-        t[0] = {a.wide(0, 0), a.wide(0, 1)};
+        g[0] = a.wide(0, 0);
+        h[0] = a.wide(0, 1);
 #pragma unroll
         for (int q = 1; q < QT; ++q) {   // deviation + reference of the sending node
-            const V2<R> dev = {a.bulk(q, PL::pcm(q)), a.bulk(q, PL::met(q))};
-            const V2<R> ref = {pcm_ref(P, a.wide(q, 0)), a.wide(q, 1)};
-            t[q] = fma2(P.wmv[QT == 5 ? 1 : q], ref, dev);   // D2Q5: one weight varpi/4 for all movers (App. B)
+            const int w = QT == 5 ? 1 : q;   // D2Q5: one weight varpi/4 for all movers (App. B)
+            g[q] = vfmac<T>(P.w_move[w], pcm_ref(P, a.wide(q, 0)), a.bulk(q, PL::pcm(q)));
+            h[q] = vfmac<T>(P.wk_move[w], a.wide(q, 1), a.bulk(q, PL::met(q)));
         }
     } else {
 #pragma unroll
-        for (int q = 0; q < QT; ++q) t[q] = {a.bulk(q, PL::pcm(q)), a.bulk(q, PL::met(q))};
+        for (int q = 0; q < QT; ++q) {
+            g[q] = a.bulk(q, PL::pcm(q));
+            h[q] = a.bulk(q, PL::met(q));
+        }
     }
-    fwd2<R, QT>(t, n.th);
-    n.Hlo = R(0);
-    n.Elo = R(0);
+    thermal_moments<T, QT>(g, n.n);
+    thermal_moments<T, QT>(h, n.k);
+    n.Hlo = bc<T>(0);
+    n.Elo = bc<T>(0);
+    n.h0 = h[0];
+    n.hs = QT == 5 ? n.k[3] : mover_sum<QT>(h);
     if constexpr (kComp<M>) {
         // H = (g_0 hi + g_0 lo) + sum of movers, without rounding loss
-        const float lo = a.bulk(0, PL::lo);
-        float g[QT];
-#pragma unroll
-        for (int q = 0; q < QT; ++q) g[q] = t[q].x;
-        const FF H = ff_accumulate<QT>(FF{g[0], lo}, g, 1.0f);
-        n.th[0].x = H.hi;
+        const FF<T> s = mover_sum_ff<QT>(g);
+        const T t = vadd(g[0], s.hi);
+        const FF<T> H = fast_two_sum(t, vadd(vadd(s.lo, sum_err(g[0], s.hi, t)), a.bulk(0, PL::lo)));
+        n.n[0] = H.hi;
         n.Hlo = H.lo;
     }
 }
 
-template <int M, int QT, bool FLOW>
-__device__ __forceinline__ void pull_moments(const StepParams<typename ModeTraits<M>::R>& P, int xs, int ys,
-                                             NodeState<M, QT, FLOW>& n) {
-    const PullAt<M, QT, FLOW> a(P, xs, ys);
-    pull_flow<M, QT, FLOW>(P, a, n);
-    pull_thermal<M, QT, FLOW>(P, a, n);
-}
-
 // Macroscopic state from the moments (Eqs. 21, 23-25, 37-39, 48, 7): the
-// thermal side (H -> T_f, f_l; T_m) and the flow side, which needs T_f and
-// f_l (buoyancy, Eq. 7; the blended momentum, Eq. 24).
-template <int M, int QT, bool FLOW>
-__device__ __forceinline__ void thermal_macro(const StepParams<typename ModeTraits<M>::R>& P,
-                                              NodeState<M, QT, FLOW>& n) {
-    n.H = n.th[0].x;
-    enthalpy_state(P, n.H, n.Tf, n.fl);
-    n.Tm = n.th[0].y;   // h_0 moment = c_pm T_m, c_pm = 1
+// thermal side (H -> T_f, f_l; T_m = k[0]) and the flow side, which needs T_f
+// and f_l (buoyancy, Eq. 7; the blended momentum, Eq. 24).
+template <int M, int QT, bool FLOW, typename T>
+__device__ __forceinline__ void buoyancy(const StepParams<typename ModeTraits<M>::R>& P, NodeState<M, QT, FLOW, T>& n) {
+    if constexpr (FLOW) n.G = vmulc<T>(P.fgb, vmul(vaddc(n.Tf, -P.T0), n.fl));
 }
 
-template <int M, int QT, bool FLOW>
-__device__ __forceinline__ void flow_macro(const StepParams<typename ModeTraits<M>::R>& P, NodeState<M, QT, FLOW>& n,
-                                           bool wall) {
-    using R = typename ModeTraits<M>::R;
+template <int M, int QT, bool FLOW, typename T>
+__device__ __forceinline__ void macro(const StepParams<typename ModeTraits<M>::R>& P, NodeState<M, QT, FLOW, T>& n) {
+    using R = typename Lane<T>::R;
+    enthalpy_state(P, n.n[0], n.Tf, n.fl);
     if constexpr (FLOW) {
-        n.drho = n.mp[0];
-        n.rho = R(1) + n.drho;
-        n.Gy = P.gbeta * (n.Tf - P.T0) * n.fl;
-        if (wall || (P.solid_scheme && n.fl <= R(0.5))) {
-            n.ux = R(0);
-            n.uy = R(0);
-            n.um = R(0);
-        } else {
-            // Eq. 24 with sum_i e_i f_i = f_l sum_i e_i f+_i (the equilibrium at rest carries no
-            // momentum); without the blend (bounce-back variant) sum_i e_i f_i = sum_i e_i f+_i
-            const R ir = fast_rcp(n.rho);
-            const R a = P.solid_scheme ? R(1) : n.fl;
-            const R vx = a * n.mp[3] * ir;
-            const R vy = a * n.mp[5] * ir + R(0.5) * P.phi * n.Gy;
-            const R vm = fast_sqrt(vx * vx + vy * vy);
-            const R den = fast_rcp(P.l0 + fast_sqrt(P.l0sq + P.l1 * vm));   // Eq. 23
-            n.ux = vx * den;
-            n.uy = vy * den;
-            n.um = vm * den;
-        }
+        constexpr R is = R(1.0 / kFlowScale<M>);
+        buoyancy<M, QT, FLOW, T>(P, n);
+        n.drho = kFlowScale<M> == 1 ? n.mp[0] : vmulc<T>(is, n.mp[0]);
+        n.rho = vaddc(n.drho, R(1));
+        // Eq. 24 with sum_i e_i f_i = f_l sum_i e_i f+_i (the equilibrium at rest carries no
+        // momentum); without the blend (bounce-back variant) sum_i e_i f_i = sum_i e_i f+_i
+        T a = n.fl;
+        if constexpr (Lane<T>::n == 1)
+            if (P.solid_scheme) a = R(1);
+        if constexpr (kFlowScale<M> != 1) a = vmulc<T>(is, a);
+        // quotients by numbers near 1 as x - x d, with a small d: rho and the denominator of
+        // Eq. 23 vary little over a run, and the rounding of their reciprocals would be the
+        // same at every node and step (measured over 200 steps of the 256^2 cavity: u off by
+        // up to 1.5e-5 in FP32 with products of reciprocals)
+        const T c = vmul(vneg(n.drho), vrcp(n.rho));
+        const T vx = vmul(a, vfma(c, n.mp[3], n.mp[3]));
+        const T vy = vfmac<T>(R(0.5), n.G, vmul(a, vfma(c, n.mp[5], n.mp[5])));
+        const T vm = vsqrt(vfma(vy, vy, vmul(vx, vx)));
+        // Eq. 23: u = v / den, den = l_0 + sqrt(l_0^2 + l_1 |v|) = 1 + (2 l_0 - 1) + l_1 |u|
+        const T r = vrcp(vaddc(vsqrt(vfma(bc<T>(P.l1), vm, bc<T>(P.l0sq))), P.l0));
+        n.um = vmul(vm, r);
+        const T d = vmul(vfma(bc<T>(P.nl1), n.um, bc<T>(P.n2l0)), r);
+        n.ux = vfma(d, vx, vx);
+        n.uy = vfma(d, vy, vy);
+        if constexpr (Lane<T>::n == 1)
+            if (P.solid_scheme && n.fl <= R(0.5)) n.ux = n.uy = n.um = R(0);
     } else {
-        n.drho = R(0);
-        n.rho = R(1);
-        n.ux = R(0);
-        n.uy = R(0);
-        n.um = R(0);
-        n.Gy = R(0);
+        n.drho = bc<T>(0);
+        n.rho = bc<T>(1);
+        n.ux = n.uy = n.um = n.G = bc<T>(0);
     }
-}
-
-template <int M, int QT, bool FLOW>
-__device__ __forceinline__ void macro(const StepParams<typename ModeTraits<M>::R>& P, NodeState<M, QT, FLOW>& n,
-                                      bool wall) {
-    thermal_macro<M, QT, FLOW>(P, n);
-    flow_macro<M, QT, FLOW>(P, n, wall);
 }
 
 // Wall nodes: x_f = x_b + inward normal (diagonal at corners) and the side
-// whose temperature rule applies (the left/right wall at corners).
+// whose temperature rule applies (the left/right wall at corners).  A node
+// pair on a left or right wall pulls both nodes at its own columns, and the
+// wall node then takes its partner's moments (its x_f).
+template <typename T> struct WallAt;
+template <typename R>
 struct WallAt {
+    bool any;            // some lane is a wall node
     bool wall;
-    int xs, ys, side;
+    int xs, ys, side;    // where to pull
+    template <typename P_>
+    __device__ __forceinline__ WallAt(const P_& P, int x, int y) {
+        const bool wx = !P.per_x && (x == 0 || x == P.nx - 1);
+        const bool wy = !P.per_y && (y == 0 || y == P.ny - 1);
+        any = wall = wx || wy;
+        xs = wx ? (x == 0 ? 1 : P.nx - 2) : x;
+        ys = wy ? (y == 0 ? 1 : P.ny - 2) : y;
+        side = wx ? (x == 0 ? 0 : 1) : (y == 0 ? 2 : 3);
+    }
+    __device__ __forceinline__ void from_inward(R&) const {}
+    __device__ __forceinline__ R of_side(const R* v) const { return v[side]; }
+    __device__ __forceinline__ bool dirichlet(const int* kind) const { return kind[side] == 0; }
+};
+template <>
+struct WallAt<W> {
+    bool any, xa, xb;    // xa, xb: the pair's first (second) node is on the left (right) wall
+    Mask2 wall;
+    int xs, ys, sa, sb;
+    __device__ __forceinline__ WallAt(const StepParams<float>& P, int x0, int y) {
+        const bool wy = !P.per_y && (y == 0 || y == P.ny - 1);
+        xa = !P.per_x && x0 == 0;
+        xb = !P.per_x && x0 + 1 == P.nx - 1;
+        wall = {xa || wy, xb || wy};
+        any = wy || xa || xb;
+        xs = x0;
+        ys = wy ? (y == 0 ? 1 : P.ny - 2) : y;
+        const int sy = y == 0 ? 2 : 3;
+        sa = xa ? 0 : sy;
+        sb = xb ? 1 : sy;
+    }
+    __device__ __forceinline__ void from_inward(W& v) const { v = {xa ? v.y : v.x, xb ? v.x : v.y}; }
+    __device__ __forceinline__ W of_side(const float* v) const { return {v[sa], v[sb]}; }
+    __device__ __forceinline__ Mask2 dirichlet(const int* kind) const {
+        return {wall.x && kind[sa] == 0, wall.y && kind[sb] == 0};
+    }
 };
 
-template <typename R>
-__device__ __forceinline__ WallAt wall_at(const StepParams<R>& P, int x, int y) {
-    const bool wx = !P.per_x && (x == 0 || x == P.nx - 1);
-    const bool wy = !P.per_y && (y == 0 || y == P.ny - 1);
-    WallAt w;
-    w.wall = wx || wy;
-    w.xs = wx ? (x == 0 ? 1 : P.nx - 2) : x;
-    w.ys = wy ? (y == 0 ? 1 : P.ny - 2) : y;
-    w.side = wx ? (x == 0 ? 0 : 1) : (y == 0 ? 2 : 3);
-    return w;
-}
-
-// Eq. 52 in moment space on the flow lattice: m+(x_b) = m+(x_f) +
-// m^eq(rho_f, u_b = 0) - m^eq(rho_f, u_f), written out so that the rho r
-// parts cancel exactly (n holds the state of x_f).
-template <int M, int QT, bool FLOW>
-__device__ __forceinline__ void flow_wall(const StepParams<typename ModeTraits<M>::R>& P, NodeState<M, QT, FLOW>& n) {
-    using R = typename ModeTraits<M>::R;
+// Eq. 52 in moment space at the wall lanes (n holds the state of x_f):
+// m+(x_b) = m+(x_f) + m^eq(rho_f, u_b = 0) - m^eq(rho_f, u_f), written out so
+// that the rho r parts cancel exactly, and likewise for the thermal moments
+// with the wall's temperature (Dirichlet: T_f = T_m = T_w, H = H(T_w);
+// adiabatic: those of x_f) and the velocity u_f in the PCM equilibrium.  The
+// other lanes of a pair go through with corrections of zero.
+template <int M, int QT, bool FLOW, typename T>
+__device__ __forceinline__ void apply_wall(const StepParams<typename ModeTraits<M>::R>& P, const WallAt<T>& w,
+                                           NodeState<M, QT, FLOW, T>& n) {
+    using R = typename Lane<T>::R;
+    const T zero = bc<T>(0);
+    const T ux = vsel(w.wall, n.ux, zero), uy = vsel(w.wall, n.uy, zero);
     if constexpr (FLOW) {
-        const R rho = n.rho, ip = P.inv_phi;
-        const R q = R(3) * rho * (n.ux * n.ux + n.uy * n.uy) * ip;
-        n.mp[1] -= q;
-        n.mp[2] += q;
-        n.mp[3] -= rho * n.ux;
-        n.mp[4] += rho * n.ux;
-        n.mp[5] -= rho * n.uy;
-        n.mp[6] += rho * n.uy;
-        n.mp[7] -= rho * (n.ux * n.ux - n.uy * n.uy) * ip;
-        n.mp[8] -= rho * n.ux * n.uy * ip;
-    }
-}
-
-// Eq. 52 on the PCM and metal lattices, with the wall's temperature
-// (Dirichlet: T_f = T_m = T_w, H = H(T_w); adiabatic: those of x_f) and the
-// velocity u_f of x_f in the PCM equilibrium.
-template <int M, int QT, bool FLOW>
-__device__ __forceinline__ void thermal_wall(const StepParams<typename ModeTraits<M>::R>& P,
-                                             NodeState<M, QT, FLOW>& n, int side) {
-    using R = typename ModeTraits<M>::R;
-    const bool dirichlet = P.wall_kind[side] == 0;
-    R Tb, Hb, Tmb;
-    if (dirichlet) {
-        Tb = P.wall_T[side];
-        Tmb = Tb;
-        Hb = P.wall_H[side];
-    } else {
-        Tb = n.Tf;
-        Hb = n.H;
-        Tmb = n.Tm;
-    }
-    R a[QT], b[QT];
-    neq_pcm<R, QT>(P, Hb, Tb, R(0), R(0), a);
-    neq_pcm<R, QT>(P, n.H, n.Tf, n.ux, n.uy, b);
-#pragma unroll
-    for (int k = 1; k < QT; ++k) n.th[k].x += a[k] - b[k];
-    if (dirichlet) {   // n_0 = H_b exactly (adiabatic: n_0 = H(x_f), unchanged)
-        n.th[0].x = P.wall_H[side];
-        n.Hlo = P.wall_H_lo[side];
-    }
-    neq_metal<R, QT>(P, Tmb, a);
-    neq_metal<R, QT>(P, n.Tm, b);
-    if constexpr (kSplit<M>) {
-#pragma unroll
-        for (int k = 1; k < QT; ++k) n.th[k].y += a[k] - b[k];
-        if (dirichlet) {   // c_pm T_m = c_pm T_b exactly (c_pm = 1)
-            n.th[0].y = P.wall_T[side];
-            n.Elo = P.wall_T_lo[side];
+        constexpr R sc = R(kFlowScale<M>);
+        T jx = vfma(n.drho, ux, ux), jy = vfma(n.drho, uy, uy);
+        if constexpr (kFlowScale<M> != 1) {
+            jx = vmulc<T>(sc, jx);
+            jy = vmulc<T>(sc, jy);
         }
+        const T a = vmul(jx, ux);
+        const T q = vmulc<T>(vmul(R(3), P.inv_phi), vfma(jy, uy, a));
+        n.mp[1] = vsub(n.mp[1], q);
+        n.mp[2] = vadd(n.mp[2], q);
+        n.mp[3] = vsub(n.mp[3], jx);
+        n.mp[4] = vadd(n.mp[4], jx);
+        n.mp[5] = vsub(n.mp[5], jy);
+        n.mp[6] = vadd(n.mp[6], jy);
+        n.mp[7] = vfmac<T>(-P.inv_phi, vfma(vneg(jy), uy, a), n.mp[7]);
+        n.mp[8] = vfmac<T>(-P.inv_phi, vmul(jx, uy), n.mp[8]);
+    }
+    const auto dir = w.dirichlet(P.wall_kind);
+    const T Tb = w.of_side(P.wall_T), Hb = w.of_side(P.wall_H);
+    const T dT = vsel(dir, vsub(Tb, n.Tf), zero), dM = vsel(dir, vsub(Tb, n.k[0]), zero);
+    const T t = vmulc<T>(P.inv_phi, n.Tf), mt = vneg(t);   // c_pl T / phi
+    if constexpr (QT == 5) {
+        n.n[1] = vfma(mt, ux, n.n[1]);
+        n.n[2] = vfma(mt, uy, n.n[2]);
+        n.n[3] = vfmac<T>(P.vcf, dT, n.n[3]);
+        n.k[3] = vfmac<T>(P.vcm, dM, n.k[3]);
     } else {
+        const T dH = vsel(dir, vsub(Hb, n.n[0]), zero);
+        const T cT = vmulc<T>(P.c_fref, dT), cM = vmulc<T>(P.c_mref, dM);
+        n.n[1] = vadd(n.n[1], vfmac<T>(R(-4), dH, vadd(cT, cT)));
+        n.n[2] = vadd(n.n[2], vfmac<T>(R(4), dH, vmulc<T>(R(-3), cT)));
+        n.n[3] = vfma(mt, ux, n.n[3]);
+        n.n[4] = vfma(t, ux, n.n[4]);
+        n.n[5] = vfma(mt, uy, n.n[5]);
+        n.n[6] = vfma(t, uy, n.n[6]);
+        n.k[1] = vadd(n.k[1], vfmac<T>(R(-4), dM, vadd(cM, cM)));
+        n.k[2] = vadd(n.k[2], vfmac<T>(R(4), dM, vmulc<T>(R(-3), cM)));
+    }
+    // n_0 = H_b and c_pm T_m = c_pm T_b exactly (adiabatic: those of x_f, unchanged)
+    n.n[0] = vsel(dir, Hb, n.n[0]);
+    n.Hlo = vsel(dir, w.of_side(P.wall_H_lo), n.Hlo);
+    n.k[0] = vsel(dir, Tb, n.k[0]);
+    if constexpr (QT == 5) n.hs = n.k[3];
+    n.h0 = vsel(dir, vsub(Tb, n.hs), n.h0);
+    if constexpr (kSplit<M>) n.Elo = vsel(dir, w.of_side(P.wall_T_lo), n.Elo);
+    enthalpy_state(P, n.n[0], n.Tf, n.fl);
+    buoyancy<M, QT, FLOW, T>(P, n);
+    n.ux = vsel(w.wall, zero, n.ux);
+    n.uy = vsel(w.wall, zero, n.uy);
+    n.um = vsel(w.wall, zero, n.um);
+}
+
+// State of a node (pair) from its pulled neighbourhood a (pulled at x_f on
+// walls, then Eq. 52 in moment space).
+template <int M, int QT, bool FLOW, typename T, typename A>
+__device__ __forceinline__ void node_state(const StepParams<typename ModeTraits<M>::R>& P, const A& a,
+                                           const WallAt<T>& w, NodeState<M, QT, FLOW, T>& n) {
+    pull_flow<M, QT, FLOW, T>(a, n);
+    pull_thermal<M, QT, FLOW, T>(P, a, n);
+    if constexpr (Lane<T>::n == 2) {
+        if (w.xa || w.xb) {
 #pragma unroll
-        for (int k = 0; k < QT; ++k) n.th[k].y += a[k] - b[k];
+            for (int q = 0; q < 9; ++q) w.from_inward(n.mp[q]);
+#pragma unroll
+            for (int q = 0; q < QT; ++q) {
+                w.from_inward(n.n[q]);
+                w.from_inward(n.k[q]);
+            }
+            w.from_inward(n.Hlo);
+        }
+    }
+    macro<M, QT, FLOW, T>(P, n);
+    if (w.any) apply_wall<M, QT, FLOW, T>(P, w, n);
+}
+
+// Full state of node (x, y) in a state copy: interior nodes pull at
+// themselves, wall nodes at x_f = x_b + inward normal.
+template <int M, int QT, bool FLOW>
+__device__ __forceinline__ void node_state_at(const StepParams<typename ModeTraits<M>::R>& P, int x, int y,
+                                              NodeState<M, QT, FLOW, Node1<M>>& n) {
+    const WallAt<Node1<M>> w(P, x, y);
+    node_state<M, QT, FLOW, Node1<M>>(P, PullAt<M, QT, FLOW>(P, w.xs, w.ys), w, n);
+}
+
+// ---------------------------------------------------------------------------
+// Collisions
+// ---------------------------------------------------------------------------
+
+// Flow collision and store of one node (pair) (Eqs. 3, 14, 18-20): f* at db,
+// the element in flow plane 0 of the next copy, PS elements from one plane to
+// the next.
+template <int M, int QT, bool FLOW, int PS, typename T>
+__device__ __forceinline__ void flow_collide(const StepParams<typename ModeTraits<M>::R>& P,
+                                             const NodeState<M, QT, FLOW, T>& n, typename ModeTraits<M>::B* db) {
+    using R = typename Lane<T>::R;
+    if constexpr (FLOW) {
+        constexpr R is = R(1.0 / kFlowScale<M>);   // takes the storage scale off the pulled moments
+        T m[9], f[9];
+        T fb = n.fl;
+        if constexpr (Lane<T>::n == 1) {
+            if (P.solid_scheme && n.fl <= R(0.5)) {
+                // bounce-back solid node: f*_i = f+_opp(i); reversing every link flips the
+                // sign of the odd moments (j, q) and keeps the even ones (deviation form too)
+#pragma unroll
+                for (int q = 0; q < 9; ++q) m[q] = vmul(q >= 3 && q <= 6 ? -is : is, n.mp[q]);
+                f_from_m9<T, kFlowScale<M>>(m, f);
+#pragma unroll
+                for (int q = 0; q < 9; ++q) put<M>(db + q * PS, f[q]);
+                return;
+            }
+            if (P.solid_scheme) fb = R(1);   // no blend in the bounce-back variant
+        }
+        const T drag = vfma(bc<T>(P.nforch), n.um, bc<T>(P.nlin));   // Eq. 3, negated
+        const T Fx = vmul(drag, n.ux), Fy = vfma(drag, n.uy, n.G);
+        const T jx = vfma(n.drho, n.ux, n.ux), jy = vfma(n.drho, n.uy, n.uy);   // rho u, rho F
+        const T fx = vfma(n.drho, Fx, Fx), fy = vfma(n.drho, Fy, Fy);
+        const T xx = vmul(jx, n.ux), fxx = vmul(jx, Fx);
+        const T up = vfma(jy, n.uy, xx), um = vfma(vneg(jy), n.uy, xx);      // j_x u_x +- j_y u_y
+        const T fp = vfma(jy, Fy, fxx), fm = vfma(vneg(jy), Fy, fxx);        // j_x F_x +- j_y F_y
+        // Eq. 14 on the blended moments (Eq. 20: f_l m+ + (1 - f_l) delta_rho r in deviation
+        // form) with the equilibria of Eq. 18 and the forcing moments of Eq. 19.  The rates of
+        // Sec. III C are constants (s_rho = s_j = 1, s_e = s_eps = 1.1, s_q = 1.2); only s_v
+        // depends on the run.  m - s (m - m^eq) is taken as (1 - s) m + s m^eq, with 1 - s
+        // exact; for e and eps the parts along r collect to (-2, 1) (delta_rho + s' f_l
+        // delta_rho), s' = s - 1.  Where s = 1 the result is m^eq + S/2 whatever the blend gave.
+        constexpr R s1 = R(1.1) - R(1), s2 = R(1.2) - R(1);
+        const T b1 = vmulc<T>(-s1 * is, fb), b2 = vmulc<T>(-s2 * is, fb), bv = vmulc<T>(P.c_v * is, fb);
+        const T K = vfma(vmulc<T>(s1, fb), n.drho, n.drho);
+        const T Q = vfmac<T>(P.k_uf, fp, vmulc<T>(P.k_uu, up));
+        m[0] = n.drho;
+        m[1] = vfma(b1, n.mp[1], vfmac<T>(R(-2), K, Q));
+        m[2] = vfma(b1, n.mp[2], vsub(K, Q));
+        m[3] = vfmac<T>(R(0.5), fx, jx);
+        m[5] = vfmac<T>(R(0.5), fy, jy);
+        m[4] = vfma(b2, n.mp[4], vfmac<T>(R(-0.4), fx, vmulc<T>(R(-1.2), jx)));
+        m[6] = vfma(b2, n.mp[6], vfmac<T>(R(-0.4), fy, vmulc<T>(R(-1.2), jy)));
+        m[7] = vfma(bv, n.mp[7], vfmac<T>(P.k_v, um, vmulc<T>(P.k_2h, fm)));
+        m[8] = vfma(bv, n.mp[8],
+                    vfmac<T>(P.k_v, vmul(jx, n.uy), vmulc<T>(P.k_h, vfma(jx, Fy, vmul(jy, Fx)))));
+        f_from_m9<T, kFlowScale<M>>(m, f);
+#pragma unroll
+        for (int q = 0; q < 9; ++q) put<M>(db + q * PS, f[q]);
     }
 }
 
-// State of a node from its pulled neighbourhood a (pulled at x_f on walls,
-// then Eq. 52 in moment space).
-template <int M, int QT, bool FLOW, typename A>
-__device__ __forceinline__ void node_state_from(const StepParams<typename ModeTraits<M>::R>& P, const A& a,
-                                                const WallAt& w, NodeState<M, QT, FLOW>& n) {
-    pull_flow<M, QT, FLOW>(P, a, n);
-    pull_thermal<M, QT, FLOW>(P, a, n);
-    macro<M, QT, FLOW>(P, n, false);
-    if (!w.wall) return;
-    flow_wall<M, QT, FLOW>(P, n);
-    thermal_wall<M, QT, FLOW>(P, n, w.side);
-    macro<M, QT, FLOW>(P, n, true);
-}
-
-// Full state of node (x, y): interior nodes pull at themselves; wall nodes pull
-// at x_f = x_b + inward normal and apply Eq. 52 in moment space.
-template <int M, int QT, bool FLOW>
-__device__ __forceinline__ void node_state(const StepParams<typename ModeTraits<M>::R>& P, int x, int y,
-                                           NodeState<M, QT, FLOW>& n, bool& wall) {
-    const WallAt w = wall_at(P, x, y);
-    wall = w.wall;
-    const PullAt<M, QT, FLOW> a(P, w.xs, w.ys);
-    node_state_from<M, QT, FLOW>(P, a, w, n);
-}
-
-// Post-collision thermal populations of both lattices from their moments
-// (x: PCM, y: metal).  n0g (hi, lo) and n0h are the conserved moments after the
-// sources.  Each rest population is the remainder n_0 - sum of the moving
-// populations as they are stored, so the stored populations carry the enthalpy
-// (internal energy) that the collision produced: the FP32 PCM rest population
-// to float-float accuracy, the FP32 metal one to one rounding, the 16-bit forms
-// to FP32 rounding as readers decode them, FP64 to FP64 rounding.  db and dw
-// point at the node's element in bulk plane 0 and wide plane 0 of the next copy
-// (PS elements from one plane to the next).
-template <int M, int QT, bool FLOW>
-__device__ __forceinline__ void store_thermal(const StepParams<typename ModeTraits<M>::R>& P,
-                                              V2<typename ModeTraits<M>::R>* nm, typename ModeTraits<M>::R n0ghi,
-                                              typename ModeTraits<M>::R n0glo, typename ModeTraits<M>::R n0h,
-                                              typename ModeTraits<M>::B* db, float* dw, int PS = kChunk) {
-    using R = typename ModeTraits<M>::R;
-    using B = typename ModeTraits<M>::B;
+// PCM and metal collisions and stores of one node (pair) (Eqs. 32, 36, 43, 47
+// with the backward difference of Remark III): dTp is the exchange history,
+// db/dw the element in bulk and wide plane 0 of the next copy; returns the new
+// history T_m - T_f.  Each rest population is the remainder n_0 - sum of the
+// moving populations as they are stored, so the stored populations carry the
+// enthalpy (internal energy) that the collision produced: the FP32 PCM rest
+// population to float-float accuracy, the FP32 metal one to one rounding, the
+// 16-bit forms to FP32 rounding as readers decode them, FP64 to FP64 rounding.
+template <int M, int QT, bool FLOW, bool PH, int PS, typename T>
+__device__ __forceinline__ T thermal_collide(const StepParams<typename ModeTraits<M>::R>& P,
+                                             const NodeState<M, QT, FLOW, T>& n, T dTp,
+                                             typename ModeTraits<M>::B* db, float* dw) {
+    using R = typename Lane<T>::R;
     using PL = Planes<M, QT, FLOW>;
-    V2<R> v[QT];
-    nm[0] = {n0ghi, n0h};
-    inv2<R, QT>(nm, v);
+    const T dTn = vsub(n.k[0], n.Tf);
+    const T S_met = vfmac<T>(P.x_now, dTn, vmulc<T>(P.x_prev, dTp));
+    // metal n_0 after its source (n_0 is conserved by the collision, Eq. 43).  The
+    // PCM takes the opposite of what the metal's n_0 actually changed by, scaled
+    // by the heat capacities (S_PCM = -(a_f/a_m) S_metal, Eqs. 36, 47), so an
+    // exchange that the metal's rounding drops moves no energy into the PCM (FP32:
+    // n_0 takes what the stored metal took, below)
+    const T hm = vadd(n.k[0], S_met);
+    const T took = kComp<M> ? S_met : vsub(hm, n.k[0]);
+    const T S_pcm = vmulc<T>(P.x_pm, took);
+    const T n0 = vfmac<T>(P.x_pm, took, n.n[0]);   // H + S_PCM (n_0 is conserved up to the source, Eq. 32)
+    T g[QT], h[QT];   // post-collision populations; g[0], h[0]: provisional rest populations
+    if constexpr (QT == 5) {
+        // n* = (1 - z) n + z n^eq + S s, the factors of M^-1 folded into the constants:
+        // a_j = n*_{1,2} / 2, a_3 = n*_3 / 4, a_4 = n*_4 / 4
+        T jx, jy, a3, a4;
+        if (PH && P.phase_k) {
+            // Eq. 9 at the node's liquid fraction -> zeta_alpha (Eq. A19) -> zeta_e (Eq. 53)
+            const T za = vrcp(vaddc(vfma(bc<T>(P.kd_c), n.fl, bc<T>(P.ks_c)), R(0.5)));
+            T z[5];
+#pragma unroll
+            for (int k = 1; k < 5; ++k) z[k] = vfma(bc<T>(P.zr_b[k]), za, bc<T>(P.zr_a[k]));
+            const T t = vmulc<T>(P.inv_phi, n.Tf);
+            const T d1 = vfma(vneg(t), n.ux, n.n[1]), d2 = vfma(vneg(t), n.uy, n.n[2]);
+            jx = vmulc<T>(R(0.5), vfma(vneg(z[1]), d1, n.n[1]));
+            jy = vmulc<T>(R(0.5), vfma(vneg(z[2]), d2, n.n[2]));
+            const T d3 = vfmac<T>(-P.vcf, n.Tf, n.n[3]);
+            a3 = vfmac<T>(P.quart_varpi, S_pcm, vmulc<T>(R(0.25), vfma(vneg(z[3]), d3, n.n[3])));
+            a4 = vmulc<T>(R(0.25), vfma(vneg(z[4]), n.n[4], n.n[4]));
+        } else {
+            jx = vmulc<T>(P.z_j, n.n[1]);
+            jy = vmulc<T>(P.z_j, n.n[2]);
+            if constexpr (FLOW) {
+                const T t = vmulc<T>(P.z_ju, n.Tf);
+                jx = vfma(t, n.ux, jx);
+                jy = vfma(t, n.uy, jy);
+            }
+            a3 = vfmac<T>(P.z_3, n.n[3], vfmac<T>(P.z_3T, n.Tf, vmulc<T>(P.quart_varpi, S_pcm)));
+            a4 = vmulc<T>(P.z_4, n.n[4]);
+        }
+        const T c3 = vfmac<T>(P.e_3, n.k[3], vfmac<T>(P.e_3T, n.k[0], vmulc<T>(P.quart_varpi, S_met)));
+        const T c4 = vmulc<T>(P.e_4, n.k[4]);
+        const T kx = vmulc<T>(P.e_j, n.k[1]), ky = vmulc<T>(P.e_j, n.k[2]);
+        const T gp = vadd(a3, a4), gm = vsub(a3, a4), hp = vadd(c3, c4), hq = vsub(c3, c4);
+        g[1] = vadd(gp, jx); g[3] = vsub(gp, jx); g[2] = vadd(gm, jy); g[4] = vsub(gm, jy);
+        h[1] = vadd(hp, kx); h[3] = vsub(hp, kx); h[2] = vadd(hq, ky); h[4] = vsub(hq, ky);
+        g[0] = vfmac<T>(R(-4), a3, n0);
+        h[0] = vfmac<T>(R(-4), c3, hm);
+    } else {
+        T a[9], c[9], z[9];
+#pragma unroll
+        for (int k = 1; k < 9; ++k) z[k] = bc<T>(P.nz[k]);
+        if (PH && P.phase_k) {
+            const T za = vrcp(vaddc(vfma(bc<T>(P.kd_c), n.fl, bc<T>(P.ks_c)), R(0.5)));
+#pragma unroll
+            for (int k = 1; k < 9; ++k) z[k] = vneg(vfma(bc<T>(P.zr_b[k]), za, bc<T>(P.zr_a[k])));
+        }
+        const T cT = vmulc<T>(P.c_fref, n.Tf), cM = vmulc<T>(P.c_mref, n.k[0]);
+        const T t = vmulc<T>(P.inv_phi, n.Tf), mt = vneg(t);
+        // distances from the equilibria of Eqs. 34 and 45 (zero for k = 7, 8)
+        const T d[9] = {n.n[0], vsub(n.n[1], vfmac<T>(R(-4), n.n[0], vadd(cT, cT))),
+                        vsub(n.n[2], vfmac<T>(R(4), n.n[0], vmulc<T>(R(-3), cT))),
+                        vfma(mt, n.ux, n.n[3]), vfma(t, n.ux, n.n[4]), vfma(mt, n.uy, n.n[5]), vfma(t, n.uy, n.n[6]),
+                        n.n[7], n.n[8]};
+        const T e[9] = {n.k[0], vsub(n.k[1], vfmac<T>(R(-4), n.k[0], vadd(cM, cM))),
+                        vsub(n.k[2], vfmac<T>(R(4), n.k[0], vmulc<T>(R(-3), cM))),
+                        n.k[3], n.k[4], n.k[5], n.k[6], n.k[7], n.k[8]};
+#pragma unroll
+        for (int k = 1; k < 9; ++k) {
+            a[k] = vfma(z[k], d[k], n.n[k]);
+            c[k] = vfma(bc<T>(P.ne[k]), e[k], n.k[k]);
+        }
+        a[1] = vfmac<T>(R(-2), S_pcm, a[1]);
+        a[2] = vadd(a[2], S_pcm);
+        c[1] = vfmac<T>(R(-2), S_met, c[1]);
+        c[2] = vadd(c[2], S_met);
+        a[0] = n0;
+        c[0] = hm;
+        f_from_m9<T>(a, g);
+        f_from_m9<T>(c, h);
+    }
     if constexpr (kSplit<M>) {
         // 16-bit deviations from the reference of the provisional rest population,
         // then the rest population readers will see the balance with.  Readers
@@ -844,170 +1020,67 @@ __device__ __forceinline__ void store_thermal(const StepParams<typename ModeTrai
         // B5 for the metal), the solution is that of H = Y: g_0 = Y - omega
         // c_ref T(Y), whose reference is c_ref T(Y).  The stored populations as
         // read then carry n_0 to FP32 rounding.
-        const V2<float> ref = {pcm_ref(P, v[0].x), v[0].y};   // v[0]: provisional rest populations
-        V2<float> sd;
+        const T ref = pcm_ref(P, g[0]);
+        T sg, sh;
 #pragma unroll
         for (int k = 1; k < QT; ++k) {
-            const V2<float> e = fma2(P.nwmv[QT == 5 ? 1 : k], ref, v[k]);
-            const B bg = from_f<B>(e.x), bh = from_f<B>(e.y);
-            db[PL::pcm(k) * PS] = bg;
-            db[PL::met(k) * PS] = bh;
-            const V2<float> d = {to_f(bg), to_f(bh)};
-            sd = k == 1 ? d : add2(sd, d);
+            const int w = QT == 5 ? 1 : k;
+            const T dg = put<M>(db + PL::pcm(k) * PS, vfmac<T>(-P.w_move[w], ref, g[k]));
+            const T dh = put<M>(db + PL::met(k) * PS, vfmac<T>(-P.wk_move[w], h[0], h[k]));
+            sg = k == 1 ? dg : vadd(sg, dg);
+            sh = k == 1 ? dh : vadd(sh, dh);
         }
-        const V2<float> Y = sub2(V2<float>{n0ghi, n0h}, sd);
-        float T, fl;
-        enthalpy_state(P, Y.x, T, fl);
-        dw[0] = Y.x - P.om_cf * T;
-        dw[PS] = Y.y * P.rest_m;
+        const T Y = vsub(n0, sg);
+        T TY, fY;
+        enthalpy_state(P, Y, TY, fY);
+        put_real(dw, vfmac<T>(-P.om_cf, TY, Y));
+        put_real(dw + PS, vmulc<T>(P.rest_m, vsub(hm, sh)));
     } else {
 #pragma unroll
         for (int k = 1; k < QT; ++k) {
-            stb<M>(db + PL::pcm(k) * PS, v[k].x);
-            stb<M>(db + PL::met(k) * PS, v[k].y);
+            put<M>(db + PL::pcm(k) * PS, g[k]);
+            put<M>(db + PL::met(k) * PS, h[k]);
         }
-        V2<R> sm = v[1];
-#pragma unroll
-        for (int k = 2; k < QT; ++k) sm = add2(sm, v[k]);
-        const V2<R> rest = sub2(V2<R>{n0ghi, n0h}, sm);
-        if constexpr (kComp<M>) {   // the FP32 PCM rest population is a float-float pair
-            float vg[QT];
-#pragma unroll
-            for (int k = 0; k < QT; ++k) vg[k] = v[k].x;
-            const FF r = ff_accumulate<QT>(FF{n0ghi, n0glo}, vg, -1.0f);
-            stb<M>(db + PL::pcm(0) * PS, r.hi);
-            stb<M>(db + PL::lo * PS, r.lo);
+        if constexpr (kComp<M>) {
+            // the metal's rest population takes what its movers give up, t, and the source,
+            // without passing through their sum with the rest population, whose rounding is
+            // coarser; what it took of the source after rounding is what the PCM gives
+            const T t = vsub(n.hs, mover_sum<QT>(h));
+            const T rh = vadd(n.h0, vadd(t, S_met));
+            put<M>(db + PL::met(0) * PS, rh);
+            const T S = vmul_alone(bc<T>(P.x_pm), vsub(vsub(rh, n.h0), t));
+            // (the PCM rest population is a float-float pair)
+            const T n0 = vadd(n.n[0], S);
+            const FF<T> s = mover_sum_ff<QT>(g);
+            const T r = vsub(n0, s.hi);
+            const T lo = vadd(vadd(sum_err(n.n[0], S, n0), n.Hlo), vsub(sum_err(n0, vneg(s.hi), r), s.lo));
+            const FF<T> rest = fast_two_sum(r, lo);
+            put<M>(db + PL::pcm(0) * PS, rest.hi);
+            put<M>(db + PL::lo * PS, rest.lo);
         } else {
-            stb<M>(db + PL::pcm(0) * PS, rest.x);
+            put<M>(db + PL::met(0) * PS, vsub(hm, mover_sum<QT>(h)));
+            put<M>(db + PL::pcm(0) * PS, vsub(n0, mover_sum<QT>(g)));
         }
-        stb<M>(db + PL::met(0) * PS, rest.y);
     }
-}
-
-// ---------------------------------------------------------------------------
-// The fused step
-// ---------------------------------------------------------------------------
-
-// Flow collision and store of one node (Eqs. 3, 14, 18-20): f* at db, this
-// node's element in flow plane 0 of the next copy.
-template <int M, int QT, bool FLOW>
-__device__ __forceinline__ void flow_collide(const StepParams<typename ModeTraits<M>::R>& P,
-                                             const NodeState<M, QT, FLOW>& n, typename ModeTraits<M>::B* db,
-                                             int PS = kChunk) {
-    using R = typename ModeTraits<M>::R;
-    if constexpr (FLOW) {
-      if (P.solid_scheme && n.fl <= R(0.5)) {
-        // bounce-back solid node: f*_i = f+_opp(i); reversing every link flips the
-        // sign of the odd moments (j, q) and keeps the even ones (deviation form too)
-        const V2<R> m[4] = {{n.mp[1], n.mp[2]}, {-n.mp[3], -n.mp[5]}, {-n.mp[4], -n.mp[6]}, {n.mp[7], n.mp[8]}};
-        R f0;
-        V2<R> F[4];
-        f_from_m9p<R, kFlowScale<M>>(n.mp[0], m, f0, F);
-        store_flow<M>(db, f0, F, PS);
-      } else {
-        // Eq. 3 at the node's velocity (u = u_b = 0 on walls)
-        const R drag = P.drag_lin + P.drag_forch * n.um;
-        const V2<R> U = {n.ux, n.uy};
-        const V2<R> F = fma2(V2<R>{-drag, -drag}, U, V2<R>{R(0), P.phi * n.Gy});   // (F_x, F_y)
-        // blended moments (Eq. 20 in moment space, deviation form); no blend in the
-        // bounce-back variant.  Pairs (e, eps), (j_x, j_y), (q_x, q_y), (p_xx, p_xy)
-        const R fb = P.solid_scheme ? R(1) : n.fl;
-        const R sol = (R(1) - fb) * n.drho;
-        const V2<R> FB = {fb, fb};
-        V2<R> m12 = fma2(FB, V2<R>{n.mp[1], n.mp[2]}, V2<R>{R(-2) * sol, sol});
-        V2<R> m46 = mul2(FB, V2<R>{n.mp[4], n.mp[6]});
-        V2<R> m78 = mul2(FB, V2<R>{n.mp[7], n.mp[8]});
-        // equilibria (Eq. 18, deviation form) and forcing moments (Eq. 19); the q
-        // pair's equilibrium and forcing are the negated j pair's
-        const R rho = n.rho, rip = rho * P.inv_phi, drho = n.drho;
-        const R q = R(3) * rip * (n.ux * n.ux + n.uy * n.uy);
-        const V2<R> me12 = {R(-2) * drho + q, drho - q};
-        const V2<R> J = mul2(V2<R>{rho, rho}, U);
-        const V2<R> me78 = mul2(V2<R>{rip, rip}, V2<R>{n.ux * n.ux - n.uy * n.uy, n.ux * n.uy});
-        const R s1 = R(6) * rip * (n.ux * F.x + n.uy * F.y);
-        const V2<R> RF = mul2(V2<R>{rho, rho}, F);
-        const V2<R> S78 = mul2(V2<R>{rip, rip}, V2<R>{R(2) * (n.ux * F.x - n.uy * F.y), n.ux * F.y + n.uy * F.x});
-        // Eq. 14: the rates of Sec. III C are constants (s_rho = s_j = 1, s_e = s_eps =
-        // 1.1, s_q = 1.2); only s_v = s[7] = s[8] depends on the run.  Where s = 1 the
-        // result is m^eq + S/2 whatever the blend gave (rho: m^eq = delta_rho, S = 0)
-        m12 = fma2(V2<R>{R(0.45), R(0.45)}, V2<R>{s1, -s1},
-                   fma2(V2<R>{R(-1.1), R(-1.1)}, sub2(m12, me12), m12));
-        const V2<R> m35 = fma2(V2<R>{R(0.5), R(0.5)}, RF, J);
-        m46 = fma2(V2<R>{R(-0.4), R(-0.4)}, RF, fma2(V2<R>{R(-1.2), R(-1.2)}, add2(m46, J), m46));
-        const R sv = P.s[7], hv = R(1) - R(0.5) * sv;
-        m78 = fma2(V2<R>{hv, hv}, S78, fma2(V2<R>{-sv, -sv}, sub2(m78, me78), m78));
-        const V2<R> m[4] = {m12, m35, m46, m78};
-        R f0;
-        V2<R> Fo[4];
-        f_from_m9p<R, kFlowScale<M>>(drho, m, f0, Fo);
-        store_flow<M>(db, f0, Fo, PS);
-      }
-    }
-}
-
-// PCM and metal collisions and stores of one node (Eqs. 32, 36, 43, 47 with
-// the backward difference of Remark III): dTp is the node's exchange history,
-// db/dw its element in bulk and wide plane 0 of the next copy; returns the new
-// history T_m - T_f.
-template <int M, int QT, bool FLOW, bool PH>
-__device__ __forceinline__ typename ModeTraits<M>::R thermal_collide(const StepParams<typename ModeTraits<M>::R>& P,
-                                                                     NodeState<M, QT, FLOW>& n,
-                                                                     typename ModeTraits<M>::R dTp,
-                                                                     typename ModeTraits<M>::B* db, float* dw,
-                                                                     int PS = kChunk) {
-    using R = typename ModeTraits<M>::R;
-    // exchange sources, Eqs. 36 and 47 with the backward difference of Remark III
-    const R dTn = n.Tm - n.Tf;
-    const R Sx = R(1.5) * dTn - R(0.5) * dTp;
-    const R S_met = -P.a_m * Sx;
-    // metal n_0 after its source (n_0 is conserved by the collision, Eq. 43).  The
-    // PCM takes the opposite of what the metal's n_0 actually changed by, scaled
-    // by the heat capacities (S_PCM = -(a_f/a_m) S_metal, Eqs. 36, 47), so an
-    // exchange that the metal's rounding drops moves no energy into the PCM
-    R hm_base;
-    if constexpr (kSplit<M>) hm_base = n.th[0].y;
-    else hm_base = n.th[0].y - P.eta[0] * (n.th[0].y - n.Tm);
-    const R hm = hm_base + S_met;
-    const R S_pcm = (hm - hm_base) * P.x_pm;
-
-    // PCM (Eq. 32) and metal (Eq. 43) collisions side by side
-    R neg[QT], nem[QT];
-    neq_pcm<R, QT>(P, n.H, n.Tf, n.ux, n.uy, neg);
-    neq_metal<R, QT>(P, n.Tm, nem);
-    V2<R> nr[QT];
-#pragma unroll
-    for (int k = 1; k < QT; ++k) nr[k] = P.nrate[QT == 5 && k == 2 ? 1 : k];   // D2Q5: j_x, j_y share a rate (App. B)
-    if (PH && P.phase_k) {
-        // Eq. 9 at the node's liquid fraction -> zeta_alpha (Eq. A19) -> zeta_e (Eq. 53)
-        const R za = fast_rcp(R(0.5) + P.ks_c + n.fl * (P.kl_c - P.ks_c));
-#pragma unroll
-        for (int k = 1; k < QT; ++k) nr[k].x = -(P.zr_a[k] + P.zr_b[k] * za);
-    }
-#pragma unroll
-    for (int k = 1; k < QT; ++k) {
-        // both equilibria vanish for k = 4 (D2Q5) and k = 7, 8 (D2Q9)
-        const bool zero = QT == 5 ? k == 4 : k >= 7;
-        const V2<R> d = zero ? n.th[k] : sub2(n.th[k], V2<R>{neg[k], nem[k]});
-        n.th[k] = fma2(nr[k], d, n.th[k]);
-    }
-    if constexpr (QT == 9) {
-        n.th[1] = fma2(V2<R>{R(-2), R(-2)}, V2<R>{S_pcm, S_met}, n.th[1]);
-        n.th[2] = add2(n.th[2], V2<R>{S_pcm, S_met});
-    } else {
-        n.th[3] = fma2(V2<R>{P.varpi, P.varpi}, V2<R>{S_pcm, S_met}, n.th[3]);
-    }
-    // n_0* = H + S_PCM (n_0 is conserved up to the source, Eq. 32)
-    R hi, lo;
-    if constexpr (kComp<M>) {
-        const FF n0 = ff_add(FF{n.th[0].x, n.Hlo}, S_pcm);
-        hi = n0.hi;
-        lo = n0.lo;
-    } else {
-        hi = n.th[0].x + S_pcm;
-        lo = R(0);
-    }
-    store_thermal<M, QT, FLOW>(P, n.th, hi, lo, hm, db, dw, PS);
     return dTn;
+}
+
+// Non-finite or runaway state: raises the sticky flag (no trap).  A NaN
+// anywhere fails a comparison; the sum overflows if any term is huge.
+template <typename R>
+__device__ __forceinline__ bool runaway(R H, R Tm, R rho, R um) {
+    return !(fabs(H) + fabs(Tm) + rho < R(1e30)) || !(rho > R(0)) || !(um <= R(0.3));
+}
+
+template <int M, int QT, bool FLOW, typename T>
+__device__ __forceinline__ void check_state(const StepParams<typename ModeTraits<M>::R>& P,
+                                            const NodeState<M, QT, FLOW, T>& n) {
+    bool bad;
+    if constexpr (Lane<T>::n == 2)
+        bad = runaway(n.n[0].x, n.k[0].x, n.rho.x, n.um.x) || runaway(n.n[0].y, n.k[0].y, n.rho.y, n.um.y);
+    else
+        bad = runaway(n.n[0], n.k[0], n.rho, n.um);
+    if (bad) atomicOr(P.status, STATUS_UNSTABLE);
 }
 
 // Node (x, y)'s element in bulk plane 0 and in wide plane 0 (16-bit modes) of
@@ -1029,32 +1102,44 @@ __device__ __forceinline__ float* next_wide(const StepParams<typename ModeTraits
     }
 }
 
-// One time step of node (x, y): steps a1-a9 (pull, walls, state, blend,
-// velocity, three collisions, store).  PH = true compiles the Eq. 9 variant's
-// per-node PCM rates in (taken where P.phase_k is set); PH = false leaves them
-// out of the kernel altogether.
+// One time step of a node (pair) whose neighbourhood the accessor a reads:
+// steps a1-a9 (pull, walls, state, blend, velocity, three collisions, store).
+// PH = true compiles the Eq. 9 variant's per-node PCM rates in (taken where
+// P.phase_k is set); PH = false leaves them out of the kernel altogether.
+// The history is read before any store: the compiler cannot move it above
+// stores that may alias it, and a load after them adds a memory round trip to
+// the step.  Returns the new history.
+template <int M, int QT, bool FLOW, bool PH, int PS, typename T, typename A>
+__device__ __forceinline__ T advance(const StepParams<typename ModeTraits<M>::R>& P, const A& a, const WallAt<T>& w,
+                                     const typename Lane<T>::R* history, typename ModeTraits<M>::B* db, float* dw) {
+    NodeState<M, QT, FLOW, T> n;
+    T dTp;
+    if constexpr (Lane<T>::n == 1) dTp = get_real<T>(history);
+    node_state<M, QT, FLOW, T>(P, a, w, n);
+    flow_collide<M, QT, FLOW, PS, T>(P, n, db);
+    if constexpr (Lane<T>::n == 2) dTp = get_real<T>(history);
+    const T dTn = thermal_collide<M, QT, FLOW, PH, PS, T>(P, n, dTp, db, dw);
+    check_state<M, QT, FLOW, T>(P, n);
+    return dTn;
+}
+
+// One time step of node (x, y) from the state copy to the next.
 template <int M, int QT, bool FLOW, bool PH = false>
 __device__ __forceinline__ void step_node(const StepParams<typename ModeTraits<M>::R>& P, int x, int y) {
-    using R = typename ModeTraits<M>::R;
-    NodeState<M, QT, FLOW> n;
-    bool wall;
-    node_state<M, QT, FLOW>(P, x, y, n, wall);
+    using T = Node1<M>;
+    const WallAt<T> w(P, x, y);
+    T* h = P.dT + (y * P.pitch + x);
+    *h = advance<M, QT, FLOW, PH, kChunk, T>(P, PullAt<M, QT, FLOW>(P, w.xs, w.ys), w, h,
+                                              next_bulk<M, QT, FLOW>(P, x, y), next_wide<M, QT, FLOW>(P, x, y));
+}
 
-    const int o = y * P.pitch + x;                                  // exchange history
-    // read before any store: the compiler cannot move it above stores that may
-    // alias it, and a load after them adds a memory round trip to the step
-    // (256^2 FP32: 2.47 -> 2.37 us per step)
-    const R dTp = P.dT[o];
-    typename ModeTraits<M>::B* db = next_bulk<M, QT, FLOW>(P, x, y);
-    float* dw = next_wide<M, QT, FLOW>(P, x, y);
-    flow_collide<M, QT, FLOW>(P, n, db);
-    P.dT[o] = thermal_collide<M, QT, FLOW, PH>(P, n, dTp, db, dw);
-
-    // non-finite or runaway state: raise the sticky flag (no trap)
-    // (a NaN anywhere fails a comparison; the sum overflows if any term is huge)
-    const bool bad = !(fabs(n.H) + fabs(n.Tm) + n.rho < R(1e30)) || !(n.rho > R(0)) ||
-                     !(n.ux * n.ux + n.uy * n.uy <= R(0.09));
-    if (bad) atomicOr(P.status, STATUS_UNSTABLE);
+// One time step of the node pair (x0, x0 + 1), x0 even, both in the grid.
+template <int M, int QT, bool PH = false>
+__device__ __forceinline__ void step_pair(const StepParams<float>& P, int x0, int y) {
+    const WallAt<W> w(P, x0, y);
+    float* h = P.dT + (y * P.pitch + x0);
+    put_real(h, advance<M, QT, true, PH, kChunk, W>(P, PairAt<M, QT>(P, x0, w.ys), w, h,
+                                                     next_bulk<M, QT, true>(P, x0, y), next_wide<M, QT, true>(P, x0, y)));
 }
 
 // Blocks of 256 threads each SM must hold, which caps the registers per
@@ -1188,9 +1273,9 @@ __device__ __forceinline__ void step2_tile(const StepParams<typename ModeTraits<
     R* sdT = reinterpret_cast<R*>(t2_smem + TL::dT_off);
     const int H = blockDim.y;   // blockDim.x == kT2W, H <= HM
     const int lx = threadIdx.x, ly = threadIdx.y, i = ly * kT2W + lx;
-    const int X0 = t2_origin(bx, kT2W - 2, P.nx), Y0 = t2_origin(by, H - 2, P.ny);
+    const int x2 = t2_origin(bx, kT2W - 2, P.nx) + lx, y2 = t2_origin(by, H - 2, P.ny) + ly;
     // step-1 node: coordinates wrapped on periodic sides, none beyond a walled side
-    int x = X0 + lx, y = Y0 + ly;
+    int x = x2, y = y2;
     bool live = true;
     if (x < 0 || x >= P.nx) {
         if (P.per_x) x = ((x % P.nx) + P.nx) % P.nx;
@@ -1202,30 +1287,17 @@ __device__ __forceinline__ void step2_tile(const StepParams<typename ModeTraits<
     }
     griddep_wait();
     if (live) {
-        NodeState<M, QT, true> n;
-        bool wall;
-        node_state<M, QT, true>(P, x, y, n, wall);
-        const R dTp = P.dT[y * P.pitch + x];
-        flow_collide<M, QT, true>(P, n, sb + i, TL::n);
-        sdT[i] = thermal_collide<M, QT, true, PH>(P, n, dTp, sb + i, kSplit<M> ? sw + i : nullptr, TL::n);
-        const bool bad = !(fabs(n.H) + fabs(n.Tm) + n.rho < R(1e30)) || !(n.rho > R(0)) ||
-                         !(n.ux * n.ux + n.uy * n.uy <= R(0.09));
-        if (bad) atomicOr(P.status, STATUS_UNSTABLE);
+        const WallAt<R> w(P, x, y);
+        sdT[i] = advance<M, QT, true, PH, TL::n, R>(P, PullAt<M, QT, true>(P, w.xs, w.ys), w, P.dT + (y * P.pitch + x),
+                                                     sb + i, sw + i);
     }
     __syncthreads();
     // step 2: the inner nodes of the tile that lie in the grid
-    const int x2 = X0 + lx, y2 = Y0 + ly;
     if (lx < 1 || lx > kT2W - 2 || ly < 1 || ly > H - 2 || x2 >= P.nx || y2 >= P.ny) return;
-    const WallAt wa = wall_at(P, x2, y2);
-    const PullTile<M, TL::n> a{sb, sw, i + (wa.ys - y2) * kT2W + (wa.xs - x2)};
-    NodeState<M, QT, true> n;
-    node_state_from<M, QT, true>(P, a, wa, n);
-    flow_collide<M, QT, true>(P, n, next_bulk<M, QT, true>(P, x2, y2));
-    P.dT_out[y2 * P.pitch + x2] =
-        thermal_collide<M, QT, true, PH>(P, n, sdT[i], next_bulk<M, QT, true>(P, x2, y2), next_wide<M, QT, true>(P, x2, y2));
-    const bool bad = !(fabs(n.H) + fabs(n.Tm) + n.rho < R(1e30)) || !(n.rho > R(0)) ||
-                     !(n.ux * n.ux + n.uy * n.uy <= R(0.09));
-    if (bad) atomicOr(P.status, STATUS_UNSTABLE);
+    const WallAt<R> w(P, x2, y2);
+    const PullTile<M, TL::n> a{sb, sw, i + (w.ys - y2) * kT2W + (w.xs - x2)};
+    P.dT_out[y2 * P.pitch + x2] = advance<M, QT, true, PH, kChunk, R>(
+        P, a, w, sdT + i, next_bulk<M, QT, true>(P, x2, y2), next_wide<M, QT, true>(P, x2, y2));
 }
 
 template <int M, int QT, bool PH, int HM>
@@ -1236,426 +1308,11 @@ __global__ void __launch_bounds__(kT2W * HM, (kT2Blocks<HM, M, QT>)) fused_step2
 // ---------------------------------------------------------------------------
 // Two nodes per thread
 // ---------------------------------------------------------------------------
-// Large grids of the default configuration (flow, D2Q5 thermal lattices,
-// volumetric blend, FP32/FP16/BF16 storage) advance node pairs (x0, x0 + 1),
-// x0 even, one pair per thread.  Every FP32 operation of the step is one
-// packed instruction for both nodes (lane x: node x0, lane y: node x0 + 1),
-// the parameter loads and the index arithmetic serve both nodes, and the pair
-// is read and written with one access per plane wherever both elements are
-// adjacent (x0 even keeps them inside one chunk, aligned).  The arithmetic is
-// that of step_node, operation for operation, except where noted; a pair with
-// a wall node (or without a second node) goes through step_node instead.
-
-using W = V2<float>;
-
-__device__ __forceinline__ W wb(float s) { return {s, s}; }
-__device__ __forceinline__ W wmin(W a, float b) { return {fminf(a.x, b), fminf(a.y, b)}; }
-__device__ __forceinline__ W wmax0(W a) { return {fmaxf(a.x, 0.0f), fmaxf(a.y, 0.0f)}; }
-__device__ __forceinline__ W wsat(W a) { return {__saturatef(a.x), __saturatef(a.y)}; }
-__device__ __forceinline__ W wrcp(W a) { return {__fdividef(1.0f, a.x), __fdividef(1.0f, a.y)}; }
-__device__ __forceinline__ W wsqrt(W a) { return {fast_sqrt(a.x), fast_sqrt(a.y)}; }
-
-// two adjacent elements of a plane (16-bit: one 32-bit access; FP32: 64-bit)
-template <int M>
-__device__ __forceinline__ W ldw(const char* p) {
-    if constexpr (M == MODE_F16) {
-        const float2 f = __half22float2(__ldg(reinterpret_cast<const __half2*>(p)));
-        return {f.x, f.y};
-    } else if constexpr (M == MODE_BF16) {
-        const float2 f = __bfloat1622float2(__ldg(reinterpret_cast<const __nv_bfloat162*>(p)));
-        return {f.x, f.y};
-    } else {
-        const float2 f = __ldg(reinterpret_cast<const float2*>(p));
-        return {f.x, f.y};
-    }
-}
-
-// stores v; returns the stored values as a reader decodes them
-template <int M>
-__device__ __forceinline__ W stw(char* p, W v) {
-    if constexpr (M == MODE_F16) {
-        const __half2 h = __floats2half2_rn(v.x, v.y);
-        *reinterpret_cast<__half2*>(p) = h;
-        const float2 f = __half22float2(h);
-        return {f.x, f.y};
-    } else if constexpr (M == MODE_BF16) {
-        const __nv_bfloat162 h = __floats2bfloat162_rn(v.x, v.y);
-        *reinterpret_cast<__nv_bfloat162*>(p) = h;
-        const float2 f = __bfloat1622float2(h);
-        return {f.x, f.y};
-    } else {
-        *reinterpret_cast<float2*>(p) = make_float2(v.x, v.y);
-        return v;
-    }
-}
-
-__device__ __forceinline__ W ldwf(const char* p) {   // two adjacent FP32 elements
-    const float2 f = __ldg(reinterpret_cast<const float2*>(p));
-    return {f.x, f.y};
-}
-
-__device__ __forceinline__ void stwf(char* p, W v) { *reinterpret_cast<float2*>(p) = make_float2(v.x, v.y); }
-
-struct FW {
-    W hi, lo;
-};
-
-__device__ __forceinline__ FW two_sum(W a, W b) {   // Knuth, lane by lane
-    const W s = add2(a, b);
-    const W bb = sub2(s, a);
-    return {s, add2(sub2(a, sub2(s, bb)), sub2(b, bb))};
-}
-
-__device__ __forceinline__ FW fast_two_sum(W a, W b) {   // Dekker, |a| >= |b|
-    const W s = add2(a, b);
-    return {s, sub2(b, sub2(s, a))};
-}
-
-// as ff_accumulate<5>
-__device__ __forceinline__ FW fw_accumulate(FW a, const W* v, float sign) {
-    W s = a.hi, c = a.lo;
-#pragma unroll
-    for (int i = 1; i < 5; ++i) {
-        const FW t = two_sum(s, sign == 1.0f ? v[i] : mul2(wb(sign), v[i]));
-        s = t.hi;
-        c = add2(c, t.lo);
-    }
-    return fast_two_sum(s, c);
-}
-
-__device__ __forceinline__ void enthalpy_state(const StepParams<float>& P, W H, W& T, W& fl) {
-    fl = wsat(mul2(sub2(H, wb(P.H_fs)), wb(P.inv_dH)));
-    T = add2(fma2(fl, wb(P.dT_sl), wmin(mul2(H, wb(P.inv_c_ps)), P.T_fs)), wmax0(sub2(H, wb(P.H_fl))));
-}
-
-__device__ __forceinline__ W pcm_ref(const StepParams<float>& P, W g0) {
-    const W a = fma2(wsat(mul2(sub2(g0, wb(P.g0_fs)), wb(P.inv_dg0))), wb(P.cr_dsl), wmin(mul2(g0, wb(P.cr_solid)), P.cr_fs));
-    return fma2(wmax0(sub2(g0, wb(P.g0_fl))), wb(P.cr_liquid), a);
-}
-
-// D2Q5 moments of one lattice (Eq. B1) and back
-__device__ __forceinline__ void m_from_f5w(const W* g, W* n) {
-    const W a = add2(g[1], g[3]), b = add2(g[2], g[4]);
-    n[1] = sub2(g[1], g[3]);
-    n[2] = sub2(g[2], g[4]);
-    n[3] = add2(a, b);
-    n[4] = sub2(a, b);
-    n[0] = add2(g[0], n[3]);
-}
-
-__device__ __forceinline__ void f_from_m5w(const W* n, W* g) {
-    const W p = mul2(add2(n[3], n[4]), wb(0.25f)), q = mul2(sub2(n[3], n[4]), wb(0.25f));
-    g[0] = sub2(n[0], n[3]);
-    g[1] = fma2(wb(0.5f), n[1], p);
-    g[3] = fma2(wb(-0.5f), n[1], p);
-    g[2] = fma2(wb(0.5f), n[2], q);
-    g[4] = fma2(wb(-0.5f), n[2], q);
-}
-
-// Source of a node pair's pulled neighbourhood in the state copy in global
-// memory: plane `plane` in source row r (0: y - 1, 1: y, 2: y + 1) of the pair
-// (x0, x0 + 1), of its west neighbours (x0 - 1, x0) and of its east ones
-// (x0 + 1, x0 + 2); the wide planes (16-bit modes) of the pair and of the
-// nodes x0 - 1, x0 + 2; the pair's exchange history.
-template <int M>
-struct PairAt {
-    using B = typename ModeTraits<M>::B;
-    using CH = Chunk<M, 5, true>;
-    static constexpr int es = (int)sizeof(B);
-    static constexpr int pb = kChunk * es;   // bytes from one bulk plane to the next
-    static constexpr int wpl = kChunk * 4;   // bytes from one wide plane to the next
-    const char* row[3];
-    int c0, cm, cp, w0, wm, wp;
-    const float* dT;
-    __device__ __forceinline__ PairAt(const StepParams<float>& P, int x0, int y) {
-        // neighbour columns of the pair (periodic wrap; no walls reach here)
-        const int xm = x0 == 0 ? P.nx - 1 : x0 - 1;   // west of x0
-        const int xp = x0 + 2 == P.nx ? 0 : x0 + 2;   // east of x0 + 1
-        const int ym = y == 0 ? P.ny - 1 : y - 1;
-        const int yp = y == P.ny - 1 ? 0 : y + 1;
-        const int rb = P.cpr * CH::bytes;
-        row[0] = P.src + (long long)ym * rb;
-        row[1] = P.src + (long long)y * rb;
-        row[2] = P.src + (long long)yp * rb;
-        c0 = col_off<M, 5, true>(x0);
-        cm = col_off<M, 5, true>(xm);
-        cp = col_off<M, 5, true>(xp);
-        w0 = c0 + CH::wide_off + (x0 & (kChunk - 1)) * 2;   // wide element of x0
-        wm = cm + CH::wide_off + (xm & (kChunk - 1)) * 2;
-        wp = cp + CH::wide_off + (xp & (kChunk - 1)) * 2;
-        dT = P.dT + (long long)y * P.pitch + x0;
-    }
-    __device__ __forceinline__ W own(int r, int q) const { return ldw<M>(row[r] + c0 + q * pb); }
-    __device__ __forceinline__ W west(int r, int q) const {
-        return W{ldb<M>(reinterpret_cast<const B*>(row[r] + cm + q * pb)),
-                 ldb<M>(reinterpret_cast<const B*>(row[r] + c0 + q * pb))};
-    }
-    __device__ __forceinline__ W east(int r, int q) const {
-        return W{ldb<M>(reinterpret_cast<const B*>(row[r] + c0 + q * pb) + 1),
-                 ldb<M>(reinterpret_cast<const B*>(row[r] + cp + q * pb))};
-    }
-    __device__ __forceinline__ W own_wide(int r, int w) const { return ldwf(row[r] + w0 + w * wpl); }
-    __device__ __forceinline__ float west_wide(int r, int w) const {
-        return __ldg(reinterpret_cast<const float*>(row[r] + wm + w * wpl));
-    }
-    __device__ __forceinline__ float east_wide(int r, int w) const {
-        return __ldg(reinterpret_cast<const float*>(row[r] + wp + w * wpl));
-    }
-    __device__ __forceinline__ W history() const { return ldwf(reinterpret_cast<const char*>(dT)); }
-};
-
-// One time step of the node pair (x0, x0 + 1) of row y, its neighbourhood
-// read through the source S (PairAt or a staged copy in shared memory); the
-// results go to the next copy and the history array in global memory.
-template <int M, bool PH, typename S>
-__device__ __forceinline__ void step_pair_from(const StepParams<float>& P, const S& src, int x0, int y) {
-    using PL = Planes<M, 5, true>;
-    using CH = Chunk<M, 5, true>;
-    constexpr int pb = kChunk * (int)sizeof(typename ModeTraits<M>::B);   // plane stride of the next copy
-    const int c0 = col_off<M, 5, true>(x0);
-    const int rb = P.cpr * CH::bytes;
-    auto own = [&](int r, int q) { return src.own(r, q); };
-    auto west = [&](int r, int q) { return src.west(r, q); };
-    auto east = [&](int r, int q) { return src.east(r, q); };
-
-    // ---- pull (Eq. 15) and flow moments (Eq. 13) ----
-    W f[9] = {own(1, 0), west(1, 1), own(0, 2), east(1, 3), own(2, 4), west(0, 5), east(0, 6), east(2, 7), west(2, 8)};
-    if constexpr (M == MODE_F16) {
-#pragma unroll
-        for (int q = 0; q < 9; ++q) f[q] = mul2(f[q], wb(1.0f / 1024.0f));
-    }
-    W m[9];
-    {
-        const W A13 = add2(f[1], f[3]), A24 = add2(f[2], f[4]), dx = sub2(f[1], f[3]), dy = sub2(f[2], f[4]);
-        const W B57 = add2(f[5], f[7]), B68 = add2(f[6], f[8]), E57 = sub2(f[5], f[7]), E68 = sub2(f[6], f[8]);
-        const W s14 = add2(A13, A24), s58 = add2(B57, B68);
-        const W ax = sub2(E57, E68), ay = add2(E57, E68);
-        m[0] = add2(add2(f[0], s14), s58);
-        m[1] = fma2(wb(2.0f), s58, fma2(wb(-1.0f), s14, mul2(wb(-4.0f), f[0])));
-        m[2] = fma2(wb(-2.0f), s14, fma2(wb(4.0f), f[0], s58));
-        m[3] = add2(dx, ax);
-        m[5] = add2(dy, ay);
-        m[4] = fma2(wb(-2.0f), dx, ax);
-        m[6] = fma2(wb(-2.0f), dy, ay);
-        m[7] = sub2(A13, A24);
-        m[8] = sub2(B57, B68);
-    }
-
-    // ---- thermal pull: PCM g, metal h (Eqs. 33, 44; App. B) ----
-    W g[5], h[5];
-    W Hlo = wb(0.0f);
-    if constexpr (kSplit<M>) {
-        const W g0o = src.own_wide(1, 0), h0o = src.own_wide(1, 1);
-        // senders' rest populations for movers 1..4 (from x - e_q)
-        const W sg[5] = {g0o, W{src.west_wide(1, 0), g0o.x}, src.own_wide(0, 0), W{g0o.y, src.east_wide(1, 0)},
-                         src.own_wide(2, 0)};
-        const W sh[5] = {h0o, W{src.west_wide(1, 1), h0o.x}, src.own_wide(0, 1), W{h0o.y, src.east_wide(1, 1)},
-                         src.own_wide(2, 1)};
-        const W dg[5] = {wb(0.0f), west(1, PL::pcm(1)), own(0, PL::pcm(2)), east(1, PL::pcm(3)), own(2, PL::pcm(4))};
-        const W dh[5] = {wb(0.0f), west(1, PL::met(1)), own(0, PL::met(2)), east(1, PL::met(3)), own(2, PL::met(4))};
-        const float wg = P.wmv[1].x, wk = P.wmv[1].y;   // D2Q5: one weight for all movers (App. B)
-        g[0] = g0o;
-        h[0] = h0o;
-#pragma unroll
-        for (int q = 1; q < 5; ++q) {
-            g[q] = fma2(wb(wg), pcm_ref(P, sg[q]), dg[q]);
-            h[q] = fma2(wb(wk), sh[q], dh[q]);
-        }
-    } else {
-        g[0] = own(1, PL::pcm(0));
-        h[0] = own(1, PL::met(0));
-        g[1] = west(1, PL::pcm(1)); g[2] = own(0, PL::pcm(2)); g[3] = east(1, PL::pcm(3)); g[4] = own(2, PL::pcm(4));
-        h[1] = west(1, PL::met(1)); h[2] = own(0, PL::met(2)); h[3] = east(1, PL::met(3)); h[4] = own(2, PL::met(4));
-    }
-    W ng[5], nh[5];
-    m_from_f5w(g, ng);
-    m_from_f5w(h, nh);
-    if constexpr (kComp<M>) {   // H = (g_0 hi + g_0 lo) + sum of movers, without rounding loss
-        const FW H = fw_accumulate(FW{g[0], own(1, PL::lo)}, g, 1.0f);
-        ng[0] = H.hi;
-        Hlo = H.lo;
-    }
-
-    // ---- macroscopic state (Eqs. 21, 23-25, 37-39, 7) ----
-    const W H = ng[0];
-    W Tf, fl;
-    enthalpy_state(P, H, Tf, fl);
-    const W Tm = nh[0];
-    const W drho = m[0];
-    const W rho = add2(wb(1.0f), drho);
-    const W Gy = mul2(mul2(wb(P.gbeta), sub2(Tf, wb(P.T0))), fl);
-    W ux, uy, um;
-    {
-        const W ir = wrcp(rho);
-        const W vx = mul2(mul2(fl, m[3]), ir);
-        const W vy = fma2(wb(0.5f * P.phi), Gy, mul2(mul2(fl, m[5]), ir));
-        const W vm = wsqrt(fma2(vy, vy, mul2(vx, vx)));
-        W r = wsqrt(fma2(wb(P.l1), vm, wb(P.l0sq)));
-        const W den = wrcp(add2(wb(P.l0), r));   // Eq. 23
-        ux = mul2(vx, den);
-        uy = mul2(vy, den);
-        um = mul2(vm, den);
-    }
-
-    // ---- flow collision (Eqs. 3, 14, 18-20) ----
-    char* dst = P.dst + (long long)y * rb;
-    {
-        const W nd = fma2(wb(-P.drag_forch), um, wb(-P.drag_lin));   // -(drag)
-        const W Fx = mul2(nd, ux), Fy = fma2(nd, uy, mul2(wb(P.phi), Gy));
-        const W sol = mul2(sub2(wb(1.0f), fl), drho);
-        W b1 = fma2(fl, m[1], mul2(wb(-2.0f), sol)), b2 = fma2(fl, m[2], sol);
-        W b4 = mul2(fl, m[4]), b6 = mul2(fl, m[6]), b7 = mul2(fl, m[7]), b8 = mul2(fl, m[8]);
-        const W rip = mul2(rho, wb(P.inv_phi));
-        const W uxx = mul2(ux, ux), uyy = mul2(uy, uy), uxy = mul2(ux, uy);
-        const W q = mul2(mul2(wb(3.0f), rip), add2(uxx, uyy));
-        const W me1 = fma2(wb(-2.0f), drho, q), me2 = sub2(drho, q);
-        const W Jx = mul2(rho, ux), Jy = mul2(rho, uy);
-        const W me7 = mul2(rip, sub2(uxx, uyy)), me8 = mul2(rip, uxy);
-        const W s1 = mul2(mul2(wb(6.0f), rip), fma2(uy, Fy, mul2(ux, Fx)));
-        const W RFx = mul2(rho, Fx), RFy = mul2(rho, Fy);
-        const W S7 = mul2(rip, mul2(wb(2.0f), sub2(mul2(ux, Fx), mul2(uy, Fy))));
-        const W S8 = mul2(rip, fma2(uy, Fx, mul2(ux, Fy)));
-        b1 = fma2(wb(0.45f), s1, fma2(wb(-1.1f), sub2(b1, me1), b1));
-        b2 = fma2(wb(-0.45f), s1, fma2(wb(-1.1f), sub2(b2, me2), b2));
-        const W b3 = fma2(wb(0.5f), RFx, Jx), b5 = fma2(wb(0.5f), RFy, Jy);
-        b4 = fma2(wb(-0.4f), RFx, fma2(wb(-1.2f), add2(b4, Jx), b4));
-        b6 = fma2(wb(-0.4f), RFy, fma2(wb(-1.2f), add2(b6, Jy), b6));
-        const float sv = P.s[7], hv = 1.0f - 0.5f * sv;
-        b7 = fma2(wb(hv), S7, fma2(wb(-sv), sub2(b7, me7), b7));
-        b8 = fma2(wb(hv), S8, fma2(wb(-sv), sub2(b8, me8), b8));
-        // f = M^-1 m* (as f_from_m9p), scaled by the storage scale
-        constexpr float sc = (float)kFlowScale<M>;
-        const W A = mul2(drho, wb(sc / 9.0f)), Bm = mul2(b1, wb(sc / 36.0f)), C = mul2(b2, wb(sc / 36.0f));
-        const W DX = mul2(b3, wb(sc / 6.0f)), QX = mul2(b4, wb(sc / 12.0f));
-        const W DY = mul2(b5, wb(sc / 6.0f)), QY = mul2(b6, wb(sc / 12.0f));
-        const W Pm = mul2(b7, wb(sc * 0.25f)), Sm = mul2(b8, wb(sc * 0.25f));
-        const W f0 = fma2(wb(4.0f), C, fma2(wb(-4.0f), Bm, A));
-        const W bb1 = fma2(wb(-2.0f), C, sub2(A, Bm));
-        const W bb5 = add2(fma2(wb(2.0f), Bm, A), C);
-        const W Tx = fma2(wb(-2.0f), QX, DX), Ty = fma2(wb(-2.0f), QY, DY);
-        const W X = add2(DX, QX), Y = add2(DY, QY);
-        const W bp = add2(bb1, Pm), bm = sub2(bb1, Pm);
-        const W G5 = add2(bb5, Sm), G6 = sub2(bb5, Sm), H5 = add2(X, Y), H6 = sub2(Y, X);
-        const W fo[9] = {f0, add2(bp, Tx), add2(bm, Ty), sub2(bp, Tx), sub2(bm, Ty),
-                         add2(G5, H5), add2(G6, H6), sub2(G5, H5), sub2(G6, H6)};
-#pragma unroll
-        for (int k = 0; k < 9; ++k) stw<M>(dst + c0 + k * pb, fo[k]);
-    }
-
-    // ---- exchange sources (Eqs. 36, 47, Remark III) ----
-    // (the history is read here, after the flow stores: read with the other
-    // loads it stays live through the step and costs FP16 a spill, 72.9
-    // against 70.2 us per step at 2048^2)
-    float* dTp_ptr = P.dT + (long long)y * P.pitch + x0;
-    const W dTn = sub2(Tm, Tf);
-    const W dTp = src.history();
-    const W Sx = fma2(wb(1.5f), dTn, mul2(wb(-0.5f), dTp));
-    const W S_met = mul2(wb(-P.a_m), Sx);
-    W hm_base;
-    if constexpr (kSplit<M>) hm_base = nh[0];
-    else hm_base = fma2(wb(-P.eta[0]), sub2(nh[0], Tm), nh[0]);
-    const W hm = add2(hm_base, S_met);
-    const W S_pcm = mul2(sub2(hm, hm_base), wb(P.x_pm));
-
-    // ---- PCM (Eq. 32) and metal (Eq. 43) collisions ----
-    {
-        const W t = mul2(Tf, wb(P.inv_phi));
-        const W ne1 = mul2(t, ux), ne2 = mul2(t, uy), ne3 = mul2(wb(P.vcf), Tf);
-        W nz[5];
-        if (PH && P.phase_k) {   // Eq. 9 -> zeta_alpha (Eq. A19) -> zeta_e (Eq. 53)
-            const W za = wrcp(add2(wb(0.5f + P.ks_c), mul2(fl, wb(P.kl_c - P.ks_c))));
-#pragma unroll
-            for (int k = 1; k < 5; ++k) nz[k] = mul2(wb(-1.0f), fma2(wb(P.zr_b[k]), za, wb(P.zr_a[k])));
-        } else {
-            nz[1] = nz[2] = wb(P.nrate[1].x);
-            nz[3] = wb(P.nrate[3].x);
-            nz[4] = wb(P.nrate[4].x);
-        }
-        ng[1] = fma2(nz[1], sub2(ng[1], ne1), ng[1]);
-        ng[2] = fma2(nz[2], sub2(ng[2], ne2), ng[2]);
-        ng[3] = fma2(nz[3], sub2(ng[3], ne3), ng[3]);
-        ng[4] = fma2(nz[4], ng[4], ng[4]);
-        const float ne_j = P.nrate[1].y;
-        nh[1] = fma2(wb(ne_j), nh[1], nh[1]);
-        nh[2] = fma2(wb(ne_j), nh[2], nh[2]);
-        nh[3] = fma2(wb(P.nrate[3].y), sub2(nh[3], mul2(wb(P.vcm), Tm)), nh[3]);
-        nh[4] = fma2(wb(P.nrate[4].y), nh[4], nh[4]);
-        ng[3] = fma2(wb(P.varpi), S_pcm, ng[3]);
-        nh[3] = fma2(wb(P.varpi), S_met, nh[3]);
-    }
-    // n_0* = H + S_PCM (Eq. 32), metal n_0* = hm
-    W n0hi, n0lo = wb(0.0f);
-    if constexpr (kComp<M>) {
-        const FW s = two_sum(ng[0], S_pcm);
-        const FW n0 = fast_two_sum(s.hi, add2(s.lo, Hlo));
-        n0hi = n0.hi;
-        n0lo = n0.lo;
-    } else {
-        n0hi = add2(ng[0], S_pcm);
-    }
-
-    // ---- thermal store: movers, then the rest populations as remainders ----
-    W vg[5], vh[5];
-    ng[0] = n0hi;
-    nh[0] = hm;
-    f_from_m5w(ng, vg);
-    f_from_m5w(nh, vh);
-    if constexpr (kSplit<M>) {
-        // as store_thermal: deviations from the provisional rest population's
-        // reference, then the rest population that closes the balance
-        const W ref = pcm_ref(P, vg[0]);
-        const float nwg = P.nwmv[1].x, nwk = P.nwmv[1].y;
-        W sdg, sdh;
-#pragma unroll
-        for (int k = 1; k < 5; ++k) {
-            const W dgk = stw<M>(dst + c0 + PL::pcm(k) * pb, fma2(wb(nwg), ref, vg[k]));
-            const W dhk = stw<M>(dst + c0 + PL::met(k) * pb, fma2(wb(nwk), vh[0], vh[k]));
-            sdg = k == 1 ? dgk : add2(sdg, dgk);
-            sdh = k == 1 ? dhk : add2(sdh, dhk);
-        }
-        const W Yg = sub2(n0hi, sdg), Yh = sub2(hm, sdh);
-        W T, f_;
-        enthalpy_state(P, Yg, T, f_);
-        const int w0 = c0 + CH::wide_off + (x0 & (kChunk - 1)) * 2;
-        stwf(dst + w0, fma2(wb(-P.om_cf), T, Yg));
-        stwf(dst + w0 + kChunk * 4, mul2(Yh, wb(P.rest_m)));
-    } else {
-#pragma unroll
-        for (int k = 1; k < 5; ++k) {
-            stw<M>(dst + c0 + PL::pcm(k) * pb, vg[k]);
-            stw<M>(dst + c0 + PL::met(k) * pb, vh[k]);
-        }
-        const W smh = add2(add2(add2(vh[1], vh[2]), vh[3]), vh[4]);
-        stw<M>(dst + c0 + PL::met(0) * pb, sub2(hm, smh));
-        if constexpr (kComp<M>) {   // the PCM rest population as a float-float pair
-            const FW r = fw_accumulate(FW{n0hi, n0lo}, vg, -1.0f);
-            stw<M>(dst + c0 + PL::pcm(0) * pb, r.hi);
-            stw<M>(dst + c0 + PL::lo * pb, r.lo);
-        } else {
-            const W smg = add2(add2(add2(vg[1], vg[2]), vg[3]), vg[4]);
-            stw<M>(dst + c0 + PL::pcm(0) * pb, sub2(n0hi, smg));
-        }
-    }
-    stwf(reinterpret_cast<char*>(dTp_ptr), dTn);
-
-    // non-finite or runaway state: raise the sticky flag (no trap)
-    const W a = add2(add2(W{fabsf(H.x), fabsf(H.y)}, W{fabsf(Tm.x), fabsf(Tm.y)}), rho);
-    const W u2 = fma2(uy, uy, mul2(ux, ux));
-    const bool bad = !(a.x < 1e30f) || !(a.y < 1e30f) || !(rho.x > 0.0f) || !(rho.y > 0.0f) ||
-                     !(u2.x <= 0.09f) || !(u2.y <= 0.09f);
-    if (bad) atomicOr(P.status, STATUS_UNSTABLE);
-}
-
-template <int M, bool PH>
-__device__ __forceinline__ void step_pair(const StepParams<float>& P, int x0, int y) {
-    const PairAt<M> src(P, x0, y);
-    step_pair_from<M, PH>(P, src, x0, y);
-}
 
 // Node pairs of the default configuration: a block of 32 x 4 threads covers
 // 64 x 4 nodes; the first of a chunk's two blocks prefetches its rows (2048^2
-// FP16 61.09 against 61.22 us per step when both do).  A pair with a wall node or without a second node (or a run
-// of the bounce-back variant) takes step_node.  Seven blocks per SM cap the
+// FP16 61.09 against 61.22 us per step when both do).  The last node of an odd
+// width steps alone.  Seven blocks per SM cap the
 // registers at 72 (measured best: 80 registers leave too few warps to hide
 // the memory latency, 64 spill).
 template <int M, bool PH>
@@ -1666,14 +1323,8 @@ __global__ void __launch_bounds__(128, 7) fused_step_pair(const __grid_constant_
     griddep_wait();
     if (P.prefetch_rows > 0 && threadIdx.x == 0 && threadIdx.y == 0 && (x0 & (kChunk - 1)) == 0)
         prefetch_rows<M, 5, true>(P, x0, y + P.prefetch_rows, blockDim.y);   // the chunk's first block
-    const bool single = P.solid_scheme || x0 + 1 >= P.nx || (!P.per_x && (x0 == 0 || x0 + 1 == P.nx - 1)) ||
-                        (!P.per_y && (y == 0 || y == P.ny - 1));
-    if (single) {
-        step_node<M, 5, true, PH>(P, x0, y);
-        if (x0 + 1 < P.nx) step_node<M, 5, true, PH>(P, x0 + 1, y);
-        return;
-    }
-    step_pair<M, PH>(P, x0, y);
+    if (x0 + 1 >= P.nx) step_node<M, 5, true, PH>(P, x0, y);
+    else step_pair<M, 5, PH>(P, x0, y);
 }
 
 // Many small runs in one launch per step, each run on the code of the
@@ -1797,11 +1448,10 @@ __global__ void __launch_bounds__(256) fields_kernel(const __grid_constant__ Ste
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x >= P.nx || y >= P.ny) return;
-    NodeState<M, QT, FLOW> n;
-    bool wall;
-    node_state<M, QT, FLOW>(P, x, y, n, wall);
+    NodeState<M, QT, FLOW, R> n;
+    node_state_at<M, QT, FLOW>(P, x, y, n);
     const long long o = (long long)y * out.ld + x;
-    const R v[7] = {n.Tf, n.Tm, n.fl, n.ux, n.uy, n.rho, n.H};   // H: high part
+    const R v[7] = {n.Tf, n.k[0], n.fl, n.ux, n.uy, n.rho, n.n[0]};   // H: high part
 #pragma unroll
     for (int i = 0; i < 7; ++i)
         if (out.mask & (1 << i)) out.dst[i][o] = v[i];
@@ -1822,20 +1472,18 @@ __global__ void __launch_bounds__(256) diag_partial(const __grid_constant__ Step
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     double v[4] = {0.0, 0.0, 0.0, 0.0};
     if (x < P.nx && y < P.ny) {
-        NodeState<M, QT, FLOW> n;
-        bool wall;
-        node_state<M, QT, FLOW>(P, x, y, n, wall);
+        NodeState<M, QT, FLOW, Node1<M>> n;
+        node_state_at<M, QT, FLOW>(P, x, y, n);
         v[0] = (double)n.fl;
-        v[1] = C.phi * C.rho_l * ((double)n.H + (double)n.Hlo) +
-               (1.0 - C.phi) * C.rho_m * C.c_pm * ((double)n.Tm + (double)n.Elo);
+        v[1] = C.phi * C.rho_l * ((double)n.n[0] + (double)n.Hlo) +
+               (1.0 - C.phi) * C.rho_m * C.c_pm * ((double)n.k[0] + (double)n.Elo);
         v[2] = 1.0 + (double)n.drho;
         if (x == 0 && C.left_wall && P.nx >= 3) {
-            NodeState<M, QT, FLOW> n1, n2;
-            bool w1, w2;
-            node_state<M, QT, FLOW>(P, 1, y, n1, w1);
-            node_state<M, QT, FLOW>(P, 2, y, n2, w2);
+            NodeState<M, QT, FLOW, Node1<M>> n1, n2;
+            node_state_at<M, QT, FLOW>(P, 1, y, n1);
+            node_state_at<M, QT, FLOW>(P, 2, y, n2);
             const double gf = 0.5 * (3.0 * (double)n.Tf - 4.0 * (double)n1.Tf + (double)n2.Tf);
-            const double gm = 0.5 * (3.0 * (double)n.Tm - 4.0 * (double)n1.Tm + (double)n2.Tm);
+            const double gm = 0.5 * (3.0 * (double)n.k[0] - 4.0 * (double)n1.k[0] + (double)n2.k[0]);
             // PCM conductivity of the wall node's own liquid fraction (Eq. 9)
             const double kw = C.k_s == C.k_f ? C.k_f : (double)n.fl * C.k_f + (1.0 - (double)n.fl) * C.k_s;
             v[3] = C.phi * kw * gf + (1.0 - C.phi) * C.k_m * gm;
