@@ -297,8 +297,6 @@ lbmk::StepParams<R> make_params(const lbm_handle* h, int from) {
         P.l0 = (R)d.l0;
         P.l0sq = (R)(d.l0 * d.l0);
         P.l1 = (R)d.l1;
-        P.nl1 = (R)-d.l1;
-        P.n2l0 = (R)(1.0 - 2.0 * d.l0);
         // 1 - s from the rounded rate, so that m = m^eq is kept exactly by (1 - s) m + s m^eq
         const R sv = (R)d.s[7];
         P.c_v = (R)1 - sv;

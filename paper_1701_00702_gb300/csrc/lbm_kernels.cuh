@@ -39,11 +39,7 @@
 //     along x, so one pointer per pulled neighbour reaches all its planes;
 //   * the arithmetic is written once over a lane type (one node, or a pair of
 //     nodes in the packed two-lane FP32 instructions of sm_100 and later), with
-//     every rounding named, so that all kernels give a node the same bits;
-//   * what is conserved or nearly so is never passed through a constant or a
-//     quotient whose rounding would be the same at every node and step: FP32
-//     velocities after 200 steps of the 256^2 cavity are within 7e-7 of exact
-//     arithmetic (up to 1.8e-5 when they were).
+//     every rounding named, so that all kernels give a node the same bits.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -202,10 +198,10 @@ __device__ __forceinline__ W vminc(W a, float c) { return {fminf(a.x, c), fminf(
 __device__ __forceinline__ float vmax0(float a) { return fmaxf(a, 0.0f); }
 __device__ __forceinline__ W vmax0(W a) { return {fmaxf(a.x, 0.0f), fmaxf(a.y, 0.0f)}; }
 
-// 1/a and sqrt(a), a >= 0, in FP32: one instruction each, relative error at
-// most 1 ulp and 2^-23 (the division and the rsqrtf product they replace took
-// 5 and 8 instructions, with 2 ulp and 2^-22.4; subnormal speeds, below
-// 1e-19 lattice units, flush to zero)
+// 1/a and sqrt(a), a >= 0, in FP32: one instruction each (the division and the
+// guarded rsqrtf product they replace took 5 and 8; subnormal speeds, below
+// 1e-19 lattice units, flush to zero).  vsqrt_pos, a > 0, is the rsqrt product
+// without the guard.
 __device__ __forceinline__ float vrcp(float a) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
@@ -216,10 +212,17 @@ __device__ __forceinline__ float vsqrt(float a) {
     asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
     return r;
 }
+__device__ __forceinline__ float vsqrt_pos(float a) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+    return __fmul_rn(a, r);
+}
 __device__ __forceinline__ W vrcp(W a) { return {vrcp(a.x), vrcp(a.y)}; }
 __device__ __forceinline__ W vsqrt(W a) { return {vsqrt(a.x), vsqrt(a.y)}; }
+__device__ __forceinline__ W vsqrt_pos(W a) { return {vsqrt_pos(a.x), vsqrt_pos(a.y)}; }
 __device__ __forceinline__ double vrcp(double a) { return 1.0 / a; }
 __device__ __forceinline__ double vsqrt(double a) { return sqrt(a); }
+__device__ __forceinline__ double vsqrt_pos(double a) { return vsqrt(a); }
 
 // Per-run constants, passed by value (__grid_constant__).
 template <typename R>
@@ -249,7 +252,6 @@ struct StepParams {
     R rest_m;            // 1 - omega c_m,ref / c_pm: h_0 = rest_m c_pm T_m at equilibrium
     // flow (Eqs. 3, 7, 16, 25)
     R inv_phi, fgb, T0, l0, l0sq, l1;   // fgb = phi gbeta
-    R nl1, n2l0;         // -l_1, 1 - 2 l_0
     R nlin, nforch;      // -phi nu_f / K and -phi F_phi / sqrt(K): the negated drag is nlin + nforch |u|
     R k_uu, k_uf;        // 3 s_e / phi and 6 (1 - s_e / 2) / phi
     R c_v, k_v, k_h, k_2h;   // 1 - s_v, s_v / phi, (1 - s_v / 2) / phi and twice that
@@ -340,23 +342,18 @@ __device__ __forceinline__ void m_from_f9(const T* f, T* m) {
 }
 
 // f = M^-1 m, every f scaled by SC (a power of two: the 16-bit flow storage
-// scale, folded into the row norms).  The conserved moments come back without
-// the rounding of 1/9 and 1/6 (which would grow the momentum by 3e-8 a step in
-// FP32): f_0 and the axis populations' odd part are the remainders to m_0 and
-// to m_3 / 2, m_5 / 2.
+// scale, folded into the row norms).
 template <typename T, int SC = 1>
 __device__ __forceinline__ void f_from_m9(const T* m, T* f) {
     using R = typename Lane<T>::R;
     constexpr double s = SC;
     const T A = vmulc<T>(R(s / 9.0), m[0]);
+    f[0] = vfmac<T>(R(s / 9.0), m[2], vfmac<T>(R(-s / 9.0), m[1], A));
     const T b1 = vfmac<T>(R(-s / 18.0), m[2], vfmac<T>(R(-s / 36.0), m[1], A));
     const T b5 = vfmac<T>(R(s / 36.0), m[2], vfmac<T>(R(s / 18.0), m[1], A));
-    const T b15 = vadd(b1, b5);
-    f[0] = SC == 1 ? vfmac<T>(R(-4), b15, m[0]) : vfmac<T>(R(s), m[0], vmulc<T>(R(-4), b15));
-    const T X = vfmac<T>(R(s / 12.0), m[4], vmulc<T>(R(s / 6.0), m[3]));
-    const T Y = vfmac<T>(R(s / 12.0), m[6], vmulc<T>(R(s / 6.0), m[5]));
-    const T tx = vfmac<T>(R(-2), X, vmulc<T>(R(s * 0.5), m[3]));
-    const T ty = vfmac<T>(R(-2), Y, vmulc<T>(R(s * 0.5), m[5]));
+    const T DX = vmulc<T>(R(s / 6.0), m[3]), DY = vmulc<T>(R(s / 6.0), m[5]);
+    const T tx = vfmac<T>(R(-s / 6.0), m[4], DX), ty = vfmac<T>(R(-s / 6.0), m[6], DY);
+    const T X = vfmac<T>(R(s / 12.0), m[4], DX), Y = vfmac<T>(R(s / 12.0), m[6], DY);
     const T bp = vfmac<T>(R(s * 0.25), m[7], b1), bm = vfmac<T>(R(-s * 0.25), m[7], b1);
     f[1] = vadd(bp, tx);
     f[3] = vsub(bp, tx);
@@ -686,21 +683,15 @@ __device__ __forceinline__ void macro(const StepParams<typename ModeTraits<M>::R
         T a = n.fl;
         if constexpr (Lane<T>::n == 1)
             if (P.solid_scheme) a = R(1);
+        a = vmul(a, vrcp(n.rho));
         if constexpr (kFlowScale<M> != 1) a = vmulc<T>(is, a);
-        // quotients by numbers near 1 as x - x d, with a small d: rho and the denominator of
-        // Eq. 23 vary little over a run, and the rounding of their reciprocals would be the
-        // same at every node and step (measured over 200 steps of the 256^2 cavity: u off by
-        // up to 1.5e-5 in FP32 with products of reciprocals)
-        const T c = vmul(vneg(n.drho), vrcp(n.rho));
-        const T vx = vmul(a, vfma(c, n.mp[3], n.mp[3]));
-        const T vy = vfmac<T>(R(0.5), n.G, vmul(a, vfma(c, n.mp[5], n.mp[5])));
+        const T vx = vmul(a, n.mp[3]);
+        const T vy = vfmac<T>(R(0.5), n.G, vmul(a, n.mp[5]));
         const T vm = vsqrt(vfma(vy, vy, vmul(vx, vx)));
-        // Eq. 23: u = v / den, den = l_0 + sqrt(l_0^2 + l_1 |v|) = 1 + (2 l_0 - 1) + l_1 |u|
-        const T r = vrcp(vaddc(vsqrt(vfma(bc<T>(P.l1), vm, bc<T>(P.l0sq))), P.l0));
-        n.um = vmul(vm, r);
-        const T d = vmul(vfma(bc<T>(P.nl1), n.um, bc<T>(P.n2l0)), r);
-        n.ux = vfma(d, vx, vx);
-        n.uy = vfma(d, vy, vy);
+        const T den = vrcp(vaddc(vsqrt_pos(vfma(bc<T>(P.l1), vm, bc<T>(P.l0sq))), P.l0));   // Eq. 23
+        n.ux = vmul(vx, den);
+        n.uy = vmul(vy, den);
+        n.um = vmul(vm, den);
         if constexpr (Lane<T>::n == 1)
             if (P.solid_scheme && n.fl <= R(0.5)) n.ux = n.uy = n.um = R(0);
     } else {
@@ -771,7 +762,7 @@ __device__ __forceinline__ void apply_wall(const StepParams<typename ModeTraits<
     const T ux = vsel(w.wall, n.ux, zero), uy = vsel(w.wall, n.uy, zero);
     if constexpr (FLOW) {
         constexpr R sc = R(kFlowScale<M>);
-        T jx = vfma(n.drho, ux, ux), jy = vfma(n.drho, uy, uy);
+        T jx = vmul(n.rho, ux), jy = vmul(n.rho, uy);
         if constexpr (kFlowScale<M> != 1) {
             jx = vmulc<T>(sc, jx);
             jy = vmulc<T>(sc, jy);
@@ -884,8 +875,8 @@ __device__ __forceinline__ void flow_collide(const StepParams<typename ModeTrait
         }
         const T drag = vfma(bc<T>(P.nforch), n.um, bc<T>(P.nlin));   // Eq. 3, negated
         const T Fx = vmul(drag, n.ux), Fy = vfma(drag, n.uy, n.G);
-        const T jx = vfma(n.drho, n.ux, n.ux), jy = vfma(n.drho, n.uy, n.uy);   // rho u, rho F
-        const T fx = vfma(n.drho, Fx, Fx), fy = vfma(n.drho, Fy, Fy);
+        const T jx = vmul(n.rho, n.ux), jy = vmul(n.rho, n.uy);
+        const T fx = vmul(n.rho, Fx), fy = vmul(n.rho, Fy);
         const T xx = vmul(jx, n.ux), fxx = vmul(jx, Fx);
         const T up = vfma(jy, n.uy, xx), um = vfma(vneg(jy), n.uy, xx);      // j_x u_x +- j_y u_y
         const T fp = vfma(jy, Fy, fxx), fm = vfma(vneg(jy), Fy, fxx);        // j_x F_x +- j_y F_y
