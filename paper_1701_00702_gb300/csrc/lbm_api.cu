@@ -329,7 +329,7 @@ lbmk::StepParams<R> make_params(const lbm_handle* h, int from) {
     P.inv_dH = (R)(1.0 / (d.H_fl - d.H_fs));
     P.dT_sl = (R)(p.T_liquidus - p.T_solidus);
     P.T_fs = (R)p.T_solidus;
-    P.T_fl = (R)p.T_liquidus;
+    P.T_off = (R)(p.T_liquidus - d.H_fl);
     P.inv_c_ps = (R)(1.0 / d.c_ps);
     P.c_fref = (R)d.c_fref;
     P.c_mref = (R)d.c_mref;

@@ -220,8 +220,27 @@ __device__ __forceinline__ float vsqrt_pos(float a) {
 __device__ __forceinline__ W vrcp(W a) { return {vrcp(a.x), vrcp(a.y)}; }
 __device__ __forceinline__ W vsqrt(W a) { return {vsqrt(a.x), vsqrt(a.y)}; }
 __device__ __forceinline__ W vsqrt_pos(W a) { return {vsqrt_pos(a.x), vsqrt_pos(a.y)}; }
-__device__ __forceinline__ double vrcp(double a) { return 1.0 / a; }
-__device__ __forceinline__ double vsqrt(double a) { return sqrt(a); }
+// In FP64, where one warp instruction occupies its scheduler's FP64 unit for 64
+// cycles (GB300: two FP64 lanes per SM and clock), from the hardware's seed y
+// (relative error below 2^-20) with one third-order step each: with e = 1 - a y,
+// 1/a = y (1 + e + e^2 + ...), and with e = 1 - a y^2, sqrt(a) = a y (1 + e/2 +
+// 3 e^2/8 + ...) (Householder, The Numerical Treatment of a Single Nonlinear
+// Equation, 1970); the neglected e^3 is below 2^-60.  3 and 5 FP64 operations
+// for the 9 and 10 of the library's correctly rounded ones, within 1 ulp.
+// sqrt gives 0 below 2^-900 (speeds below 1e-135 lattice units).
+__device__ __forceinline__ double vrcp(double a) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+    const double e = vfma(-a, y, 1.0);
+    return vfma(y, vfma(e, e, e), y);
+}
+__device__ __forceinline__ double vsqrt(double a) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+    const double s = vmul(a, y), e = vfma(-s, y, 1.0);
+    const double r = vfma(s, vmul(e, vfma(0.375, e, 0.5)), s);
+    return __double2hiint(a) < (1023 - 900) << 20 ? 0.0 : r;   // (a >= 0; NaN and infinity pass)
+}
 __device__ __forceinline__ double vsqrt_pos(double a) { return vsqrt(a); }
 
 // Per-run constants, passed by value (__grid_constant__).
@@ -257,7 +276,7 @@ struct StepParams {
     R c_v, k_v, k_h, k_2h;   // 1 - s_v, s_v / phi, (1 - s_v / 2) / phi and twice that
     // thermal (Eqs. 38-39, 34, 45, App. B)
     // (c_pl = c_pm = 1 in the lattice units of Eq. 54, so they appear nowhere below)
-    R H_fs, H_fl, inv_dH, T_fs, T_fl, dT_sl, inv_c_ps;   // dT_sl = T_fl - T_fs
+    R H_fs, H_fl, inv_dH, T_fs, T_off, dT_sl, inv_c_ps;   // T_off = T_fl - H_fl, dT_sl = T_fl - T_fs
     R c_fref, c_mref, varpi;
     R vcf, vcm;          // varpi c_f,ref and varpi c_m,ref (D2Q5 equilibria, Eqs. B2, B4)
     R nz[9], ne[9];      // -zeta_k, -eta_k (D2Q9)
@@ -397,9 +416,21 @@ __device__ __forceinline__ void enthalpy_state(const StepParams<float>& P, T H, 
     Tf = vadd(vfmac<T>(P.dT_sl, fl, vminc(vmulc<T>(P.inv_c_ps, H), P.T_fs)), vmax0(vaddc(H, -P.H_fl)));
 }
 
+// In FP64 the branch is chosen by comparing bit patterns (order_key keeps the
+// order of the numbers it maps), which takes no FP64 operation, and T is one
+// multiply-add of the branch's own slope and offset.
+__device__ __forceinline__ long long order_key(double v) {
+    const long long b = __double_as_longlong(v);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+
 __device__ __forceinline__ void enthalpy_state(const StepParams<double>& P, double H, double& Tf, double& fl) {
-    fl = fmin(fmax((H - P.H_fs) * P.inv_dH, 0.0), 1.0);
-    Tf = fmin(H * P.inv_c_ps, P.T_fs) + fl * P.dT_sl + fmax(H - P.H_fl, 0.0);
+    const long long k = order_key(H);
+    const bool solid = k <= order_key(P.H_fs), liquid = !solid && k >= order_key(P.H_fl);
+    const double f = vmul(vsub(H, P.H_fs), P.inv_dH);
+    fl = solid ? 0.0 : liquid || __double_as_longlong(f) > __double_as_longlong(1.0) ? 1.0 : f;
+    Tf = vfma(solid || liquid ? H : fl, solid ? P.inv_c_ps : liquid ? 1.0 : P.dT_sl,
+              solid ? 0.0 : liquid ? P.T_off : P.T_fs);
 }
 
 // c_f,ref T at equilibrium as a function of the PCM rest population g_0: the
@@ -781,10 +812,12 @@ __device__ __forceinline__ void apply_wall(const StepParams<typename ModeTraits<
     const auto dir = w.dirichlet(P.wall_kind);
     const T Tb = w.of_side(P.wall_T), Hb = w.of_side(P.wall_H);
     const T dT = vsel(dir, vsub(Tb, n.Tf), zero), dM = vsel(dir, vsub(Tb, n.k[0]), zero);
-    const T t = vmulc<T>(P.inv_phi, n.Tf), mt = vneg(t);   // c_pl T / phi
+    const T t = FLOW ? vmulc<T>(P.inv_phi, n.Tf) : zero, mt = vneg(t);   // c_pl T / phi
     if constexpr (QT == 5) {
-        n.n[1] = vfma(mt, ux, n.n[1]);
-        n.n[2] = vfma(mt, uy, n.n[2]);
+        if constexpr (FLOW) {
+            n.n[1] = vfma(mt, ux, n.n[1]);
+            n.n[2] = vfma(mt, uy, n.n[2]);
+        }
         n.n[3] = vfmac<T>(P.vcf, dT, n.n[3]);
         n.k[3] = vfmac<T>(P.vcm, dM, n.k[3]);
     } else {
@@ -792,10 +825,12 @@ __device__ __forceinline__ void apply_wall(const StepParams<typename ModeTraits<
         const T cT = vmulc<T>(P.c_fref, dT), cM = vmulc<T>(P.c_mref, dM);
         n.n[1] = vadd(n.n[1], vfmac<T>(R(-4), dH, vadd(cT, cT)));
         n.n[2] = vadd(n.n[2], vfmac<T>(R(4), dH, vmulc<T>(R(-3), cT)));
-        n.n[3] = vfma(mt, ux, n.n[3]);
-        n.n[4] = vfma(t, ux, n.n[4]);
-        n.n[5] = vfma(mt, uy, n.n[5]);
-        n.n[6] = vfma(t, uy, n.n[6]);
+        if constexpr (FLOW) {
+            n.n[3] = vfma(mt, ux, n.n[3]);
+            n.n[4] = vfma(t, ux, n.n[4]);
+            n.n[5] = vfma(mt, uy, n.n[5]);
+            n.n[6] = vfma(t, uy, n.n[6]);
+        }
         n.k[1] = vadd(n.k[1], vfmac<T>(R(-4), dM, vadd(cM, cM)));
         n.k[2] = vadd(n.k[2], vfmac<T>(R(4), dM, vmulc<T>(R(-3), cM)));
     }
@@ -982,8 +1017,8 @@ __device__ __forceinline__ T thermal_collide(const StepParams<typename ModeTrait
         // distances from the equilibria of Eqs. 34 and 45 (zero for k = 7, 8)
         const T d[9] = {n.n[0], vsub(n.n[1], vfmac<T>(R(-4), n.n[0], vadd(cT, cT))),
                         vsub(n.n[2], vfmac<T>(R(4), n.n[0], vmulc<T>(R(-3), cT))),
-                        vfma(mt, n.ux, n.n[3]), vfma(t, n.ux, n.n[4]), vfma(mt, n.uy, n.n[5]), vfma(t, n.uy, n.n[6]),
-                        n.n[7], n.n[8]};
+                        FLOW ? vfma(mt, n.ux, n.n[3]) : n.n[3], FLOW ? vfma(t, n.ux, n.n[4]) : n.n[4],
+                        FLOW ? vfma(mt, n.uy, n.n[5]) : n.n[5], FLOW ? vfma(t, n.uy, n.n[6]) : n.n[6], n.n[7], n.n[8]};
         const T e[9] = {n.k[0], vsub(n.k[1], vfmac<T>(R(-4), n.k[0], vadd(cM, cM))),
                         vsub(n.k[2], vfmac<T>(R(4), n.k[0], vmulc<T>(R(-3), cM))),
                         n.k[3], n.k[4], n.k[5], n.k[6], n.k[7], n.k[8]};
@@ -1060,6 +1095,13 @@ __device__ __forceinline__ T thermal_collide(const StepParams<typename ModeTrait
 // anywhere fails a comparison; the sum overflows if any term is huge.
 template <typename R>
 __device__ __forceinline__ bool runaway(R H, R Tm, R rho, R um) {
+    if constexpr (sizeof(R) == 8) {   // nothing large (2^97), on the high words: no FP64 operation
+        const int big = (1023 + 97) << 20;
+        const unsigned h = __double2hiint(rho), u = __double2hiint(um);
+        if ((__double2hiint(H) & 0x7fffffff) < big && (__double2hiint(Tm) & 0x7fffffff) < big && h - 1 < big - 1 &&
+            u < (unsigned)__double2hiint(0.3))
+            return false;
+    }
     return !(fabs(H) + fabs(Tm) + rho < R(1e30)) || !(rho > R(0)) || !(um <= R(0.3));
 }
 
