@@ -728,6 +728,7 @@ int lbm_diag(lbm_handle* h, double* melt_frac, double* nu_hot, double* enthalpy,
     C.k_s = h->d.k_s;
     C.k_m = h->d.k_m;
     C.left_wall = (!p.periodic_x && p.nx >= 3) ? 1 : 0;
+    C.rows = lbmk::diag_rows(p.nx, p.ny);
     cudaError_t e;
     const int q = p.thermal_q, fl = p.flow;
     if (p.precision == LBM_F64) {

@@ -1490,58 +1490,86 @@ __global__ void __launch_bounds__(256) fields_kernel(const __grid_constant__ Ste
         if (out.mask & (1 << i)) out.dst[i][o] = v[i];
 }
 
-// Diagnostics: per-block FP64 partial sums of f_l, enthalpy, mass and the
-// left-wall heat flux, written to scratch[block][4] in a fixed order.
+// Diagnostics: FP64 sums of f_l, enthalpy, mass and the left-wall heat flux.
+// An FP64 operation occupies a scheduler's FP64 unit for 64 cycles (two lanes
+// per SM and clock), so the sums are arranged around their number: the
+// conversions from FP32 are integer operations, the enthalpy's weights are
+// applied to a thread's sums instead of to each node's terms, a thread takes
+// up to eight rows before its block reduces, and the warp reduces its four
+// sums in 6 additions instead of 20 (each exchange halves the sums a lane
+// keeps).  The wall flux, three node states per row, has blocks of its own
+// (the last column of blocks), beside the others instead of in their chains.
 struct DiagConst {
     double phi, rho_l, rho_m, c_pm, k_f, k_s, k_m;   // k_f: liquid PCM conductivity, k_s: solid (Eq. 9)
     int left_wall;  // 1 when x = 0 is a wall (Nusselt number defined)
+    int rows;       // rows of nodes per thread
 };
 
-template <int M, int QT, bool FLOW>
-__global__ void __launch_bounds__(256) diag_partial(const __grid_constant__ StepParams<typename ModeTraits<M>::R> P,
-                                                    const __grid_constant__ DiagConst C,
-                                                    double* __restrict__ scratch) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    double v[4] = {0.0, 0.0, 0.0, 0.0};
-    if (x < P.nx && y < P.ny) {
-        NodeState<M, QT, FLOW, Node1<M>> n;
-        node_state_at<M, QT, FLOW>(P, x, y, n);
-        v[0] = (double)n.fl;
-        v[1] = C.phi * C.rho_l * ((double)n.n[0] + (double)n.Hlo) +
-               (1.0 - C.phi) * C.rho_m * C.c_pm * ((double)n.k[0] + (double)n.Elo);
-        v[2] = 1.0 + (double)n.drho;
-        if (x == 0 && C.left_wall && P.nx >= 3) {
-            NodeState<M, QT, FLOW, Node1<M>> n1, n2;
-            node_state_at<M, QT, FLOW>(P, 1, y, n1);
-            node_state_at<M, QT, FLOW>(P, 2, y, n2);
-            const double gf = 0.5 * (3.0 * (double)n.Tf - 4.0 * (double)n1.Tf + (double)n2.Tf);
-            const double gm = 0.5 * (3.0 * (double)n.k[0] - 4.0 * (double)n1.k[0] + (double)n2.k[0]);
-            // PCM conductivity of the wall node's own liquid fraction (Eq. 9)
-            const double kw = C.k_s == C.k_f ? C.k_f : (double)n.fl * C.k_f + (1.0 - (double)n.fl) * C.k_s;
-            v[3] = C.phi * kw * gf + (1.0 - C.phi) * C.k_m * gm;
-        }
-    }
-    __shared__ double red[4][32];
-    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-    const int lane = tid & 31, warp = tid >> 5;
-    const int nwarps = (blockDim.x * blockDim.y + 31) >> 5;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        double a = v[i];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) a += __shfl_down_sync(0xffffffffu, a, off);
-        if (lane == 0) red[i][warp] = a;
-    }
-    __syncthreads();
-    if (tid < 4) {
-        double a = 0.0;
-        for (int w = 0; w < nwarps; ++w) a += red[tid][w];
-        scratch[(long long)(blockIdx.y * gridDim.x + blockIdx.x) * 4 + tid] = a;
-    }
+// v as a double, by integer operations for zero and normal numbers.
+__device__ __forceinline__ double to_double(double v) { return v; }
+__device__ __forceinline__ double to_double(float v) {
+    const unsigned u = __float_as_uint(v), m = u & 0x7fffffffu;
+    if (m - 0x00800000u >= 0x7f000000u) return m ? (double)v : 0.0;   // subnormal, infinite, NaN; zero
+    return __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(u << 29));
 }
 
-// Sums the partials in a fixed order (one block of 256 threads).
-__global__ void diag_finalize(const double* __restrict__ scratch, int nblocks, double* __restrict__ out);
+template <int M, int QT, bool FLOW>
+__global__ void __launch_bounds__(128) diag_partial(const __grid_constant__ StepParams<typename ModeTraits<M>::R> P,
+                                                    const __grid_constant__ DiagConst C,
+                                                    double* __restrict__ scratch) {
+    const int x = blockIdx.x * 128 + threadIdx.x;
+    double fl = 0.0, H = 0.0, Tm = 0.0, drho = 0.0, flux = 0.0;
+    const int y0 = blockIdx.y * C.rows, y1 = min(y0 + C.rows, P.ny);
+    if (blockIdx.x == gridDim.x - 1) {   // the left wall's heat flux, a row per thread
+        const int y = y0 + threadIdx.x;
+        if (C.left_wall && y < y1) {
+            double tf[3], tm[3], kw = 0.0;
+#pragma unroll 1
+            for (int k = 0; k < 3; ++k) {
+                NodeState<M, QT, FLOW, Node1<M>> n;
+                node_state_at<M, QT, FLOW>(P, k, y, n);
+                tf[k] = (double)n.Tf;
+                tm[k] = (double)n.k[0];
+                // PCM conductivity of the wall node's own liquid fraction (Eq. 9)
+                if (k == 0) kw = C.k_s == C.k_f ? C.k_f : (double)n.fl * C.k_f + (1.0 - (double)n.fl) * C.k_s;
+            }
+            const double gf = 0.5 * (3.0 * tf[0] - 4.0 * tf[1] + tf[2]);
+            const double gm = 0.5 * (3.0 * tm[0] - 4.0 * tm[1] + tm[2]);
+            flux = C.phi * kw * gf + (1.0 - C.phi) * C.k_m * gm;
+        }
+    } else if (x < P.nx) {
+#pragma unroll 1
+        for (int y = y0; y < y1; ++y) {
+            NodeState<M, QT, FLOW, Node1<M>> n;
+            node_state_at<M, QT, FLOW>(P, x, y, n);
+            fl += to_double(n.fl);
+            H += to_double(n.n[0]);
+            Tm += to_double(n.k[0]);
+            if constexpr (M != MODE_F64) H += to_double(n.Hlo);
+            if constexpr (kSplit<M>) Tm += to_double(n.Elo);
+            if constexpr (FLOW) drho += to_double(n.drho);
+        }
+    }
+    const double E = C.phi * C.rho_l * H + (1.0 - C.phi) * C.rho_m * C.c_pm * Tm;
+    // lanes 0-15 take (fl, E), 16-31 (drho, flux); then each eight lanes one of the two
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool h16 = lane & 16, h8 = lane & 8;
+    const double a = (h16 ? drho : fl) + __shfl_xor_sync(0xffffffffu, h16 ? fl : drho, 16);
+    const double b = (h16 ? flux : E) + __shfl_xor_sync(0xffffffffu, h16 ? E : flux, 16);
+    double v = (h8 ? b : a) + __shfl_xor_sync(0xffffffffu, h8 ? a : b, 8);
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    __shared__ double red[4][4];
+    if ((lane & 7) == 0) red[warp][lane >> 3] = v;
+    __syncthreads();
+    if (threadIdx.x < 4)
+        scratch[(long long)(blockIdx.y * gridDim.x + blockIdx.x) * 4 + threadIdx.x] =
+            (red[0][threadIdx.x] + red[1][threadIdx.x]) + (red[2][threadIdx.x] + red[3][threadIdx.x]);
+}
+
+// Sums the partials in a fixed order (one block of 512 threads, four sums side
+// by side): out[0..3] = sum f_l, sum enthalpy, nodes + sum delta_rho, sum
+// left-wall flux.
+__global__ void diag_finalize(const double* __restrict__ scratch, int nblocks, double nodes, double* __restrict__ out);
 
 }  // namespace lbmk

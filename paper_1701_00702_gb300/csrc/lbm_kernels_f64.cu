@@ -6,22 +6,20 @@ namespace lbmk {
 LBMK_INSTANTIATE(MODE_F64)
 LBMK_INSTANTIATE_CONVERT(MODE_F64)
 
-// Fixed-order sum of the per-block partials: thread t adds blocks t, t+256, ...
-// then a shared-memory tree combines the 256 thread sums; out[0..3] =
-// sum f_l, sum enthalpy, sum rho, sum left-wall flux.
-__global__ void diag_finalize(const double* __restrict__ scratch, int nblocks, double* __restrict__ out) {
-    __shared__ double red[4][256];
+// Fixed-order sum of the per-block partials: thread t adds sum t mod 4 of the
+// blocks t / 4, t / 4 + 128, ..., then a shared-memory tree combines the 128
+// threads of each sum.
+__global__ void diag_finalize(const double* __restrict__ scratch, int nblocks, double nodes, double* __restrict__ out) {
+    __shared__ double red[512];
     const int t = threadIdx.x;
-    double a[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int b = t; b < nblocks; b += blockDim.x)
-        for (int i = 0; i < 4; ++i) a[i] += scratch[(long long)b * 4 + i];
-    for (int i = 0; i < 4; ++i) red[i][t] = a[i];
+    double a = 0.0;
+    for (int i = t; i < 4 * nblocks; i += 512) a += scratch[i];
+    red[t] = a;
     __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (t < w)
-            for (int i = 0; i < 4; ++i) red[i][t] += red[i][t + w];
+    for (int w = 256; w >= 4; w >>= 1) {
+        if (t < w) red[t] += red[t + w];
         __syncthreads();
     }
-    if (t < 4) out[t] = red[t][0];
+    if (t < 4) out[t] = t == 2 ? nodes + red[t] : red[t];
 }
 }  // namespace lbmk

@@ -13,8 +13,21 @@ inline dim3 grid_for(int nx, int ny) {
     return dim3((unsigned)((nx + kBlockX - 1) / kBlockX), (unsigned)((ny + kBlockY - 1) / kBlockY), 1u);
 }
 
+// Rows per thread of the diagnostics: one where the grid hardly fills the
+// device, up to eight where blocks abound (a block's reduction costs as much
+// FP64 time as two rows).
+inline int diag_rows(int nx, int ny) {
+    const long long nodes = (long long)nx * ny;
+    return nodes <= 65536 && ny <= 32768 ? 1 : nodes <= 524288 ? 4 : 8;   // (at most 65,535 blocks along y)
+}
+
+inline dim3 diag_grid(int nx, int ny) {
+    const int r = diag_rows(nx, ny);
+    return dim3((unsigned)((nx + 127) / 128 + 1), (unsigned)((ny + r - 1) / r), 1u);   // and a column for the wall flux
+}
+
 inline int diag_blocks(int nx, int ny) {
-    const dim3 g = grid_for(nx, ny);
+    const dim3 g = diag_grid(nx, ny);
     return (int)(g.x * g.y);
 }
 
@@ -411,13 +424,13 @@ cudaError_t launch_fields(const StepParams<typename ModeTraits<M>::R>& P,
 template <int M>
 cudaError_t launch_diag(const StepParams<typename ModeTraits<M>::R>& P, const DiagConst& C, double* scratch,
                         double* out, int qt, int flow, cudaStream_t s) {
-    const dim3 g = grid_for(P.nx, P.ny), b(kBlockX, kBlockY);
+    const dim3 g = diag_grid(P.nx, P.ny);
     cudaError_t e = dispatch<M>(qt, flow, [&]<int MM, int Q, bool F>() {
-        diag_partial<MM, Q, F><<<g, b, 0, s>>>(P, C, scratch);
+        diag_partial<MM, Q, F><<<g, 128, 0, s>>>(P, C, scratch);
         return cudaGetLastError();
     });
     if (e != cudaSuccess) return e;
-    diag_finalize<<<1, 256, 0, s>>>(scratch, (int)(g.x * g.y), out);
+    diag_finalize<<<1, 512, 0, s>>>(scratch, (int)(g.x * g.y), (double)P.nx * P.ny, out);
     return cudaGetLastError();
 }
 
