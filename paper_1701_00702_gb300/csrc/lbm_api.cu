@@ -2,6 +2,7 @@
 // device state, graph-replayed stepping, fields, diagnostics, state I/O.
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstdint>
 #include <cstring>
 #include <memory>
@@ -158,7 +159,7 @@ struct Layout {
     size_t chunk_bytes;   // one chunk: every plane of kChunk nodes
     size_t elem;      // bytes of one bulk element (8, 4 or 2)
     size_t relem;     // bytes of one arithmetic element (8 or 4): history, fields, state I/O
-    size_t copy_bytes, dT_bytes, off_buf1, off_dT, off_status, off_scratch, off_out, total;
+    size_t copy_bytes, dT_bytes, off_buf1, off_dT, off_status, off_scratch, total;
     int nblocks;
 };
 
@@ -186,8 +187,7 @@ Layout layout_of(const lbm_params& p) {
     L.off_dT = 2 * L.copy_bytes;
     L.off_status = L.off_dT + L.dT_bytes;
     L.off_scratch = L.off_status + kAlign;
-    L.off_out = L.off_scratch + align_up((size_t)L.nblocks * 4 * sizeof(double));
-    L.total = L.off_out + kAlign;
+    L.total = L.off_scratch + align_up((size_t)L.nblocks * 4 * sizeof(double));
     return L;
 }
 
@@ -446,11 +446,21 @@ int build_graph(lbm_handle* h) {
     return LBM_OK;
 }
 
-int sync_and_check(lbm_handle* h) {
-    if (cudaStreamSynchronize(h->stream) != cudaSuccess) return cuda_fail(h);
-    unsigned int st = 0;
-    if (cudaMemcpy(&st, h->status, sizeof st, cudaMemcpyDeviceToHost) != cudaSuccess) return cuda_fail(h);
-    if (st & lbmk::STATUS_UNSTABLE) h->sticky = LBM_ERR_UNSTABLE;
+// Waits for the run's stream and takes the sticky status, with the
+// diagnostics' four sums when wanted: they lie behind the flag (kSumsOffset),
+// so that one copy in the stream brings both and the wait that follows is the
+// only one (a copy of the flag after the wait is a second round trip).
+constexpr size_t kSumsOffset = 64;
+
+int sync_and_check(lbm_handle* h, double* sums = nullptr) {
+    struct { unsigned int flag; char pad[kSumsOffset - 4]; double sums[4]; } back;
+    static_assert(offsetof(decltype(back), sums) == kSumsOffset && sizeof back <= kAlign, "behind the flag");
+    const size_t n = sums ? sizeof back : sizeof back.flag;
+    if (cudaMemcpyAsync(&back, h->status, n, cudaMemcpyDeviceToHost, h->stream) != cudaSuccess ||
+        cudaStreamSynchronize(h->stream) != cudaSuccess)
+        return cuda_fail(h);
+    if (sums) std::memcpy(sums, back.sums, sizeof back.sums);
+    if (back.flag & lbmk::STATUS_UNSTABLE) h->sticky = LBM_ERR_UNSTABLE;
     return h->sticky;
 }
 
@@ -584,7 +594,7 @@ int lbm_create_ex(const lbm_params* p, void* cuda_stream, lbm_alloc_fn alloc, lb
     h->dT = h->base + h->L.off_dT;
     h->status = reinterpret_cast<unsigned int*>(h->base + h->L.off_status);
     h->scratch = reinterpret_cast<double*>(h->base + h->L.off_scratch);
-    h->diag_out = reinterpret_cast<double*>(h->base + h->L.off_out);
+    h->diag_out = reinterpret_cast<double*>(h->base + h->L.off_status + kSumsOffset);
     // zero everything once: row padding is never written by the kernels, so
     // checkpoints of equal states are equal byte for byte
     cudaError_t e = cudaMemsetAsync(h->base, 0, h->L.total, h->stream);
@@ -744,9 +754,8 @@ int lbm_diag(lbm_handle* h, double* melt_frac, double* nu_hot, double* enthalpy,
             e = lbmk::launch_diag<lbmk::MODE_BF16>(P, C, h->scratch, h->diag_out, q, fl, h->stream);
     }
     double s[4] = {0, 0, 0, 0};
-    if (e == cudaSuccess) e = cudaMemcpyAsync(s, h->diag_out, sizeof s, cudaMemcpyDeviceToHost, h->stream);
     if (e != cudaSuccess) return cuda_fail(h);
-    int rc = sync_and_check(h);
+    int rc = sync_and_check(h, s);
     if (rc == LBM_ERR_CUDA) return rc;
     const double k_e = p.porosity * p.k_f + (1.0 - p.porosity) * h->d.k_m;
     if (melt_frac) *melt_frac = s[0] / ((double)p.nx * p.ny);
