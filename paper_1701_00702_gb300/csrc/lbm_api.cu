@@ -1252,7 +1252,7 @@ long long fill_group(const lbm_batch* b, const std::vector<int>& g, int parity, 
             acc += lbmk::group2_blocks(h->p.nx, h->p.ny);
         } else {
             G.tile[i] = lbmk::group_tile(h->p.nx);
-            acc += lbmk::group_blocks(h->p.nx, h->p.ny, G.tile[i]);
+            acc += lbmk::group_blocks(h->p.nx, h->p.ny, G.tile[i], lbmk::group_pairs(b->precision, b->qt, b->flow));
         }
     }
     G.first_block[g.size()] = (int)acc;

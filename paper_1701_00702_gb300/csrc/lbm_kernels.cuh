@@ -1342,22 +1342,41 @@ __global__ void __launch_bounds__(kT2W * HM, (kT2Blocks<HM, M, QT>)) fused_step2
 // Two nodes per thread
 // ---------------------------------------------------------------------------
 
-// Node pairs of the default configuration: a block of 32 x 4 threads covers
-// 64 x 4 nodes; the first of a chunk's two blocks prefetches its rows (2048^2
-// FP16 61.09 against 61.22 us per step when both do).  The last node of an odd
-// width steps alone.  Seven blocks per SM cap the
-// registers at 72 (measured best: 80 registers leave too few warps to hide
-// the memory latency, 64 spill).
+// Runs of the default configuration (flow, D2Q5 thermal lattices, volumetric
+// blend, FP32/FP16/BF16 storage) may advance node pairs (x0, x0 + 1), x0 even,
+// one pair per thread: the parameter loads and the index arithmetic serve both
+// nodes, and the pair is read and written with one access per plane wherever
+// both elements are adjacent (x0 even keeps them inside one chunk, aligned).
+// The last node of an odd width, and both nodes of a bounce-back run, step
+// one by one.
 template <int M, bool PH>
-__global__ void __launch_bounds__(128, 7) fused_step_pair(const __grid_constant__ StepParams<float> P) {
+__device__ __forceinline__ void step_pair_or_nodes(const StepParams<float>& P, int x0, int y) {
+    if (!P.solid_scheme && x0 + 1 < P.nx) {
+        step_pair<M, 5, PH>(P, x0, y);
+    } else {
+#pragma unroll 1
+        for (int x = x0; x < min(x0 + 2, P.nx); ++x) step_node<M, 5, true, PH>(P, x, y);
+    }
+}
+
+// Blocks of pairs per SM: six of 128 threads cap the registers at 80.  Seven
+// (72 registers) spill some 50 bytes: 2048^2 FP16 59.5 against 58.5 us per
+// step, BF16 60.4 against 57.8 (56.9 at the copy bandwidth on the 92 bytes the
+// form moves); eight, 78; three blocks of 256 threads, 61.7.
+constexpr int kPairBlocks = 6;
+
+// A block of 32 x 4 threads covers 64 x 4 nodes; the first of a chunk's two
+// blocks prefetches its rows (2048^2 FP16 61.09 against 61.22 us per step when
+// both did).
+template <int M, bool PH>
+__global__ void __launch_bounds__(128, kPairBlocks) fused_step_pair(const __grid_constant__ StepParams<float> P) {
     const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x0 >= P.nx || y >= P.ny) return;
     griddep_wait();
     if (P.prefetch_rows > 0 && threadIdx.x == 0 && threadIdx.y == 0 && (x0 & (kChunk - 1)) == 0)
         prefetch_rows<M, 5, true>(P, x0, y + P.prefetch_rows, blockDim.y);   // the chunk's first block
-    if (x0 + 1 >= P.nx) step_node<M, 5, true, PH>(P, x0, y);
-    else step_pair<M, 5, PH>(P, x0, y);
+    step_pair_or_nodes<M, PH>(P, x0, y);
 }
 
 // Many small runs in one launch per step, each run on the code of the
@@ -1381,18 +1400,23 @@ struct GroupParams {
     StepParams<R> run[kGroupRuns<R>];
 };
 
-template <int M, int QT, bool FLOW, bool PH>
-__global__ void __launch_bounds__(128, 2 * kMinBlocks<M, QT, FLOW>) group_step(
-    const __grid_constant__ GroupParams<typename ModeTraits<M>::R> G) {
-    using R = typename ModeTraits<M>::R;
-    const int b = blockIdx.x;
-    int lo = 0, hi = G.nruns - 1;   // the last run whose first block is <= b
+// The run of block b: the last one whose first block is <= b.
+template <typename R>
+__device__ __forceinline__ int group_run(const GroupParams<R>& G, int b) {
+    int lo = 0, hi = G.nruns - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (G.first_block[mid] <= b) lo = mid;
         else hi = mid - 1;
     }
-    const StepParams<R>& P = G.run[lo];
+    return lo;
+}
+
+template <int M, int QT, bool FLOW, bool PH>
+__global__ void __launch_bounds__(128, 2 * kMinBlocks<M, QT, FLOW>) group_step(
+    const __grid_constant__ GroupParams<typename ModeTraits<M>::R> G) {
+    const int b = blockIdx.x, lo = group_run(G, b);
+    const StepParams<typename ModeTraits<M>::R>& P = G.run[lo];
     const int lb = b - G.first_block[lo];
     const int lw = 5 + G.tile[lo];   // log2 of the tile width
     const int t = (int)threadIdx.x;
@@ -1404,6 +1428,25 @@ __global__ void __launch_bounds__(128, 2 * kMinBlocks<M, QT, FLOW>) group_step(
     step_node<M, QT, FLOW, PH>(P, x, y);
 }
 
+// The same for runs in 16-bit storage with flow and the D2Q5 thermal lattices,
+// a node pair per thread: tiles of w x 256 / w nodes, w = 32 << tile.  These
+// runs are bound by instruction issue, and a pair takes some 650 instructions
+// where its nodes one by one take 1,000.
+template <int M, bool PH>
+__global__ void __launch_bounds__(128, kPairBlocks) group_step_pair(const __grid_constant__ GroupParams<float> G) {
+    const int b = blockIdx.x, lo = group_run(G, b);
+    const StepParams<float>& P = G.run[lo];
+    const int lb = b - G.first_block[lo];
+    const int lw = 5 + G.tile[lo], lp = lw - 1;   // log2 of the tile width in nodes and in pairs
+    const int t = (int)threadIdx.x;
+    const int gx = (P.nx + (1 << lw) - 1) >> lw;
+    const int x0 = (lb % gx) * (1 << lw) + 2 * (t & ((1 << lp) - 1));
+    const int y = (lb / gx) * (128 >> lp) + (t >> lp);
+    if (x0 >= P.nx || y >= P.ny) return;
+    griddep_wait();
+    step_pair_or_nodes<M, PH>(P, x0, y);
+}
+
 // Batch map 5: the grouped launch of the two-step form.  Run k owns blocks
 // first_block[k] .. first_block[k + 1] - 1, one per two-step tile (blocks of
 // kT2W x kT2HMany threads, inner tiles of (kT2W - 2) x (kT2HMany - 2) nodes,
@@ -1412,15 +1455,8 @@ __global__ void __launch_bounds__(128, 2 * kMinBlocks<M, QT, FLOW>) group_step(
 template <int M, int QT, bool PH>
 __global__ void __launch_bounds__(kT2W * kT2HMany, (kT2Blocks<kT2HMany, M, QT>)) group_step2(
     const __grid_constant__ GroupParams<typename ModeTraits<M>::R> G) {
-    using R = typename ModeTraits<M>::R;
-    const int b = blockIdx.x;
-    int lo = 0, hi = G.nruns - 1;   // the last run whose first block is <= b
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (G.first_block[mid] <= b) lo = mid;
-        else hi = mid - 1;
-    }
-    const StepParams<R>& P = G.run[lo];
+    const int b = blockIdx.x, lo = group_run(G, b);
+    const StepParams<typename ModeTraits<M>::R>& P = G.run[lo];
     const int lb = b - G.first_block[lo];
     const int gx = t2_count(P.nx, kT2W - 2);
     step2_tile<M, QT, PH, kT2HMany>(P, lb % gx, lb / gx);

@@ -165,16 +165,21 @@ inline dim3 step_block(int nx, int ny) {
     return (long long)nx * ny <= 40000 ? dim3(64, 2) : dim3(128, 1);
 }
 
-// Step forms: one node per thread (fused_step) or node pairs
-// (fused_step_pair, the default configuration only: flow, D2Q5, volumetric
-// blend, FP32 arithmetic).  Automatic: node pairs, with the L2 prefetch, for
-// the 16-bit forms from 1536 x 1024 nodes up (measured on GB300, us per step:
-// FP16 2048^2 62.1 against 72.7, 2048 x 1024 34.1 against 38.1, 1448^2 37.3
-// against 39.2; at 1024^2, whose state nearly fits in L2, one node per thread
-// is faster, 18.9 against 19.4; in FP32, bound by HBM, one node per thread is
-// faster at every size).
+// Step forms.  FORM_SINGLE is one step per launch, FORM_PAIRS that with node
+// pairs (fused_step_pair, the default configuration only: flow, D2Q5,
+// volumetric blend, FP32 arithmetic) and the L2 prefetch.  Automatic: pairs
+// with the prefetch for the 16-bit forms from 1536 x 1024 nodes up (at 1024^2,
+// whose state nearly fits in L2, the prefetch gains nothing; in FP32, bound by
+// HBM, one node per thread is faster at every size).
 enum : int { FORM_AUTO = 0, FORM_SINGLE = 1, FORM_PAIRS = 2, FORM_TWO_STEPS = 3 };
 constexpr long long kPairMinNodes = 3ll << 19;
+
+// FORM_SINGLE too takes pairs, without the prefetch, for 16-bit runs from
+// kPairPlainMinNodes nodes, where instruction issue and not one warp's chain
+// bounds the step (GB300, us per step, one node / pairs: FP16 384^2 3.37 / 3.27,
+// 512^2 5.09 / 4.93, 1024^2 17.9 / 16.1, BF16 with Eq. 9 777 x 501 7.80 / 7.62;
+// in FP32 512^2 5.0 / 5.2, 1024^2 26.5 / 26.9).
+constexpr long long kPairPlainMinNodes = 1ll << 17;
 
 // The rule (host code; lbm_step_form_for reports it): the form a run takes,
 // FORM_SINGLE or FORM_PAIRS.  mode: MODE_*.
@@ -209,9 +214,12 @@ inline bool two_steps_for(int mode, int qt, int flow, long long nodes, int form)
     return nodes <= kTwoStepSmallMaxNodes || (mode == MODE_F32 && nodes >= kTwoStepF32MinNodes);
 }
 
+// Whether a run's one-step kernel takes node pairs.
 template <int M>
-inline int form_of(const StepParams<typename ModeTraits<M>::R>& P, int qt, int flow, int form) {
-    return form_for(M, qt, flow, P.solid_scheme, (long long)P.nx * P.ny, form);
+inline bool pairs_of(const StepParams<typename ModeTraits<M>::R>& P, int qt, int flow, int form) {
+    const long long nodes = (long long)P.nx * P.ny;
+    if (form_for(M, qt, flow, P.solid_scheme, nodes, form) == FORM_PAIRS) return true;
+    return kSplit<M> && qt == 5 && flow && !P.solid_scheme && nodes >= kPairPlainMinNodes;
 }
 
 // L2 prefetch distance of the node-pair kernel in rows (0: off): grids of at
@@ -227,7 +235,7 @@ inline int prefetch_rows_for(int mode, int qt, int flow, int solid_scheme, long 
     return form_for(mode, qt, flow, solid_scheme, nodes, form) == FORM_PAIRS ? kPrefetchRowsPairs : 0;
 }
 
-// The step kernel of a run, with its grid: one node per thread in blocks of
+// The one-step kernel of a run, with its grid: one node per thread in blocks of
 // b threads, or node pairs in blocks of 32 x 4.
 struct StepLaunch {
     const void* fn;
@@ -238,7 +246,7 @@ template <int M>
 StepLaunch step_launch(const StepParams<typename ModeTraits<M>::R>& P, int qt, int flow, int form, dim3 b) {
     StepLaunch L{nullptr, dim3(), b};
     if constexpr (M != MODE_F64) {
-        if (form_of<M>(P, qt, flow, form) == FORM_PAIRS) {
+        if (pairs_of<M>(P, qt, flow, form)) {
             L.fn = P.phase_k ? (const void*)fused_step_pair<M, true> : (const void*)fused_step_pair<M, false>;
             L.block = dim3(32, 4);   // 2048^2 FP16 61.25 us per step (64 x 2: 61.98)
             L.grid = dim3((unsigned)(((P.nx + 1) / 2 + 31) / 32), (unsigned)((P.ny + 3) / 4), 1u);
@@ -275,15 +283,21 @@ inline int group_tile(int nx) {
     return best;
 }
 
-// Blocks of one run in a grouped launch (blocks of 128 threads).
-inline long long group_blocks(int nx, int ny, int tile) {
-    const int w = 32 << tile;
-    return (long long)((nx + w - 1) / w) * ((ny + (128 / w) - 1) / (128 / w));
+// Whether the grouped launches of a mode's runs take node pairs.
+inline bool group_pairs(int mode, int qt, int flow) { return (mode == MODE_F16 || mode == MODE_BF16) && qt == 5 && flow; }
+
+// Blocks of one run in a grouped launch (blocks of 128 threads, one node or one
+// pair each).
+inline long long group_blocks(int nx, int ny, int tile, bool pairs) {
+    const int w = 32 << tile, h = (pairs ? 256 : 128) / w;
+    return (long long)((nx + w - 1) / w) * ((ny + h - 1) / h);
 }
 
 template <int M>
 const void* group_kernel(int qt, int flow, int ph) {
     const void* fn = nullptr;
+    if constexpr (kSplit<M>)
+        if (group_pairs(M, qt, flow)) return ph ? (const void*)group_step_pair<M, true> : (const void*)group_step_pair<M, false>;
     dispatch_step<M>(qt, flow, ph, [&]<int MM, int Q, bool F, bool PH>() {
         fn = (const void*)group_step<MM, Q, F, PH>;
         return cudaSuccess;
