@@ -963,6 +963,18 @@ const char* lbm_strerror(int code) {
 // Batches: many runs advanced by one launch per time step
 // ---------------------------------------------------------------------------
 
+namespace {
+// The launch configuration and the parameters of one grouped launch.
+struct GroupArgs {
+    std::vector<char> params;   // a GroupParams of the group's size class
+    void* args[1];
+    dim3 grid, block;
+    size_t smem = 0;
+    const void* fn = nullptr;
+};
+
+}  // namespace
+
 struct lbm_batch {
     std::vector<lbm_handle*> runs;
     int precision = 0, qt = 0, flow = 0;
@@ -977,7 +989,9 @@ struct lbm_batch {
     std::vector<int> flip;        // run's current copy relative to the batch parity
     std::vector<int> form;        // each run's step form when the parameters were uploaded
     std::vector<int> shape;       // map 3: block shape of each run (index into kShapes)
-    std::vector<std::vector<int>> groups;   // map 4: the runs of each grouped launch
+    std::vector<std::vector<int>> groups;   // maps 4, 5: the runs of each grouped launch in graphs
+    std::vector<std::vector<int>> inline_groups;   // the same outside graphs
+    std::vector<GroupArgs> launches[4];     // their launches outside graphs, filled on first use: one step from parity 0 or 1, two steps there or back
     std::vector<int> solo;                  // map 4: runs that keep their own step kernel
     lbmk::Tile* tiles = nullptr;
     size_t tile_capacity = 0;     // tiles that fit in the allocation
@@ -1107,22 +1121,42 @@ int batch_blocks_per_sm(const lbm_batch* b) {
 // contiguous chunks of tiles, 2 persistent blocks striding over the tiles,
 // 3 one single-run kernel per run and step, the runs' chains concurrent in
 // one graph.
-// Map 4: the runs below kGroupMaxNodes nodes in order, at most kGroupRuns per
-// grouped launch; the larger runs keep their own step kernel.
 // Map 4: the runs below kGroupMaxNodes in groups of at most kGroupRuns, the
-// others solo.  Map 5: every run in groups (its kernel takes any size).
+// others solo.  Map 5: every run in groups (its kernel takes any size).  The
+// groups' chains run side by side in the graph, so that one group's launch
+// ramp and last blocks overlap another's work: at least two groups under map 4
+// and four under map 5, balanced by nodes (12 cavities of 106-471 nodes a side,
+// us per step with 1 / 2 / 4 / 8 groups: FP16 map 4 21.2 / 17.5 / 17.6 / 18.0,
+// FP32 map 5 24.9 / 22.6 / 21.9 / 21.5; 64 cavities: FP16 map 4 with 2 / 4 / 8
+// groups 123.1 / 128.5 / 129.4, FP32 map 5 146.7 / 145.5 / 144.5).
 void make_groups(lbm_batch* b) {
     b->groups.clear();
+    b->inline_groups.clear();
     b->solo.clear();
-    const int cap = b->precision == LBM_F64 ? lbmk::kGroupRuns<double> : lbmk::kGroupRuns<float>;
+    const size_t cap = b->precision == LBM_F64 ? lbmk::kGroupRuns<double> : lbmk::kGroupRuns<float>;
+    auto nodes = [&](int r) { return (long long)b->runs[r]->p.nx * b->runs[r]->p.ny; };
     std::vector<int> small;
     for (int r = 0; r < (int)b->runs.size(); ++r) {
-        const lbm_params& p = b->runs[r]->p;
-        if (b->mapping == 5 || (long long)p.nx * p.ny < lbmk::kGroupMaxNodes) small.push_back(r);
+        if (b->mapping == 5 || nodes(r) < lbmk::kGroupMaxNodes) small.push_back(r);
         else b->solo.push_back(r);
     }
+    if (small.empty()) return;
+    // outside graphs, one launch after another in the stream, as few groups as hold the runs
     for (size_t i = 0; i < small.size(); i += cap)
-        b->groups.emplace_back(small.begin() + i, small.begin() + std::min(small.size(), i + cap));
+        b->inline_groups.emplace_back(small.begin() + i, small.begin() + std::min(small.size(), i + cap));
+    const size_t apart = b->mapping == 5 ? 4 : 2;
+    const size_t few = lbmk::kGroupFew, per = small.size() <= 3 * few ? few : cap;   // few runs: small parameters
+    const size_t ng = std::min(small.size(), std::max(apart, (small.size() + per - 1) / per));
+    std::stable_sort(small.begin(), small.end(), [&](int x, int y) { return nodes(x) > nodes(y); });
+    std::vector<long long> load(ng, 0);
+    b->groups.resize(ng);
+    for (int r : small) {   // the largest first, each to the group with the fewest nodes
+        size_t g = ng;
+        for (size_t k = 0; k < ng; ++k)
+            if (b->groups[k].size() < per && (g == ng || load[k] < load[g])) g = k;
+        b->groups[g].push_back(r);
+        load[g] += nodes(r);
+    }
 }
 
 void set_mapping(lbm_batch* b, int mapping, int resident_blocks) {
@@ -1140,7 +1174,9 @@ void set_mapping(lbm_batch* b, int mapping, int resident_blocks) {
     }
 }
 
+// Drops everything that bakes in the runs' parameters: the graph and the kept launches.
 void batch_destroy_graph(lbm_batch* b) {
+    for (auto& l : b->launches) l.clear();
     if (b->graph) cudaGraphExecDestroy(b->graph);
     b->graph = nullptr;
 }
@@ -1237,10 +1273,11 @@ int build_chain_graph(lbm_batch* b, int steps, cudaGraphExec_t* out) {
 // sums of their block counts.  two: a launch of the two-step kernel, whose
 // history goes from h->dT to h->dT2 (back = 0) or back (back = 1).  Returns the
 // launch's block count.
-template <typename R>
-long long fill_group(const lbm_batch* b, const std::vector<int>& g, int parity, lbmk::GroupParams<R>& G,
+template <typename R, int NR>
+long long fill_group(const lbm_batch* b, const std::vector<int>& g, int parity, std::vector<char>& store,
                      bool two, bool back) {
-    std::memset(&G, 0, sizeof G);
+    store.assign(sizeof(lbmk::GroupParams<R, NR>), 0);
+    lbmk::GroupParams<R, NR>& G = *reinterpret_cast<lbmk::GroupParams<R, NR>*>(store.data());
     G.nruns = (int)g.size();
     long long acc = 0;
     for (size_t i = 0; i < g.size(); ++i) {
@@ -1259,13 +1296,13 @@ long long fill_group(const lbm_batch* b, const std::vector<int>& g, int parity, 
     return acc;
 }
 
-const void* group_fn(const lbm_batch* b) {
+const void* group_fn(const lbm_batch* b, bool few) {
     const int ph = batch_phase(b);
     switch (b->precision) {
-        case LBM_F64: return lbmk::group_kernel<lbmk::MODE_F64>(b->qt, b->flow, ph);
-        case LBM_F32: return lbmk::group_kernel<lbmk::MODE_F32>(b->qt, b->flow, ph);
-        case LBM_F16: return lbmk::group_kernel<lbmk::MODE_F16>(b->qt, b->flow, ph);
-        default: return lbmk::group_kernel<lbmk::MODE_BF16>(b->qt, b->flow, ph);
+        case LBM_F64: return lbmk::group_kernel<lbmk::MODE_F64>(b->qt, b->flow, ph, few);
+        case LBM_F32: return lbmk::group_kernel<lbmk::MODE_F32>(b->qt, b->flow, ph, few);
+        case LBM_F16: return lbmk::group_kernel<lbmk::MODE_F16>(b->qt, b->flow, ph, few);
+        default: return lbmk::group_kernel<lbmk::MODE_BF16>(b->qt, b->flow, ph, few);
     }
 }
 
@@ -1281,12 +1318,12 @@ int ensure_batch_dT2(lbm_batch* b) {
     return LBM_OK;
 }
 
-const void* group2_fn(const lbm_batch* b) {
+const void* group2_fn(const lbm_batch* b, bool few) {
     const int ph = batch_phase(b);
     switch (b->precision) {
-        case LBM_F32: return lbmk::group2_kernel<lbmk::MODE_F32>(b->qt, ph);
-        case LBM_F16: return lbmk::group2_kernel<lbmk::MODE_F16>(b->qt, ph);
-        case LBM_BF16: return lbmk::group2_kernel<lbmk::MODE_BF16>(b->qt, ph);
+        case LBM_F32: return lbmk::group2_kernel<lbmk::MODE_F32>(b->qt, ph, few);
+        case LBM_F16: return lbmk::group2_kernel<lbmk::MODE_F16>(b->qt, ph, few);
+        case LBM_BF16: return lbmk::group2_kernel<lbmk::MODE_BF16>(b->qt, ph, few);
         default: return nullptr;
     }
 }
@@ -1300,45 +1337,35 @@ size_t group2_smem(const lbm_batch* b) {
     }
 }
 
-// The launch configuration and the parameters of one grouped launch.
-struct GroupArgs {
-    std::unique_ptr<lbmk::GroupParams<double>> d;
-    std::unique_ptr<lbmk::GroupParams<float>> f;
-    void* args[1];
-    dim3 grid, block;
-    size_t smem = 0;
-    const void* fn = nullptr;
-};
-
 cudaError_t group_args(const lbm_batch* b, const std::vector<int>& g, int parity, GroupArgs& a, bool two = false,
                        bool back = false) {
+    using namespace lbmk;
+    const bool few = g.size() <= (size_t)kGroupFew;
     long long blocks;
-    if (b->precision == LBM_F64) {
-        if (!a.d) a.d = std::make_unique<lbmk::GroupParams<double>>();
-        blocks = fill_group<double>(b, g, parity, *a.d, false, false);
-        a.args[0] = a.d.get();
-    } else {
-        if (!a.f) a.f = std::make_unique<lbmk::GroupParams<float>>();
-        blocks = fill_group<float>(b, g, parity, *a.f, two, back);
-        a.args[0] = a.f.get();
-    }
+    if (b->precision == LBM_F64)
+        blocks = few ? fill_group<double, kGroupFew>(b, g, parity, a.params, false, false)
+                     : fill_group<double, kGroupRuns<double>>(b, g, parity, a.params, false, false);
+    else
+        blocks = few ? fill_group<float, kGroupFew>(b, g, parity, a.params, two, back)
+                     : fill_group<float, kGroupRuns<float>>(b, g, parity, a.params, two, back);
+    a.args[0] = a.params.data();
     a.grid = dim3((unsigned)blocks, 1u, 1u);
     if (!two) {
         a.block = dim3(128, 1, 1);
         a.smem = 0;
-        a.fn = group_fn(b);
+        a.fn = group_fn(b, few);
         return cudaSuccess;
     }
     a.block = dim3((unsigned)lbmk::kT2W, (unsigned)lbmk::kT2HMany, 1u);
     a.smem = group2_smem(b);
-    a.fn = group2_fn(b);
+    a.fn = group2_fn(b, few);
     if (!a.fn) return cudaErrorInvalidConfiguration;
     return cudaFuncSetAttribute(a.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)a.smem);
 }
 
 // One batched step under map 4 (each group's launch and each large run's
-// own step) or two steps under map 5 (two = true: each group's two-step
-// launch), as programmatic dependents of the previous launch in the stream.
+// own step) or two steps under map 5 (two = true, parity = back: each group's
+// two-step launch), as programmatic dependents of the previous launch in the stream.
 // Single steps under map 5 take each run's one-step kernel (one node per
 // thread), which rounds exactly as the two-step kernel does.
 cudaError_t group_step_all(lbm_batch* b, int parity, cudaStream_t s, bool two = false, bool back = false) {
@@ -1349,10 +1376,18 @@ cudaError_t group_step_all(lbm_batch* b, int parity, cudaStream_t s, bool two = 
         }
         return cudaSuccess;
     }
-    GroupArgs a;
-    for (const std::vector<int>& g : b->groups) {
-        cudaError_t e = group_args(b, g, parity, a, two, back);
-        if (e != cudaSuccess) return e;
+    // filling a launch's parameters (every run's block) takes the host longer than the launch
+    // takes the device, so they are kept until the runs' parameters change
+    std::vector<GroupArgs>& kept = b->launches[two ? 2 + (back ? 1 : 0) : parity];
+    if (kept.empty()) {
+        std::vector<GroupArgs> fresh(b->inline_groups.size());
+        for (size_t i = 0; i < fresh.size(); ++i) {
+            const cudaError_t e = group_args(b, b->inline_groups[i], parity, fresh[i], two, back);
+            if (e != cudaSuccess) return e;
+        }
+        kept.swap(fresh);
+    }
+    for (GroupArgs& a : kept) {
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -1363,7 +1398,7 @@ cudaError_t group_step_all(lbm_batch* b, int parity, cudaStream_t s, bool two = 
         cfg.stream = s;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        e = cudaLaunchKernelExC(&cfg, a.fn, a.args);
+        const cudaError_t e = cudaLaunchKernelExC(&cfg, a.fn, a.args);
         if (e != cudaSuccess) return e;
     }
     for (int r : b->solo) {
@@ -1381,14 +1416,14 @@ int build_group_graph(lbm_batch* b, int steps, cudaGraphExec_t* out) {
     cudaGraph_t g = nullptr;
     if (cudaGraphCreate(&g, 0) != cudaSuccess) return LBM_ERR_CUDA;
     cudaError_t e = cudaSuccess;
-    GroupArgs a;
     const bool two = b->mapping == 5;
     const int launches = two ? steps / 2 : steps;
     for (size_t gi = 0; gi < b->groups.size() && e == cudaSuccess; ++gi) {
+        GroupArgs args[2];   // the chain alternates between two launches
+        for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = group_args(b, b->groups[gi], k, args[k], two, k != 0);
         cudaGraphNode_t prev = nullptr;
         for (int k = 0; k < launches && e == cudaSuccess; ++k) {
-            e = group_args(b, b->groups[gi], k & 1, a, two, (k & 1) != 0);
-            if (e != cudaSuccess) break;
+            GroupArgs& a = args[k & 1];
             cudaKernelNodeParams kp = {};
             kp.func = const_cast<void*>(a.fn);
             kp.gridDim = a.grid;

@@ -1392,17 +1392,23 @@ __global__ void __launch_bounds__(128, kPairBlocks) fused_step_pair(const __grid
 template <typename R>
 constexpr int kGroupRuns = (32000 - 16) / (int)(sizeof(StepParams<R>) + 2 * sizeof(int));
 
-template <typename R>
+// Groups of up to kGroupFew runs have a build of their own with smaller
+// parameters: a launch and a graph node copy all of them, 30 KB at full size
+// (12 FP16 cavities in two groups, first 64 steps with the graph's build 1.92
+// ms at full size).
+constexpr int kGroupFew = 8;
+
+template <typename R, int NR>
 struct GroupParams {
     int nruns;
-    int first_block[kGroupRuns<R> + 1];
-    int tile[kGroupRuns<R>];
-    StepParams<R> run[kGroupRuns<R>];
+    int first_block[NR + 1];
+    int tile[NR];
+    StepParams<R> run[NR];
 };
 
 // The run of block b: the last one whose first block is <= b.
-template <typename R>
-__device__ __forceinline__ int group_run(const GroupParams<R>& G, int b) {
+template <typename R, int NR>
+__device__ __forceinline__ int group_run(const GroupParams<R, NR>& G, int b) {
     int lo = 0, hi = G.nruns - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
@@ -1412,9 +1418,9 @@ __device__ __forceinline__ int group_run(const GroupParams<R>& G, int b) {
     return lo;
 }
 
-template <int M, int QT, bool FLOW, bool PH>
+template <int M, int QT, bool FLOW, bool PH, int NR>
 __global__ void __launch_bounds__(128, 2 * kMinBlocks<M, QT, FLOW>) group_step(
-    const __grid_constant__ GroupParams<typename ModeTraits<M>::R> G) {
+    const __grid_constant__ GroupParams<typename ModeTraits<M>::R, NR> G) {
     const int b = blockIdx.x, lo = group_run(G, b);
     const StepParams<typename ModeTraits<M>::R>& P = G.run[lo];
     const int lb = b - G.first_block[lo];
@@ -1432,8 +1438,8 @@ __global__ void __launch_bounds__(128, 2 * kMinBlocks<M, QT, FLOW>) group_step(
 // a node pair per thread: tiles of w x 256 / w nodes, w = 32 << tile.  These
 // runs are bound by instruction issue, and a pair takes some 650 instructions
 // where its nodes one by one take 1,000.
-template <int M, bool PH>
-__global__ void __launch_bounds__(128, kPairBlocks) group_step_pair(const __grid_constant__ GroupParams<float> G) {
+template <int M, bool PH, int NR>
+__global__ void __launch_bounds__(128, kPairBlocks) group_step_pair(const __grid_constant__ GroupParams<float, NR> G) {
     const int b = blockIdx.x, lo = group_run(G, b);
     const StepParams<float>& P = G.run[lo];
     const int lb = b - G.first_block[lo];
@@ -1452,9 +1458,9 @@ __global__ void __launch_bounds__(128, kPairBlocks) group_step_pair(const __grid
 // kT2W x kT2HMany threads, inner tiles of (kT2W - 2) x (kT2HMany - 2) nodes,
 // row-major over the run's tiles); each block advances its tile two steps as
 // fused_step2 does, with its run's parameter block.
-template <int M, int QT, bool PH>
+template <int M, int QT, bool PH, int NR>
 __global__ void __launch_bounds__(kT2W * kT2HMany, (kT2Blocks<kT2HMany, M, QT>)) group_step2(
-    const __grid_constant__ GroupParams<typename ModeTraits<M>::R> G) {
+    const __grid_constant__ GroupParams<typename ModeTraits<M>::R, NR> G) {
     const int b = blockIdx.x, lo = group_run(G, b);
     const StepParams<typename ModeTraits<M>::R>& P = G.run[lo];
     const int lb = b - G.first_block[lo];

@@ -293,16 +293,24 @@ inline long long group_blocks(int nx, int ny, int tile, bool pairs) {
     return (long long)((nx + w - 1) / w) * ((ny + h - 1) / h);
 }
 
-template <int M>
-const void* group_kernel(int qt, int flow, int ph) {
-    const void* fn = nullptr;
+template <int M, int NR>
+const void* group_kernel_nr(int qt, int flow, int ph) {
     if constexpr (kSplit<M>)
-        if (group_pairs(M, qt, flow)) return ph ? (const void*)group_step_pair<M, true> : (const void*)group_step_pair<M, false>;
+        if (group_pairs(M, qt, flow))
+            return ph ? (const void*)group_step_pair<M, true, NR> : (const void*)group_step_pair<M, false, NR>;
+    const void* fn = nullptr;
     dispatch_step<M>(qt, flow, ph, [&]<int MM, int Q, bool F, bool PH>() {
-        fn = (const void*)group_step<MM, Q, F, PH>;
+        if constexpr (!(kSplit<MM> && Q == 5 && F)) fn = (const void*)group_step<MM, Q, F, PH, NR>;
         return cudaSuccess;
     });
     return fn;
+}
+
+// few: the build for at most kGroupFew runs.
+template <int M>
+const void* group_kernel(int qt, int flow, int ph, bool few) {
+    return few ? group_kernel_nr<M, kGroupFew>(qt, flow, ph)
+               : group_kernel_nr<M, kGroupRuns<typename ModeTraits<M>::R>>(qt, flow, ph);
 }
 
 // Launched as a programmatic dependent of the previous step (the kernels wait
@@ -389,12 +397,16 @@ size_t step2_smem(int qt, int h) {
 
 // Batch map 5: the grouped two-step kernel and its shared memory (the 12-row
 // build; blocks of kT2W x kT2HMany threads).
+template <int M, int NR>
+const void* group2_kernel_nr(int qt, int phase_k) {
+    if (qt == 5) return phase_k ? (const void*)group_step2<M, 5, true, NR> : (const void*)group_step2<M, 5, false, NR>;
+    return phase_k ? (const void*)group_step2<M, 9, true, NR> : (const void*)group_step2<M, 9, false, NR>;
+}
+
 template <int M>
-const void* group2_kernel(int qt, int phase_k) {
-    if constexpr (M != MODE_F64) {
-        if (qt == 5) return phase_k ? (const void*)group_step2<M, 5, true> : (const void*)group_step2<M, 5, false>;
-        return phase_k ? (const void*)group_step2<M, 9, true> : (const void*)group_step2<M, 9, false>;
-    }
+const void* group2_kernel(int qt, int phase_k, bool few) {
+    if constexpr (M != MODE_F64)
+        return few ? group2_kernel_nr<M, kGroupFew>(qt, phase_k) : group2_kernel_nr<M, kGroupRuns<float>>(qt, phase_k);
     return nullptr;
 }
 
@@ -502,9 +514,9 @@ int batch_blocks_per_sm(int qt, int flow, int ph) {
     KW template cudaError_t launch_batch<M>(const StepParams<ModeTraits<M>::R>*, const Tile*, int, int, int, int, int, \
                                          int, int, cudaStream_t);                                               \
     KW template int batch_blocks_per_sm<M>(int, int, int);                                                   \
-    KW template const void* group_kernel<M>(int, int, int);                                                    \
+    KW template const void* group_kernel<M>(int, int, int, bool);                                                    \
     KW template cudaError_t launch_step2<M>(const StepParams<ModeTraits<M>::R>&, int, int, cudaStream_t);     \
-    KW template const void* group2_kernel<M>(int, int);                                                        \
+    KW template const void* group2_kernel<M>(int, int, bool);                                                        \
     KW template size_t step2_smem<M>(int, int);                                                                \
     KW template StepLaunch step_launch<M>(const StepParams<ModeTraits<M>::R>&, int, int, int, dim3);
 
