@@ -393,6 +393,7 @@ cudaError_t enqueue_two(lbm_handle* h, int from, int back, cudaStream_t s) {
     const int q = h->p.thermal_q;
     auto run = [&](auto P, auto tag) {
         if (back) std::swap(P.dT, P.dT_out);
+        P.prefetch_rows = lbmk::prefetch_rows_two_steps(decltype(tag)::value, (long long)P.nx * P.ny);
         return lbmk::launch_step2<decltype(tag)::value>(P, q, h->t2h, s);
     };
     switch (h->p.precision) {
@@ -1285,6 +1286,7 @@ long long fill_group(const lbm_batch* b, const std::vector<int>& g, int parity, 
         G.first_block[i] = (int)acc;
         G.run[i] = make_params<R>(h, b->flip[g[i]] ^ parity);
         if (two) {
+            G.run[i].prefetch_rows = 0;   // a group's blocks of one run start at about the same time
             if (back) std::swap(G.run[i].dT, G.run[i].dT_out);
             acc += lbmk::group2_blocks(h->p.nx, h->p.ny);
         } else {

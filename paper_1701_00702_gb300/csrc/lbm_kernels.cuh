@@ -1193,8 +1193,8 @@ constexpr int kMinBlocks = (QT == 5 && FLOW) ? (M == MODE_F64 ? 1 : 5) : 1;
 // 2.50).
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// L2 prefetch ahead of the blocks that will run next (node pairs on large
-// grids): a block's first thread asks L2, by bulk prefetches
+// L2 prefetch ahead of the blocks that will run next (node pairs and two steps
+// per launch on large grids): a block's first thread asks L2, by bulk prefetches
 // (cp.async.bulk.prefetch.L2), for the chunk of x in `rows` rows starting at
 // y0 and for their exchange history, so that the block launched for those
 // rows later finds them in L2 instead of waiting for HBM.  No registers or
@@ -1319,6 +1319,9 @@ __device__ __forceinline__ void step2_tile(const StepParams<typename ModeTraits<
         else live = false;
     }
     griddep_wait();
+    // the tile's rows, prefetch_rows further on, of the chunk that starts at its first inner column
+    if (P.prefetch_rows > 0 && lx == 1 && (x2 & (kChunk - 1)) == 0 && ly >= 1 && ly <= H - 2)
+        prefetch_rows<M, QT, true>(P, x2, y2 + P.prefetch_rows, 1);
     if (live) {
         const WallAt<R> w(P, x, y);
         sdT[i] = advance<M, QT, true, PH, TL::n, R>(P, PullAt<M, QT, true>(P, w.xs, w.ys), w, P.dT + (y * P.pitch + x),

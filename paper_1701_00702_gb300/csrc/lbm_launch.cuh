@@ -235,6 +235,17 @@ inline int prefetch_rows_for(int mode, int qt, int flow, int solid_scheme, long 
     return form_for(mode, qt, flow, solid_scheme, nodes, form) == FORM_PAIRS ? kPrefetchRowsPairs : 0;
 }
 
+// The two-step kernel's distance, for FP32 grids whose state exceeds L2 (GB300,
+// us per step without / with: 900 x 880 17.0 / 16.4, 1024^2 21.7 / 19.5, 2048^2
+// 80.8 / 71.3, 4096^2 317 / 279, 256 x 4096 21.8 / 19.9, 8192 x 128 21.9 /
+// 20.2; distances of 10 to 40 rows within 1 % of each other but for the
+// widest).  The blocks that read the rows start about 2 us later.
+constexpr int kPrefetchRowsTwoSteps = 20;
+
+inline int prefetch_rows_two_steps(int mode, long long nodes) {
+    return mode == MODE_F32 && nodes >= kTwoStepF32MinNodes ? kPrefetchRowsTwoSteps : 0;
+}
+
 // The one-step kernel of a run, with its grid: one node per thread in blocks of
 // b threads, or node pairs in blocks of 32 x 4.
 struct StepLaunch {
