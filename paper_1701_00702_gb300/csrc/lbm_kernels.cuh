@@ -865,6 +865,8 @@ __device__ __forceinline__ void node_state(const StepParams<typename ModeTraits<
                 w.from_inward(n.k[q]);
             }
             w.from_inward(n.Hlo);
+            w.from_inward(n.h0);
+            w.from_inward(n.hs);
         }
     }
     macro<M, QT, FLOW, T>(P, n);
