@@ -206,7 +206,7 @@ struct lbm_handle {
     void* buf[2] = {nullptr, nullptr};
     void* dT = nullptr;
     void* dT2 = nullptr;   // second history array of the two-step form (allocated on first use)
-    int t2h = 0;              // its block height (chosen with dT2)
+    lbmk::T2Shape t2 = {};    // its block shape and build (chosen with dT2)
     unsigned int* status = nullptr;
     double* scratch = nullptr;
     double* diag_out = nullptr;
@@ -394,7 +394,7 @@ cudaError_t enqueue_two(lbm_handle* h, int from, int back, cudaStream_t s) {
     auto run = [&](auto P, auto tag) {
         if (back) std::swap(P.dT, P.dT_out);
         P.prefetch_rows = lbmk::prefetch_rows_two_steps(decltype(tag)::value, (long long)P.nx * P.ny);
-        return lbmk::launch_step2<decltype(tag)::value>(P, q, h->t2h, s);
+        return lbmk::launch_step2<decltype(tag)::value>(P, q, h->t2, s);
     };
     switch (h->p.precision) {
         case LBM_F32: return run(make_params<float>(h, from), std::integral_constant<int, lbmk::MODE_F32>{});
@@ -415,7 +415,7 @@ int ensure_dT2(lbm_handle* h) {
     int dev = 0, nsm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return cuda_fail(h);
-    h->t2h = lbmk::t2_block(h->p.nx, h->p.ny, nsm);
+    h->t2 = lbmk::t2_block(h->p.nx, h->p.ny, nsm);
     h->dT2 = dev_alloc(h, h->L.dT_bytes);
     return h->dT2 ? LBM_OK : LBM_ERR_OOM;
 }
@@ -1332,9 +1332,9 @@ const void* group2_fn(const lbm_batch* b, bool few) {
 
 size_t group2_smem(const lbm_batch* b) {
     switch (b->precision) {
-        case LBM_F32: return lbmk::step2_smem<lbmk::MODE_F32>(b->qt, lbmk::kT2HMany);
-        case LBM_F16: return lbmk::step2_smem<lbmk::MODE_F16>(b->qt, lbmk::kT2HMany);
-        case LBM_BF16: return lbmk::step2_smem<lbmk::MODE_BF16>(b->qt, lbmk::kT2HMany);
+        case LBM_F32: return lbmk::step2_smem<lbmk::MODE_F32>(b->qt, true);
+        case LBM_F16: return lbmk::step2_smem<lbmk::MODE_F16>(b->qt, true);
+        case LBM_BF16: return lbmk::step2_smem<lbmk::MODE_BF16>(b->qt, true);
         default: return 0;
     }
 }
@@ -1610,10 +1610,13 @@ int lbm_batch_create(lbm_handle* const* runs, int32_t n_runs, int32_t autotune, 
         b->flip.push_back(runs[r]->cur);
         b->form.push_back(runs[r]->form);
     }
-    // the single-run kernel's own shape rule until tuned (64 x 2 small, 128 x 1 large)
+    // the single-run kernel's own shape rule until tuned
     for (int r = 0; r < n_runs; ++r) {
-        const dim3 sb = lbmk::step_block(runs[r]->p.nx, runs[r]->p.ny);
-        b->shape.push_back(sb.x == 64 ? 5 : 4);
+        const dim3 sb = lbmk::step_block(b->precision, runs[r]->p.nx, runs[r]->p.ny);
+        int id = 0;
+        for (int k = 0; k < kNumShapes; ++k)
+            if (kShapes[k][0] == (int)sb.x && kShapes[k][1] == (int)sb.y) id = k;
+        b->shape.push_back(id);
     }
     b->params_stride = b->precision == LBM_F64 ? sizeof(lbmk::StepParams<double>) : sizeof(lbmk::StepParams<float>);
     for (lbm_handle* h : b->runs)

@@ -157,12 +157,22 @@ inline cudaError_t dispatch_step(int qt, int flow, int ph, Fn&& fn) {
     });
 }
 
-// Block shape of the single-run step kernel by grid size (measured on GB300,
-// us per step: 128^2 and 192^2 finish sooner in 64 x 2 blocks, 1.63 and 1.86
-// against 1.73 and 2.11 in 128 x 1; from 256^2 up one-row blocks do as well or
-// better, 2.37 against 2.47 at 256^2).
-inline dim3 step_block(int nx, int ny) {
-    return (long long)nx * ny <= 40000 ? dim3(64, 2) : dim3(128, 1);
+// Block shape of the one-node-per-thread step kernel (GB300, us per step).
+// FP64: 64 x 1; two warps spread over the SMs' schedulers better than four where
+// each scheduler has only a few, 64 cycles an operation each (128 x 1 / 64 x 1:
+// 150^2 15.9 / 12.6, 256^2 30.1 / 28.3).  Others: 64 x 2 up to 40,000 nodes
+// (128^2 in one step per launch 1.63, 128 x 1 1.73); 128 x 1 from there; where
+// the grid takes more than a wave of blocks, the width of 128, 64 and 32 that
+// leaves the fewest columns idle (128 x 1 / 64 x 1 / 32 x 2, FP32: 400 x 390
+// 4.11 / 3.62 / 3.61, 777 x 501 7.10 / 7.03 / 6.80, 512^2 5.00 all).
+inline dim3 step_block(int mode, int nx, int ny) {
+    const long long nodes = (long long)nx * ny;
+    if (mode == MODE_F64) return dim3(64, 1);
+    if (nodes <= 40000) return dim3(64, 2);
+    if (nodes <= 1ll << 17) return dim3(128, 1);
+    auto cover = [&](int w) { return (nx + w - 1) / w * w; };
+    if (cover(128) <= cover(64)) return dim3(128, 1);
+    return cover(64) <= cover(32) ? dim3(64, 1) : dim3(32, 2);
 }
 
 // Step forms.  FORM_SINGLE is one step per launch, FORM_PAIRS that with node
@@ -328,7 +338,7 @@ const void* group_kernel(int qt, int flow, int ph, bool few) {
 // for it before touching the state), so the launch overlaps its tail.
 template <int M>
 cudaError_t launch_step(const StepParams<typename ModeTraits<M>::R>& P, int qt, int flow, int form, cudaStream_t s) {
-    const StepLaunch L = step_launch<M>(P, qt, flow, form, step_block(P.nx, P.ny));
+    const StepLaunch L = step_launch<M>(P, qt, flow, form, step_block(M, P.nx, P.ny));
     void* args[1] = {const_cast<StepParams<typename ModeTraits<M>::R>*>(&P)};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -363,9 +373,14 @@ inline dim3 t2_grid(int nx, int ny, int h) {
     return dim3((unsigned)t2_tiles(nx, kT2W - 2), (unsigned)t2_tiles(ny, h - 2), 1u);
 }
 
-inline int t2_block(int nx, int ny, int nsm) {
+struct T2Shape {
+    int h;       // block height
+    bool many;   // the many-tiles build
+};
+
+inline T2Shape t2_block(int nx, int ny, int nsm) {
     if (nsm < 1) nsm = 1;
-    int best = kT2HMany;
+    T2Shape best = {kT2HMany, true};
     double best_cost = -1.0;
     for (int h = 4; h <= kT2H; ++h) {
         const long long tiles = t2_tiles(nx, kT2W - 2) * t2_tiles(ny, h - 2);
@@ -374,15 +389,16 @@ inline int t2_block(int nx, int ny, int nsm) {
         const long long work = per_sm * ((kT2W * h + 31) / 32 * 32 + (long long)(kT2W - 2) * (h - 2));
         const double cost = per_sm > 1 ? kT2Overlap * (double)work : (double)work;
         if (best_cost < 0.0 || cost < best_cost) {
-            best = h;
+            best = {h, false};
             best_cost = cost;
         }
     }
     return best;
 }
 
-// The build of the kernel for block height h (h == kT2HMany: the many-tiles
-// build) and its dynamic shared memory.
+// The build of the kernel (many: the many-tiles build, for kT2HMany rows and
+// launch bounds for three blocks per SM; 300^2 with 12 rows and two tiles per
+// SM takes 2.53 us per step in it) and its dynamic shared memory.
 template <int M, int HM>
 const void* step2_kernel_hm(int qt, int phase_k) {
     if (qt == 5) return phase_k ? (const void*)fused_step2<M, 5, true, HM> : (const void*)fused_step2<M, 5, false, HM>;
@@ -390,17 +406,17 @@ const void* step2_kernel_hm(int qt, int phase_k) {
 }
 
 template <int M>
-const void* step2_kernel(int qt, int phase_k, int h) {
+const void* step2_kernel(int qt, int phase_k, bool many) {
     if constexpr (M != MODE_F64) {
-        return h == kT2HMany ? step2_kernel_hm<M, kT2HMany>(qt, phase_k) : step2_kernel_hm<M, kT2H>(qt, phase_k);
+        return many ? step2_kernel_hm<M, kT2HMany>(qt, phase_k) : step2_kernel_hm<M, kT2H>(qt, phase_k);
     }
     return nullptr;
 }
 
 template <int M>
-size_t step2_smem(int qt, int h) {
+size_t step2_smem(int qt, bool many) {
     if constexpr (M != MODE_F64) {
-        if (h == kT2HMany) return qt == 5 ? Tile2<M, 5, kT2HMany>::bytes : Tile2<M, 9, kT2HMany>::bytes;
+        if (many) return qt == 5 ? Tile2<M, 5, kT2HMany>::bytes : Tile2<M, 9, kT2HMany>::bytes;
         return qt == 5 ? Tile2<M, 5, kT2H>::bytes : Tile2<M, 9, kT2H>::bytes;
     }
     return 0;
@@ -424,14 +440,14 @@ const void* group2_kernel(int qt, int phase_k, bool few) {
 inline long long group2_blocks(int nx, int ny) { return t2_tiles(nx, kT2W - 2) * t2_tiles(ny, kT2HMany - 2); }
 
 // Two steps from copy P.src to P.dst, history P.dT -> P.dT_out, in blocks of
-// kT2W x h threads, as a programmatic dependent of the previous launch in the
+// kT2W x t.h threads, as a programmatic dependent of the previous launch in the
 // stream.
 template <int M>
-cudaError_t launch_step2(const StepParams<typename ModeTraits<M>::R>& P, int qt, int h, cudaStream_t s) {
-    if (h < 4 || h > kT2H) return cudaErrorInvalidConfiguration;
-    const void* fn = step2_kernel<M>(qt, P.phase_k, h);
+cudaError_t launch_step2(const StepParams<typename ModeTraits<M>::R>& P, int qt, T2Shape t, cudaStream_t s) {
+    if (t.h < 4 || t.h > (t.many ? kT2HMany : kT2H)) return cudaErrorInvalidConfiguration;
+    const void* fn = step2_kernel<M>(qt, P.phase_k, t.many);
     if (!fn) return cudaErrorInvalidConfiguration;
-    const size_t smem = step2_smem<M>(qt, h);
+    const size_t smem = step2_smem<M>(qt, t.many);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     void* args[1] = {const_cast<StepParams<typename ModeTraits<M>::R>*>(&P)};
@@ -439,8 +455,8 @@ cudaError_t launch_step2(const StepParams<typename ModeTraits<M>::R>& P, int qt,
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = t2_grid(P.nx, P.ny, h);
-    cfg.blockDim = dim3((unsigned)kT2W, (unsigned)h, 1u);
+    cfg.gridDim = t2_grid(P.nx, P.ny, t.h);
+    cfg.blockDim = dim3((unsigned)kT2W, (unsigned)t.h, 1u);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cfg.attrs = attr;
@@ -526,9 +542,9 @@ int batch_blocks_per_sm(int qt, int flow, int ph) {
                                          int, int, cudaStream_t);                                               \
     KW template int batch_blocks_per_sm<M>(int, int, int);                                                   \
     KW template const void* group_kernel<M>(int, int, int, bool);                                                    \
-    KW template cudaError_t launch_step2<M>(const StepParams<ModeTraits<M>::R>&, int, int, cudaStream_t);     \
+    KW template cudaError_t launch_step2<M>(const StepParams<ModeTraits<M>::R>&, int, T2Shape, cudaStream_t); \
     KW template const void* group2_kernel<M>(int, int, bool);                                                        \
-    KW template size_t step2_smem<M>(int, int);                                                                \
+    KW template size_t step2_smem<M>(int, bool);                                                               \
     KW template StepLaunch step_launch<M>(const StepParams<ModeTraits<M>::R>&, int, int, int, dim3);
 
 #define LBMK_CONVERT_TEMPLATES(KW, M)                                                                         \
