@@ -1321,8 +1321,9 @@ __device__ __forceinline__ void step2_tile(const StepParams<typename ModeTraits<
         else live = false;
     }
     griddep_wait();
-    // the tile's rows, prefetch_rows further on, of the chunk that starts at its first inner column
-    if (P.prefetch_rows > 0 && lx == 1 && (x2 & (kChunk - 1)) == 0 && ly >= 1 && ly <= H - 2)
+    // the tile's rows, prefetch_rows further on, of the chunk that starts at its first inner
+    // column (in the many-tiles build only: the test costs 64^2 0.03 us a step)
+    if (HM == kT2HMany && P.prefetch_rows > 0 && lx == 1 && (x2 & (kChunk - 1)) == 0 && ly >= 1 && ly <= H - 2)
         prefetch_rows<M, QT, true>(P, x2, y2 + P.prefetch_rows, 1);
     if (live) {
         const WallAt<R> w(P, x, y);
