@@ -416,6 +416,15 @@ int ensure_dT2(lbm_handle* h) {
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return cuda_fail(h);
     h->t2 = lbmk::t2_block(h->p.nx, h->p.ny, nsm);
+    cudaError_t e = cudaSuccess;
+    const int q = h->p.thermal_q, ph = phase_k_of(h);
+    switch (h->p.precision) {
+        case LBM_F32: e = lbmk::prepare_step2<lbmk::MODE_F32>(q, ph, h->t2); break;
+        case LBM_F16: e = lbmk::prepare_step2<lbmk::MODE_F16>(q, ph, h->t2); break;
+        case LBM_BF16: e = lbmk::prepare_step2<lbmk::MODE_BF16>(q, ph, h->t2); break;
+        default: break;   // (no two-step kernel)
+    }
+    if (e != cudaSuccess) return cuda_fail(h);
     h->dT2 = dev_alloc(h, h->L.dT_bytes);
     return h->dT2 ? LBM_OK : LBM_ERR_OOM;
 }

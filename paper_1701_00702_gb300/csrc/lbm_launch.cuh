@@ -439,6 +439,15 @@ const void* group2_kernel(int qt, int phase_k, bool few) {
 
 inline long long group2_blocks(int nx, int ny) { return t2_tiles(nx, kT2W - 2) * t2_tiles(ny, kT2HMany - 2); }
 
+// Lets the kernel of a run's two-step launches take its shared memory; once,
+// before the first of them on the device.
+template <int M>
+cudaError_t prepare_step2(int qt, int phase_k, T2Shape t) {
+    const void* fn = step2_kernel<M>(qt, phase_k, t.many);
+    if (!fn) return cudaErrorInvalidConfiguration;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)step2_smem<M>(qt, t.many));
+}
+
 // Two steps from copy P.src to P.dst, history P.dT -> P.dT_out, in blocks of
 // kT2W x t.h threads, as a programmatic dependent of the previous launch in the
 // stream.
@@ -448,8 +457,6 @@ cudaError_t launch_step2(const StepParams<typename ModeTraits<M>::R>& P, int qt,
     const void* fn = step2_kernel<M>(qt, P.phase_k, t.many);
     if (!fn) return cudaErrorInvalidConfiguration;
     const size_t smem = step2_smem<M>(qt, t.many);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     void* args[1] = {const_cast<StepParams<typename ModeTraits<M>::R>*>(&P)};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -543,6 +550,7 @@ int batch_blocks_per_sm(int qt, int flow, int ph) {
     KW template int batch_blocks_per_sm<M>(int, int, int);                                                   \
     KW template const void* group_kernel<M>(int, int, int, bool);                                                    \
     KW template cudaError_t launch_step2<M>(const StepParams<ModeTraits<M>::R>&, int, T2Shape, cudaStream_t); \
+    KW template cudaError_t prepare_step2<M>(int, int, T2Shape);                                              \
     KW template const void* group2_kernel<M>(int, int, bool);                                                        \
     KW template size_t step2_smem<M>(int, bool);                                                               \
     KW template StepLaunch step_launch<M>(const StepParams<ModeTraits<M>::R>&, int, int, int, dim3);
