@@ -1226,6 +1226,69 @@ __global__ void __launch_bounds__(256, (kMinBlocks<M, QT, FLOW>)) fused_step(con
     step_node<M, QT, FLOW, PH>(P, x, y);
 }
 
+// FP64 runs without flow on grids that leave most schedulers idle: two lanes
+// per node, the even one with the PCM, the odd one with the metal lattice.  One
+// warp's chain of FP64 operations, 64 cycles each whatever its lanes do, is the
+// step's time there (200 x 4: 58 operations a warp, 3.46 us a step), and the two
+// lattices take the same operations with constants of their own; the
+// temperatures cross by shuffle.  Operation for operation step_node's, D2Q5
+// with constant PCM properties.
+template <int M>   // MODE_F64
+__global__ void __launch_bounds__(64) conduction_step_lanes(const __grid_constant__ StepParams<double> P) {
+    const int xr = blockIdx.x * 32 + (threadIdx.x >> 1), y = blockIdx.y;
+    const bool metal = threadIdx.x & 1, live = xr < P.nx;
+    const int x = live ? xr : P.nx - 1;   // lanes beyond the grid go along and put nothing
+    griddep_wait();
+    const WallAt<double> w(P, x, y);
+    const PullAt<M, 5, false> a(P, w.xs, w.ys);
+    double* h = P.dT + (y * P.pitch + x);
+    const double dTp = *h;
+    const int first = metal ? 5 : 0;   // the lattice's first plane
+    double g[5], n[5];
+#pragma unroll
+    for (int q = 0; q < 5; ++q) g[q] = __ldg(a.src(q) + (first + q) * kChunk);
+    thermal_moments<double, 5>(g, n);
+    double Tf, fl;
+    enthalpy_state(P, n[0], Tf, fl);
+    auto exchange = [&]() {   // both temperatures on both lanes
+        const double mine = metal ? n[0] : Tf, other = __shfl_xor_sync(0xffffffffu, mine, 1);
+        Tf = metal ? other : mine;
+        return metal ? mine : other;
+    };
+    double Tm = exchange();
+    if (__any_sync(0xffffffffu, w.wall && P.wall_kind[w.side] == 0)) {
+        if (w.wall && P.wall_kind[w.side] == 0) {   // Eq. 52 (an adiabatic wall at rest keeps x_f's moments)
+            const double Tb = P.wall_T[w.side];
+            n[3] = vfma(metal ? P.vcm : P.vcf, vsub(Tb, metal ? Tm : Tf), n[3]);
+            n[0] = metal ? Tb : P.wall_H[w.side];
+            enthalpy_state(P, n[0], Tf, fl);
+        }
+        Tm = exchange();
+    }
+    const double S_met = vfma(P.x_now, vsub(Tm, Tf), vmul(P.x_prev, dTp));
+    const double hm = vadd(Tm, S_met), took = vsub(hm, Tm);
+    const double S = metal ? S_met : vmul(P.x_pm, took), n0 = metal ? hm : vfma(P.x_pm, took, n[0]);
+    const double zj = metal ? P.e_j : P.z_j;
+    const double jx = vmul(zj, n[1]), jy = vmul(zj, n[2]);
+    const double a3 = vfma(metal ? P.e_3 : P.z_3, n[3],
+                           vfma(metal ? P.e_3T : P.z_3T, metal ? Tm : Tf, vmul(P.quart_varpi, S)));
+    const double a4 = vmul(metal ? P.e_4 : P.z_4, n[4]);
+    const double p = vadd(a3, a4), q = vsub(a3, a4);
+    const double v1 = vadd(p, jx), v3 = vsub(p, jx), v2 = vadd(q, jy), v4 = vsub(q, jy);
+    __syncwarp();   // both lanes have read the history that one of them writes
+    if (!live) return;
+    double* db = next_bulk<M, 5, false>(P, x, y) + first * kChunk;
+    db[0] = vsub(n0, vadd(vadd(v1, v3), vadd(v2, v4)));
+    db[kChunk] = v1;
+    db[2 * kChunk] = v2;
+    db[3 * kChunk] = v3;
+    db[4 * kChunk] = v4;
+    if (!metal) {
+        *h = vsub(Tm, Tf);
+        if (runaway(n[0], Tm, 1.0, 0.0)) atomicOr(P.status, STATUS_UNSTABLE);
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Two time steps per launch
 // ---------------------------------------------------------------------------

@@ -256,6 +256,11 @@ inline int prefetch_rows_two_steps(int mode, long long nodes) {
     return mode == MODE_F32 && nodes >= kTwoStepF32MinNodes ? kPrefetchRowsTwoSteps : 0;
 }
 
+// FP64 runs without flow take conduction_step_lanes while its warps, of 16
+// nodes, find a scheduler each (152 SMs x 4); beyond, two warps of 33 FP64
+// operations in turn take longer than one of 50.
+constexpr long long kConductionLanesMaxNodes = 152 * 4 * 16;
+
 // The one-step kernel of a run, with its grid: one node per thread in blocks of
 // b threads, or node pairs in blocks of 32 x 4.
 struct StepLaunch {
@@ -271,6 +276,14 @@ StepLaunch step_launch(const StepParams<typename ModeTraits<M>::R>& P, int qt, i
             L.fn = P.phase_k ? (const void*)fused_step_pair<M, true> : (const void*)fused_step_pair<M, false>;
             L.block = dim3(32, 4);   // 2048^2 FP16 61.25 us per step (64 x 2: 61.98)
             L.grid = dim3((unsigned)(((P.nx + 1) / 2 + 31) / 32), (unsigned)((P.ny + 3) / 4), 1u);
+            return L;
+        }
+    }
+    if constexpr (M == MODE_F64) {
+        if (qt == 5 && !flow && !P.phase_k && (long long)P.nx * P.ny <= kConductionLanesMaxNodes) {
+            L.fn = (const void*)conduction_step_lanes<M>;
+            L.block = dim3(64, 1);
+            L.grid = dim3((unsigned)((P.nx + 31) / 32), (unsigned)P.ny, 1u);
             return L;
         }
     }

@@ -133,3 +133,24 @@ def test_diagnostics_are_the_sums_of_the_fields(lbm, shape, prec):
         k_e = phi * p["k_f"] + (1 - phi) * c["k_m"]
         nu = p["L_char"] / k_e * (phi * p["k_f"] * g[0] + (1 - phi) * c["k_m"] * g[1]).mean()
         assert abs(d["nu_hot"] - nu) <= 1e-11 * max(1.0, abs(nu))
+
+
+@pytest.mark.parametrize("shape", [(1, 1, 1, 1), (3, 3, 0, 0), (31, 5, 0, 1), (33, 4, 1, 0), (200, 4, 0, 1), (97, 100, 0, 0),
+                                   (608, 16, 0, 1), (609, 16, 0, 1)])
+@pytest.mark.parametrize("kinds", [(0, 0, 1, 1), (1, 0, 0, 1)])
+def test_conduction_lanes_equal_one_node_per_thread(lbm, shape, kinds):
+    """FP64 runs without flow up to 9,728 nodes step with two lanes per node; the
+    tile-list batch steps one node per thread.  Equal checkpoints after five
+    steps, on both sides of the limit and with either wall on every side."""
+    nx, ny, px, py = shape
+    p = inputs.conduction_1d(nx, ny, periodic_x=px, periodic_y=py, wall_kind=list(kinds), wall_T=[1.0, 0.0, 0.4, 0.7],
+                             T_solidus=0.29, T_liquidus=0.31, L_char=100.0)
+    _, G, H, dT = inputs.random_state(nx, ny, 5, seed=nx + ny, H_range=(0.0, 1.6))
+    s = lbm.Solver(p)
+    s.set_state(None, G, H, dT)
+    t = twin(lbm, s, 0)
+    b = lbm.Batch([t], autotune=False).configure(128, 0)
+    s.step(5)
+    b.step(5)
+    assert s.status() == 0 and np.array_equal(s.save(), t.save())
+    b.close()
