@@ -971,8 +971,8 @@ __device__ __forceinline__ T thermal_collide(const StepParams<typename ModeTrait
     T g[QT], h[QT];   // post-collision populations; g[0], h[0]: provisional rest populations
     if constexpr (QT == 5) {
         // n* = (1 - z) n + z n^eq + S s, the factors of M^-1 folded into the constants:
-        // a_j = n*_{1,2} / 2, a_3 = n*_3 / 4, a_4 = n*_4 / 4
-        T jx, jy, a3, a4;
+        // j = n*_{1,2} / 2, a3 = n*_3 / 4, and with z4 n_4 = n*_4 / 4 the movers are a3 +- z4 n_4 +- j
+        T jx, jy, a3, z4 = bc<T>(P.z_4);
         if (PH && P.phase_k) {
             // Eq. 9 at the node's liquid fraction -> zeta_alpha (Eq. A19) -> zeta_e (Eq. 53)
             const T za = vrcp(vaddc(vfma(bc<T>(P.kd_c), n.fl, bc<T>(P.ks_c)), R(0.5)));
@@ -985,7 +985,7 @@ __device__ __forceinline__ T thermal_collide(const StepParams<typename ModeTrait
             jy = vmulc<T>(R(0.5), vfma(vneg(z[2]), d2, n.n[2]));
             const T d3 = vfmac<T>(-P.vcf, n.Tf, n.n[3]);
             a3 = vfmac<T>(P.quart_varpi, S_pcm, vmulc<T>(R(0.25), vfma(vneg(z[3]), d3, n.n[3])));
-            a4 = vmulc<T>(R(0.25), vfma(vneg(z[4]), n.n[4], n.n[4]));
+            z4 = vmulc<T>(R(0.25), vaddc(vneg(z[4]), R(1)));
         } else {
             jx = vmulc<T>(P.z_j, n.n[1]);
             jy = vmulc<T>(P.z_j, n.n[2]);
@@ -995,14 +995,18 @@ __device__ __forceinline__ T thermal_collide(const StepParams<typename ModeTrait
                 jy = vfma(t, n.uy, jy);
             }
             a3 = vfmac<T>(P.z_3, n.n[3], vfmac<T>(P.z_3T, n.Tf, vmulc<T>(P.quart_varpi, S_pcm)));
-            a4 = vmulc<T>(P.z_4, n.n[4]);
         }
         const T c3 = vfmac<T>(P.e_3, n.k[3], vfmac<T>(P.e_3T, n.k[0], vmulc<T>(P.quart_varpi, S_met)));
-        const T c4 = vmulc<T>(P.e_4, n.k[4]);
-        const T kx = vmulc<T>(P.e_j, n.k[1]), ky = vmulc<T>(P.e_j, n.k[2]);
-        const T gp = vadd(a3, a4), gm = vsub(a3, a4), hp = vadd(c3, c4), hq = vsub(c3, c4);
-        g[1] = vadd(gp, jx); g[3] = vsub(gp, jx); g[2] = vadd(gm, jy); g[4] = vsub(gm, jy);
-        h[1] = vadd(hp, kx); h[3] = vsub(hp, kx); h[2] = vadd(hq, ky); h[4] = vsub(hq, ky);
+        const T gp = vfma(z4, n.n[4], a3), gm = vfma(vneg(z4), n.n[4], a3);
+        const T hp = vfmac<T>(P.e_4, n.k[4], c3), hq = vfmac<T>(-P.e_4, n.k[4], c3);
+        if (FLOW || (PH && P.phase_k)) {
+            g[1] = vadd(gp, jx); g[3] = vsub(gp, jx); g[2] = vadd(gm, jy); g[4] = vsub(gm, jy);
+        } else {
+            g[1] = vfmac<T>(P.z_j, n.n[1], gp); g[3] = vfmac<T>(-P.z_j, n.n[1], gp);
+            g[2] = vfmac<T>(P.z_j, n.n[2], gm); g[4] = vfmac<T>(-P.z_j, n.n[2], gm);
+        }
+        h[1] = vfmac<T>(P.e_j, n.k[1], hp); h[3] = vfmac<T>(-P.e_j, n.k[1], hp);
+        h[2] = vfmac<T>(P.e_j, n.k[2], hq); h[4] = vfmac<T>(-P.e_j, n.k[2], hq);
         g[0] = vfmac<T>(R(-4), a3, n0);
         h[0] = vfmac<T>(R(-4), c3, hm);
     } else {
@@ -1269,12 +1273,11 @@ __global__ void __launch_bounds__(64) conduction_step_lanes(const __grid_constan
     const double hm = vadd(Tm, S_met), took = vsub(hm, Tm);
     const double S = metal ? S_met : vmul(P.x_pm, took), n0 = metal ? hm : vfma(P.x_pm, took, n[0]);
     const double zj = metal ? P.e_j : P.z_j;
-    const double jx = vmul(zj, n[1]), jy = vmul(zj, n[2]);
     const double a3 = vfma(metal ? P.e_3 : P.z_3, n[3],
                            vfma(metal ? P.e_3T : P.z_3T, metal ? Tm : Tf, vmul(P.quart_varpi, S)));
-    const double a4 = vmul(metal ? P.e_4 : P.z_4, n[4]);
-    const double p = vadd(a3, a4), q = vsub(a3, a4);
-    const double v1 = vadd(p, jx), v3 = vsub(p, jx), v2 = vadd(q, jy), v4 = vsub(q, jy);
+    const double z4 = metal ? P.e_4 : P.z_4;
+    const double p = vfma(z4, n[4], a3), q = vfma(-z4, n[4], a3);
+    const double v1 = vfma(zj, n[1], p), v3 = vfma(-zj, n[1], p), v2 = vfma(zj, n[2], q), v4 = vfma(-zj, n[2], q);
     __syncwarp();   // both lanes have read the history that one of them writes
     if (!live) return;
     double* db = next_bulk<M, 5, false>(P, x, y) + first * kChunk;
