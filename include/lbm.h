@@ -189,40 +189,46 @@ int lbm_create_ex(const lbm_params* p, void* cuda_stream, lbm_alloc_fn alloc,
  * on the host (LBM_ERR_UNSTABLE after any synchronising call saw the device
  * flag).  Large nsteps are replayed from a captured CUDA graph.  Each step is
  * launched as a programmatic dependent of the previous one in the stream.
- * The step kernel runs one node per thread in blocks of 64 x 2 threads on
- * grids of up to 40,000 nodes and 128 x 1 on larger ones, or node pairs, or
- * two steps per launch (see lbm_set_step_form). */
+ * The step kernel runs one node per thread (FP64: blocks of 64 x 1 threads;
+ * the others: 64 x 2 on grids of up to 40,000 nodes, 128 x 1 on larger ones,
+ * and beyond 131,072 nodes the one of 128 x 1, 64 x 1 and 32 x 2 that leaves
+ * the fewest columns idle), two nodes per thread, or two steps per launch (see
+ * lbm_set_step_form); FP64 runs without flow, with D2Q5 lattices and constant
+ * conductivity, take two threads per node on grids of up to 9,728 nodes. */
 int lbm_step(lbm_handle* h, int64_t nsteps);
 
 /* Step form of a run (the paper has no counterpart: an implementation
- * choice).  LBM_STEP_FORM_SINGLE: one node per thread.  LBM_STEP_FORM_PAIRS:
- * two neighbouring nodes per thread, each FP32 operation one packed
- * instruction for both; taken only by runs in the default configuration (flow,
- * D2Q5 thermal lattices, volumetric blend, FP32/FP16/BF16 storage), the others
- * keep one node per thread.  On grids of at least 1,572,864 nodes (state far
- * beyond L2) each node-pair block also asks L2 for the rows that blocks 48
- * rows further on will read (bulk L2 prefetch).  LBM_STEP_FORM_TWO_STEPS:
- * two time steps per launch for runs with flow in FP32/FP16/BF16 storage (the
- * others step one node per thread): each block of 34 x H threads advances its
- * tile and the one-node ring around it one step into shared memory, then the
- * tile's 32 x (H - 2) inner nodes a second step into the other state copy (H
- * from 4 to 16 per grid, at most two tiles per SM where the grid allows, else
- * H = 12);
+ * choice).  LBM_STEP_FORM_SINGLE: one step per launch, one node per thread, or
+ * two neighbouring nodes (as the next form, without its prefetch) in FP16/BF16
+ * runs of at least 131,072 nodes that could take that form.
+ * LBM_STEP_FORM_PAIRS: two neighbouring nodes per thread, each FP32 operation
+ * one packed instruction for both; taken only by runs in the default
+ * configuration (flow, D2Q5 thermal lattices, volumetric blend,
+ * FP32/FP16/BF16 storage), the others keep one node per thread.  On grids of at
+ * least 1,572,864 nodes (state far beyond L2) each node-pair block also asks L2
+ * for the rows that blocks 48 rows further on will read (bulk L2 prefetch).
+ * LBM_STEP_FORM_TWO_STEPS: two time steps per launch for runs with flow in
+ * FP32/FP16/BF16 storage (the others step one node per thread): each block of
+ * 34 x H threads advances its tile and the one-node ring around it one step
+ * into shared memory, then the tile's 32 x (H - 2) inner nodes a second step
+ * into the other state copy (H from 4 to 16 per grid, at most two tiles per SM
+ * where the grid allows, else H = 12; FP32 grids of at least 786,432 nodes
+ * prefetch the rows 20 further on into L2);
  * lbm_step takes it for 4 steps or more (an odd remainder and steps that bring
  * the run back to state copy 0 are single steps).  LBM_STEP_FORM_AUTO (the
  * default), for runs with flow and the D2Q5 thermal lattices: two steps per
  * launch on grids of up to 102,400 nodes in FP32/FP16/BF16 and on FP32 grids
  * of at least 786,432 nodes (state beyond L2); node pairs for FP16/BF16 runs
- * of at least 1,572,864 (1536 x 1024) nodes; otherwise one node per thread.
- * Two steps per launch give the states of one step per launch bit for bit;
- * node pairs agree with them to within a few roundings of the FP32
- * arithmetic.  A run that steps two steps per launch keeps a second
- * exchange-history array (4 bytes per node of row pitch), allocated on the
- * run's allocator at the first lbm_step that uses the form (LBM_ERR_OOM if
- * that fails; nothing stepped).  Applies to later lbm_step calls and to
- * batches created afterwards (batches advance one step per launch: a run in
- * the two-step form steps there one node per thread); synchronises the run's
- * stream when it drops a captured graph.  LBM_ERR_ARG for another value. */
+ * of at least 1,572,864 (1536 x 1024) nodes; otherwise LBM_STEP_FORM_SINGLE.
+ * Every form gives the same states bit for bit: all kernels share one node
+ * update in which each rounding is fixed.  A run that steps two steps per
+ * launch keeps a second exchange-history array (4 bytes per node of row
+ * pitch), allocated on the run's allocator at the first lbm_step that uses the
+ * form (LBM_ERR_OOM if that fails; nothing stepped).  Applies to later lbm_step
+ * calls and to batches created afterwards (batches advance one step per launch
+ * except under map 5: a run in the two-step form steps there as
+ * LBM_STEP_FORM_SINGLE); synchronises the run's stream when it drops a captured
+ * graph.  LBM_ERR_ARG for another value. */
 #define LBM_STEP_FORM_AUTO 0
 #define LBM_STEP_FORM_SINGLE 1
 #define LBM_STEP_FORM_PAIRS 2
@@ -309,33 +315,29 @@ const char* lbm_strerror(int code);
  * run's kernel takes one of the block shapes 128 x 2, 64 x 4, 32 x 8, 256 x 1
  * (256 threads), 128 x 1, 64 x 2, 32 x 4 (128) or 64 x 1, 32 x 2 (64).  Map
  * 4 steps the runs below 1,048,576 nodes in grouped launches, one kernel per
- * step for up to about 40 runs (23 in FP64) at a time, their parameter
- * blocks in the launch's own parameters, each run in tiles of w x 128/w
- * nodes (w = 32, 64 or 128, whichever leaves the fewest of the run's threads
- * idle); each group of runs is a chain of its own in the graph, and larger
- * runs keep their own step kernel in chains of their own, as under map 3.
- * Map 5 (runs with flow in FP32/FP16/BF16 storage) advances every run two
- * steps per launch in grouped launches of the two-step kernel (blocks of 34
- * x 12 threads, inner tiles of 32 x 10 nodes; see lbm_set_step_form), 32
- * launches per 64 steps, each run keeping a second exchange-history array
- * (allocated on its allocator when map 5 is chosen; LBM_ERR_OOM if that
- * fails); steps that align the batch to an even parity, and an odd
- * remainder, take each run's one-step kernel (one node per thread).
+ * step for up to 54 runs (29 in FP64) at a time, their parameter blocks in the
+ * launch's own parameters, each run in tiles of w x 128/w nodes (FP16/BF16 with
+ * flow and D2Q5: w x 256/w, two nodes per thread; w = 32, 64 or 128, whichever
+ * leaves the fewest of the run's threads idle).  In the replayed graph the runs
+ * form at least two groups of about equal size, each a chain of its own, so
+ * that one chain's launch overlaps another's tail; larger runs keep their own
+ * step kernel in chains of their own, as under map 3.  Map 5 (runs with flow in
+ * FP32/FP16/BF16 storage) advances every run two steps per launch in grouped
+ * launches of the two-step kernel (blocks of 34 x 12 threads, inner tiles of
+ * 32 x 10 nodes; see lbm_set_step_form), at least four groups side by side and
+ * 32 launches of each per 64 steps, each run keeping a second exchange-history
+ * array (allocated on its allocator when map 5 is chosen; LBM_ERR_OOM if that
+ * fails); steps that align the batch to an even parity, and an odd remainder,
+ * take each run's one-step kernel.
  * With autotune = 1 the call times, on freshly created copies of the runs (the
  * runs themselves do not move, but the copies hold as much device memory
  * again while tuning), map 3 with the block shape chosen per size class
  * (grid width <= 64, <= 128, <= 256, wider; one class at a time, keeping the
  * fastest shape), map 4, map 5 where it applies, and every combination of
  * tile-width cap (64, 128, 256) and map 0-2, and keeps the fastest; otherwise it takes width cap 128,
- * map 0, and for map 3 lbm_step's own block shapes (64 x 2 up to 40,000
- * nodes, 128 x 1 above).  Under map 3 a batched step equals lbm_step on each
- * run bit for bit.  Maps 0-2, 4 and 5 inline the same per-node code into
- * another kernel, where the compiler may fuse a few multiply-adds
- * differently: their states can differ from lbm_step's by a few roundings of
- * the arithmetic (FP32: 1-3 ulps in about 1e-4 of the flow populations per
- * step), which a 16-bit store sometimes carries into the last stored bit.  A
- * run's steps under maps 4 and 5 do not depend on the other runs of its
- * launch.
+ * map 0, and for map 3 lbm_step's own block shapes.  Under every map a
+ * batched step equals lbm_step on each run bit for bit, and a run's steps do not
+ * depend on the other runs of its batch.
  *
  * lbm_batch_step enqueues nsteps steps of every run on the batch's stream
  * and advances each run's step count.  Use the runs' own calls (fields,
@@ -382,17 +384,15 @@ int lbm_batch_destroy(lbm_batch* b);
  *   2. advances all active runs together by min(quantum, the smallest number
  *      of steps any active run still needs) through one lbm_batch (batched =
  *      1; the batch is rebuilt when membership changes, with the tile width
- *      cap and map of lbm_server_configure, default 128 and map 4, every
- *      active run in one grouped launch per step), then synchronises the
+ *      cap and map of lbm_server_configure, default 128 and map 4, its
+ *      active runs below 1,048,576 nodes in grouped launches), then synchronises the
  *      stream;
  *   3. retires every run that has taken its steps: its FP64 diagnostics
  *      (lbm_diag) go into a result record and its device memory is freed.
  * A request that arrives while others run joins them at the next tick.
  * With batched = 0 the engine is the plain form: one request at a time, in
  * arrival order, each advanced by lbm_step.  A run's result is the same
- * alone and in the mix, bit for bit: under map 4 (the default) a run's steps
- * do not depend on the other runs of the launch, under map 3 they equal
- * lbm_step's.
+ * alone and in the mix, bit for bit, under every map.
  *
  * All requests of a server share precision, thermal_q and flow (LBM_ERR_ARG
  * otherwise); a request that the budget can never hold (its state, plus

@@ -186,7 +186,7 @@ Layout layout_of(const lbm_params& p) {
     L.off_buf1 = L.copy_bytes;
     L.off_dT = 2 * L.copy_bytes;
     L.off_status = L.off_dT + L.dT_bytes;
-    L.off_scratch = L.off_status + kAlign;
+    L.off_scratch = L.off_status + 2 * kAlign;   // the flag and the diagnostics' results
     L.total = L.off_scratch + align_up((size_t)L.nblocks * 4 * sizeof(double));
     return L;
 }
@@ -1377,8 +1377,8 @@ cudaError_t group_args(const lbm_batch* b, const std::vector<int>& g, int parity
 // One batched step under map 4 (each group's launch and each large run's
 // own step) or two steps under map 5 (two = true, parity = back: each group's
 // two-step launch), as programmatic dependents of the previous launch in the stream.
-// Single steps under map 5 take each run's one-step kernel (one node per
-// thread), which rounds exactly as the two-step kernel does.
+// Single steps under map 5 take each run's one-step kernel (every kernel gives
+// the same bits).
 cudaError_t group_step_all(lbm_batch* b, int parity, cudaStream_t s, bool two = false, bool back = false) {
     if (b->mapping == 5 && !two) {
         for (size_t r = 0; r < b->runs.size(); ++r) {

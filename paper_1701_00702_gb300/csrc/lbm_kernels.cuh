@@ -547,9 +547,7 @@ __device__ __forceinline__ int col_off(int x) {
 // Pull streaming around node (xs, ys): the population along e_i comes from
 // xs - e_i.  The index wrap is also correct for interior nodes of a walled
 // direction, which never reach the edge.  PullAt holds the addressing (one
-// 64-bit row pointer per source row, one 32-bit offset per source column);
-// pull_flow and pull_thermal load one side each, so that the flow and the
-// thermal lattices of a node can also be pulled by two different threads.
+// 64-bit row pointer per source row, one 32-bit offset per source column).
 // Source column and row (x - e_x, y - e_y) of direction q, D2Q9 order of Eq. 11,
 // as 0 (x - 1 or y - 1), 1 (x or y), 2 (x + 1 or y + 1): columns 1 0 1 2 1 0 2 2 0,
 // rows 1 1 0 1 2 0 0 2 2, two bits per direction.
@@ -1182,9 +1180,9 @@ __device__ __forceinline__ void step_pair(const StepParams<float>& P, int x0, in
 }
 
 // Blocks of 256 threads each SM must hold, which caps the registers per
-// thread: five for the FP32 and 16-bit forms of D2Q5 with flow (48 registers;
-// with the packed arithmetic 40 registers and six blocks measured ~1 % slower
-// at 256^2 and 2048^2 in FP32); the others take what their registers allow.
+// thread: five for the FP32 and 16-bit forms of D2Q5 with flow (48 registers,
+// where the FP32 step at 2048^2 runs at the copy bandwidth); the others take
+// what their registers allow (FP64 and the D2Q9 forms are bound by arithmetic).
 template <int M, int QT, bool FLOW>
 constexpr int kMinBlocks = (QT == 5 && FLOW) ? (M == MODE_F64 ? 1 : 5) : 1;
 
@@ -1219,8 +1217,14 @@ __device__ __forceinline__ void prefetch_rows(const StepParams<typename ModeTrai
     }
 }
 
-// One run: one thread per node, 256 threads per block (128 x 2 by default;
-// the batch's map 3 may take other shapes).
+// One run: one thread per node, in blocks of the launcher's choice (step_block;
+// up to 256 threads, the batch's map 3 may take any of its shapes).  FP32 grids
+// beyond L2 are bound by HBM (2048^2 100 us per step, 160 B per update at
+// 6.7 TB/s); smaller ones by the launch floor, one warp's chain and instruction
+// issue (256^2 2.41 us per step before the update was written in named
+// multiply-adds and single-instruction reciprocals and roots, 2.15 now).  FP64
+// is bound by its two lanes per SM and clock: 252 FP64 operations per node took
+// 39.7 us per step at 256^2, 187 take 27.8 (in 64 x 1 blocks).
 template <int M, int QT, bool FLOW, bool PH>
 __global__ void __launch_bounds__(256, (kMinBlocks<M, QT, FLOW>)) fused_step(const __grid_constant__ StepParams<typename ModeTraits<M>::R> P) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1233,10 +1237,10 @@ __global__ void __launch_bounds__(256, (kMinBlocks<M, QT, FLOW>)) fused_step(con
 // FP64 runs without flow on grids that leave most schedulers idle: two lanes
 // per node, the even one with the PCM, the odd one with the metal lattice.  One
 // warp's chain of FP64 operations, 64 cycles each whatever its lanes do, is the
-// step's time there (200 x 4: 58 operations a warp, 3.46 us a step), and the two
-// lattices take the same operations with constants of their own; the
-// temperatures cross by shuffle.  Operation for operation step_node's, D2Q5
-// with constant PCM properties.
+// step's time there (200 x 4: both lattices in one lane 3.46 us a step, one
+// each 2.63, 4.96 before either), and the two lattices take the same operations
+// with constants of their own; the temperatures cross by shuffle.  Operation for
+// operation step_node's, D2Q5 with constant PCM properties.
 template <int M>   // MODE_F64
 __global__ void __launch_bounds__(64) conduction_step_lanes(const __grid_constant__ StepParams<double> P) {
     const int xr = blockIdx.x * 32 + (threadIdx.x >> 1), y = blockIdx.y;
@@ -1319,7 +1323,13 @@ __global__ void __launch_bounds__(64) conduction_step_lanes(const __grid_constan
 // take it) and HM = kT2HMany (H = 12 for grids of many tiles per SM, launch
 // bounds that leave three FP32 D2Q5 blocks resident: at 52 registers only two
 // fit, 2048^2 FP32 104 against 84 us per step; two blocks of the other builds,
-// which would spill under the three-block cap).
+// which would spill under the three-block cap).  Small grids are bound by the
+// launch floor and two dependency chains (64^2 FP32 1.315 us per step before
+// the update was written in named multiply-adds, 1.09 now; 256^2 2.05 / 1.86),
+// grids beyond L2 by instruction issue once their rows are prefetched (2048^2
+// 79.9 us per step before, 71.1 now; 49.5 at the copy bandwidth).  Two nodes
+// per thread in the tile, side by side or one above the other, were slower
+// (2048^2 77.0 and 73.3, 64^2 1.37): more registers, fewer warps.
 constexpr int kT2W = 34, kT2H = 16, kT2HMany = 12;
 
 template <int HM, int M, int QT>
@@ -1420,7 +1430,10 @@ __global__ void __launch_bounds__(kT2W * HM, (kT2Blocks<HM, M, QT>)) fused_step2
 // nodes, and the pair is read and written with one access per plane wherever
 // both elements are adjacent (x0 even keeps them inside one chunk, aligned).
 // The last node of an odd width, and both nodes of a bounce-back run, step
-// one by one.
+// one by one.  Bound by instruction issue up to L2's size and by HBM beyond
+// (us per step, before / with the update in named multiply-adds and 80
+// registers: FP16 512^2 5.52 / 4.77 (before: one node per thread), 1024^2 18.4 /
+// 15.2, 2048^2 61.2 / 57.5, BF16 2048^2 61.3 / 57.6).
 template <int M, bool PH>
 __device__ __forceinline__ void step_pair_or_nodes(const StepParams<float>& P, int x0, int y) {
     if (!P.solid_scheme && x0 + 1 < P.nx) {
@@ -1457,10 +1470,10 @@ __global__ void __launch_bounds__(128, kPairBlocks) fused_step_pair(const __grid
 // bank, up to 32 KB), with the prefix sums of the runs' block counts; block b
 // finds its run by a binary search over them (uniform across the block) and
 // takes block b - first_block[run] of that run's tiles: w x (128 / w) nodes,
-// one node per thread (fused_step's arithmetic), w = 32 << tile[run] chosen so
-// that the run's width leaves the fewest threads idle.  With all small runs in
-// one grid the device sees one large launch instead of many small ones, each
-// bound by the latency of a few warps.
+// one node per thread, w = 32 << tile[run] chosen so that the run's width
+// leaves the fewest threads idle.  With all small runs in one grid the device
+// sees one large launch instead of many small ones, each bound by the latency
+// of a few warps.
 template <typename R>
 constexpr int kGroupRuns = (32000 - 16) / (int)(sizeof(StepParams<R>) + 2 * sizeof(int));
 
@@ -1509,7 +1522,9 @@ __global__ void __launch_bounds__(128, 2 * kMinBlocks<M, QT, FLOW>) group_step(
 // The same for runs in 16-bit storage with flow and the D2Q5 thermal lattices,
 // a node pair per thread: tiles of w x 256 / w nodes, w = 32 << tile.  These
 // runs are bound by instruction issue, and a pair takes some 650 instructions
-// where its nodes one by one take 1,000.
+// where its nodes one by one take 1,000 (64 cavities of 64-512 nodes a side,
+// FP16: 132.7 us per step of all with one node per thread, 123.1 with pairs;
+// 12 cavities 22.2 and 17.5 with the groups side by side as well).
 template <int M, bool PH, int NR>
 __global__ void __launch_bounds__(128, kPairBlocks) group_step_pair(const __grid_constant__ GroupParams<float, NR> G) {
     const int b = blockIdx.x, lo = group_run(G, b);
@@ -1612,7 +1627,10 @@ __global__ void __launch_bounds__(256) fields_kernel(const __grid_constant__ Ste
 // up to eight rows before its block reduces, and the warp reduces its four
 // sums in 6 additions instead of 20 (each exchange halves the sums a lane
 // keeps).  The wall flux, three node states per row, has blocks of its own
-// (the last column of blocks), beside the others instead of in their chains.
+// (the last column of blocks), beside the others instead of in their chains; they
+// write their row's flux sum into the first column's partials.  GB300, us per
+// lbm_diag call with the copy of the results, before / with this arrangement:
+// FP32 64^2 38 / 30, 1024^2 115 / 54, 2048^2 359 / 130.
 struct DiagConst {
     double phi, rho_l, rho_m, c_pm, k_f, k_s, k_m;   // k_f: liquid PCM conductivity, k_s: solid (Eq. 9)
     int left_wall;  // 1 when x = 0 is a wall (Nusselt number defined)
@@ -1628,15 +1646,15 @@ __device__ __forceinline__ double to_double(float v) {
 }
 
 template <int M, int QT, bool FLOW>
-__global__ void __launch_bounds__(128) diag_partial(const __grid_constant__ StepParams<typename ModeTraits<M>::R> P,
+__global__ void __launch_bounds__(256) diag_partial(const __grid_constant__ StepParams<typename ModeTraits<M>::R> P,
                                                     const __grid_constant__ DiagConst C,
                                                     double* __restrict__ scratch) {
     const int x = blockIdx.x * 128 + threadIdx.x;
     double fl = 0.0, H = 0.0, Tm = 0.0, drho = 0.0, flux = 0.0;
-    const int y0 = blockIdx.y * C.rows, y1 = min(y0 + C.rows, P.ny);
-    if (blockIdx.x == gridDim.x - 1) {   // the left wall's heat flux, a row per thread
-        const int y = y0 + threadIdx.x;
-        if (C.left_wall && y < y1) {
+    const bool wall = blockIdx.x == gridDim.x - 1;
+    if (wall) {   // the left wall's heat flux, a row per thread
+        const int rows = blockDim.y * C.rows, y = blockIdx.y * rows + threadIdx.x;
+        if (C.left_wall && threadIdx.y == 0 && threadIdx.x < rows && y < P.ny) {
             double tf[3], tm[3], kw = 0.0;
 #pragma unroll 1
             for (int k = 0; k < 3; ++k) {
@@ -1652,6 +1670,7 @@ __global__ void __launch_bounds__(128) diag_partial(const __grid_constant__ Step
             flux = C.phi * kw * gf + (1.0 - C.phi) * C.k_m * gm;
         }
     } else if (x < P.nx) {
+        const int y0 = (blockIdx.y * blockDim.y + threadIdx.y) * C.rows, y1 = min(y0 + C.rows, P.ny);
 #pragma unroll 1
         for (int y = y0; y < y1; ++y) {
             NodeState<M, QT, FLOW, Node1<M>> n;
@@ -1666,19 +1685,28 @@ __global__ void __launch_bounds__(128) diag_partial(const __grid_constant__ Step
     }
     const double E = C.phi * C.rho_l * H + (1.0 - C.phi) * C.rho_m * C.c_pm * Tm;
     // lanes 0-15 take (fl, E), 16-31 (drho, flux); then each eight lanes one of the two
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.y * 4 + (threadIdx.x >> 5);
     const bool h16 = lane & 16, h8 = lane & 8;
     const double a = (h16 ? drho : fl) + __shfl_xor_sync(0xffffffffu, h16 ? fl : drho, 16);
     const double b = (h16 ? flux : E) + __shfl_xor_sync(0xffffffffu, h16 ? E : flux, 16);
     double v = (h8 ? b : a) + __shfl_xor_sync(0xffffffffu, h8 ? a : b, 8);
 #pragma unroll
     for (int off = 4; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    __shared__ double red[4][4];
+    __shared__ double red[8][4];
     if ((lane & 7) == 0) red[warp][lane >> 3] = v;
     __syncthreads();
-    if (threadIdx.x < 4)
-        scratch[(long long)(blockIdx.y * gridDim.x + blockIdx.x) * 4 + threadIdx.x] =
-            (red[0][threadIdx.x] + red[1][threadIdx.x]) + (red[2][threadIdx.x] + red[3][threadIdx.x]);
+    const int i = threadIdx.x;
+    if (threadIdx.y != 0 || i >= 4) return;
+    double t = (red[0][i] + red[1][i]) + (red[2][i] + red[3][i]);
+    if (blockDim.y == 2) t += (red[4][i] + red[5][i]) + (red[6][i] + red[7][i]);
+    // partial sums [row of blocks][column of nodes' blocks][4]; the flux, slot 3, is the wall block's
+    const int columns = gridDim.x - 1;
+    double* out = scratch + (long long)blockIdx.y * columns * 4 + i;
+    if (wall) {
+        if (i == 3) *out = t;
+    } else if (i < 3 || blockIdx.x > 0) {
+        out[blockIdx.x * 4] = t;
+    }
 }
 
 // Sums the partials in a fixed order (one block of 512 threads, four sums side

@@ -14,22 +14,23 @@ inline dim3 grid_for(int nx, int ny) {
 }
 
 // Rows per thread of the diagnostics: one where the grid hardly fills the
-// device, up to eight where blocks abound (a block's reduction costs as much
-// FP64 time as two rows).
+// device (in blocks of 128 x 2 threads), up to eight where blocks abound (a
+// block's reduction costs as much FP64 time as two rows), in blocks of 128 x 1.
 inline int diag_rows(int nx, int ny) {
     const long long nodes = (long long)nx * ny;
     return nodes <= 65536 && ny <= 32768 ? 1 : nodes <= 524288 ? 4 : 8;   // (at most 65,535 blocks along y)
 }
 
+inline dim3 diag_block(int nx, int ny) { return dim3(128, diag_rows(nx, ny) == 1 ? 2 : 1); }
+
 inline dim3 diag_grid(int nx, int ny) {
-    const int r = diag_rows(nx, ny);
+    const int r = diag_rows(nx, ny) * (int)diag_block(nx, ny).y;
     return dim3((unsigned)((nx + 127) / 128 + 1), (unsigned)((ny + r - 1) / r), 1u);   // and a column for the wall flux
 }
 
-inline int diag_blocks(int nx, int ny) {
-    const dim3 g = diag_grid(nx, ny);
-    return (int)(g.x * g.y);
-}
+// Rows of four partial sums that a run's scratch holds: one per 128 x 2 nodes,
+// which every grid above needs at most.
+inline int diag_blocks(int nx, int ny) { return ((nx + 127) / 128) * ((ny + 1) / 2); }
 
 // Uniform initial state: one value per logical population (9 flow, Q PCM, Q
 // metal, in the order of Eq. 11), the low part of the PCM rest population
@@ -208,11 +209,13 @@ inline int form_for(int mode, int qt, int flow, int solid_scheme, long long node
 // least kTwoStepF32MinNodes (two state copies, 168 bytes per node, exceed the
 // 129 MB L2, and two steps per launch move the state through HBM once per two
 // steps).  Between the two the state sits in L2 and the step is bound by
-// instruction issue, which the redundant ring only adds to (us per step, one
-// against two steps per launch; FP32: 256^2 2.40 / 2.02, 320^2 3.01 / 2.74,
+// instruction issue, which the redundant ring only adds to.  The thresholds
+// were set on an earlier node update's times (us per step, one against two
+// steps per launch; FP32: 256^2 2.40 / 2.02, 320^2 3.01 / 2.74,
 // 352^2 3.16 / 3.30, 384^2 3.39 / 4.26, 512^2 4.99 / 5.98, 768^2 11.1 / 12.2,
 // 896^2 19.1 / 16.9, 1024^2 26.5 / 21.9, 2048^2 99.7 / 81.2; FP16: 320^2
-// 3.14 / 2.91, 352^2 3.20 / 4.25).  Single steps (an odd remainder, batches)
+// 3.14 / 2.91, 352^2 3.20 / 4.25); the current one takes FP32 256^2 2.15 / 1.86,
+// 2048^2 100 / 71.1.  Single steps (an odd remainder, batches)
 // keep the form above.
 constexpr long long kTwoStepSmallMaxNodes = 320 * 320;
 constexpr long long kTwoStepF32MinNodes = 3ll << 18;
@@ -257,8 +260,10 @@ inline int prefetch_rows_two_steps(int mode, long long nodes) {
 }
 
 // FP64 runs without flow take conduction_step_lanes while its warps, of 16
-// nodes, find a scheduler each (152 SMs x 4); beyond, two warps of 33 FP64
-// operations in turn take longer than one of 50.
+// nodes, find a scheduler each (152 SMs x 4; 200 x 4 2.63 us per step against
+// 3.46 with one lane per node); beyond, two warps of one lattice's FP64
+// operations in turn take longer than one warp of both lattices', which share
+// some.
 constexpr long long kConductionLanesMaxNodes = 152 * 4 * 16;
 
 // The one-step kernel of a run, with its grid: one node per thread in blocks of
@@ -373,8 +378,8 @@ cudaError_t launch_step(const StepParams<typename ModeTraits<M>::R>& P, int qt, 
 // block's warps for the first step and the inner tile for the second), with
 // the work of two tiles per SM counted at kT2Overlap: two resident blocks
 // overlap each other's L2 loads and barrier.  On 152 SMs: 128^2 takes H = 6
-// (128 tiles), 192^2 H = 10 (144), 256^2 H = 9 (296; FP32 2.04 against 2.21 us
-// per step for H = 16 and one tile per SM).  Grids that need more than two
+// (128 tiles), 192^2 H = 10 (144), 256^2 H = 9 (296; fitted on FP32 times of
+// 2.04 us per step against 2.21 for H = 16 and one tile per SM, now 1.86).  Grids that need more than two
 // tiles per SM take H = kT2HMany = 12, measured fastest there (FP32: three
 // resident blocks of 13 warps per SM; 1024^2 and 2048^2 against H = 6, 8,
 // 10, 14, 16).
@@ -497,13 +502,13 @@ cudaError_t launch_fields(const StepParams<typename ModeTraits<M>::R>& P,
 template <int M>
 cudaError_t launch_diag(const StepParams<typename ModeTraits<M>::R>& P, const DiagConst& C, double* scratch,
                         double* out, int qt, int flow, cudaStream_t s) {
-    const dim3 g = diag_grid(P.nx, P.ny);
+    const dim3 g = diag_grid(P.nx, P.ny), b = diag_block(P.nx, P.ny);
     cudaError_t e = dispatch<M>(qt, flow, [&]<int MM, int Q, bool F>() {
-        diag_partial<MM, Q, F><<<g, 128, 0, s>>>(P, C, scratch);
+        diag_partial<MM, Q, F><<<g, b, 0, s>>>(P, C, scratch);
         return cudaGetLastError();
     });
     if (e != cudaSuccess) return e;
-    diag_finalize<<<1, 512, 0, s>>>(scratch, (int)(g.x * g.y), (double)P.nx * P.ny, out);
+    diag_finalize<<<1, 512, 0, s>>>(scratch, (int)((g.x - 1) * g.y), (double)P.nx * P.ny, out);
     return cudaGetLastError();
 }
 

@@ -213,8 +213,9 @@ def derive(p: dict) -> dict:
 
 
 def step_form_for(p: dict, form: int = 0) -> int:
-    """The step form (1: one node per thread, 2: node pairs) a run with
-    parameters p takes when set to `form` (lbm_step_form_for; no GPU needed)."""
+    """The step form (1: one step per launch, 2: that with node pairs and their
+    prefetch, 3: two steps per launch) a run with parameters p takes when set
+    to `form` (lbm_step_form_for; no GPU needed)."""
     used = ctypes.c_int32()
     _check(lib().lbm_step_form_for(ctypes.byref(to_struct(p)), int(form), ctypes.byref(used)), "lbm_step_form_for")
     return int(used.value)
