@@ -211,7 +211,7 @@ int lbm_step(lbm_handle* h, int64_t nsteps);
  * FP32/FP16/BF16 storage (the others step one node per thread): each block of
  * 34 x H threads advances its tile and the one-node ring around it one step
  * into shared memory, then the tile's 32 x (H - 2) inner nodes a second step
- * into the other state copy (H from 4 to 16 per grid, at most two tiles per SM
+ * into the other state copy (H from 4 to 15 per grid, at most two tiles per SM
  * where the grid allows, else H = 12; FP32 grids of at least 786,432 nodes
  * prefetch the rows 20 further on into L2);
  * lbm_step takes it for 4 steps or more (an odd remainder and steps that bring

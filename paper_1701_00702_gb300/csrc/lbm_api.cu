@@ -408,14 +408,14 @@ bool two_steps(const lbm_handle* h) {
     return lbmk::two_steps_for(h->p.precision, h->p.thermal_q, h->p.flow, (long long)h->p.nx * h->p.ny, h->form);
 }
 
-// The second history array and the block height of the two-step form, on
+// The second history array and the block shape of the two-step form, on
 // first use (the SM count of the current device).
 int ensure_dT2(lbm_handle* h) {
     if (h->dT2) return LBM_OK;
     int dev = 0, nsm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return cuda_fail(h);
-    h->t2 = lbmk::t2_block(h->p.nx, h->p.ny, nsm);
+    h->t2 = lbmk::t2_block(h->p.precision, h->p.thermal_q, h->p.nx, h->p.ny, nsm);
     cudaError_t e = cudaSuccess;
     const int q = h->p.thermal_q, ph = phase_k_of(h);
     switch (h->p.precision) {
@@ -1341,9 +1341,9 @@ const void* group2_fn(const lbm_batch* b, bool few) {
 
 size_t group2_smem(const lbm_batch* b) {
     switch (b->precision) {
-        case LBM_F32: return lbmk::step2_smem<lbmk::MODE_F32>(b->qt, true);
-        case LBM_F16: return lbmk::step2_smem<lbmk::MODE_F16>(b->qt, true);
-        case LBM_BF16: return lbmk::step2_smem<lbmk::MODE_BF16>(b->qt, true);
+        case LBM_F32: return lbmk::step2_smem<lbmk::MODE_F32>(b->qt, lbmk::kT2HMany);
+        case LBM_F16: return lbmk::step2_smem<lbmk::MODE_F16>(b->qt, lbmk::kT2HMany);
+        case LBM_BF16: return lbmk::step2_smem<lbmk::MODE_BF16>(b->qt, lbmk::kT2HMany);
         default: return 0;
     }
 }

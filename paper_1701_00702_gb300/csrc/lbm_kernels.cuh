@@ -1318,22 +1318,26 @@ __global__ void __launch_bounds__(64) conduction_step_lanes(const __grid_constan
 // are computed by both blocks with the same inputs and code, and written with
 // the same values.  The history is read from P.dT and written to P.dT_out:
 // other blocks still read the previous history of their rings.  Flow runs
-// only.  The host picks H per grid (t2_block in the launcher).  Two builds of
-// the kernel: HM = kT2H (any H up to 16; one block per SM on the grids that
-// take it) and HM = kT2HMany (H = 12 for grids of many tiles per SM, launch
-// bounds that leave three FP32 D2Q5 blocks resident: at 52 registers only two
-// fit, 2048^2 FP32 104 against 84 us per step; two blocks of the other builds,
-// which would spill under the three-block cap).  Small grids are bound by the
+// only.  The host picks H per grid (t2_block in the launcher).  Three builds of
+// the kernel: HM = kT2H (any H up to 15, registers as they come: fastest where
+// one or two blocks per SM fit anyway); HM = kT2HTwo (tiles of up to 14 rows,
+// two per SM, capped at 64 registers for two resident blocks where the first
+// build's registers would leave one: FP16 320^2 3.40 -> 2.62 us per step, 334 x
+// 303 3.55 -> 2.90; on smaller tiles the cap costs, 64^2 1.186 -> 1.218); and HM =
+// kT2HMany (H = 12 for grids of many tiles per SM, launch bounds that leave
+// three FP32 D2Q5 blocks resident: at 52 registers only two fit, 2048^2 FP32
+// 104 against 84 us per step; two blocks of the other builds, which would spill
+// under the three-block cap).  Small grids are bound by the
 // launch floor and two dependency chains (64^2 FP32 1.315 us per step before
 // the update was written in named multiply-adds, 1.09 now; 256^2 2.05 / 1.86),
 // grids beyond L2 by instruction issue once their rows are prefetched (2048^2
 // 79.9 us per step before, 71.1 now; 49.5 at the copy bandwidth).  Two nodes
 // per thread in the tile, side by side or one above the other, were slower
 // (2048^2 77.0 and 73.3, 64^2 1.37): more registers, fewer warps.
-constexpr int kT2W = 34, kT2H = 16, kT2HMany = 12;
+constexpr int kT2W = 34, kT2H = 15, kT2HTwo = 14, kT2HMany = 12;
 
 template <int HM, int M, int QT>
-constexpr int kT2Blocks = HM == kT2HMany ? (M == MODE_F32 && QT == 5 ? 3 : 2) : 1;
+constexpr int kT2Blocks = HM == kT2HMany ? (M == MODE_F32 && QT == 5 ? 3 : 2) : HM == kT2HTwo ? 2 : 1;
 
 // Dynamic shared memory of a two-step block of up to HM rows, planes
 // kT2W * HM elements apart: the bulk planes (storage type), the wide planes
@@ -1341,7 +1345,7 @@ constexpr int kT2Blocks = HM == kT2HMany ? (M == MODE_F32 && QT == 5 ? 3 : 2) : 
 template <int M, int QT, int HM>
 struct Tile2 {
     using PL = Planes<M, QT, true>;
-    static constexpr int n = kT2W * HM;
+    static constexpr int n = (kT2W * HM + 7) / 8 * 8;
     static constexpr size_t wide_off = (size_t)PL::bulk * n * sizeof(typename ModeTraits<M>::B);
     static constexpr size_t dT_off = wide_off + (size_t)PL::wide * n * sizeof(float);
     static constexpr size_t bytes = dT_off + (size_t)n * sizeof(typename ModeTraits<M>::R);

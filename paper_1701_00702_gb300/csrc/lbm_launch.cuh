@@ -379,10 +379,11 @@ cudaError_t launch_step(const StepParams<typename ModeTraits<M>::R>& P, int qt, 
 // the work of two tiles per SM counted at kT2Overlap: two resident blocks
 // overlap each other's L2 loads and barrier.  On 152 SMs: 128^2 takes H = 6
 // (128 tiles), 192^2 H = 10 (144), 256^2 H = 9 (296; fitted on FP32 times of
-// 2.04 us per step against 2.21 for H = 16 and one tile per SM, now 1.86).  Grids that need more than two
-// tiles per SM take H = kT2HMany = 12, measured fastest there (FP32: three
-// resident blocks of 13 warps per SM; 1024^2 and 2048^2 against H = 6, 8,
-// 10, 14, 16).
+// 2.04 us per step against 2.21 for H = 16 and one tile per SM, now 1.86).  One
+// tile per SM takes up to kT2H rows, two up to kT2HTwo (what their registers
+// allow).  Other grids take H = kT2HMany = 12, measured fastest there (FP32:
+// three resident blocks of 13 warps per SM; 1024^2 and 2048^2 against H = 6, 8,
+// 10, 14, 16; 65 x 1400, two tiles of 16 rows per SM before: 3.37 / 3.17).
 constexpr double kT2Overlap = 0.87;
 
 inline long long t2_tiles(int n, int inner) { return t2_count(n, inner); }
@@ -392,50 +393,62 @@ inline dim3 t2_grid(int nx, int ny, int h) {
 }
 
 struct T2Shape {
-    int h;       // block height
-    bool many;   // the many-tiles build
+    int h;    // block height
+    int hm;   // the build, kT2H, kT2HTwo or kT2HMany
 };
 
-inline T2Shape t2_block(int nx, int ny, int nsm) {
+// Height from which two blocks of the first build don't fit an SM's registers
+// (FP32 64, with D2Q9 76; 16-bit 75, with D2Q9 94), so that two tiles per SM take
+// the build capped for them.
+inline int t2_two_from(int mode, int qt) { return mode == MODE_F32 ? (qt == 5 ? kT2HTwo + 1 : 12) : (qt == 5 ? 12 : 10); }
+
+inline T2Shape t2_block(int mode, int qt, int nx, int ny, int nsm) {
     if (nsm < 1) nsm = 1;
-    T2Shape best = {kT2HMany, true};
+    T2Shape best = {kT2HMany, kT2HMany};
     double best_cost = -1.0;
     for (int h = 4; h <= kT2H; ++h) {
         const long long tiles = t2_tiles(nx, kT2W - 2) * t2_tiles(ny, h - 2);
         const long long per_sm = (tiles + nsm - 1) / nsm;
-        if (per_sm > 2) continue;
+        if (per_sm > 2 || (per_sm == 2 && h > kT2HTwo)) continue;
         const long long work = per_sm * ((kT2W * h + 31) / 32 * 32 + (long long)(kT2W - 2) * (h - 2));
         const double cost = per_sm > 1 ? kT2Overlap * (double)work : (double)work;
         if (best_cost < 0.0 || cost < best_cost) {
-            best = {h, false};
+            best = {h, per_sm == 2 && h >= t2_two_from(mode, qt) ? kT2HTwo : kT2H};
             best_cost = cost;
         }
     }
     return best;
 }
 
-// The build of the kernel (many: the many-tiles build, for kT2HMany rows and
-// launch bounds for three blocks per SM; 300^2 with 12 rows and two tiles per
-// SM takes 2.53 us per step in it) and its dynamic shared memory.
+// The build of the kernel and its dynamic shared memory (300^2 with 12 rows and
+// two tiles per SM takes 2.53 us per step in the many-tiles build, 2.44 in the
+// first).
 template <int M, int HM>
 const void* step2_kernel_hm(int qt, int phase_k) {
-    if (qt == 5) return phase_k ? (const void*)fused_step2<M, 5, true, HM> : (const void*)fused_step2<M, 5, false, HM>;
-    return phase_k ? (const void*)fused_step2<M, 9, true, HM> : (const void*)fused_step2<M, 9, false, HM>;
+    if (qt == 9) return phase_k ? (const void*)fused_step2<M, 9, true, HM> : (const void*)fused_step2<M, 9, false, HM>;
+    if constexpr (HM == kT2HTwo && M == MODE_F32) return nullptr;   // (two blocks of up to 14 rows fit as they are)
+    else return phase_k ? (const void*)fused_step2<M, 5, true, HM> : (const void*)fused_step2<M, 5, false, HM>;
 }
 
 template <int M>
-const void* step2_kernel(int qt, int phase_k, bool many) {
+const void* step2_kernel(int qt, int phase_k, int hm) {
     if constexpr (M != MODE_F64) {
-        return many ? step2_kernel_hm<M, kT2HMany>(qt, phase_k) : step2_kernel_hm<M, kT2H>(qt, phase_k);
+        if (hm == kT2HMany) return step2_kernel_hm<M, kT2HMany>(qt, phase_k);
+        return hm == kT2HTwo ? step2_kernel_hm<M, kT2HTwo>(qt, phase_k) : step2_kernel_hm<M, kT2H>(qt, phase_k);
     }
     return nullptr;
 }
 
+template <int M, int HM>
+constexpr size_t step2_smem_hm(int qt) {
+    return qt == 5 ? Tile2<M, 5, HM>::bytes : Tile2<M, 9, HM>::bytes;
+}
+
 template <int M>
-size_t step2_smem(int qt, bool many) {
+size_t step2_smem(int qt, int hm) {
     if constexpr (M != MODE_F64) {
-        if (many) return qt == 5 ? Tile2<M, 5, kT2HMany>::bytes : Tile2<M, 9, kT2HMany>::bytes;
-        return qt == 5 ? Tile2<M, 5, kT2H>::bytes : Tile2<M, 9, kT2H>::bytes;
+        if (hm == kT2HMany) return step2_smem_hm<M, kT2HMany>(qt);
+        return hm == kT2HTwo ? step2_smem_hm<M, kT2HTwo>(qt) : step2_smem_hm<M, kT2H>(qt);
     }
     return 0;
 }
@@ -461,9 +474,9 @@ inline long long group2_blocks(int nx, int ny) { return t2_tiles(nx, kT2W - 2) *
 // before the first of them on the device.
 template <int M>
 cudaError_t prepare_step2(int qt, int phase_k, T2Shape t) {
-    const void* fn = step2_kernel<M>(qt, phase_k, t.many);
+    const void* fn = step2_kernel<M>(qt, phase_k, t.hm);
     if (!fn) return cudaErrorInvalidConfiguration;
-    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)step2_smem<M>(qt, t.many));
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)step2_smem<M>(qt, t.hm));
 }
 
 // Two steps from copy P.src to P.dst, history P.dT -> P.dT_out, in blocks of
@@ -471,10 +484,10 @@ cudaError_t prepare_step2(int qt, int phase_k, T2Shape t) {
 // stream.
 template <int M>
 cudaError_t launch_step2(const StepParams<typename ModeTraits<M>::R>& P, int qt, T2Shape t, cudaStream_t s) {
-    if (t.h < 4 || t.h > (t.many ? kT2HMany : kT2H)) return cudaErrorInvalidConfiguration;
-    const void* fn = step2_kernel<M>(qt, P.phase_k, t.many);
+    if (t.h < 4 || t.h > t.hm) return cudaErrorInvalidConfiguration;
+    const void* fn = step2_kernel<M>(qt, P.phase_k, t.hm);
     if (!fn) return cudaErrorInvalidConfiguration;
-    const size_t smem = step2_smem<M>(qt, t.many);
+    const size_t smem = step2_smem<M>(qt, t.hm);
     void* args[1] = {const_cast<StepParams<typename ModeTraits<M>::R>*>(&P)};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -570,7 +583,7 @@ int batch_blocks_per_sm(int qt, int flow, int ph) {
     KW template cudaError_t launch_step2<M>(const StepParams<ModeTraits<M>::R>&, int, T2Shape, cudaStream_t); \
     KW template cudaError_t prepare_step2<M>(int, int, T2Shape);                                              \
     KW template const void* group2_kernel<M>(int, int, bool);                                                        \
-    KW template size_t step2_smem<M>(int, bool);                                                               \
+    KW template size_t step2_smem<M>(int, int);                                                               \
     KW template StepLaunch step_launch<M>(const StepParams<ModeTraits<M>::R>&, int, int, int, dim3);
 
 #define LBMK_CONVERT_TEMPLATES(KW, M)                                                                         \

@@ -52,6 +52,18 @@ def test_step_forms_give_the_same_bits(lbm, shape, kinds, prec):
         assert np.array_equal(want, r.save())
 
 
+@pytest.mark.parametrize("shape", [(287, 301), (320, 320), (334, 303), (65, 1400), (256, 242)])
+@pytest.mark.parametrize("prec,q,eq9", [(1, 5, 0), (1, 9, 0), (2, 5, 0), (2, 9, 0), (3, 5, 1)])
+def test_two_step_builds_of_tall_tiles(lbm, shape, prec, q, eq9):
+    """Tiles of 12 to 15 rows: two per SM at registers capped for it (16-bit,
+    D2Q9), one per SM, and the many-tiles build, against one step per launch."""
+    s = random_run(lbm, *shape, prec, seed=9, qt=q, **(dict(ks_over_kl=0.7) if eq9 else {}))
+    a, b = twin(lbm, s, 1), twin(lbm, s, 3)
+    a.step(4)
+    b.step(4)
+    assert b.status() == 0 and np.array_equal(a.save(), b.save())
+
+
 @pytest.mark.parametrize("shape", [(1025, 768), (900, 874)])
 def test_two_steps_with_prefetch_beyond_l2(lbm, shape):
     """FP32 grids of at least 786,432 nodes, whose two-step tiles prefetch rows
