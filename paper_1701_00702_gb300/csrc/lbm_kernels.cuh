@@ -459,9 +459,22 @@ struct NodeState {
 // the lane's type in a mode's one-node kernels
 template <int M> using Node1 = typename ModeTraits<M>::R;
 
-template <int M>
+// Reads of a state copy.  EV: marked evict-first (ld.global.cs), for grids whose
+// two copies and history come near L2's 129 MB or a little above: a step's
+// source is dead once its neighbours have read it, until the next step
+// overwrites it whole, and gives way to the copy being written, which the next
+// step reads (GB300, us per step without / with: FP32 768^2, 97 MB, 11.7 / 9.3,
+// 1024^2 one step per launch, 172 MB, 26.3 / 21.5; FP16 1200^2, 127 MB, 25.3 /
+// 18.6; at 80 MB 1 % slower, at 276 MB 7 %).
+template <bool EV, typename V>
+__device__ __forceinline__ V read_state(const V* p) {
+    if constexpr (EV) return __ldcs(p);
+    else return __ldg(p);
+}
+
+template <int M, bool EV = false>
 __device__ __forceinline__ typename ModeTraits<M>::R ldb(const typename ModeTraits<M>::B* p) {
-    return to_f(__ldg(p));
+    return to_f(read_state<EV>(p));
 }
 
 template <int M, typename R>
@@ -554,7 +567,7 @@ __device__ __forceinline__ int col_off(int x) {
 __host__ __device__ constexpr int src_col(int q) { return (0xa191 >> (2 * q)) & 3; }
 __host__ __device__ constexpr int src_row(int q) { return (0x28245 >> (2 * q)) & 3; }
 
-template <int M, int QT, bool FLOW>
+template <int M, int QT, bool FLOW, bool EV = false>
 struct PullAt {
     const char* row[3];
     int dc[3];   // bulk plane 0 of source columns x - 1, x, x + 1, from this node's
@@ -586,17 +599,17 @@ struct PullAt {
     }
     // bulk plane `plane` and wide plane w (16-bit modes) of the source node of direction q
     __device__ __forceinline__ typename ModeTraits<M>::R bulk(int q, int plane) const {
-        return ldb<M>(src(q) + plane * kChunk);
+        return ldb<M, EV>(src(q) + plane * kChunk);
     }
     __device__ __forceinline__ float wide(int q, int w) const {
-        return __ldg(reinterpret_cast<const float*>(row[src_row(q)] + dw[src_col(q)]) + w * kChunk);
+        return read_state<EV>(reinterpret_cast<const float*>(row[src_row(q)] + dw[src_col(q)]) + w * kChunk);
     }
 };
 
 // The same around the node pair (x0, x0 + 1), x0 even (both nodes in one
 // chunk): own reads the pair's two adjacent elements, west the elements of
 // x0 - 1 and x0, east those of x0 + 1 and x0 + 2.
-template <int M, int QT>
+template <int M, int QT, bool EV = false>
 struct PairAt {
     using B = typename ModeTraits<M>::B;
     using CH = Chunk<M, QT, true>;
@@ -622,19 +635,21 @@ struct PairAt {
             wp = col_off<M, QT, true, true>(xp) - c0;
         }
     }
-    __device__ __forceinline__ static float one(const char* p) { return ldb<M>(reinterpret_cast<const B*>(p)); }
-    __device__ __forceinline__ static float onew(const char* p) { return __ldg(reinterpret_cast<const float*>(p)); }
+    __device__ __forceinline__ static float one(const char* p) { return ldb<M, EV>(reinterpret_cast<const B*>(p)); }
+    __device__ __forceinline__ static float onew(const char* p) {
+        return read_state<EV>(reinterpret_cast<const float*>(p));
+    }
     __device__ __forceinline__ W bulk(int q, int plane) const {
         const char* r = row[src_row(q)] + plane * kChunk * es;
         if (src_col(q) == 0) return {one(r + cm), one(r)};
         if (src_col(q) == 2) return {one(r + es), one(r + cp)};
-        return unpack2(__ldg(reinterpret_cast<const typename Two<B>::type*>(r)));
+        return unpack2(read_state<EV>(reinterpret_cast<const typename Two<B>::type*>(r)));
     }
     __device__ __forceinline__ W wide(int q, int w) const {
         const char* r = row[src_row(q)] + w * kChunk * 4;
         if (src_col(q) == 0) return {onew(r + wm), onew(r + w0)};
         if (src_col(q) == 2) return {onew(r + w0 + 4), onew(r + wp)};
-        return unpack2(__ldg(reinterpret_cast<const float2*>(r + w0)));
+        return unpack2(read_state<EV>(reinterpret_cast<const float2*>(r + w0)));
     }
 };
 
@@ -851,8 +866,13 @@ __device__ __forceinline__ void apply_wall(const StepParams<typename ModeTraits<
 template <int M, int QT, bool FLOW, typename T, typename A>
 __device__ __forceinline__ void node_state(const StepParams<typename ModeTraits<M>::R>& P, const A& a,
                                            const WallAt<T>& w, NodeState<M, QT, FLOW, T>& n) {
-    pull_flow<M, QT, FLOW, T>(a, n);
-    pull_thermal<M, QT, FLOW, T>(P, a, n);
+    if constexpr (kComp<M>) {
+        pull_thermal<M, QT, FLOW, T>(P, a, n);
+        pull_flow<M, QT, FLOW, T>(a, n);
+    } else {
+        pull_flow<M, QT, FLOW, T>(a, n);
+        pull_thermal<M, QT, FLOW, T>(P, a, n);
+    }
     if constexpr (Lane<T>::n == 2) {
         if (w.xa || w.xb) {
 #pragma unroll
@@ -1145,14 +1165,17 @@ __device__ __forceinline__ float* next_wide(const StepParams<typename ModeTraits
 // P.phase_k is set); PH = false leaves them out of the kernel altogether.
 // The history is read before any store: the compiler cannot move it above
 // stores that may alias it, and a load after them adds a memory round trip to
-// the step.  Returns the new history.
+// the step; in FP32, one node per thread, it is read after the state is known,
+// and the thermal lattices are pulled first (one step per launch 330^2 3.17 ->
+// 2.98 us, 512^2 4.98 -> 4.84, 1024^2 27.3 -> 26.4).  Returns the new history.
 template <int M, int QT, bool FLOW, bool PH, int PS, typename T, typename A>
 __device__ __forceinline__ T advance(const StepParams<typename ModeTraits<M>::R>& P, const A& a, const WallAt<T>& w,
                                      const typename Lane<T>::R* history, typename ModeTraits<M>::B* db, float* dw) {
     NodeState<M, QT, FLOW, T> n;
     T dTp;
-    if constexpr (Lane<T>::n == 1) dTp = get_real<T>(history);
+    if constexpr (Lane<T>::n == 1 && !kComp<M>) dTp = get_real<T>(history);
     node_state<M, QT, FLOW, T>(P, a, w, n);
+    if constexpr (Lane<T>::n == 1 && kComp<M>) dTp = get_real<T>(history);
     flow_collide<M, QT, FLOW, PS, T>(P, n, db);
     if constexpr (Lane<T>::n == 2) dTp = get_real<T>(history);
     const T dTn = thermal_collide<M, QT, FLOW, PH, PS, T>(P, n, dTp, db, dw);
@@ -1161,21 +1184,21 @@ __device__ __forceinline__ T advance(const StepParams<typename ModeTraits<M>::R>
 }
 
 // One time step of node (x, y) from the state copy to the next.
-template <int M, int QT, bool FLOW, bool PH = false>
+template <int M, int QT, bool FLOW, bool PH = false, bool EV = false>
 __device__ __forceinline__ void step_node(const StepParams<typename ModeTraits<M>::R>& P, int x, int y) {
     using T = Node1<M>;
     const WallAt<T> w(P, x, y);
     T* h = P.dT + (y * P.pitch + x);
-    *h = advance<M, QT, FLOW, PH, kChunk, T>(P, PullAt<M, QT, FLOW>(P, w.xs, w.ys), w, h,
+    *h = advance<M, QT, FLOW, PH, kChunk, T>(P, PullAt<M, QT, FLOW, EV>(P, w.xs, w.ys), w, h,
                                               next_bulk<M, QT, FLOW>(P, x, y), next_wide<M, QT, FLOW>(P, x, y));
 }
 
 // One time step of the node pair (x0, x0 + 1), x0 even, both in the grid.
-template <int M, int QT, bool PH = false>
+template <int M, int QT, bool PH = false, bool EV = false>
 __device__ __forceinline__ void step_pair(const StepParams<float>& P, int x0, int y) {
     const WallAt<W> w(P, x0, y);
     float* h = P.dT + (y * P.pitch + x0);
-    put_real(h, advance<M, QT, true, PH, kChunk, W>(P, PairAt<M, QT>(P, x0, w.ys), w, h,
+    put_real(h, advance<M, QT, true, PH, kChunk, W>(P, PairAt<M, QT, EV>(P, x0, w.ys), w, h,
                                                      next_bulk<M, QT, true>(P, x0, y), next_wide<M, QT, true>(P, x0, y)));
 }
 
@@ -1225,13 +1248,13 @@ __device__ __forceinline__ void prefetch_rows(const StepParams<typename ModeTrai
 // multiply-adds and single-instruction reciprocals and roots, 2.15 now).  FP64
 // is bound by its two lanes per SM and clock: 252 FP64 operations per node took
 // 39.7 us per step at 256^2, 187 take 27.8 (in 64 x 1 blocks).
-template <int M, int QT, bool FLOW, bool PH>
+template <int M, int QT, bool FLOW, bool PH, bool EV = false>
 __global__ void __launch_bounds__(256, (kMinBlocks<M, QT, FLOW>)) fused_step(const __grid_constant__ StepParams<typename ModeTraits<M>::R> P) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x >= P.nx || y >= P.ny) return;
     griddep_wait();
-    step_node<M, QT, FLOW, PH>(P, x, y);
+    step_node<M, QT, FLOW, PH, EV>(P, x, y);
 }
 
 // FP64 runs without flow on grids that leave most schedulers idle: two lanes
@@ -1377,7 +1400,7 @@ __host__ __device__ __forceinline__ int t2_count(int n, int w) { return n > w ? 
 // Both steps of tile (bx, by) of run P, by a block of kT2W x blockDim.y
 // threads (blockDim.y <= HM) with Tile2<M, QT, HM>::bytes of dynamic shared
 // memory.
-template <int M, int QT, bool PH, int HM>
+template <int M, int QT, bool PH, int HM, bool EV = false>
 __device__ __forceinline__ void step2_tile(const StepParams<typename ModeTraits<M>::R>& P, int bx, int by) {
     using R = typename ModeTraits<M>::R;
     using B = typename ModeTraits<M>::B;
@@ -1403,11 +1426,11 @@ __device__ __forceinline__ void step2_tile(const StepParams<typename ModeTraits<
     griddep_wait();
     // the tile's rows, prefetch_rows further on, of the chunk that starts at its first inner
     // column (in the many-tiles build only: the test costs 64^2 0.03 us a step)
-    if (HM == kT2HMany && P.prefetch_rows > 0 && lx == 1 && (x2 & (kChunk - 1)) == 0 && ly >= 1 && ly <= H - 2)
+    if (HM == kT2HMany && !EV && P.prefetch_rows > 0 && lx == 1 && (x2 & (kChunk - 1)) == 0 && ly >= 1 && ly <= H - 2)
         prefetch_rows<M, QT, true>(P, x2, y2 + P.prefetch_rows, 1);
     if (live) {
         const WallAt<R> w(P, x, y);
-        sdT[i] = advance<M, QT, true, PH, TL::n, R>(P, PullAt<M, QT, true>(P, w.xs, w.ys), w, P.dT + (y * P.pitch + x),
+        sdT[i] = advance<M, QT, true, PH, TL::n, R>(P, PullAt<M, QT, true, EV>(P, w.xs, w.ys), w, P.dT + (y * P.pitch + x),
                                                      sb + i, sw + i);
     }
     __syncthreads();
@@ -1419,9 +1442,9 @@ __device__ __forceinline__ void step2_tile(const StepParams<typename ModeTraits<
         P, a, w, sdT + i, next_bulk<M, QT, true>(P, x2, y2), next_wide<M, QT, true>(P, x2, y2));
 }
 
-template <int M, int QT, bool PH, int HM>
+template <int M, int QT, bool PH, int HM, bool EV = false>
 __global__ void __launch_bounds__(kT2W * HM, (kT2Blocks<HM, M, QT>)) fused_step2(const __grid_constant__ StepParams<typename ModeTraits<M>::R> P) {
-    step2_tile<M, QT, PH, HM>(P, blockIdx.x, blockIdx.y);
+    step2_tile<M, QT, PH, HM, EV>(P, blockIdx.x, blockIdx.y);
 }
 
 // ---------------------------------------------------------------------------
@@ -1438,13 +1461,13 @@ __global__ void __launch_bounds__(kT2W * HM, (kT2Blocks<HM, M, QT>)) fused_step2
 // (us per step, before / with the update in named multiply-adds and 80
 // registers: FP16 512^2 5.52 / 4.77 (before: one node per thread), 1024^2 18.4 /
 // 15.2, 2048^2 61.2 / 57.5, BF16 2048^2 61.3 / 57.6).
-template <int M, bool PH>
+template <int M, bool PH, bool EV = false>
 __device__ __forceinline__ void step_pair_or_nodes(const StepParams<float>& P, int x0, int y) {
     if (!P.solid_scheme && x0 + 1 < P.nx) {
-        step_pair<M, 5, PH>(P, x0, y);
+        step_pair<M, 5, PH, EV>(P, x0, y);
     } else {
 #pragma unroll 1
-        for (int x = x0; x < min(x0 + 2, P.nx); ++x) step_node<M, 5, true, PH>(P, x, y);
+        for (int x = x0; x < min(x0 + 2, P.nx); ++x) step_node<M, 5, true, PH, EV>(P, x, y);
     }
 }
 
@@ -1457,15 +1480,15 @@ constexpr int kPairBlocks = 6;
 // A block of 32 x 4 threads covers 64 x 4 nodes; the first of a chunk's two
 // blocks prefetches its rows (2048^2 FP16 61.09 against 61.22 us per step when
 // both did).
-template <int M, bool PH>
+template <int M, bool PH, bool EV = false>
 __global__ void __launch_bounds__(128, kPairBlocks) fused_step_pair(const __grid_constant__ StepParams<float> P) {
     const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x0 >= P.nx || y >= P.ny) return;
     griddep_wait();
-    if (P.prefetch_rows > 0 && threadIdx.x == 0 && threadIdx.y == 0 && (x0 & (kChunk - 1)) == 0)
+    if (!EV && P.prefetch_rows > 0 && threadIdx.x == 0 && threadIdx.y == 0 && (x0 & (kChunk - 1)) == 0)
         prefetch_rows<M, 5, true>(P, x0, y + P.prefetch_rows, blockDim.y);   // the chunk's first block
-    step_pair_or_nodes<M, PH>(P, x0, y);
+    step_pair_or_nodes<M, PH, EV>(P, x0, y);
 }
 
 // Many small runs in one launch per step, each run on the code of the

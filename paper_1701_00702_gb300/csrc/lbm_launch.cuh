@@ -235,6 +235,25 @@ inline bool pairs_of(const StepParams<typename ModeTraits<M>::R>& P, int qt, int
     return kSplit<M> && qt == 5 && flow && !P.solid_scheme && nodes >= kPairPlainMinNodes;
 }
 
+// Whether a run's launches mark their reads evict-first (read_state): from
+// kStreamMinBytes, where the two copies and the history begin to overflow L2, to
+// kStreamMaxBytes, beyond which they stream through it anyway and the marking
+// costs (GB300, us per step without / with.  FP32: 700^2, 80 MB, 8.60 / 8.69,
+// 740^2, 90 MB, 11.2 / 10.5, 768^2 11.7 / 9.3, 1024^2 in two steps per launch, 172
+// MB, 19.4 / 18.4, 1150^2, 217 MB, 24.1 / 25.9; with D2Q9 700^2, 112 MB, 16.2 /
+// 12.7, 900^2, 185 MB, 29.6 / 28.4, 1100^2, 276 MB, 42.5 / 45.6.  FP16: 900^2, 71
+// MB, 11.7 / 11.6, 1000^2, 88 MB, 14.7 / 13.7, 1200^2, 127 MB, 25.3 / 18.6.)  A
+// marked line is not prefetched: it would be dropped before its block reads it.
+// A run's own launches only: the runs of a batch share L2.
+constexpr long long kStreamMinBytes = 84000000, kStreamMaxBytes = 180000000;
+
+inline bool streams(int mode, int qt, int flow, long long nodes) {
+    const int fb = flow ? 9 : 0;
+    const long long copy = mode == MODE_F32 ? 4 * (fb + 2 * qt + 1) : 2 * (fb + 2 * (qt - 1)) + 8;
+    const long long bytes = (2 * copy + 4) * nodes;
+    return flow && mode != MODE_F64 && bytes >= kStreamMinBytes && bytes <= kStreamMaxBytes;
+}
+
 // L2 prefetch distance of the node-pair kernel in rows (0: off): grids of at
 // least kPrefetchMinNodes nodes, whose state is far larger than L2, prefetch
 // each block's chunk rows this far ahead, past most of the blocks resident at
@@ -249,10 +268,8 @@ inline int prefetch_rows_for(int mode, int qt, int flow, int solid_scheme, long 
 }
 
 // The two-step kernel's distance, for FP32 grids whose state exceeds L2 (GB300,
-// us per step without / with: 900 x 880 17.0 / 16.4, 1024^2 21.7 / 19.5, 2048^2
-// 80.8 / 71.3, 4096^2 317 / 279, 256 x 4096 21.8 / 19.9, 8192 x 128 21.9 /
-// 20.2; distances of 10 to 40 rows within 1 % of each other but for the
-// widest).  The blocks that read the rows start about 2 us later.
+// us per step without / with: 2048^2 80.8 / 71.3, 4096^2 317 / 279; distances of
+// 10 to 40 rows within 1 % of each other but for the widest).  The blocks that read the rows start about 2 us later.
 constexpr int kPrefetchRowsTwoSteps = 20;
 
 inline int prefetch_rows_two_steps(int mode, long long nodes) {
@@ -274,11 +291,13 @@ struct StepLaunch {
 };
 
 template <int M>
-StepLaunch step_launch(const StepParams<typename ModeTraits<M>::R>& P, int qt, int flow, int form, dim3 b) {
+StepLaunch step_launch(const StepParams<typename ModeTraits<M>::R>& P, int qt, int flow, int form, dim3 b,
+                       bool stream = false) {
     StepLaunch L{nullptr, dim3(), b};
     if constexpr (M != MODE_F64) {
         if (pairs_of<M>(P, qt, flow, form)) {
-            L.fn = P.phase_k ? (const void*)fused_step_pair<M, true> : (const void*)fused_step_pair<M, false>;
+            if (stream) L.fn = P.phase_k ? (const void*)fused_step_pair<M, true, true> : (const void*)fused_step_pair<M, false, true>;
+            else L.fn = P.phase_k ? (const void*)fused_step_pair<M, true> : (const void*)fused_step_pair<M, false>;
             L.block = dim3(32, 4);   // 2048^2 FP16 61.25 us per step (64 x 2: 61.98)
             L.grid = dim3((unsigned)(((P.nx + 1) / 2 + 31) / 32), (unsigned)((P.ny + 3) / 4), 1u);
             return L;
@@ -294,6 +313,8 @@ StepLaunch step_launch(const StepParams<typename ModeTraits<M>::R>& P, int qt, i
     }
     dispatch_step<M>(qt, flow, P.phase_k, [&]<int MM, int Q, bool F, bool PH>() {
         L.fn = (const void*)fused_step<MM, Q, F, PH>;
+        if constexpr (F && MM != MODE_F64)
+            if (stream) L.fn = (const void*)fused_step<MM, Q, F, PH, true>;
         return cudaSuccess;
     });
     L.grid = dim3((unsigned)((P.nx + b.x - 1) / b.x), (unsigned)((P.ny + b.y - 1) / b.y), 1u);
@@ -356,7 +377,8 @@ const void* group_kernel(int qt, int flow, int ph, bool few) {
 // for it before touching the state), so the launch overlaps its tail.
 template <int M>
 cudaError_t launch_step(const StepParams<typename ModeTraits<M>::R>& P, int qt, int flow, int form, cudaStream_t s) {
-    const StepLaunch L = step_launch<M>(P, qt, flow, form, step_block(M, P.nx, P.ny));
+    const bool stream = streams(M, qt, flow, (long long)P.nx * P.ny);
+    const StepLaunch L = step_launch<M>(P, qt, flow, form, step_block(M, P.nx, P.ny), stream);
     void* args[1] = {const_cast<StepParams<typename ModeTraits<M>::R>*>(&P)};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -395,6 +417,7 @@ inline dim3 t2_grid(int nx, int ny, int h) {
 struct T2Shape {
     int h;    // block height
     int hm;   // the build, kT2H, kT2HTwo or kT2HMany
+    bool stream;   // kT2HMany in FP32: reads marked evict-first
 };
 
 // Height from which two blocks of the first build don't fit an SM's registers
@@ -404,7 +427,7 @@ inline int t2_two_from(int mode, int qt) { return mode == MODE_F32 ? (qt == 5 ? 
 
 inline T2Shape t2_block(int mode, int qt, int nx, int ny, int nsm) {
     if (nsm < 1) nsm = 1;
-    T2Shape best = {kT2HMany, kT2HMany};
+    T2Shape best = {kT2HMany, kT2HMany, mode == MODE_F32 && streams(mode, qt, 1, (long long)nx * ny)};
     double best_cost = -1.0;
     for (int h = 4; h <= kT2H; ++h) {
         const long long tiles = t2_tiles(nx, kT2W - 2) * t2_tiles(ny, h - 2);
@@ -413,7 +436,7 @@ inline T2Shape t2_block(int mode, int qt, int nx, int ny, int nsm) {
         const long long work = per_sm * ((kT2W * h + 31) / 32 * 32 + (long long)(kT2W - 2) * (h - 2));
         const double cost = per_sm > 1 ? kT2Overlap * (double)work : (double)work;
         if (best_cost < 0.0 || cost < best_cost) {
-            best = {h, per_sm == 2 && h >= t2_two_from(mode, qt) ? kT2HTwo : kT2H};
+            best = {h, per_sm == 2 && h >= t2_two_from(mode, qt) ? kT2HTwo : kT2H, false};
             best_cost = cost;
         }
     }
@@ -423,15 +446,19 @@ inline T2Shape t2_block(int mode, int qt, int nx, int ny, int nsm) {
 // The build of the kernel and its dynamic shared memory (300^2 with 12 rows and
 // two tiles per SM takes 2.53 us per step in the many-tiles build, 2.44 in the
 // first).
-template <int M, int HM>
+template <int M, int HM, bool EV = false>
 const void* step2_kernel_hm(int qt, int phase_k) {
-    if (qt == 9) return phase_k ? (const void*)fused_step2<M, 9, true, HM> : (const void*)fused_step2<M, 9, false, HM>;
+    if (qt == 9)
+        return phase_k ? (const void*)fused_step2<M, 9, true, HM, EV> : (const void*)fused_step2<M, 9, false, HM, EV>;
     if constexpr (HM == kT2HTwo && M == MODE_F32) return nullptr;   // (two blocks of up to 14 rows fit as they are)
-    else return phase_k ? (const void*)fused_step2<M, 5, true, HM> : (const void*)fused_step2<M, 5, false, HM>;
+    else return phase_k ? (const void*)fused_step2<M, 5, true, HM, EV> : (const void*)fused_step2<M, 5, false, HM, EV>;
 }
 
 template <int M>
-const void* step2_kernel(int qt, int phase_k, int hm) {
+const void* step2_kernel(int qt, int phase_k, T2Shape t) {
+    const int hm = t.hm;
+    if constexpr (M == MODE_F32)
+        if (t.stream) return step2_kernel_hm<M, kT2HMany, true>(qt, phase_k);
     if constexpr (M != MODE_F64) {
         if (hm == kT2HMany) return step2_kernel_hm<M, kT2HMany>(qt, phase_k);
         return hm == kT2HTwo ? step2_kernel_hm<M, kT2HTwo>(qt, phase_k) : step2_kernel_hm<M, kT2H>(qt, phase_k);
@@ -474,7 +501,7 @@ inline long long group2_blocks(int nx, int ny) { return t2_tiles(nx, kT2W - 2) *
 // before the first of them on the device.
 template <int M>
 cudaError_t prepare_step2(int qt, int phase_k, T2Shape t) {
-    const void* fn = step2_kernel<M>(qt, phase_k, t.hm);
+    const void* fn = step2_kernel<M>(qt, phase_k, t);
     if (!fn) return cudaErrorInvalidConfiguration;
     return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)step2_smem<M>(qt, t.hm));
 }
@@ -485,7 +512,7 @@ cudaError_t prepare_step2(int qt, int phase_k, T2Shape t) {
 template <int M>
 cudaError_t launch_step2(const StepParams<typename ModeTraits<M>::R>& P, int qt, T2Shape t, cudaStream_t s) {
     if (t.h < 4 || t.h > t.hm) return cudaErrorInvalidConfiguration;
-    const void* fn = step2_kernel<M>(qt, P.phase_k, t.hm);
+    const void* fn = step2_kernel<M>(qt, P.phase_k, t);
     if (!fn) return cudaErrorInvalidConfiguration;
     const size_t smem = step2_smem<M>(qt, t.hm);
     void* args[1] = {const_cast<StepParams<typename ModeTraits<M>::R>*>(&P)};
@@ -584,7 +611,7 @@ int batch_blocks_per_sm(int qt, int flow, int ph) {
     KW template cudaError_t prepare_step2<M>(int, int, T2Shape);                                              \
     KW template const void* group2_kernel<M>(int, int, bool);                                                        \
     KW template size_t step2_smem<M>(int, int);                                                               \
-    KW template StepLaunch step_launch<M>(const StepParams<ModeTraits<M>::R>&, int, int, int, dim3);
+    KW template StepLaunch step_launch<M>(const StepParams<ModeTraits<M>::R>&, int, int, int, dim3, bool);
 
 #define LBMK_CONVERT_TEMPLATES(KW, M)                                                                         \
     KW template cudaError_t launch_convert<M>(const StepParams<ModeTraits<M>::R>&, const DenseState<ModeTraits<M>::R>&, \

@@ -64,6 +64,22 @@ def test_two_step_builds_of_tall_tiles(lbm, shape, prec, q, eq9):
     assert b.status() == 0 and np.array_equal(a.save(), b.save())
 
 
+@pytest.mark.parametrize("shape,prec,q,form,bounce", [
+    ((769, 701), 1, 5, 1, 0), ((641, 643), 1, 9, 1, 0), ((900, 874), 1, 5, 3, 0), ((1011, 999), 2, 5, 1, 0),
+    ((1301, 1210), 2, 5, 2, 0), ((1000, 803), 3, 9, 1, 0), ((1000, 1003), 3, 5, 1, 1)])
+def test_reads_marked_evict_first(lbm, shape, prec, q, form, bounce):
+    """Grids whose state is about L2's size, where lbm_step marks its reads
+    evict-first, against a batch of one run, which does not."""
+    s = random_run(lbm, *shape, prec, seed=3, qt=q, solid_scheme=bounce)
+    a, b = twin(lbm, s, form), twin(lbm, s, 1)
+    batch = lbm.Batch([b], autotune=False).configure(128, 3)
+    a.step(4)
+    batch.step(64)   # (the graph's launches)
+    a.step(60)
+    assert a.status() == 0 and np.array_equal(a.save(), b.save())
+    batch.close()
+
+
 @pytest.mark.parametrize("shape", [(1025, 768), (900, 874)])
 def test_two_steps_with_prefetch_beyond_l2(lbm, shape):
     """FP32 grids of at least 786,432 nodes, whose two-step tiles prefetch rows
