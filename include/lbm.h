@@ -207,13 +207,15 @@ int lbm_step(lbm_handle* h, int64_t nsteps);
  * FP32/FP16/BF16 storage), the others keep one node per thread.  On grids of at
  * least 1,572,864 nodes (state far beyond L2) each node-pair block also asks L2
  * for the rows that blocks 48 rows further on will read (bulk L2 prefetch).
+ * lbm_step's launches of a run with flow in FP32/FP16/BF16 whose state takes 84
+ * to 180 MB mark their reads evict-first instead.
  * LBM_STEP_FORM_TWO_STEPS: two time steps per launch for runs with flow in
  * FP32/FP16/BF16 storage (the others step one node per thread): each block of
  * 34 x H threads advances its tile and the one-node ring around it one step
  * into shared memory, then the tile's 32 x (H - 2) inner nodes a second step
  * into the other state copy (H from 4 to 15 per grid, at most two tiles per SM
- * where the grid allows, else H = 12; FP32 grids of at least 786,432 nodes
- * prefetch the rows 20 further on into L2);
+ * where the grid allows, else H = 12; larger FP32 grids prefetch the rows 20
+ * further on into L2);
  * lbm_step takes it for 4 steps or more (an odd remainder and steps that bring
  * the run back to state copy 0 are single steps).  LBM_STEP_FORM_AUTO (the
  * default), for runs with flow and the D2Q5 thermal lattices: two steps per

@@ -1167,8 +1167,9 @@ __device__ __forceinline__ float* next_wide(const StepParams<typename ModeTraits
 // stores that may alias it, and a load after them adds a memory round trip to
 // the step; in FP32, one node per thread, it is read after the state is known,
 // and the thermal lattices are pulled first (one step per launch 330^2 3.17 ->
-// 2.98 us, 512^2 4.98 -> 4.84, 1024^2 27.3 -> 26.4).  Returns the new history.
-template <int M, int QT, bool FLOW, bool PH, int PS, typename T, typename A>
+// 2.98 us, 512^2 4.98 -> 4.84, 1024^2 27.3 -> 26.4).  TF: the thermal lattices
+// collide before the flow.  Returns the new history.
+template <int M, int QT, bool FLOW, bool PH, int PS, typename T, bool TF = false, typename A>
 __device__ __forceinline__ T advance(const StepParams<typename ModeTraits<M>::R>& P, const A& a, const WallAt<T>& w,
                                      const typename Lane<T>::R* history, typename ModeTraits<M>::B* db, float* dw) {
     NodeState<M, QT, FLOW, T> n;
@@ -1176,9 +1177,10 @@ __device__ __forceinline__ T advance(const StepParams<typename ModeTraits<M>::R>
     if constexpr (Lane<T>::n == 1 && !kComp<M>) dTp = get_real<T>(history);
     node_state<M, QT, FLOW, T>(P, a, w, n);
     if constexpr (Lane<T>::n == 1 && kComp<M>) dTp = get_real<T>(history);
-    flow_collide<M, QT, FLOW, PS, T>(P, n, db);
+    if constexpr (!TF) flow_collide<M, QT, FLOW, PS, T>(P, n, db);
     if constexpr (Lane<T>::n == 2) dTp = get_real<T>(history);
     const T dTn = thermal_collide<M, QT, FLOW, PH, PS, T>(P, n, dTp, db, dw);
+    if constexpr (TF) flow_collide<M, QT, FLOW, PS, T>(P, n, db);
     check_state<M, QT, FLOW, T>(P, n);
     return dTn;
 }
@@ -1400,7 +1402,7 @@ __host__ __device__ __forceinline__ int t2_count(int n, int w) { return n > w ? 
 // Both steps of tile (bx, by) of run P, by a block of kT2W x blockDim.y
 // threads (blockDim.y <= HM) with Tile2<M, QT, HM>::bytes of dynamic shared
 // memory.
-template <int M, int QT, bool PH, int HM, bool EV = false>
+template <int M, int QT, bool PH, int HM, bool EV = false, bool TF = false>
 __device__ __forceinline__ void step2_tile(const StepParams<typename ModeTraits<M>::R>& P, int bx, int by) {
     using R = typename ModeTraits<M>::R;
     using B = typename ModeTraits<M>::B;
@@ -1430,7 +1432,7 @@ __device__ __forceinline__ void step2_tile(const StepParams<typename ModeTraits<
         prefetch_rows<M, QT, true>(P, x2, y2 + P.prefetch_rows, 1);
     if (live) {
         const WallAt<R> w(P, x, y);
-        sdT[i] = advance<M, QT, true, PH, TL::n, R>(P, PullAt<M, QT, true, EV>(P, w.xs, w.ys), w, P.dT + (y * P.pitch + x),
+        sdT[i] = advance<M, QT, true, PH, TL::n, R, TF>(P, PullAt<M, QT, true, EV>(P, w.xs, w.ys), w, P.dT + (y * P.pitch + x),
                                                      sb + i, sw + i);
     }
     __syncthreads();
@@ -1438,13 +1440,13 @@ __device__ __forceinline__ void step2_tile(const StepParams<typename ModeTraits<
     if (lx < 1 || lx > kT2W - 2 || ly < 1 || ly > H - 2 || x2 >= P.nx || y2 >= P.ny) return;
     const WallAt<R> w(P, x2, y2);
     const PullTile<M, TL::n> a{sb, sw, i + (w.ys - y2) * kT2W + (w.xs - x2)};
-    P.dT_out[y2 * P.pitch + x2] = advance<M, QT, true, PH, kChunk, R>(
+    P.dT_out[y2 * P.pitch + x2] = advance<M, QT, true, PH, kChunk, R, TF>(
         P, a, w, sdT + i, next_bulk<M, QT, true>(P, x2, y2), next_wide<M, QT, true>(P, x2, y2));
 }
 
-template <int M, int QT, bool PH, int HM, bool EV = false>
+template <int M, int QT, bool PH, int HM, bool EV = false, bool TF = false>
 __global__ void __launch_bounds__(kT2W * HM, (kT2Blocks<HM, M, QT>)) fused_step2(const __grid_constant__ StepParams<typename ModeTraits<M>::R> P) {
-    step2_tile<M, QT, PH, HM, EV>(P, blockIdx.x, blockIdx.y);
+    step2_tile<M, QT, PH, HM, EV, TF>(P, blockIdx.x, blockIdx.y);
 }
 
 // ---------------------------------------------------------------------------

@@ -418,6 +418,7 @@ struct T2Shape {
     int h;    // block height
     int hm;   // the build, kT2H, kT2HTwo or kT2HMany
     bool stream;   // kT2HMany in FP32: reads marked evict-first
+    bool thermal;  // kT2H in FP32, D2Q5: the thermal lattices collide first
 };
 
 // Height from which two blocks of the first build don't fit an SM's registers
@@ -425,9 +426,18 @@ struct T2Shape {
 // the build capped for them.
 inline int t2_two_from(int mode, int qt) { return mode == MODE_F32 ? (qt == 5 ? kT2HTwo + 1 : 12) : (qt == 5 ? 12 : 10); }
 
+// Rows of tiles per SM from which the FP32 D2Q5 tiles let the thermal lattices
+// collide first: with the schedulers full the order that frees registers
+// early wins, with a few warps the one whose chain is shorter (us per step,
+// flow / thermal lattices first: 64^2, 4 rows, 1.09 / 1.12, 128^2, 6, 1.22 / 1.25,
+// 150^2, 7, and 200^2, 10, the same, 256 x 242, 15, 1.89 / 1.86, 256^2, 18, 1.86 /
+// 1.83, 300^2, 24, 2.41 / 2.39, 320^2, 26, 2.47 / 2.43; with Eq. 9 256^2 1.89 /
+// 1.91, not taken).
+constexpr int kT2ThermalRows = 15;
+
 inline T2Shape t2_block(int mode, int qt, int nx, int ny, int nsm) {
     if (nsm < 1) nsm = 1;
-    T2Shape best = {kT2HMany, kT2HMany, mode == MODE_F32 && streams(mode, qt, 1, (long long)nx * ny)};
+    T2Shape best = {kT2HMany, kT2HMany, mode == MODE_F32 && streams(mode, qt, 1, (long long)nx * ny), false};
     double best_cost = -1.0;
     for (int h = 4; h <= kT2H; ++h) {
         const long long tiles = t2_tiles(nx, kT2W - 2) * t2_tiles(ny, h - 2);
@@ -436,7 +446,8 @@ inline T2Shape t2_block(int mode, int qt, int nx, int ny, int nsm) {
         const long long work = per_sm * ((kT2W * h + 31) / 32 * 32 + (long long)(kT2W - 2) * (h - 2));
         const double cost = per_sm > 1 ? kT2Overlap * (double)work : (double)work;
         if (best_cost < 0.0 || cost < best_cost) {
-            best = {h, per_sm == 2 && h >= t2_two_from(mode, qt) ? kT2HTwo : kT2H, false};
+            best = {h, per_sm == 2 && h >= t2_two_from(mode, qt) ? kT2HTwo : kT2H, false,
+                    mode == MODE_F32 && qt == 5 && per_sm * h >= kT2ThermalRows};
             best_cost = cost;
         }
     }
@@ -457,8 +468,10 @@ const void* step2_kernel_hm(int qt, int phase_k) {
 template <int M>
 const void* step2_kernel(int qt, int phase_k, T2Shape t) {
     const int hm = t.hm;
-    if constexpr (M == MODE_F32)
+    if constexpr (M == MODE_F32) {
         if (t.stream) return step2_kernel_hm<M, kT2HMany, true>(qt, phase_k);
+        if (t.thermal && !phase_k) return (const void*)fused_step2<M, 5, false, kT2H, false, true>;
+    }
     if constexpr (M != MODE_F64) {
         if (hm == kT2HMany) return step2_kernel_hm<M, kT2HMany>(qt, phase_k);
         return hm == kT2HTwo ? step2_kernel_hm<M, kT2HTwo>(qt, phase_k) : step2_kernel_hm<M, kT2H>(qt, phase_k);
