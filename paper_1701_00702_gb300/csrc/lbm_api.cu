@@ -1002,6 +1002,7 @@ struct lbm_batch {
     std::vector<std::vector<int>> groups;   // maps 4, 5: the runs of each grouped launch in graphs
     std::vector<std::vector<int>> inline_groups;   // the same outside graphs
     std::vector<GroupArgs> launches[4];     // their launches outside graphs, filled on first use: one step from parity 0 or 1, two steps there or back
+    bool streams = false;                   // grouped launches mark their reads evict-first
     std::vector<int> solo;                  // map 4: runs that keep their own step kernel
     lbmk::Tile* tiles = nullptr;
     size_t tile_capacity = 0;     // tiles that fit in the allocation
@@ -1146,6 +1147,9 @@ void make_groups(lbm_batch* b) {
     const size_t cap = b->precision == LBM_F64 ? lbmk::kGroupRuns<double> : lbmk::kGroupRuns<float>;
     auto nodes = [&](int r) { return (long long)b->runs[r]->p.nx * b->runs[r]->p.ny; };
     std::vector<int> small;
+    long long all = 0;
+    for (int r = 0; r < (int)b->runs.size(); ++r) all += nodes(r);
+    b->streams = lbmk::streams(b->precision, b->qt, b->flow, all);
     for (int r = 0; r < (int)b->runs.size(); ++r) {
         if (b->mapping == 5 || nodes(r) < lbmk::kGroupMaxNodes) small.push_back(r);
         else b->solo.push_back(r);
@@ -1310,10 +1314,10 @@ long long fill_group(const lbm_batch* b, const std::vector<int>& g, int parity, 
 const void* group_fn(const lbm_batch* b, bool few) {
     const int ph = batch_phase(b);
     switch (b->precision) {
-        case LBM_F64: return lbmk::group_kernel<lbmk::MODE_F64>(b->qt, b->flow, ph, few);
-        case LBM_F32: return lbmk::group_kernel<lbmk::MODE_F32>(b->qt, b->flow, ph, few);
-        case LBM_F16: return lbmk::group_kernel<lbmk::MODE_F16>(b->qt, b->flow, ph, few);
-        default: return lbmk::group_kernel<lbmk::MODE_BF16>(b->qt, b->flow, ph, few);
+        case LBM_F64: return lbmk::group_kernel<lbmk::MODE_F64>(b->qt, b->flow, ph, few, b->streams);
+        case LBM_F32: return lbmk::group_kernel<lbmk::MODE_F32>(b->qt, b->flow, ph, few, b->streams);
+        case LBM_F16: return lbmk::group_kernel<lbmk::MODE_F16>(b->qt, b->flow, ph, few, b->streams);
+        default: return lbmk::group_kernel<lbmk::MODE_BF16>(b->qt, b->flow, ph, few, b->streams);
     }
 }
 
@@ -1332,9 +1336,9 @@ int ensure_batch_dT2(lbm_batch* b) {
 const void* group2_fn(const lbm_batch* b, bool few) {
     const int ph = batch_phase(b);
     switch (b->precision) {
-        case LBM_F32: return lbmk::group2_kernel<lbmk::MODE_F32>(b->qt, ph, few);
-        case LBM_F16: return lbmk::group2_kernel<lbmk::MODE_F16>(b->qt, ph, few);
-        case LBM_BF16: return lbmk::group2_kernel<lbmk::MODE_BF16>(b->qt, ph, few);
+        case LBM_F32: return lbmk::group2_kernel<lbmk::MODE_F32>(b->qt, ph, few, b->streams);
+        case LBM_F16: return lbmk::group2_kernel<lbmk::MODE_F16>(b->qt, ph, few, b->streams);
+        case LBM_BF16: return lbmk::group2_kernel<lbmk::MODE_BF16>(b->qt, ph, few, b->streams);
         default: return nullptr;
     }
 }

@@ -1532,7 +1532,7 @@ __device__ __forceinline__ int group_run(const GroupParams<R, NR>& G, int b) {
     return lo;
 }
 
-template <int M, int QT, bool FLOW, bool PH, int NR>
+template <int M, int QT, bool FLOW, bool PH, int NR, bool EV>
 __global__ void __launch_bounds__(128, 2 * kMinBlocks<M, QT, FLOW>) group_step(
     const __grid_constant__ GroupParams<typename ModeTraits<M>::R, NR> G) {
     const int b = blockIdx.x, lo = group_run(G, b);
@@ -1545,7 +1545,7 @@ __global__ void __launch_bounds__(128, 2 * kMinBlocks<M, QT, FLOW>) group_step(
     const int y = (lb / gx) * (128 >> lw) + (t >> lw);
     if (x >= P.nx || y >= P.ny) return;
     griddep_wait();
-    step_node<M, QT, FLOW, PH>(P, x, y);
+    step_node<M, QT, FLOW, PH, EV>(P, x, y);
 }
 
 // The same for runs in 16-bit storage with flow and the D2Q5 thermal lattices,
@@ -1554,7 +1554,7 @@ __global__ void __launch_bounds__(128, 2 * kMinBlocks<M, QT, FLOW>) group_step(
 // where its nodes one by one take 1,000 (64 cavities of 64-512 nodes a side,
 // FP16: 132.7 us per step of all with one node per thread, 123.1 with pairs;
 // 12 cavities 22.2 and 17.5 with the groups side by side as well).
-template <int M, bool PH, int NR>
+template <int M, bool PH, int NR, bool EV>
 __global__ void __launch_bounds__(128, kPairBlocks) group_step_pair(const __grid_constant__ GroupParams<float, NR> G) {
     const int b = blockIdx.x, lo = group_run(G, b);
     const StepParams<float>& P = G.run[lo];
@@ -1566,7 +1566,7 @@ __global__ void __launch_bounds__(128, kPairBlocks) group_step_pair(const __grid
     const int y = (lb / gx) * (128 >> lp) + (t >> lp);
     if (x0 >= P.nx || y >= P.ny) return;
     griddep_wait();
-    step_pair_or_nodes<M, PH>(P, x0, y);
+    step_pair_or_nodes<M, PH, EV>(P, x0, y);
 }
 
 // Batch map 5: the grouped launch of the two-step form.  Run k owns blocks
@@ -1574,14 +1574,14 @@ __global__ void __launch_bounds__(128, kPairBlocks) group_step_pair(const __grid
 // kT2W x kT2HMany threads, inner tiles of (kT2W - 2) x (kT2HMany - 2) nodes,
 // row-major over the run's tiles); each block advances its tile two steps as
 // fused_step2 does, with its run's parameter block.
-template <int M, int QT, bool PH, int NR>
+template <int M, int QT, bool PH, int NR, bool EV>
 __global__ void __launch_bounds__(kT2W * kT2HMany, (kT2Blocks<kT2HMany, M, QT>)) group_step2(
     const __grid_constant__ GroupParams<typename ModeTraits<M>::R, NR> G) {
     const int b = blockIdx.x, lo = group_run(G, b);
     const StepParams<typename ModeTraits<M>::R>& P = G.run[lo];
     const int lb = b - G.first_block[lo];
     const int gx = t2_count(P.nx, kT2W - 2);
-    step2_tile<M, QT, PH, kT2HMany>(P, lb % gx, lb / gx);
+    step2_tile<M, QT, PH, kT2HMany, EV>(P, lb % gx, lb / gx);
 }
 
 // Many runs in one launch.  A tile is w x (256 / w) nodes of one run (w a

@@ -244,7 +244,10 @@ inline bool pairs_of(const StepParams<typename ModeTraits<M>::R>& P, int qt, int
 // 12.7, 900^2, 185 MB, 29.6 / 28.4, 1100^2, 276 MB, 42.5 / 45.6.  FP16: 900^2, 71
 // MB, 11.7 / 11.6, 1000^2, 88 MB, 14.7 / 13.7, 1200^2, 127 MB, 25.3 / 18.6.)  A
 // marked line is not prefetched: it would be dropped before its block reads it.
-// A run's own launches only: the runs of a batch share L2.
+// The runs of a batch share L2: grouped launches go by the nodes of all runs
+// (12 cavities of 106-471 nodes a side, us per step of all: FP16 map 4, 90 MB,
+// 17.7 / 16.1, FP32 map 5, 167 MB, 22.8 / 20.0, FP32 map 4 25.5 / 24.5), the other
+// maps' kernels don't mark.
 constexpr long long kStreamMinBytes = 84000000, kStreamMaxBytes = 180000000;
 
 inline bool streams(int mode, int qt, int flow, long long nodes) {
@@ -353,14 +356,15 @@ inline long long group_blocks(int nx, int ny, int tile, bool pairs) {
     return (long long)((nx + w - 1) / w) * ((ny + h - 1) / h);
 }
 
-template <int M, int NR>
+// stream: reads marked evict-first (runs with flow, not in FP64).
+template <int M, int NR, bool EV>
 const void* group_kernel_nr(int qt, int flow, int ph) {
     if constexpr (kSplit<M>)
         if (group_pairs(M, qt, flow))
-            return ph ? (const void*)group_step_pair<M, true, NR> : (const void*)group_step_pair<M, false, NR>;
+            return ph ? (const void*)group_step_pair<M, true, NR, EV> : (const void*)group_step_pair<M, false, NR, EV>;
     const void* fn = nullptr;
     dispatch_step<M>(qt, flow, ph, [&]<int MM, int Q, bool F, bool PH>() {
-        if constexpr (!(kSplit<MM> && Q == 5 && F)) fn = (const void*)group_step<MM, Q, F, PH, NR>;
+        if constexpr (!(kSplit<MM> && Q == 5 && F)) fn = (const void*)group_step<MM, Q, F, PH, NR, (EV && F)>;
         return cudaSuccess;
     });
     return fn;
@@ -368,9 +372,11 @@ const void* group_kernel_nr(int qt, int flow, int ph) {
 
 // few: the build for at most kGroupFew runs.
 template <int M>
-const void* group_kernel(int qt, int flow, int ph, bool few) {
-    return few ? group_kernel_nr<M, kGroupFew>(qt, flow, ph)
-               : group_kernel_nr<M, kGroupRuns<typename ModeTraits<M>::R>>(qt, flow, ph);
+const void* group_kernel(int qt, int flow, int ph, bool few, bool stream) {
+    constexpr int all = kGroupRuns<typename ModeTraits<M>::R>;
+    if constexpr (M != MODE_F64)
+        if (stream) return few ? group_kernel_nr<M, kGroupFew, true>(qt, flow, ph) : group_kernel_nr<M, all, true>(qt, flow, ph);
+    return few ? group_kernel_nr<M, kGroupFew, false>(qt, flow, ph) : group_kernel_nr<M, all, false>(qt, flow, ph);
 }
 
 // Launched as a programmatic dependent of the previous step (the kernels wait
@@ -495,16 +501,21 @@ size_t step2_smem(int qt, int hm) {
 
 // Batch map 5: the grouped two-step kernel and its shared memory (the 12-row
 // build; blocks of kT2W x kT2HMany threads).
-template <int M, int NR>
+template <int M, int NR, bool EV>
 const void* group2_kernel_nr(int qt, int phase_k) {
-    if (qt == 5) return phase_k ? (const void*)group_step2<M, 5, true, NR> : (const void*)group_step2<M, 5, false, NR>;
-    return phase_k ? (const void*)group_step2<M, 9, true, NR> : (const void*)group_step2<M, 9, false, NR>;
+    if (qt == 5) return phase_k ? (const void*)group_step2<M, 5, true, NR, EV> : (const void*)group_step2<M, 5, false, NR, EV>;
+    return phase_k ? (const void*)group_step2<M, 9, true, NR, EV> : (const void*)group_step2<M, 9, false, NR, EV>;
 }
 
 template <int M>
-const void* group2_kernel(int qt, int phase_k, bool few) {
+const void* group2_kernel(int qt, int phase_k, bool few, bool stream) {
+    if constexpr (M == MODE_F32)
+        if (stream)
+            return few ? group2_kernel_nr<M, kGroupFew, true>(qt, phase_k)
+                       : group2_kernel_nr<M, kGroupRuns<float>, true>(qt, phase_k);
     if constexpr (M != MODE_F64)
-        return few ? group2_kernel_nr<M, kGroupFew>(qt, phase_k) : group2_kernel_nr<M, kGroupRuns<float>>(qt, phase_k);
+        return few ? group2_kernel_nr<M, kGroupFew, false>(qt, phase_k)
+                   : group2_kernel_nr<M, kGroupRuns<float>, false>(qt, phase_k);
     return nullptr;
 }
 
@@ -619,10 +630,10 @@ int batch_blocks_per_sm(int qt, int flow, int ph) {
     KW template cudaError_t launch_batch<M>(const StepParams<ModeTraits<M>::R>*, const Tile*, int, int, int, int, int, \
                                          int, int, cudaStream_t);                                               \
     KW template int batch_blocks_per_sm<M>(int, int, int);                                                   \
-    KW template const void* group_kernel<M>(int, int, int, bool);                                                    \
+    KW template const void* group_kernel<M>(int, int, int, bool, bool);                                                    \
     KW template cudaError_t launch_step2<M>(const StepParams<ModeTraits<M>::R>&, int, T2Shape, cudaStream_t); \
     KW template cudaError_t prepare_step2<M>(int, int, T2Shape);                                              \
-    KW template const void* group2_kernel<M>(int, int, bool);                                                        \
+    KW template const void* group2_kernel<M>(int, int, bool, bool);                                                        \
     KW template size_t step2_smem<M>(int, int);                                                               \
     KW template StepLaunch step_launch<M>(const StepParams<ModeTraits<M>::R>&, int, int, int, dim3, bool);
 

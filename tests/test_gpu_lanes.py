@@ -80,6 +80,21 @@ def test_reads_marked_evict_first(lbm, shape, prec, q, form, bounce):
     batch.close()
 
 
+@pytest.mark.parametrize("prec,q,mapping,shape", [(2, 5, 4, (701, 720)), (1, 5, 5, (501, 524)), (1, 5, 4, (501, 524)),
+                                                 (3, 9, 4, (611, 600)), (1, 9, 5, (433, 480))])
+def test_grouped_reads_marked_evict_first(lbm, prec, q, mapping, shape):
+    """Two runs whose states are about L2's size together, in grouped launches
+    that mark their reads, against lbm_step on each, which does not."""
+    runs = [random_run(lbm, *shape, prec, seed=k, qt=q) for k in (1, 2)]
+    twins = [twin(lbm, s, 1) for s in runs]
+    b = lbm.Batch(runs, autotune=False).configure(128, mapping)
+    b.step(66)
+    for s, t in zip(runs, twins):
+        t.step(66)
+        assert s.status() == 0 and np.array_equal(s.save(), t.save())
+    b.close()
+
+
 @pytest.mark.parametrize("shape", [(1025, 768), (900, 874)])
 def test_two_steps_with_prefetch_beyond_l2(lbm, shape):
     """FP32 grids of at least 786,432 nodes, whose two-step tiles prefetch rows
