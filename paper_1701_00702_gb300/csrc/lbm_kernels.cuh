@@ -1354,9 +1354,9 @@ __global__ void __launch_bounds__(64) conduction_step_lanes(const __grid_constan
 // 104 against 84 us per step; two blocks of the other builds, which would spill
 // under the three-block cap).  Small grids are bound by the
 // launch floor and two dependency chains (64^2 FP32 1.315 us per step before
-// the update was written in named multiply-adds, 1.09 now; 256^2 2.05 / 1.86),
+// the update was written in named multiply-adds, 1.09 now; 256^2 2.05 / 1.83),
 // grids beyond L2 by instruction issue once their rows are prefetched (2048^2
-// 79.9 us per step before, 71.1 now; 49.5 at the copy bandwidth).  Two nodes
+// 79.9 us per step before, 70.6 now; 49.5 at the copy bandwidth).  Two nodes
 // per thread in the tile, side by side or one above the other, were slower
 // (2048^2 77.0 and 73.3, 64^2 1.37): more registers, fewer warps.
 constexpr int kT2W = 34, kT2H = 15, kT2HTwo = 14, kT2HMany = 12;

@@ -214,8 +214,9 @@ inline int form_for(int mode, int qt, int flow, int solid_scheme, long long node
 // steps per launch; FP32: 256^2 2.40 / 2.02, 320^2 3.01 / 2.74,
 // 352^2 3.16 / 3.30, 384^2 3.39 / 4.26, 512^2 4.99 / 5.98, 768^2 11.1 / 12.2,
 // 896^2 19.1 / 16.9, 1024^2 26.5 / 21.9, 2048^2 99.7 / 81.2; FP16: 320^2
-// 3.14 / 2.91, 352^2 3.20 / 4.25); the current one takes FP32 256^2 2.15 / 1.86,
-// 2048^2 100 / 71.1.  Single steps (an odd remainder, batches)
+// 3.14 / 2.91, 352^2 3.20 / 4.25); the current one takes FP32 256^2 2.26 / 1.82,
+// 320^2 2.75 / 2.43, 352^2 2.91 / 3.07, 768^2 9.3 / 10.8, 896^2 13.1 / 14.2, 1024^2
+// 21.6 / 18.1, 2048^2 99.4 / 70.5, FP16 320^2 2.91 / 2.62, 352^2 2.98 / 3.71.  Single steps (an odd remainder, batches)
 // keep the form above.
 constexpr long long kTwoStepSmallMaxNodes = 320 * 320;
 constexpr long long kTwoStepF32MinNodes = 3ll << 18;
