@@ -198,9 +198,7 @@ int lbm_create_ex(const lbm_params* p, void* cuda_stream, lbm_alloc_fn alloc,
 int lbm_step(lbm_handle* h, int64_t nsteps);
 
 /* Step form of a run (the paper has no counterpart: an implementation
- * choice).  LBM_STEP_FORM_SINGLE: one step per launch, one node per thread, or
- * two neighbouring nodes (as the next form, without its prefetch) in FP16/BF16
- * runs of at least 131,072 nodes that could take that form.
+ * choice).  LBM_STEP_FORM_SINGLE: one step per launch, one node per thread.
  * LBM_STEP_FORM_PAIRS: two neighbouring nodes per thread, each FP32 operation
  * one packed instruction for both; taken only by runs in the default
  * configuration (flow, D2Q5 thermal lattices, volumetric blend,
@@ -221,16 +219,20 @@ int lbm_step(lbm_handle* h, int64_t nsteps);
  * default), for runs with flow and the D2Q5 thermal lattices: two steps per
  * launch on grids of up to 102,400 nodes in FP32/FP16/BF16 and on FP32 grids
  * of at least 786,432 nodes (state beyond L2); node pairs for FP16/BF16 runs
- * of at least 1,572,864 (1536 x 1024) nodes; otherwise LBM_STEP_FORM_SINGLE.
+ * of at least 1,572,864 (1536 x 1024) nodes; otherwise one step per launch, one
+ * node per thread or, in FP16/BF16 runs of at least 131,072 nodes that could take
+ * pairs, those without their prefetch (lbm_step_form_for reports
+ * LBM_STEP_FORM_SINGLE for both).
  * Every form gives the same states bit for bit: all kernels share one node
  * update in which each rounding is fixed.  A run that steps two steps per
  * launch keeps a second exchange-history array (4 bytes per node of row
  * pitch), allocated on the run's allocator at the first lbm_step that uses the
  * form (LBM_ERR_OOM if that fails; nothing stepped).  Applies to later lbm_step
  * calls and to batches created afterwards (batches advance one step per launch
- * except under map 5: a run in the two-step form steps there as
- * LBM_STEP_FORM_SINGLE); synchronises the run's stream when it drops a captured
- * graph.  LBM_ERR_ARG for another value. */
+ * except under map 5: a run in the two-step form steps there, and in its single
+ * steps, as LBM_STEP_FORM_AUTO's one step per launch without the prefetch);
+ * synchronises the run's stream when it drops a captured graph.  LBM_ERR_ARG for
+ * another value. */
 #define LBM_STEP_FORM_AUTO 0
 #define LBM_STEP_FORM_SINGLE 1
 #define LBM_STEP_FORM_PAIRS 2

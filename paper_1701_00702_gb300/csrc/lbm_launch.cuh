@@ -176,24 +176,26 @@ inline dim3 step_block(int mode, int nx, int ny) {
     return cover(64) <= cover(32) ? dim3(64, 1) : dim3(32, 2);
 }
 
-// Step forms.  FORM_SINGLE is one step per launch, FORM_PAIRS that with node
-// pairs (fused_step_pair, the default configuration only: flow, D2Q5,
-// volumetric blend, FP32 arithmetic) and the L2 prefetch.  Automatic: pairs
+// Step forms.  FORM_SINGLE is one step per launch, one node per thread,
+// FORM_PAIRS that with node pairs (fused_step_pair, the default configuration
+// only: flow, D2Q5, volumetric blend, FP32 arithmetic) and the L2 prefetch.
+// Automatic: pairs
 // with the prefetch for the 16-bit forms from 1536 x 1024 nodes up (at 1024^2,
 // whose state nearly fits in L2, the prefetch gains nothing; in FP32, bound by
 // HBM, one node per thread is faster at every size).
 enum : int { FORM_AUTO = 0, FORM_SINGLE = 1, FORM_PAIRS = 2, FORM_TWO_STEPS = 3 };
 constexpr long long kPairMinNodes = 3ll << 19;
 
-// FORM_SINGLE too takes pairs, without the prefetch, for 16-bit runs from
-// kPairPlainMinNodes nodes, where instruction issue and not one warp's chain
-// bounds the step (GB300, us per step, one node / pairs: FP16 384^2 3.37 / 3.27,
+// The automatic single step, and the single steps of FORM_TWO_STEPS, take pairs
+// too, without the prefetch, for 16-bit runs from kPairPlainMinNodes nodes, where
+// instruction issue and not one warp's chain bounds the step (GB300, us per step, one node / pairs: FP16 384^2 3.37 / 3.27,
 // 512^2 5.09 / 4.93, 1024^2 17.9 / 16.1, BF16 with Eq. 9 777 x 501 7.80 / 7.62;
 // in FP32 512^2 5.0 / 5.2, 1024^2 26.5 / 26.9).
 constexpr long long kPairPlainMinNodes = 1ll << 17;
 
 // The rule (host code; lbm_step_form_for reports it): the form a run takes,
-// FORM_SINGLE or FORM_PAIRS.  mode: MODE_*.
+// FORM_SINGLE (one step per launch, pairs without the prefetch among them) or
+// FORM_PAIRS.  mode: MODE_*.
 inline int form_for(int mode, int qt, int flow, int solid_scheme, long long nodes, int form) {
     const bool pairs = mode != MODE_F64 && qt == 5 && flow && !solid_scheme;
     if (form == FORM_PAIRS) return pairs ? FORM_PAIRS : FORM_SINGLE;
@@ -233,7 +235,7 @@ template <int M>
 inline bool pairs_of(const StepParams<typename ModeTraits<M>::R>& P, int qt, int flow, int form) {
     const long long nodes = (long long)P.nx * P.ny;
     if (form_for(M, qt, flow, P.solid_scheme, nodes, form) == FORM_PAIRS) return true;
-    return kSplit<M> && qt == 5 && flow && !P.solid_scheme && nodes >= kPairPlainMinNodes;
+    return form != FORM_SINGLE && kSplit<M> && qt == 5 && flow && !P.solid_scheme && nodes >= kPairPlainMinNodes;
 }
 
 // Whether a run's launches mark their reads evict-first (read_state): from

@@ -1,11 +1,12 @@
-"""Edges of the launch rules and of the node update: block edges of the
-two-lane FP64 conduction step, compared with the general path."""
+"""Edges of the launch rules and of the node update, compared with the general
+path: block edges, sizes about a rule's line, special values."""
 import numpy as np
 import pytest
 
 from paper_1701_00702_gb300 import inputs
 
 pytestmark = pytest.mark.gpu
+W9 = np.array([4 / 9] + [1 / 9] * 4 + [1 / 36] * 4)
 
 
 @pytest.fixture(scope="module")
@@ -37,3 +38,24 @@ def test_conduction_lanes_beyond_the_grid(lbm, nx):
     b.step(197)
     assert s.status() == 0 and np.array_equal(s.save(), t.save())
     b.close()
+
+
+@pytest.mark.parametrize("shape", [(512, 256), (513, 256), (545, 545), (577, 579), (1025, 1026), (1601, 1030)])
+@pytest.mark.parametrize("prec,eq9", [(2, 0), (3, 0), (2, 1)])
+def test_pairs_equal_one_node_per_thread(lbm, shape, prec, eq9):
+    """16-bit runs about and above the sizes where automatic single steps take
+    node pairs, with and without the prefetch and the evict-first reads: forms 0
+    and 2 against form 1, which steps one node per thread, from a random state."""
+    nx, ny = shape
+    p = inputs.cavity(max(nx, ny), ny=ny, precision=prec, L_char=100.0, Ra=1e7, wall_kind=[0, 1, 1, 0],
+                      **(dict(ks_over_kl=0.7, cps_over_cpl=0.9) if eq9 else {}))
+    p["nx"] = nx
+    F, G, H, dT = inputs.random_state(nx, ny, 5, seed=nx, H_range=(0.0, 1.6), f_base=W9)
+    s = lbm.Solver(p)
+    s.set_state(F - W9[:, None, None], G, H, dT)
+    runs = [twin(lbm, s, form) for form in (1, 0, 2)]
+    for r in runs:
+        r.step(3)
+        assert r.status() == 0
+    want = runs[0].save()
+    assert np.array_equal(want, runs[1].save()) and np.array_equal(want, runs[2].save())

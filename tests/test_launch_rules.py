@@ -1,0 +1,51 @@
+"""The one-step kernel's launch rules on the CPU: which kernel and blocks a run
+takes, from the library's own rule (tests/launch_rules.cu calls it)."""
+import ctypes
+import subprocess
+
+import pytest
+
+from paper_1701_00702_gb300 import build
+
+
+@pytest.fixture(scope="module")
+def rules(tmp_path_factory):
+    lib = build.build()
+    out = tmp_path_factory.mktemp("rules") / "launch_rules.so"
+    src = build.ROOT / "tests" / "launch_rules.cu"
+    subprocess.run([build.nvcc(), *build.GENCODE, "-std=c++20", "-O1", "-shared", "-Xcompiler", "-fPIC", "-I",
+                    str(build.CSRC), "-o", str(out), str(src), str(lib), f"-Xlinker=-rpath={lib.parent}"],
+                   check=True, capture_output=True)
+    L = ctypes.CDLL(str(out))
+
+    def step(nx, ny, prec, form=0, qt=5, flow=1, bounce=0, block=(0, 0)):
+        o = (ctypes.c_int * 4)()
+        L.rule_step(prec, qt, flow, bounce, nx, ny, form, *block, o)
+        return tuple(o)
+
+    return step
+
+
+def takes_pairs(launch, nx):
+    """Blocks of 32 x 4 threads that cover two columns each (no rule gives one
+    node per thread blocks of 32 x 4)."""
+    gx, _, bx, by = launch
+    return (bx, by) == (32, 4) and gx == -(-nx // 64)
+
+
+@pytest.mark.parametrize("prec", [2, 3])
+@pytest.mark.parametrize("shape", [(512, 256), (577, 577), (1024, 1024), (1600, 1024), (2048, 2048)])
+def test_single_is_one_node_per_thread(rules, shape, prec):
+    """Form 1 keeps one node per thread at every size, form 2 pairs."""
+    assert not takes_pairs(rules(*shape, prec, form=1), shape[0])
+    assert takes_pairs(rules(*shape, prec, form=2), shape[0])
+
+
+@pytest.mark.parametrize("prec", [2, 3])
+@pytest.mark.parametrize("shape", [(577, 577), (640, 640), (1024, 1024), (2048, 2048)])
+def test_automatic_single_steps_take_pairs(rules, shape, prec):
+    for form in (0, 3):
+        assert takes_pairs(rules(*shape, prec, form=form), shape[0])
+        assert not takes_pairs(rules(*shape, prec, form=form, bounce=1), shape[0])
+        assert not takes_pairs(rules(*shape, prec, form=form, qt=9), shape[0])
+        assert not takes_pairs(rules(*shape, 1, form=form), shape[0])
