@@ -321,8 +321,9 @@ const char* lbm_strerror(int code);
  * 4 steps the runs below 1,048,576 nodes in grouped launches, one kernel per
  * step for up to 54 runs (29 in FP64) at a time, their parameter blocks in the
  * launch's own parameters, each run in tiles of w x 128/w nodes (FP16/BF16 with
- * flow and D2Q5: w x 256/w, two nodes per thread; w = 32, 64 or 128, whichever
- * leaves the fewest of the run's threads idle).  In the replayed graph the runs
+ * flow and D2Q5 where these runs have 458,752 nodes or more together: w x 256/w,
+ * two nodes per thread; w = 32, 64 or 128, whichever leaves the fewest of the
+ * run's threads idle).  In the replayed graph the runs
  * form at least two groups of about equal size, each a chain of its own, so
  * that one chain's launch overlaps another's tail; larger runs keep their own
  * step kernel in chains of their own, as under map 3.  Map 5 (runs with flow in

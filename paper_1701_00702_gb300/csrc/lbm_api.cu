@@ -1003,6 +1003,7 @@ struct lbm_batch {
     std::vector<std::vector<int>> inline_groups;   // the same outside graphs
     std::vector<GroupArgs> launches[4];     // their launches outside graphs, filled on first use: one step from parity 0 or 1, two steps there or back
     bool streams = false;                   // grouped launches mark their reads evict-first
+    bool pairs = false;                     // map 4: grouped launches take node pairs
     std::vector<int> solo;                  // map 4: runs that keep their own step kernel
     lbmk::Tile* tiles = nullptr;
     size_t tile_capacity = 0;     // tiles that fit in the allocation
@@ -1155,6 +1156,9 @@ void make_groups(lbm_batch* b) {
         else b->solo.push_back(r);
     }
     if (small.empty()) return;
+    long long grouped = 0;
+    for (int r : small) grouped += nodes(r);
+    b->pairs = lbmk::group_pairs(b->precision, b->qt, b->flow, grouped);
     // outside graphs, one launch after another in the stream, as few groups as hold the runs
     for (size_t i = 0; i < small.size(); i += cap)
         b->inline_groups.emplace_back(small.begin() + i, small.begin() + std::min(small.size(), i + cap));
@@ -1304,7 +1308,7 @@ long long fill_group(const lbm_batch* b, const std::vector<int>& g, int parity, 
             acc += lbmk::group2_blocks(h->p.nx, h->p.ny);
         } else {
             G.tile[i] = lbmk::group_tile(h->p.nx);
-            acc += lbmk::group_blocks(h->p.nx, h->p.ny, G.tile[i], lbmk::group_pairs(b->precision, b->qt, b->flow));
+            acc += lbmk::group_blocks(h->p.nx, h->p.ny, G.tile[i], b->pairs);
         }
     }
     G.first_block[g.size()] = (int)acc;
@@ -1314,10 +1318,10 @@ long long fill_group(const lbm_batch* b, const std::vector<int>& g, int parity, 
 const void* group_fn(const lbm_batch* b, bool few) {
     const int ph = batch_phase(b);
     switch (b->precision) {
-        case LBM_F64: return lbmk::group_kernel<lbmk::MODE_F64>(b->qt, b->flow, ph, few, b->streams);
-        case LBM_F32: return lbmk::group_kernel<lbmk::MODE_F32>(b->qt, b->flow, ph, few, b->streams);
-        case LBM_F16: return lbmk::group_kernel<lbmk::MODE_F16>(b->qt, b->flow, ph, few, b->streams);
-        default: return lbmk::group_kernel<lbmk::MODE_BF16>(b->qt, b->flow, ph, few, b->streams);
+        case LBM_F64: return lbmk::group_kernel<lbmk::MODE_F64>(b->qt, b->flow, ph, few, b->streams, b->pairs);
+        case LBM_F32: return lbmk::group_kernel<lbmk::MODE_F32>(b->qt, b->flow, ph, few, b->streams, b->pairs);
+        case LBM_F16: return lbmk::group_kernel<lbmk::MODE_F16>(b->qt, b->flow, ph, few, b->streams, b->pairs);
+        default: return lbmk::group_kernel<lbmk::MODE_BF16>(b->qt, b->flow, ph, few, b->streams, b->pairs);
     }
 }
 

@@ -1549,8 +1549,8 @@ __global__ void __launch_bounds__(128, 2 * kMinBlocks<M, QT, FLOW>) group_step(
 }
 
 // The same for runs in 16-bit storage with flow and the D2Q5 thermal lattices,
-// a node pair per thread: tiles of w x 256 / w nodes, w = 32 << tile.  These
-// runs are bound by instruction issue, and a pair takes some 650 instructions
+// a node pair per thread: tiles of w x 256 / w nodes, w = 32 << tile.  Batches
+// with nodes enough (group_pairs) are bound by instruction issue, and a pair takes some 650 instructions
 // where its nodes one by one take 1,000 (64 cavities of 64-512 nodes a side,
 // FP16: 132.7 us per step of all with one node per thread, 123.1 with pairs;
 // 12 cavities 22.2 and 17.5 with the groups side by side as well).

@@ -349,8 +349,17 @@ inline int group_tile(int nx) {
     return best;
 }
 
-// Whether the grouped launches of a mode's runs take node pairs.
-inline bool group_pairs(int mode, int qt, int flow) { return (mode == MODE_F16 || mode == MODE_BF16) && qt == 5 && flow; }
+// Whether the grouped launches of a batch take node pairs, by the nodes of all
+// its grouped runs, whose launches run side by side: below kGroupPairsMinNodes
+// one warp's chain bounds them, not instruction issue (GB300, us per step of all,
+// one node / pairs, FP16: one run of 25,600 nodes 2.05 / 2.29, two of 17,416 together
+// 2.11 / 3.15, 8 of 284,456 5.44 / 5.96, 3 of 380,495 6.72 / 6.98, 16 of 560,742 10.72 /
+// 9.17, 5 of 580,808 10.21 / 8.74, 30 of 2,683,681 53.9 / 51.1; BF16 within 3 % of these).
+constexpr long long kGroupPairsMinNodes = 7ll << 16;
+
+inline bool group_pairs(int mode, int qt, int flow, long long nodes) {
+    return (mode == MODE_F16 || mode == MODE_BF16) && qt == 5 && flow && nodes >= kGroupPairsMinNodes;
+}
 
 // Blocks of one run in a grouped launch (blocks of 128 threads, one node or one
 // pair each).
@@ -359,15 +368,16 @@ inline long long group_blocks(int nx, int ny, int tile, bool pairs) {
     return (long long)((nx + w - 1) / w) * ((ny + h - 1) / h);
 }
 
-// stream: reads marked evict-first (runs with flow, not in FP64).
+// stream: reads marked evict-first (runs with flow, not in FP64; 16-bit runs of
+// D2Q5 then take pairs, since they are beyond kGroupPairsMinNodes).
 template <int M, int NR, bool EV>
-const void* group_kernel_nr(int qt, int flow, int ph) {
+const void* group_kernel_nr(int qt, int flow, int ph, bool pairs) {
     if constexpr (kSplit<M>)
-        if (group_pairs(M, qt, flow))
+        if (pairs)
             return ph ? (const void*)group_step_pair<M, true, NR, EV> : (const void*)group_step_pair<M, false, NR, EV>;
     const void* fn = nullptr;
     dispatch_step<M>(qt, flow, ph, [&]<int MM, int Q, bool F, bool PH>() {
-        if constexpr (!(kSplit<MM> && Q == 5 && F)) fn = (const void*)group_step<MM, Q, F, PH, NR, (EV && F)>;
+        fn = (const void*)group_step<MM, Q, F, PH, NR, (EV && F && !(kSplit<MM> && Q == 5))>;
         return cudaSuccess;
     });
     return fn;
@@ -375,11 +385,14 @@ const void* group_kernel_nr(int qt, int flow, int ph) {
 
 // few: the build for at most kGroupFew runs.
 template <int M>
-const void* group_kernel(int qt, int flow, int ph, bool few, bool stream) {
+const void* group_kernel(int qt, int flow, int ph, bool few, bool stream, bool pairs) {
     constexpr int all = kGroupRuns<typename ModeTraits<M>::R>;
     if constexpr (M != MODE_F64)
-        if (stream) return few ? group_kernel_nr<M, kGroupFew, true>(qt, flow, ph) : group_kernel_nr<M, all, true>(qt, flow, ph);
-    return few ? group_kernel_nr<M, kGroupFew, false>(qt, flow, ph) : group_kernel_nr<M, all, false>(qt, flow, ph);
+        if (stream)
+            return few ? group_kernel_nr<M, kGroupFew, true>(qt, flow, ph, pairs)
+                       : group_kernel_nr<M, all, true>(qt, flow, ph, pairs);
+    return few ? group_kernel_nr<M, kGroupFew, false>(qt, flow, ph, pairs)
+               : group_kernel_nr<M, all, false>(qt, flow, ph, pairs);
 }
 
 // Launched as a programmatic dependent of the previous step (the kernels wait
@@ -633,7 +646,7 @@ int batch_blocks_per_sm(int qt, int flow, int ph) {
     KW template cudaError_t launch_batch<M>(const StepParams<ModeTraits<M>::R>*, const Tile*, int, int, int, int, int, \
                                          int, int, cudaStream_t);                                               \
     KW template int batch_blocks_per_sm<M>(int, int, int);                                                   \
-    KW template const void* group_kernel<M>(int, int, int, bool, bool);                                                    \
+    KW template const void* group_kernel<M>(int, int, int, bool, bool, bool);                                                  \
     KW template cudaError_t launch_step2<M>(const StepParams<ModeTraits<M>::R>&, int, T2Shape, cudaStream_t); \
     KW template cudaError_t prepare_step2<M>(int, int, T2Shape);                                              \
     KW template const void* group2_kernel<M>(int, int, bool, bool);                                                        \

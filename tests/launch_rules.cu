@@ -32,3 +32,8 @@ extern "C" void rule_step(int mode, int qt, int flow, int bounce, int nx, int ny
     out[2] = (int)L.block.x;
     out[3] = (int)L.block.y;
 }
+
+// Whether grouped launches over `nodes` nodes take node pairs.
+extern "C" int rule_group_pairs(int mode, int qt, int flow, long long nodes) {
+    return lbmk::group_pairs(mode, qt, flow, nodes) ? 1 : 0;
+}

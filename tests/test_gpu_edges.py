@@ -59,3 +59,27 @@ def test_pairs_equal_one_node_per_thread(lbm, shape, prec, eq9):
         assert r.status() == 0
     want = runs[0].save()
     assert np.array_equal(want, runs[1].save()) and np.array_equal(want, runs[2].save())
+
+
+@pytest.mark.parametrize("shapes", [[(401, 333), (300, 290), (512, 200), (333, 300), (65, 900), (129, 64)],
+                                    [(401, 333), (300, 290), (129, 64)]])
+@pytest.mark.parametrize("prec,eq9", [(2, 0), (3, 1)])
+def test_grouped_launches_on_both_sides_of_the_pair_rule(lbm, shapes, prec, eq9):
+    """Map 4 over 558,000 and 235,000 nodes in 16-bit storage (node pairs, one
+    node per thread), a bounce-back run among them: each run equals lbm_step's."""
+    runs, twins = [], []
+    for k, (nx, ny) in enumerate(shapes):
+        p = inputs.cavity(max(nx, ny), ny=ny, precision=prec, L_char=100.0, Ra=1e7, solid_scheme=1 if k == 1 else 0,
+                          **(dict(ks_over_kl=0.7) if eq9 and k else {}))
+        p["nx"] = nx
+        F, G, H, dT = inputs.random_state(nx, ny, 5, seed=k, H_range=(0.0, 1.6), f_base=W9)
+        s = lbm.Solver(p)
+        s.set_state(F - W9[:, None, None], G, H, dT)
+        runs.append(s)
+        twins.append(twin(lbm, s, 1))
+    b = lbm.Batch(runs, autotune=False).configure(128, 4)
+    b.step(67)
+    for s, t in zip(runs, twins):
+        t.step(67)
+        assert s.status() == 0 and np.array_equal(s.save(), t.save())
+    b.close()

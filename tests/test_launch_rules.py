@@ -23,6 +23,7 @@ def rules(tmp_path_factory):
         L.rule_step(prec, qt, flow, bounce, nx, ny, form, *block, o)
         return tuple(o)
 
+    step.lib = L
     return step
 
 
@@ -49,3 +50,13 @@ def test_automatic_single_steps_take_pairs(rules, shape, prec):
         assert not takes_pairs(rules(*shape, prec, form=form, bounce=1), shape[0])
         assert not takes_pairs(rules(*shape, prec, form=form, qt=9), shape[0])
         assert not takes_pairs(rules(*shape, 1, form=form), shape[0])
+
+
+@pytest.mark.parametrize("prec", [2, 3])
+def test_grouped_launches_take_pairs_where_nodes_abound(rules, prec):
+    """Batches whose grouped runs have few nodes together step one node per
+    thread: there one warp's chain is the time, which pairs lengthen."""
+    pairs = lambda nodes, prec=prec, qt=5, flow=1: rules.lib.rule_group_pairs(prec, qt, flow, ctypes.c_longlong(nodes))
+    assert not any(pairs(n) for n in (9, 17416, 114024, 284456, 380495))
+    assert all(pairs(n) for n in (560742, 1 << 20, 1 << 30))
+    assert not pairs(1 << 20, prec=1) and not pairs(1 << 20, qt=9) and not pairs(1 << 20, flow=0)
