@@ -221,8 +221,9 @@ int lbm_step(lbm_handle* h, int64_t nsteps);
  * of at least 786,432 nodes (state beyond L2); node pairs for FP16/BF16 runs
  * of at least 1,572,864 (1536 x 1024) nodes; otherwise one step per launch, one
  * node per thread or, in FP16/BF16 runs of at least 131,072 nodes that could take
- * pairs, those without their prefetch (lbm_step_form_for reports
- * LBM_STEP_FORM_SINGLE for both).
+ * pairs, those without their prefetch wherever they are the faster (by the blocks
+ * of the busiest SM; odd widths mostly from 360,000 nodes).  lbm_step_form_for
+ * reports LBM_STEP_FORM_SINGLE for both.
  * Every form gives the same states bit for bit: all kernels share one node
  * update in which each rounding is fixed.  A run that steps two steps per
  * launch keeps a second exchange-history array (4 bytes per node of row

@@ -186,13 +186,6 @@ inline dim3 step_block(int mode, int nx, int ny) {
 enum : int { FORM_AUTO = 0, FORM_SINGLE = 1, FORM_PAIRS = 2, FORM_TWO_STEPS = 3 };
 constexpr long long kPairMinNodes = 3ll << 19;
 
-// The automatic single step, and the single steps of FORM_TWO_STEPS, take pairs
-// too, without the prefetch, for 16-bit runs from kPairPlainMinNodes nodes, where
-// instruction issue and not one warp's chain bounds the step (GB300, us per step, one node / pairs: FP16 384^2 3.37 / 3.27,
-// 512^2 5.09 / 4.93, 1024^2 17.9 / 16.1, BF16 with Eq. 9 777 x 501 7.80 / 7.62;
-// in FP32 512^2 5.0 / 5.2, 1024^2 26.5 / 26.9).
-constexpr long long kPairPlainMinNodes = 1ll << 17;
-
 // The rule (host code; lbm_step_form_for reports it): the form a run takes,
 // FORM_SINGLE (one step per launch, pairs without the prefetch among them) or
 // FORM_PAIRS.  mode: MODE_*.
@@ -230,12 +223,40 @@ inline bool two_steps_for(int mode, int qt, int flow, long long nodes, int form)
     return nodes <= kTwoStepSmallMaxNodes || (mode == MODE_F32 && nodes >= kTwoStepF32MinNodes);
 }
 
+// The automatic single step, and the single steps of FORM_TWO_STEPS, take pairs
+// without the prefetch too, in 16-bit runs of kPairPlainMinNodes nodes and more
+// where they are the faster form (GB300, us per step, one node / pairs, FP16):
+//   * beyond about one wave of one-node blocks (10 of 128 threads per SM) always:
+//     1000 x 200 4.42 / 3.98, 512^2 5.1 / 4.7, 640^2 7.33 / 6.35, 1217 x 1011 20.3 / 16.3;
+//   * within the wave, where a step takes as long as the busiest SM's blocks one
+//     after another, if those of pairs are half as many or fewer: 600 x 240 (8 and
+//     4) 3.45 / 3.27, 600 x 300 (10 and 5) 3.93 / 3.63, but 512 x 256 (7 and 4) 3.02 /
+//     3.40, 512 x 340 (9 and 5) 3.62 / 3.78, 448 x 300 (7 and 4) 3.02 / 3.28;
+//   * in odd widths the last node is a second chain for its warp of pairs, unless
+//     it has the warp for itself (nx mod 64 = 1: 513 x 300 3.69 / 3.54, 577^2 6.64 /
+//     5.85): from kPairOddMinNodes (333 x 700 5.27 / 5.87, 593 x 411 5.14 / 5.37, 901 x
+//     360 6.22 / 6.27, 1201 x 300 6.63 / 6.35, 777 x 501 7.24 / 7.15, 865 x 801 11.9 / 10.7).
+// In FP32 one node per thread is faster (512^2 4.83 / 5.23).
+constexpr long long kPairPlainMinNodes = 1ll << 17, kPairOddMinNodes = 360000;
+constexpr int kNumSMs = 152;
+
+inline bool plain_pairs(int nx, int ny) {
+    const long long nodes = (long long)nx * ny;
+    if (nodes < kPairPlainMinNodes) return false;
+    if (nx & 1) return nx % 64 == 1 || nodes >= kPairOddMinNodes;
+    const dim3 b = step_block(MODE_F16, nx, ny);
+    auto busiest = [](long long blocks) { return (blocks + kNumSMs - 1) / kNumSMs; };
+    auto blocks = [&](int w, int h) { return (long long)((nx + w - 1) / w) * ((ny + h - 1) / h); };
+    // in blocks of 64 threads, as which those of 128 count twice
+    const long long one = busiest(blocks((int)b.x, (int)b.y)) * (b.x * b.y / 64), pairs = 2 * busiest(blocks(64, 4));
+    return one > 18 || 2 * pairs <= one;
+}
+
 // Whether a run's one-step kernel takes node pairs.
 template <int M>
 inline bool pairs_of(const StepParams<typename ModeTraits<M>::R>& P, int qt, int flow, int form) {
-    const long long nodes = (long long)P.nx * P.ny;
-    if (form_for(M, qt, flow, P.solid_scheme, nodes, form) == FORM_PAIRS) return true;
-    return form != FORM_SINGLE && kSplit<M> && qt == 5 && flow && !P.solid_scheme && nodes >= kPairPlainMinNodes;
+    if (form_for(M, qt, flow, P.solid_scheme, (long long)P.nx * P.ny, form) == FORM_PAIRS) return true;
+    return form != FORM_SINGLE && kSplit<M> && qt == 5 && flow && !P.solid_scheme && plain_pairs(P.nx, P.ny);
 }
 
 // Whether a run's launches mark their reads evict-first (read_state): from
@@ -287,7 +308,7 @@ inline int prefetch_rows_two_steps(int mode, long long nodes) {
 // 3.46 with one lane per node); beyond, two warps of one lattice's FP64
 // operations in turn take longer than one warp of both lattices', which share
 // some.
-constexpr long long kConductionLanesMaxNodes = 152 * 4 * 16;
+constexpr long long kConductionLanesMaxNodes = kNumSMs * 4 * 16;
 
 // The one-step kernel of a run, with its grid: one node per thread in blocks of
 // b threads, or node pairs in blocks of 32 x 4.

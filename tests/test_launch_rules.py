@@ -53,6 +53,21 @@ def test_automatic_single_steps_take_pairs(rules, shape, prec):
 
 
 @pytest.mark.parametrize("prec", [2, 3])
+@pytest.mark.parametrize("shape,pairs", [
+    # within a wave of one-node blocks, by the blocks of the busiest SM
+    ((363, 361), 0), ((512, 256), 0), ((448, 300), 0), ((512, 340), 0), ((514, 256), 0), ((600, 240), 1), ((600, 300), 1),
+    ((1000, 180), 1), ((900, 160), 1),
+    # beyond it
+    ((1000, 200), 1), ((512, 512), 1), ((128, 2000), 1), ((1024, 1024), 1), ((1606, 1000), 1),
+    # odd widths: a second chain in the last node's warp, unless it is alone there
+    ((333, 700), 0), ((593, 411), 0), ((515, 511), 0), ((777, 501), 1), ((1201, 301), 1), ((865, 801), 1),
+    ((513, 300), 1), ((577, 577), 1), ((65, 3000), 1),
+])
+def test_automatic_pairs_where_they_are_the_faster(rules, shape, pairs, prec):
+    assert takes_pairs(rules(*shape, prec), shape[0]) == bool(pairs)
+
+
+@pytest.mark.parametrize("prec", [2, 3])
 def test_grouped_launches_take_pairs_where_nodes_abound(rules, prec):
     """Batches whose grouped runs have few nodes together step one node per
     thread: there one warp's chain is the time, which pairs lengthen."""
