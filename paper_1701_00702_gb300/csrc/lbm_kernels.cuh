@@ -1206,10 +1206,20 @@ __device__ __forceinline__ void step_pair(const StepParams<float>& P, int x0, in
 
 // Blocks of 256 threads each SM must hold, which caps the registers per
 // thread: five for the FP32 and 16-bit forms of D2Q5 with flow (48 registers,
-// where the FP32 step at 2048^2 runs at the copy bandwidth); the others take
-// what their registers allow (FP64 and the D2Q9 forms are bound by arithmetic).
+// where the FP32 step at 2048^2 runs at the copy bandwidth) and four for 16-bit
+// D2Q9 (64: at the 72 it takes uncapped, fewer warps stay resident: 512^2 FP16 7.08 /
+// 6.80 us per step, 2048^2 BF16 101.4 / 98.1, a batch of 60 runs under map 3 48.9 / 45.9);
+// the others take what their registers allow (FP64 and FP32 D2Q9, where four
+// blocks cost single runs 1-4 %, are bound by arithmetic).
 template <int M, int QT, bool FLOW>
-constexpr int kMinBlocks = (QT == 5 && FLOW) ? (M == MODE_F64 ? 1 : 5) : 1;
+constexpr int kMinBlocks = !FLOW || M == MODE_F64 ? 1 : QT == 5 ? 5 : kSplit<M> ? 4 : 1;
+
+// The same of grouped launches' blocks of 128 threads: the D2Q9 forms, whose many
+// runs fill the device, at 64 registers (60 runs under map 4, us per step of all,
+// uncapped, FP32 73 and 16-bit 96 registers / 64: FP32 58.0 / 55.3, FP16 55.8 / 47.1,
+// BF16 56.4 / 47.1; 12 runs FP32 10.8 / 9.9, FP16 10.9 / 9.2).
+template <int M, int QT, bool FLOW>
+constexpr int kGroupBlocks = QT == 9 && FLOW && M != MODE_F64 ? 8 : 2 * kMinBlocks<M, QT, FLOW>;
 
 // Programmatic dependent launch (sm_90 and later): the step kernels are
 // launched as programmatic dependents of the previous step, so their launch
@@ -1533,7 +1543,7 @@ __device__ __forceinline__ int group_run(const GroupParams<R, NR>& G, int b) {
 }
 
 template <int M, int QT, bool FLOW, bool PH, int NR, bool EV>
-__global__ void __launch_bounds__(128, 2 * kMinBlocks<M, QT, FLOW>) group_step(
+__global__ void __launch_bounds__(128, (kGroupBlocks<M, QT, FLOW>)) group_step(
     const __grid_constant__ GroupParams<typename ModeTraits<M>::R, NR> G) {
     const int b = blockIdx.x, lo = group_run(G, b);
     const StepParams<typename ModeTraits<M>::R>& P = G.run[lo];

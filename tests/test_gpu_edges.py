@@ -83,3 +83,26 @@ def test_grouped_launches_on_both_sides_of_the_pair_rule(lbm, shapes, prec, eq9)
         t.step(67)
         assert s.status() == 0 and np.array_equal(s.save(), t.save())
     b.close()
+
+
+@pytest.mark.parametrize("prec,mapping", [(1, 3), (1, 4), (2, 3), (2, 4), (3, 4)])
+def test_d2q9_batches_equal_their_runs(lbm, prec, mapping):
+    """The register-capped D2Q9 kernels of single runs and of grouped launches,
+    runs with Eq. 9 and with constant properties together: each equals lbm_step's."""
+    runs, twins = [], []
+    for k in range(10):
+        nx, ny = 17 + 13 * k, 70 - 6 * k
+        p = inputs.cavity(max(nx, ny), ny=ny, precision=prec, thermal_q=9, L_char=100.0, Ra=1e7,
+                          **(dict(ks_over_kl=0.7, cps_over_cpl=0.9) if k % 3 == 0 else {}))
+        p["nx"] = nx
+        F, G, H, dT = inputs.random_state(nx, ny, 9, seed=k, H_range=(0.0, 1.6), f_base=W9)
+        s = lbm.Solver(p)
+        s.set_state(F - W9[:, None, None], G, H, dT)
+        runs.append(s)
+        twins.append(twin(lbm, s, 1))
+    b = lbm.Batch(runs, autotune=False).configure(128, mapping)
+    b.step(67)
+    for s, t in zip(runs, twins):
+        t.step(67)
+        assert s.status() == 0 and np.array_equal(s.save(), t.save())
+    b.close()
