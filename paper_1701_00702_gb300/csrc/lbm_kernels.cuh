@@ -862,11 +862,12 @@ __device__ __forceinline__ void apply_wall(const StepParams<typename ModeTraits<
 }
 
 // State of a node (pair) from its pulled neighbourhood a (pulled at x_f on
-// walls, then Eq. 52 in moment space).
-template <int M, int QT, bool FLOW, typename T, typename A>
+// walls, then Eq. 52 in moment space).  LATE: the thermal lattices are pulled
+// first.
+template <int M, int QT, bool FLOW, typename T, bool LATE = kComp<M>, typename A>
 __device__ __forceinline__ void node_state(const StepParams<typename ModeTraits<M>::R>& P, const A& a,
                                            const WallAt<T>& w, NodeState<M, QT, FLOW, T>& n) {
-    if constexpr (kComp<M>) {
+    if constexpr (LATE) {
         pull_thermal<M, QT, FLOW, T>(P, a, n);
         pull_flow<M, QT, FLOW, T>(a, n);
     } else {
@@ -1165,18 +1166,18 @@ __device__ __forceinline__ float* next_wide(const StepParams<typename ModeTraits
 // P.phase_k is set); PH = false leaves them out of the kernel altogether.
 // The history is read before any store: the compiler cannot move it above
 // stores that may alias it, and a load after them adds a memory round trip to
-// the step; in FP32, one node per thread, it is read after the state is known,
+// the step; LATE (FP32, one node per thread), it is read after the state is known,
 // and the thermal lattices are pulled first (one step per launch 330^2 3.17 ->
 // 2.98 us, 512^2 4.98 -> 4.84, 1024^2 27.3 -> 26.4).  TF: the thermal lattices
 // collide before the flow.  Returns the new history.
-template <int M, int QT, bool FLOW, bool PH, int PS, typename T, bool TF = false, typename A>
+template <int M, int QT, bool FLOW, bool PH, int PS, typename T, bool TF = false, bool LATE = kComp<M>, typename A>
 __device__ __forceinline__ T advance(const StepParams<typename ModeTraits<M>::R>& P, const A& a, const WallAt<T>& w,
                                      const typename Lane<T>::R* history, typename ModeTraits<M>::B* db, float* dw) {
     NodeState<M, QT, FLOW, T> n;
     T dTp;
-    if constexpr (Lane<T>::n == 1 && !kComp<M>) dTp = get_real<T>(history);
-    node_state<M, QT, FLOW, T>(P, a, w, n);
-    if constexpr (Lane<T>::n == 1 && kComp<M>) dTp = get_real<T>(history);
+    if constexpr (Lane<T>::n == 1 && !LATE) dTp = get_real<T>(history);
+    node_state<M, QT, FLOW, T, LATE>(P, a, w, n);
+    if constexpr (Lane<T>::n == 1 && LATE) dTp = get_real<T>(history);
     if constexpr (!TF) flow_collide<M, QT, FLOW, PS, T>(P, n, db);
     if constexpr (Lane<T>::n == 2) dTp = get_real<T>(history);
     const T dTn = thermal_collide<M, QT, FLOW, PH, PS, T>(P, n, dTp, db, dw);
@@ -1186,12 +1187,12 @@ __device__ __forceinline__ T advance(const StepParams<typename ModeTraits<M>::R>
 }
 
 // One time step of node (x, y) from the state copy to the next.
-template <int M, int QT, bool FLOW, bool PH = false, bool EV = false>
+template <int M, int QT, bool FLOW, bool PH = false, bool EV = false, bool TF = false, bool LATE = kComp<M>>
 __device__ __forceinline__ void step_node(const StepParams<typename ModeTraits<M>::R>& P, int x, int y) {
     using T = Node1<M>;
     const WallAt<T> w(P, x, y);
     T* h = P.dT + (y * P.pitch + x);
-    *h = advance<M, QT, FLOW, PH, kChunk, T>(P, PullAt<M, QT, FLOW, EV>(P, w.xs, w.ys), w, h,
+    *h = advance<M, QT, FLOW, PH, kChunk, T, TF, LATE>(P, PullAt<M, QT, FLOW, EV>(P, w.xs, w.ys), w, h,
                                               next_bulk<M, QT, FLOW>(P, x, y), next_wide<M, QT, FLOW>(P, x, y));
 }
 
@@ -1606,8 +1607,13 @@ struct Tile {
     int run, x0, y0, log2w_flip;   // log2 w in bits 0-7, flip in bit 8
 };
 
+// The order of a node's reads and collisions and the register bound are what
+// measured best with the parameters in shared memory (us per step of all, FP32
+// D2Q5 with LATE / without: 12 runs under map 0 10.0 / 9.8, 60 runs 55.6 / 55.0;
+// FP16 D2Q5 flow / thermal lattices first: 12 runs 11.3 / 11.1, 60 runs 51.8 / 50.2; FP32
+// D2Q9 unbounded / with three blocks per SM: 12 runs 15.7 / 15.2, 60 runs 76.2 / 72.5).
 template <int M, int QT, bool FLOW, bool PH>
-__global__ void __launch_bounds__(256) batch_step(const StepParams<typename ModeTraits<M>::R>* __restrict__ runs,
+__global__ void __launch_bounds__(256, (M == MODE_F32 && QT == 9 && FLOW ? 3 : 0)) batch_step(const StepParams<typename ModeTraits<M>::R>* __restrict__ runs,
                                                   const Tile* __restrict__ tiles, int ntiles, int chunk, int parity) {
     using R = typename ModeTraits<M>::R;
     __shared__ StepParams<R> P;
@@ -1630,7 +1636,8 @@ __global__ void __launch_bounds__(256) batch_step(const StepParams<typename Mode
         const int lg = tl.log2w_flip & 0xff;
         const int x = tl.x0 + (threadIdx.x & ((1 << lg) - 1));
         const int y = tl.y0 + (threadIdx.x >> lg);
-        if (x < P.nx && y < P.ny) step_node<M, QT, FLOW, PH>(P, x, y);
+        if (x < P.nx && y < P.ny)
+            step_node<M, QT, FLOW, PH, false, M == MODE_F16 && QT == 5, kComp<M> && QT == 9>(P, x, y);
     }
 }
 

@@ -106,3 +106,30 @@ def test_d2q9_batches_equal_their_runs(lbm, prec, mapping):
         t.step(67)
         assert s.status() == 0 and np.array_equal(s.save(), t.save())
     b.close()
+
+
+@pytest.mark.parametrize("mapping", [0, 1, 2])
+@pytest.mark.parametrize("prec,qt,flow", [(0, 5, 1), (0, 9, 1), (1, 5, 1), (1, 9, 1), (2, 5, 1), (2, 9, 1), (3, 5, 1), (3, 9, 1),
+                                          (0, 5, 0), (1, 5, 0), (2, 9, 0)])
+def test_tile_lists_equal_their_runs(lbm, prec, qt, flow, mapping):
+    """Maps 0 to 2 in every storage type, lattice and with flow or without, runs
+    with Eq. 9 and with constant properties together (the kernel with per-node
+    rates serves both): each equals lbm_step's bit for bit."""
+    runs, twins = [], []
+    for k in range(7):
+        nx, ny = 9 + 21 * k, 60 - 7 * k
+        over = dict(ks_over_kl=0.7, cps_over_cpl=0.9) if k % 2 else {}
+        p = inputs.cavity(max(nx, ny), ny=ny, precision=prec, thermal_q=qt, L_char=100.0, Ra=1e7, flow=flow,
+                          periodic_y=int(k == 2), **over)
+        p["nx"] = nx
+        F, G, H, dT = inputs.random_state(nx, ny, qt, seed=k, H_range=(0.0, 1.6), f_base=W9)
+        s = lbm.Solver(p)
+        s.set_state(F - W9[:, None, None] if flow else None, G, H, dT)
+        runs.append(s)
+        twins.append(twin(lbm, s, 1))
+    b = lbm.Batch(runs, autotune=False).configure(64, mapping)
+    b.step(69)
+    for s, t in zip(runs, twins):
+        t.step(69)
+        assert s.status() == 0 and np.array_equal(s.save(), t.save())
+    b.close()
