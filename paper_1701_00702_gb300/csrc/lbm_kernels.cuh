@@ -227,7 +227,9 @@ __device__ __forceinline__ W vsqrt_pos(W a) { return {vsqrt_pos(a.x), vsqrt_pos(
 // 3 e^2/8 + ...) (Householder, The Numerical Treatment of a Single Nonlinear
 // Equation, 1970); the neglected e^3 is below 2^-60.  3 and 5 FP64 operations
 // for the 9 and 10 of the library's correctly rounded ones, within 1 ulp.
-// sqrt gives 0 below 2^-900 (speeds below 1e-135 lattice units).
+// sqrt takes a >= 0, gives 0 below 2^-900 (speeds below 1e-135 lattice units) and
+// leaves infinity and NaN what they are; 1/a is for normal numbers below 2^1022
+// (zero and infinity give NaN, which the state's check reports).
 __device__ __forceinline__ double vrcp(double a) {
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
@@ -239,7 +241,9 @@ __device__ __forceinline__ double vsqrt(double a) {
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
     const double s = vmul(a, y), e = vfma(-s, y, 1.0);
     const double r = vfma(s, vmul(e, vfma(0.375, e, 0.5)), s);
-    return __double2hiint(a) < (1023 - 900) << 20 ? 0.0 : r;   // (a >= 0; NaN and infinity pass)
+    // by the unsigned high word, as which a NaN of either sign is large; infinity's seed is zero
+    const unsigned hi = __double2hiint(a);
+    return hi < (1023u - 900u) << 20 ? 0.0 : hi == 0x7ff00000u ? a : r;
 }
 __device__ __forceinline__ double vsqrt_pos(double a) { return vsqrt(a); }
 
