@@ -198,10 +198,9 @@ __device__ __forceinline__ W vminc(W a, float c) { return {fminf(a.x, c), fminf(
 __device__ __forceinline__ float vmax0(float a) { return fmaxf(a, 0.0f); }
 __device__ __forceinline__ W vmax0(W a) { return {fmaxf(a.x, 0.0f), fmaxf(a.y, 0.0f)}; }
 
-// 1/a and sqrt(a), a >= 0, in FP32: one instruction each (the division and the
-// guarded rsqrtf product they replace took 5 and 8; subnormal speeds, below
-// 1e-19 lattice units, flush to zero).  vsqrt_pos, a > 0, is the rsqrt product
-// without the guard.
+// 1/a (within 1 ulp) and sqrt(a), a >= 0 (within 2^-23), in FP32: one instruction
+// each; subnormal speeds, below 1e-19 lattice units, flush to zero.  vsqrt_pos,
+// a > 0, is a times 1/sqrt(a) (within 2^-22.4).
 __device__ __forceinline__ float vrcp(float a) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
@@ -221,12 +220,15 @@ __device__ __forceinline__ W vrcp(W a) { return {vrcp(a.x), vrcp(a.y)}; }
 __device__ __forceinline__ W vsqrt(W a) { return {vsqrt(a.x), vsqrt(a.y)}; }
 __device__ __forceinline__ W vsqrt_pos(W a) { return {vsqrt_pos(a.x), vsqrt_pos(a.y)}; }
 // In FP64, where one warp instruction occupies its scheduler's FP64 unit for 64
-// cycles (GB300: two FP64 lanes per SM and clock), from the hardware's seed y
-// (relative error below 2^-20) with one third-order step each: with e = 1 - a y,
-// 1/a = y (1 + e + e^2 + ...), and with e = 1 - a y^2, sqrt(a) = a y (1 + e/2 +
-// 3 e^2/8 + ...) (Householder, The Numerical Treatment of a Single Nonlinear
-// Equation, 1970); the neglected e^3 is below 2^-60.  3 and 5 FP64 operations
-// for the 9 and 10 of the library's correctly rounded ones, within 1 ulp.
+// cycles (GB300: two FP64 lanes per SM and clock), 3 and 5 FP64 operations from
+// the hardware's seed y (relative error below 2^-20).  1/a by one third-order step
+// (Householder, The Numerical Treatment of a Single Nonlinear Equation, 1970):
+// with e = 1 - a y, 1/a = y (1 + e + e^2 + ...), the neglected e^3 below 2^-60.
+// sqrt(a) by two steps of Newton's method for s^2 = a from s = a y, with y / 2 for
+// the 1 / (2 s) of both: the first leaves 3/2 2^-40, the second takes a - s^2 in one
+// rounding and leaves less than 2^-59.  Both are so within 0.5 + 2^-6 ulp of the
+// exact value (a third-order step for the root, as many operations, keeps half
+// the rounding of a y: 0.75 ulp).
 // sqrt takes a >= 0, gives 0 below 2^-900 (speeds below 1e-135 lattice units) and
 // leaves infinity and NaN what they are; 1/a is for normal numbers below 2^1022
 // (zero and infinity give NaN, which the state's check reports).
@@ -239,8 +241,10 @@ __device__ __forceinline__ double vrcp(double a) {
 __device__ __forceinline__ double vsqrt(double a) {
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-    const double s = vmul(a, y), e = vfma(-s, y, 1.0);
-    const double r = vfma(s, vmul(e, vfma(0.375, e, 0.5)), s);
+    const double h = __hiloint2double(__double2hiint(y) - (1 << 20), __double2loint(y));   // y / 2
+    const double s0 = vmul(a, y);
+    const double s = vfma(s0, vfma(-s0, h, 0.5), s0);
+    const double r = vfma(vfma(-s, s, a), h, s);
     // by the unsigned high word, as which a NaN of either sign is large; infinity's seed is zero
     const unsigned hi = __double2hiint(a);
     return hi < (1023u - 900u) << 20 ? 0.0 : hi == 0x7ff00000u ? a : r;
