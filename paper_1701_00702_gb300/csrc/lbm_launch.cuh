@@ -320,6 +320,7 @@ struct StepLaunch {
 template <int M>
 StepLaunch step_launch(const StepParams<typename ModeTraits<M>::R>& P, int qt, int flow, int form, dim3 b,
                        bool stream = false) {
+    while (P.ny > 65535ll * b.y) b = dim3(b.x / 2, b.y * 2);   // (65,536 rows are admitted, 65,535 blocks along y)
     StepLaunch L{nullptr, dim3(), b};
     if constexpr (M != MODE_F64) {
         if (pairs_of<M>(P, qt, flow, form)) {

@@ -133,3 +133,23 @@ def test_tile_lists_equal_their_runs(lbm, prec, qt, flow, mapping):
         t.step(69)
         assert s.status() == 0 and np.array_equal(s.save(), t.save())
     b.close()
+
+
+@pytest.mark.parametrize("prec,flow", [(0, 1), (0, 0), (1, 1), (2, 1)])
+def test_the_tallest_grid_steps(lbm, prec, flow):
+    """65,536 rows, one more than a grid has blocks along y: single steps, graph
+    replays and map 3 with one-row blocks equal the tile list."""
+    p = inputs.cavity(100, precision=prec, flow=flow, L_char=100.0)
+    p["nx"], p["ny"] = 3, 65536
+    runs = [lbm.Solver(p) for _ in range(3)]
+    lists = lbm.Batch([runs[1]], autotune=False).configure(128, 0)
+    chain = lbm.Batch([runs[2]], autotune=False).configure(128, 3).set_block(0, 256, 1)
+    runs[0].step(67)
+    lists.step(67)
+    chain.step(67)
+    want = runs[0].save()
+    assert all(r.status() == 0 for r in runs)
+    assert all(np.array_equal(want, r.save()) for r in runs[1:])
+    d = runs[0].diag()
+    assert np.isfinite([d["melt_frac"], d["enthalpy"], d["mass"], d["nu_hot"]]).all()
+    lists.close(), chain.close()

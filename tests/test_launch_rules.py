@@ -75,3 +75,20 @@ def test_grouped_launches_take_pairs_where_nodes_abound(rules, prec):
     assert not any(pairs(n) for n in (9, 17416, 114024, 284456, 380495))
     assert all(pairs(n) for n in (560742, 1 << 20, 1 << 30))
     assert not pairs(1 << 20, prec=1) and not pairs(1 << 20, qt=9) and not pairs(1 << 20, flow=0)
+
+
+SHAPES = [(0, 0), (128, 2), (64, 4), (32, 8), (256, 1), (128, 1), (64, 2), (32, 4), (64, 1), (32, 2)]
+
+
+@pytest.mark.parametrize("prec", [0, 1, 2, 3])
+@pytest.mark.parametrize("nx,ny", [(3, 65536), (128, 65536), (1000, 65536), (128, 65535), (65536, 3)])
+def test_grids_stay_within_the_launch_limits(rules, nx, ny, prec):
+    """65,536 rows are admitted, 65,535 blocks along y: the run's own block shape
+    and every shape a batch may choose cover the grid within the limit."""
+    for qt, flow in ((5, 1), (5, 0), (9, 1)):
+        for form in (0, 1, 2):
+            for block in SHAPES:
+                launch = rules(nx, ny, prec, form=form, qt=qt, flow=flow, block=block)
+                gx, gy, bx, by = launch
+                assert gy <= 65535 and gy * by >= ny and bx * by <= 256
+                assert gx * bx * (2 if takes_pairs(launch, nx) else 1) >= nx
