@@ -373,8 +373,12 @@ int lbm_batch_configure(lbm_batch* b, int32_t width_cap, int32_t mapping);
 int lbm_batch_info(const lbm_batch* b, int32_t* n_tiles, int32_t* width_cap, int32_t* mapping, int32_t* grid,
                    double* tuned_us_per_step);
 /* Block shape of run `run` under map 3: one of the shapes listed above
- * (LBM_ERR_ARG otherwise).  The shape changes no result.  set synchronises
- * the batch's stream. */
+ * (LBM_ERR_ARG otherwise).  A run whose shape was set, or tuned, steps one node
+ * per thread in it (in half the width and twice the rows where the grid has more
+ * than 65,535 blocks along y), but for one whose form is LBM_STEP_FORM_PAIRS or
+ * which takes that form by its size; until then the run keeps lbm_step's own
+ * kernel, and get gives the shape of its one-node blocks.  The shape changes no
+ * result.  set synchronises the batch's stream. */
 int lbm_batch_set_block(lbm_batch* b, int32_t run, int32_t block_x, int32_t block_y);
 int lbm_batch_get_block(const lbm_batch* b, int32_t run, int32_t* block_x, int32_t* block_y);
 int lbm_batch_destroy(lbm_batch* b);

@@ -999,6 +999,7 @@ struct lbm_batch {
     std::vector<int> flip;        // run's current copy relative to the batch parity
     std::vector<int> form;        // each run's step form when the parameters were uploaded
     std::vector<int> shape;       // map 3: block shape of each run (index into kShapes)
+    std::vector<char> shaped;     // map 3: the shape was set or tuned, so the run steps one node per thread in it
     std::vector<std::vector<int>> groups;   // maps 4, 5: the runs of each grouped launch in graphs
     std::vector<std::vector<int>> inline_groups;   // the same outside graphs
     std::vector<GroupArgs> launches[4];     // their launches outside graphs, filled on first use: one step from parity 0 or 1, two steps there or back
@@ -1233,12 +1234,13 @@ cudaError_t add_run_chains(lbm_batch* b, cudaGraph_t g, const std::vector<int>& 
                 args[0] = &Pf;
             }
             const dim3 blk((unsigned)kShapes[b->shape[r]][0], (unsigned)kShapes[b->shape[r]][1], 1u);
+            const bool own = b->shaped[r] != 0;
             lbmk::StepLaunch L;
             switch (b->precision) {   // the kernel and grid lbm_step would launch for this run
-                case LBM_F64: L = lbmk::step_launch<lbmk::MODE_F64>(Pd, b->qt, b->flow, h->form, blk); break;
-                case LBM_F32: L = lbmk::step_launch<lbmk::MODE_F32>(Pf, b->qt, b->flow, h->form, blk); break;
-                case LBM_F16: L = lbmk::step_launch<lbmk::MODE_F16>(Pf, b->qt, b->flow, h->form, blk); break;
-                default: L = lbmk::step_launch<lbmk::MODE_BF16>(Pf, b->qt, b->flow, h->form, blk); break;
+                case LBM_F64: L = lbmk::step_launch<lbmk::MODE_F64>(Pd, b->qt, b->flow, h->form, blk, false, own); break;
+                case LBM_F32: L = lbmk::step_launch<lbmk::MODE_F32>(Pf, b->qt, b->flow, h->form, blk, false, own); break;
+                case LBM_F16: L = lbmk::step_launch<lbmk::MODE_F16>(Pf, b->qt, b->flow, h->form, blk, false, own); break;
+                default: L = lbmk::step_launch<lbmk::MODE_BF16>(Pf, b->qt, b->flow, h->form, blk, false, own); break;
             }
             cudaKernelNodeParams kp = {};
             kp.func = const_cast<void*>(L.fn);
@@ -1635,6 +1637,7 @@ int lbm_batch_create(lbm_handle* const* runs, int32_t n_runs, int32_t autotune, 
             if (kShapes[k][0] == (int)sb.x && kShapes[k][1] == (int)sb.y) id = k;
         b->shape.push_back(id);
     }
+    b->shaped.assign(n_runs, 0);
     b->params_stride = b->precision == LBM_F64 ? sizeof(lbmk::StepParams<double>) : sizeof(lbmk::StepParams<float>);
     for (lbm_handle* h : b->runs)
         if (cudaStreamSynchronize(h->stream) != cudaSuccess) {
@@ -1692,14 +1695,17 @@ int lbm_batch_create(lbm_handle* const* runs, int32_t n_runs, int32_t autotune, 
                     for (int r : members) start.push_back(b->shape[r]);
                     int chosen = -1;
                     for (int sh = 0; sh < kNumShapes; ++sh) {
-                        for (int r : members) b->shape[r] = sh;
+                        for (int r : members) b->shape[r] = sh, b->shaped[r] = 1;
                         const double us = time_batch(b, 16);
                         if (us < t3) {
                             t3 = us;
                             chosen = sh;
                         }
                     }
-                    for (size_t i = 0; i < members.size(); ++i) b->shape[members[i]] = chosen >= 0 ? chosen : start[i];
+                    for (size_t i = 0; i < members.size(); ++i) {
+                        b->shape[members[i]] = chosen >= 0 ? chosen : start[i];
+                        b->shaped[members[i]] = chosen >= 0;
+                    }
                 }
                 if (t3 < best) {
                     best = t3;
@@ -1814,6 +1820,7 @@ int lbm_batch_set_block(lbm_batch* b, int32_t run, int32_t block_x, int32_t bloc
     }
     batch_destroy_graph(b);
     b->shape[run] = id;
+    b->shaped[run] = 1;
     return LBM_OK;
 }
 

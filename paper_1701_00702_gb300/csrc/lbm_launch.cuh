@@ -252,11 +252,11 @@ inline bool plain_pairs(int nx, int ny) {
     return one > 18 || 2 * pairs <= one;
 }
 
-// Whether a run's one-step kernel takes node pairs.
+// Whether a run's one-step kernel takes node pairs (chosen: see step_launch).
 template <int M>
-inline bool pairs_of(const StepParams<typename ModeTraits<M>::R>& P, int qt, int flow, int form) {
+inline bool pairs_of(const StepParams<typename ModeTraits<M>::R>& P, int qt, int flow, int form, bool chosen) {
     if (form_for(M, qt, flow, P.solid_scheme, (long long)P.nx * P.ny, form) == FORM_PAIRS) return true;
-    return form != FORM_SINGLE && kSplit<M> && qt == 5 && flow && !P.solid_scheme && plain_pairs(P.nx, P.ny);
+    return form != FORM_SINGLE && !chosen && kSplit<M> && qt == 5 && flow && !P.solid_scheme && plain_pairs(P.nx, P.ny);
 }
 
 // Whether a run's launches mark their reads evict-first (read_state): from
@@ -311,7 +311,9 @@ inline int prefetch_rows_two_steps(int mode, long long nodes) {
 constexpr long long kConductionLanesMaxNodes = kNumSMs * 4 * 16;
 
 // The one-step kernel of a run, with its grid: one node per thread in blocks of
-// b threads, or node pairs in blocks of 32 x 4.
+// b threads, node pairs in blocks of 32 x 4, or two lanes per node.  chosen: b is
+// the caller's choice for this run, which then steps one node per thread unless
+// its form is FORM_PAIRS.
 struct StepLaunch {
     const void* fn;
     dim3 grid, block;
@@ -319,11 +321,11 @@ struct StepLaunch {
 
 template <int M>
 StepLaunch step_launch(const StepParams<typename ModeTraits<M>::R>& P, int qt, int flow, int form, dim3 b,
-                       bool stream = false) {
+                       bool stream = false, bool chosen = false) {
     while (P.ny > 65535ll * b.y) b = dim3(b.x / 2, b.y * 2);   // (65,536 rows are admitted, 65,535 blocks along y)
     StepLaunch L{nullptr, dim3(), b};
     if constexpr (M != MODE_F64) {
-        if (pairs_of<M>(P, qt, flow, form)) {
+        if (pairs_of<M>(P, qt, flow, form, chosen)) {
             if (stream) L.fn = P.phase_k ? (const void*)fused_step_pair<M, true, true> : (const void*)fused_step_pair<M, false, true>;
             else L.fn = P.phase_k ? (const void*)fused_step_pair<M, true> : (const void*)fused_step_pair<M, false>;
             L.block = dim3(32, 4);   // 2048^2 FP16 61.25 us per step (64 x 2: 61.98)
@@ -332,7 +334,7 @@ StepLaunch step_launch(const StepParams<typename ModeTraits<M>::R>& P, int qt, i
         }
     }
     if constexpr (M == MODE_F64) {
-        if (qt == 5 && !flow && !P.phase_k && (long long)P.nx * P.ny <= kConductionLanesMaxNodes) {
+        if (!chosen && qt == 5 && !flow && !P.phase_k && (long long)P.nx * P.ny <= kConductionLanesMaxNodes) {
             L.fn = (const void*)conduction_step_lanes<M>;
             L.block = dim3(64, 1);
             L.grid = dim3((unsigned)((P.nx + 31) / 32), (unsigned)P.ny, 1u);
@@ -673,7 +675,7 @@ int batch_blocks_per_sm(int qt, int flow, int ph) {
     KW template cudaError_t prepare_step2<M>(int, int, T2Shape);                                              \
     KW template const void* group2_kernel<M>(int, int, bool, bool);                                                        \
     KW template size_t step2_smem<M>(int, int);                                                               \
-    KW template StepLaunch step_launch<M>(const StepParams<ModeTraits<M>::R>&, int, int, int, dim3, bool);
+    KW template StepLaunch step_launch<M>(const StepParams<ModeTraits<M>::R>&, int, int, int, dim3, bool, bool);
 
 #define LBMK_CONVERT_TEMPLATES(KW, M)                                                                         \
     KW template cudaError_t launch_convert<M>(const StepParams<ModeTraits<M>::R>&, const DenseState<ModeTraits<M>::R>&, \

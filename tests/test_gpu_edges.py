@@ -153,3 +153,21 @@ def test_the_tallest_grid_steps(lbm, prec, flow):
     d = runs[0].diag()
     assert np.isfinite([d["melt_frac"], d["enthalpy"], d["mass"], d["nu_hot"]]).all()
     lists.close(), chain.close()
+
+
+@pytest.mark.parametrize("nx,ny,prec,flow", [(577, 300, 2, 1), (200, 4, 0, 0)])
+def test_block_shapes_of_runs_with_a_kernel_of_their_own(lbm, nx, ny, prec, flow):
+    """Map 3 with a shape set for a run that otherwise takes node pairs or two
+    lanes per node, the graph's steps and those outside it, against lbm_step."""
+    p = inputs.cavity(max(nx, ny), ny=ny, precision=prec, flow=flow, L_char=100.0, periodic_y=1 - flow)
+    p["nx"] = nx
+    s = lbm.Solver(p)
+    for block in ((32, 8), (256, 1), (32, 2)):
+        r = twin(lbm, s)
+        b = lbm.Batch([r], autotune=False).configure(128, 3).set_block(0, *block)
+        assert b.blocks() == [block]
+        t = twin(lbm, s)
+        b.step(131)
+        t.step(131)
+        assert np.array_equal(r.save(), t.save())
+        b.close()

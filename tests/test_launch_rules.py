@@ -92,3 +92,15 @@ def test_grids_stay_within_the_launch_limits(rules, nx, ny, prec):
                 gx, gy, bx, by = launch
                 assert gy <= 65535 and gy * by >= ny and bx * by <= 256
                 assert gx * bx * (2 if takes_pairs(launch, nx) else 1) >= nx
+
+
+@pytest.mark.parametrize("block", SHAPES[1:])
+def test_a_chosen_block_shape_is_the_one_launched(rules, block):
+    """One node per thread in the chosen shape, also in runs whose own kernel
+    would be node pairs or two lanes per node; pairs by form or size stay."""
+    bx, by = block
+    for nx, ny, prec, form, flow in ((512, 512, 2, 0, 1), (1024, 1000, 3, 0, 1), (600, 600, 2, 1, 1), (256, 256, 1, 0, 1),
+                                     (200, 4, 0, 0, 0), (700, 700, 0, 0, 1)):
+        assert rules(nx, ny, prec, form=form, flow=flow, block=block) == (-(-nx // bx), -(-ny // by), bx, by)
+    for nx, ny, form in ((2048, 2048, 0), (256, 256, 2)):
+        assert takes_pairs(rules(nx, ny, 2, form=form, block=block), nx)
