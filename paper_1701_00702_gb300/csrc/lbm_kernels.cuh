@@ -129,8 +129,9 @@ struct Chunk {
 // operation is one packed instruction for both nodes (the .f32x2 add, multiply
 // and fused multiply-add of sm_100 and later), which halves the issue slots of
 // the arithmetic; scalar constants broadcast, negations and lane swaps cost
-// nothing in packed operands.  Every operation names its rounding, so no
-// multiply and add are contracted by the compiler, and a node's result is the
+// nothing in packed operands.  Every operation names its rounding, and a product
+// whose sum with something is a rounding of its own is taken with vmul_alone,
+// since a packed one would be contracted all the same; so a node's result is the
 // same bit for bit in every kernel and lane type.
 template <typename R>
 struct alignas(2 * sizeof(R)) V2 {
@@ -172,11 +173,14 @@ __device__ __forceinline__ W vmul(W a, W b) {
     const float2 r = __fmul2_rn(f2(a), f2(b));
     return {r.x, r.y};
 }
-// A product that goes into an error-free sum: ptxas 13.0 fuses a packed
-// multiply with the addition of its product although both name their rounding
-// (-fmad=false does not stop it), and the error taken would be another
-// number's.  One scalar multiply per lane is left alone.
+// A product that is then added or subtracted (not an fma's addend, and not one by
+// a power of two, which is exact): ptxas 13.0 may fuse a packed multiply with the
+// addition of its product although both name their rounding (-fmad=false does not
+// stop it), and the pair's sum would be rounded once where a single node's is
+// rounded twice; in an error-free sum the error taken would be another number's.
+// One scalar multiply per lane is left alone.
 __device__ __forceinline__ float vmul_alone(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double vmul_alone(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ W vmul_alone(W a, W b) { return {__fmul_rn(a.x, b.x), __fmul_rn(a.y, b.y)}; }
 __device__ __forceinline__ float vneg(float a) { return -a; }
 __device__ __forceinline__ double vneg(double a) { return -a; }
@@ -814,13 +818,13 @@ __device__ __forceinline__ void apply_wall(const StepParams<typename ModeTraits<
     const T ux = vsel(w.wall, n.ux, zero), uy = vsel(w.wall, n.uy, zero);
     if constexpr (FLOW) {
         constexpr R sc = R(kFlowScale<M>);
-        T jx = vmul(n.rho, ux), jy = vmul(n.rho, uy);
+        T jx = vmul_alone(n.rho, ux), jy = vmul_alone(n.rho, uy);
         if constexpr (kFlowScale<M> != 1) {
             jx = vmulc<T>(sc, jx);
             jy = vmulc<T>(sc, jy);
         }
         const T a = vmul(jx, ux);
-        const T q = vmulc<T>(vmul(R(3), P.inv_phi), vfma(jy, uy, a));
+        const T q = vmul_alone(bc<T>(vmul(R(3), P.inv_phi)), vfma(jy, uy, a));
         n.mp[1] = vsub(n.mp[1], q);
         n.mp[2] = vadd(n.mp[2], q);
         n.mp[3] = vsub(n.mp[3], jx);

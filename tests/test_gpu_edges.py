@@ -171,3 +171,25 @@ def test_block_shapes_of_runs_with_a_kernel_of_their_own(lbm, nx, ny, prec, flow
         t.step(131)
         assert np.array_equal(r.save(), t.save())
         b.close()
+
+
+@pytest.mark.parametrize("kinds", [(0, 0, 1, 1), (1, 1, 0, 0)])
+@pytest.mark.parametrize("shape", [(3, 3), (4, 5), (34, 21), (130, 8)])
+@pytest.mark.parametrize("prec", [1, 2, 3])
+@pytest.mark.parametrize("eq9", [0, 1])
+def test_pairs_on_walls_round_as_single_nodes(lbm, shape, kinds, prec, eq9):
+    """Fast flow next to walls, where the wall rule subtracts products: node pairs
+    and two steps per launch against one node per thread, bit for bit."""
+    nx, ny = shape
+    p = inputs.cavity(max(nx, ny), ny=ny, precision=prec, L_char=100.0, Ra=1e7, wall_kind=list(kinds), porosity=0.85,
+                      wall_T=[1.0, 0.0, 0.9, 0.1], **(dict(ks_over_kl=0.7, cps_over_cpl=0.9) if eq9 else {}))
+    p["nx"] = nx
+    F, G, H, dT = inputs.random_state(nx, ny, 5, seed=nx + eq9, H_range=(0.9, 1.9), u_amp=0.3, f_base=W9)
+    s = lbm.Solver(p)
+    s.set_state(F - W9[:, None, None], G, H, dT)
+    runs = [twin(lbm, s, form) for form in (1, 2, 3)]
+    for r in runs:
+        r.step(4)
+        assert r.status() == 0
+    want = runs[0].save()
+    assert np.array_equal(want, runs[1].save()) and np.array_equal(want, runs[2].save())
