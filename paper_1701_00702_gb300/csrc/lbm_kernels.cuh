@@ -1293,12 +1293,14 @@ template <int M>   // MODE_F64
 __global__ void __launch_bounds__(64) conduction_step_lanes(const __grid_constant__ StepParams<double> P) {
     const int xr = blockIdx.x * 32 + (threadIdx.x >> 1), y = blockIdx.y;
     const bool metal = threadIdx.x & 1, live = xr < P.nx;
-    const int x = live ? xr : P.nx - 1;   // lanes beyond the grid go along and touch no history, which another warp writes
+    // a warp without a node returns: it would read the history that another warp writes, in no order
+    if (blockIdx.x * 32 + (threadIdx.x >> 5) * 16 >= P.nx) return;
+    const int x = live ? xr : P.nx - 1;   // lanes beyond the grid go along with their own warp and put nothing
     griddep_wait();
     const WallAt<double> w(P, x, y);
     const PullAt<M, 5, false> a(P, w.xs, w.ys);
     double* h = P.dT + (y * P.pitch + x);
-    const double dTp = live ? *h : 0.0;
+    const double dTp = *h;
     const int first = metal ? 5 : 0;   // the lattice's first plane
     double g[5], n[5];
 #pragma unroll
