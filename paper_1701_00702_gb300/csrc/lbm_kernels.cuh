@@ -1270,7 +1270,7 @@ __device__ __forceinline__ void prefetch_rows(const StepParams<typename ModeTrai
 // beyond L2 are bound by HBM (2048^2 100 us per step, 160 B per update at
 // 6.7 TB/s); smaller ones by the launch floor, one warp's chain and instruction
 // issue (256^2 2.41 us per step before the update was written in named
-// multiply-adds and single-instruction reciprocals and roots, 2.15 now).  FP64
+// multiply-adds and single-instruction reciprocals and roots, 2.21 now).  FP64
 // is bound by its two lanes per SM and clock: 252 FP64 operations per node took
 // 39.7 us per step at 256^2, 187 take 27.8 (in 64 x 1 blocks).
 template <int M, int QT, bool FLOW, bool PH, bool EV = false>
@@ -1379,7 +1379,7 @@ __global__ void __launch_bounds__(64) conduction_step_lanes(const __grid_constan
 // 104 against 84 us per step; two blocks of the other builds, which would spill
 // under the three-block cap).  Small grids are bound by the
 // launch floor and two dependency chains (64^2 FP32 1.315 us per step before
-// the update was written in named multiply-adds, 1.09 now; 256^2 2.05 / 1.83),
+// the update was written in named multiply-adds, 1.09 now; 256^2 2.05 and 1.82),
 // grids beyond L2 by instruction issue once their rows are prefetched (2048^2
 // 79.9 us per step before, 70.6 now; 49.5 at the copy bandwidth).  Two nodes
 // per thread in the tile, side by side or one above the other, were slower

@@ -209,10 +209,11 @@ inline int form_for(int mode, int qt, int flow, int solid_scheme, long long node
 // steps per launch; FP32: 256^2 2.40 / 2.02, 320^2 3.01 / 2.74,
 // 352^2 3.16 / 3.30, 384^2 3.39 / 4.26, 512^2 4.99 / 5.98, 768^2 11.1 / 12.2,
 // 896^2 19.1 / 16.9, 1024^2 26.5 / 21.9, 2048^2 99.7 / 81.2; FP16: 320^2
-// 3.14 / 2.91, 352^2 3.20 / 4.25); the current one takes FP32 256^2 2.26 / 1.82,
-// 320^2 2.75 / 2.43, 352^2 2.91 / 3.07, 768^2 9.3 / 10.8, 896^2 13.1 / 14.2, 1024^2
-// 21.6 / 18.1, 2048^2 99.4 / 70.5, FP16 320^2 2.91 / 2.62, 352^2 2.98 / 3.71.  Single steps (an odd remainder, batches)
-// keep the form above.
+// 3.14 / 2.91, 352^2 3.20 / 4.25).  The current one takes FP32 256^2 2.21 / 1.82,
+// 320^2 2.83 / 2.43, 352^2 2.94 / 3.10, 768^2 9.3 / 10.9, 896^2 13.1 / 14.2, 1024^2
+// 21.6 / 18.2, 2048^2 99.3 / 70.5, FP16 320^2 2.97 / 2.62, 352^2 2.98 / 3.72: by it the
+// FP32 line would lie some way above 896^2 (802,816 nodes).  Single steps (an odd
+// remainder, batches) keep the form above.
 constexpr long long kTwoStepSmallMaxNodes = 320 * 320;
 constexpr long long kTwoStepF32MinNodes = 3ll << 18;
 
@@ -265,7 +266,8 @@ inline bool pairs_of(const StepParams<typename ModeTraits<M>::R>& P, int qt, int
 // costs (GB300, us per step without / with.  FP32: 700^2, 80 MB, 8.60 / 8.69,
 // 740^2, 90 MB, 11.2 / 10.5, 768^2 11.7 / 9.3, 1024^2 in two steps per launch, 172
 // MB, 19.4 / 18.4, 1150^2, 217 MB, 24.1 / 25.9; with D2Q9 700^2, 112 MB, 16.2 /
-// 12.7, 900^2, 185 MB, 29.6 / 28.4, 1100^2, 276 MB, 42.5 / 45.6.  FP16: 900^2, 71
+// 12.7, 900^2, 185 MB, 29.6 / 28.4, 1100^2, 276 MB, 42.5 / 45.6, in two steps per
+// launch (forced) 700^2 16.3 / 15.2, 800^2, 146 MB, 20.2 / 18.2.  FP16: 900^2, 71
 // MB, 11.7 / 11.6, 1000^2, 88 MB, 14.7 / 13.7, 1200^2, 127 MB, 25.3 / 18.6.)  A
 // marked line is not prefetched: it would be dropped before its block reads it.
 // The runs of a batch share L2: grouped launches go by the nodes of all runs
@@ -447,7 +449,7 @@ cudaError_t launch_step(const StepParams<typename ModeTraits<M>::R>& P, int qt, 
 // the work of two tiles per SM counted at kT2Overlap: two resident blocks
 // overlap each other's L2 loads and barrier.  On 152 SMs: 128^2 takes H = 6
 // (128 tiles), 192^2 H = 10 (144), 256^2 H = 9 (296; fitted on FP32 times of
-// 2.04 us per step against 2.21 for H = 16 and one tile per SM, now 1.86).  One
+// 2.04 us per step against 2.21 for H = 16 and one tile per SM, now 1.82).  One
 // tile per SM takes up to kT2H rows, two up to kT2HTwo (what their registers
 // allow).  Other grids take H = kT2HMany = 12, measured fastest there (FP32:
 // three resident blocks of 13 warps per SM; 1024^2 and 2048^2 against H = 6, 8,
@@ -469,7 +471,9 @@ struct T2Shape {
 
 // Height from which two blocks of the first build don't fit an SM's registers
 // (FP32 64, with D2Q9 76; 16-bit 75, with D2Q9 94), so that two tiles per SM take
-// the build capped for them.
+// the build capped for them (D2Q9, us per step uncapped / capped: FP32 300^2 4.04 /
+// 3.30, 320^2 4.20 / 3.39, 334 x 303 4.39 / 3.74, FP16 300 x 260 3.91 / 3.21, 320^2 4.55 /
+// 3.75, BF16 334 x 303 4.68 / 4.08).
 inline int t2_two_from(int mode, int qt) { return mode == MODE_F32 ? (qt == 5 ? kT2HTwo + 1 : 12) : (qt == 5 ? 12 : 10); }
 
 // Rows of tiles per SM from which the FP32 D2Q5 tiles let the thermal lattices
@@ -477,7 +481,7 @@ inline int t2_two_from(int mode, int qt) { return mode == MODE_F32 ? (qt == 5 ? 
 // early wins, with a few warps the one whose chain is shorter (us per step,
 // flow / thermal lattices first: 64^2, 4 rows, 1.09 / 1.12, 128^2, 6, 1.22 / 1.25,
 // 150^2, 7, and 200^2, 10, the same, 256 x 242, 15, 1.89 / 1.86, 256^2, 18, 1.86 /
-// 1.83, 300^2, 24, 2.41 / 2.39, 320^2, 26, 2.47 / 2.43; with Eq. 9 256^2 1.89 /
+// 1.82, 300^2, 24, 2.41 / 2.38, 320^2, 26, 2.47 / 2.43; with Eq. 9 256^2 1.89 /
 // 1.91, not taken).
 constexpr int kT2ThermalRows = 15;
 
