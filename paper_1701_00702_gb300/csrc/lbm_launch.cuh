@@ -163,15 +163,19 @@ inline cudaError_t dispatch_step(int qt, int flow, int ph, Fn&& fn) {
 // each scheduler has only a few, 64 cycles an operation each (128 x 1 / 64 x 1:
 // 150^2 15.9 / 12.6, 256^2 30.1 / 28.3).  Others: 64 x 2 up to 40,000 nodes
 // (128^2 in one step per launch 1.63, 128 x 1 1.73); 128 x 1 from there; where
-// the grid takes more than a wave of blocks, the width of 128, 64 and 32 that
+// the grid takes more than a wave of blocks (131,072 nodes, or columns so idle
+// that its blocks of 128 x 1 are more than 8 per SM), the width of 128, 64 and 32 that
 // leaves the fewest columns idle (128 x 1 / 64 x 1 / 32 x 2, FP32: 400 x 390
-// 4.11 / 3.62 / 3.61, 777 x 501 7.10 / 7.03 / 6.80, 512^2 5.00 all).
+// 4.11 / 3.62 / 3.61, 777 x 501 7.10 / 7.03 / 6.80, 512^2 5.00 all; 128 x 1 / chosen,
+// D2Q9 137 x 689 4.76 / 3.37, 290 x 420 4.30 / 3.72, D2Q5 150 x 800 3.95 / 3.02).
+constexpr int kNumSMs = 152;
+
 inline dim3 step_block(int mode, int nx, int ny) {
     const long long nodes = (long long)nx * ny;
     if (mode == MODE_F64) return dim3(64, 1);
     if (nodes <= 40000) return dim3(64, 2);
-    if (nodes <= 1ll << 17) return dim3(128, 1);
     auto cover = [&](int w) { return (nx + w - 1) / w * w; };
+    if (nodes <= 1ll << 17 && cover(128) / 128 * (long long)ny <= 8 * kNumSMs) return dim3(128, 1);
     if (cover(128) <= cover(64)) return dim3(128, 1);
     return cover(64) <= cover(32) ? dim3(64, 1) : dim3(32, 2);
 }
@@ -239,7 +243,6 @@ inline bool two_steps_for(int mode, int qt, int flow, long long nodes, int form)
 //     360 6.22 / 6.27, 1201 x 300 6.63 / 6.35, 777 x 501 7.24 / 7.15, 865 x 801 11.9 / 10.7).
 // In FP32 one node per thread is faster (512^2 4.83 / 5.23).
 constexpr long long kPairPlainMinNodes = 1ll << 17, kPairOddMinNodes = 360000;
-constexpr int kNumSMs = 152;
 
 inline bool plain_pairs(int nx, int ny) {
     const long long nodes = (long long)nx * ny;

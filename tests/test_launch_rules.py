@@ -104,3 +104,15 @@ def test_a_chosen_block_shape_is_the_one_launched(rules, block):
         assert rules(nx, ny, prec, form=form, flow=flow, block=block) == (-(-nx // bx), -(-ny // by), bx, by)
     for nx, ny, form in ((2048, 2048, 0), (256, 256, 2)):
         assert takes_pairs(rules(nx, ny, 2, form=form, block=block), nx)
+
+
+@pytest.mark.parametrize("shape,block", [
+    ((64, 64), (64, 2)), ((200, 200), (64, 2)), ((256, 256), (128, 1)), ((360, 360), (128, 1)), ((160, 300), (128, 1)),
+    ((137, 689), (32, 2)), ((290, 420), (64, 1)), ((190, 660), (64, 1)), ((24, 2000), (32, 2)), ((400, 390), (32, 2)),
+    ((512, 512), (128, 1)),
+])
+def test_blocks_leave_few_columns_idle_beyond_a_wave(rules, shape, block):
+    """Where blocks of 128 x 1 are more than a wave, by nodes or by idle columns,
+    the widest of 128, 64 and 32 that leaves the fewest columns idle."""
+    for prec, qt in ((1, 5), (1, 9), (2, 9)):
+        assert rules(*shape, prec, form=1, qt=qt)[2:] == block
