@@ -97,16 +97,16 @@ def stored_bytes_per_update(qt: int, flow: int, precision: int) -> int:
 # taken for the kernel sources whose code hash is given; the bench reports
 # them only while the sources still hash to that value.
 ROOFLINE_TRAFFIC = {
-    "bytes_per_launch": 352023040 + 297974784,
-    "kernel_sources_sha256_16": "32f3001db8f058e8",
+    "bytes_per_launch": 352021248 + 298989568,
+    "kernel_sources_sha256_16": "1e78d175a5c7ef7d",
     "gpu__dram_throughput_pct": 83.8,
     "captured": "2026-12-05, ncu --set full --clock-control none, one launch after two "
                 "(profiles/fused_step_cavity2048_fp32.md)",
 }
 TWO_STEP_TRAFFIC = {
-    "bytes_per_launch": 352225792 + 307002368,
-    "kernel_sources_sha256_16": "32f3001db8f058e8",
-    "gpu__dram_throughput_pct": 57.4,
+    "bytes_per_launch": 352233728 + 306928896,
+    "kernel_sources_sha256_16": "1e78d175a5c7ef7d",
+    "gpu__dram_throughput_pct": 57.8,
     "captured": "2026-12-05, ncu --set full --clock-control none, one launch after two "
                 "(profiles/fused_step2_cavity2048_fp32.md)",
 }

@@ -191,8 +191,9 @@ int lbm_create_ex(const lbm_params* p, void* cuda_stream, lbm_alloc_fn alloc,
  * launched as a programmatic dependent of the previous one in the stream.
  * The step kernel runs one node per thread (FP64: blocks of 64 x 1 threads;
  * the others: 64 x 2 on grids of up to 40,000 nodes, 128 x 1 on larger ones,
- * and beyond 131,072 nodes the one of 128 x 1, 64 x 1 and 32 x 2 that leaves
- * the fewest columns idle), two nodes per thread, or two steps per launch (see
+ * and beyond 131,072 nodes, or 1,216 blocks of 128 x 1, the one of 128 x 1, 64 x 1
+ * and 32 x 2 that leaves the fewest columns idle; grids of 65,536 rows take at
+ * least two rows per block), two nodes per thread, or two steps per launch (see
  * lbm_set_step_form); FP64 runs without flow, with D2Q5 lattices and constant
  * conductivity, take two threads per node on grids of up to 9,728 nodes. */
 int lbm_step(lbm_handle* h, int64_t nsteps);

@@ -1272,7 +1272,7 @@ __device__ __forceinline__ void prefetch_rows(const StepParams<typename ModeTrai
 // issue (256^2 2.41 us per step before the update was written in named
 // multiply-adds and single-instruction reciprocals and roots, 2.21 now).  FP64
 // is bound by its two lanes per SM and clock: 252 FP64 operations per node took
-// 39.7 us per step at 256^2, 187 take 27.8 (in 64 x 1 blocks).
+// 39.7 us per step at 256^2, 187 take 27.6 (in 64 x 1 blocks).
 template <int M, int QT, bool FLOW, bool PH, bool EV = false>
 __global__ void __launch_bounds__(256, (kMinBlocks<M, QT, FLOW>)) fused_step(const __grid_constant__ StepParams<typename ModeTraits<M>::R> P) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
